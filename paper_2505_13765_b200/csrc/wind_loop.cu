@@ -72,7 +72,8 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
     __shared__ unsigned long long win_key[FULL ? kMaxWindow : 1];
     __shared__ int s_red[8];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
+    const uint32_t el = lane == 0;             // the lane that executes the CTA-level instructions of an issuing warp
     const int cta = blockIdx.x, G = gridDim.x;
     // a length outside [0, T] (found by the init kernel, which ran before this launch): the status is set, no CTA starts
     if (p.ctrl->bad_input) return;
@@ -224,7 +225,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
 
     // ----- TMA issuer (warp 0, lane 0) -----
     auto acquire = [&](uint32_t sb) -> uint8_t* {   // next free stage, nullptr when giving up
-        if (!mbar_wait(&empty_bar[cur], (pe_bits >> cur) & 1u, &s_abort)) return nullptr;
+        if (!mbar_wait_warp(&empty_bar[cur], (pe_bits >> cur) & 1u, &s_abort)) return nullptr;
         pe_bits ^= 1u << cur;
         return ring + (size_t)cur * sb;
     };
@@ -241,10 +242,10 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                     uint8_t* a_dst = acquire(sb_lp);
                     if (!a_dst) return false;
                     uint8_t* b_dst = a_dst + LOOP_A_BYTES;
-                    mbar_expect_tx(&full_bar[cur], LOOP_A_BYTES + b_bytes);
-                    tma_load_2d(a_dst, ma, kb * BK, mt * 128, &full_bar[cur]);
+                    mbar_expect_tx(&full_bar[cur], LOOP_A_BYTES + b_bytes, el);
+                    tma_load_2d(a_dst, ma, kb * BK, mt * 128, &full_bar[cur], el);
                     for (int g = 0; g < 4; ++g)
-                        tma_load_2d(b_dst + (size_t)g * p.slots * 128, mb, kb * BK, g * p.P + ug * p.ul, &full_bar[cur]);
+                        tma_load_2d(b_dst + (size_t)g * p.slots * 128, mb, kb * BK, g * p.P + ug * p.ul, &full_bar[cur], el);
                     cur = cur + 1 == S_lp ? 0 : cur + 1;
                 }
             }
@@ -253,13 +254,13 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
     };
     // ----- MMA issuer (warp 1, lane 0) -----
     auto consume = [&]() -> bool {
-        if (!mbar_wait(&full_bar[cur], (cf_bits >> cur) & 1u, &s_abort)) return false;
+        if (!mbar_wait_warp(&full_bar[cur], (cf_bits >> cur) & 1u, &s_abort)) return false;
         cf_bits ^= 1u << cur;
         tc_fence_after();
         return true;
     };
     auto begin_acc = [&](int k) -> bool {   // the epilogue has drained the previous use of accumulator k
-        if (!mbar_wait(&acc_empty[k], (acc_n[k] & 1u) ^ 1u, &s_abort)) return false;
+        if (!mbar_wait_warp(&acc_empty[k], (acc_n[k] & 1u) ^ 1u, &s_abort)) return false;
         tc_fence_after();
         return true;
     };
@@ -275,11 +276,11 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                 const uint64_t bdesc = smem_desc_sw128(a_addr + LOOP_A_BYTES);
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tm_l, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
-                tc_commit(&empty_bar[cur]);
+                    tc_mma_bf16(tm_l, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
+                tc_commit(&empty_bar[cur], el);
                 cur = cur + 1 == S_lp ? 0 : cur + 1;
             }
-            tc_commit(&acc_full[1]);
+            tc_commit(&acc_full[1], el);
             ++acc_n[1];
         }
         return true;
@@ -491,8 +492,8 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
         cur = 0;
         uint8_t* dst = acquire(0);
         if (!dst) return false;
-        mbar_expect_tx(&full_bar[0], bytes);
-        tma_load_3d(dst, map, 0, row0, 0, &full_bar[0]);
+        mbar_expect_tx(&full_bar[0], bytes, el);
+        tma_load_3d(dst, map, 0, row0, 0, &full_bar[0], el);
         return true;
     };
     // One issuing thread's share of a GEMM: K blocks [kb_lo, kb_hi) into the accumulator at tm_d.  Two threads call
@@ -500,7 +501,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
     // separate accumulator copies that the epilogue adds; an empty range only takes part in the commits.
     auto mma_part = [&](int k_acc, uint32_t tm_d, int n_tile, int kb_lo, int kb_hi, bool a_tmem) -> bool {
         const uint32_t idesc = idesc_bf16(a_tmem ? 128 : 64, n_tile);
-        if (!a_tmem && !mbar_wait(&stat_bar, 0, &s_abort)) return false;
+        if (!a_tmem && !mbar_wait_warp(&stat_bar, 0, &s_abort)) return false;
         if (!begin_acc(k_acc)) return false;
         cur = 0;
         if (!consume()) return false;
@@ -512,16 +513,16 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
                     tc_mma_bf16_ts(tm_d, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
-                                   kb != kb_lo || k != 0);
+                                   kb != kb_lo || k != 0, el);
             } else {
                 const uint64_t adesc = smem_desc_sw128(smem_u32(stat + (size_t)kb * RES_A_BYTES));
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0);
+                    tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0, el);
             }
         }
-        tc_commit(&empty_bar[0]);
-        tc_commit(&acc_full[k_acc]);
+        tc_commit(&empty_bar[0], el);
+        tc_commit(&acc_full[k_acc], el);
         ++acc_n[k_acc];
         return true;
     };
@@ -997,13 +998,13 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
     // next control step) and, with two layers, layer 1's recurrent term (stored by store_res_h1)
     auto early_res = [&]() {
         if (warp == 0) {
-            if (lane == 0 && (res_l || res_h1)) {
+            if (res_l || res_h1) {
                 fence_proxy_async_all();
                 if (produce_one(res_l ? &M.hb_l3[pin] : &M.hb_l3_1[pin], r_ql * p.nl, (uint32_t)p.nl * (uint32_t)p.P * 2u))
                     mma_part(1, tm_l, p.nl, p.kb_p, p.kb_p, false);   // one accumulator: warp 1 issues all of it
             }
         } else if (warp == 1) {
-            if (lane == 0 && (res_l || res_h1)) mma_part(1, tm_l, p.nl, 0, p.kb_p, false);
+            if (res_l || res_h1) mma_part(1, tm_l, p.nl, 0, p.kb_p, false);
         } else if (res_h1) {
             store_res_h1();
         }
@@ -1019,9 +1020,9 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
         early_res();
     } else if (early) {
         if (warp == 0) {
-            if (lane == 0) { fence_proxy_async_all(); cur = 0; produce_L(0); }
+            fence_proxy_async_all(); cur = 0; produce_L(0);
         } else if (warp == 1) {
-            if (lane == 0) { cur = 0; mma_L(0); }
+            cur = 0; mma_L(0);
         }
     }
 
@@ -1041,13 +1042,13 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
             if (p.L == 2) {
                 // layer 1: W_ih[1] . (new layer-0 state) on the x1 CTAs, then their cell update
                 if (warp == 0) {
-                    if (lane == 0 && res_x1) {
+                    if (res_x1) {
                         fence_proxy_async_all();
                         if (produce_one(&M.hb_l3[pin ^ 1], r_ql * p.nl, (uint32_t)p.nl * (uint32_t)p.P * 2u))
                             mma_part(1, tm_l, p.nl, p.kb_p, p.kb_p, false);
                     }
                 } else if (warp == 1) {
-                    if (lane == 0 && res_x1) mma_part(1, tm_l, p.nl, 0, p.kb_p, false);
+                    if (res_x1) mma_part(1, tm_l, p.nl, 0, p.kb_p, false);
                 } else if (res_x1) {
                     epilogue_res_L(1, false);
                 }
@@ -1057,9 +1058,9 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
         for (int l = 0; l < p.L && !RES; ++l) {
             const bool gemm_here = l > 0 || !early;
             if (warp == 0) {
-                if (lane == 0 && gemm_here) { fence_proxy_async_all(); cur = 0; produce_L(l); }
+                if (gemm_here) { fence_proxy_async_all(); cur = 0; produce_L(l); }
             } else if (warp == 1) {
-                if (lane == 0 && gemm_here) { cur = 0; mma_L(l); }
+                if (gemm_here) { cur = 0; mma_L(l); }
             } else {
                 if (e == 0) if constexpr (FULL) trace_event(p, 2, tr_n, step, TR_L, EV_START);
                 epilogue_L(l);
@@ -1073,9 +1074,9 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                 early_res();
             } else if (early) {
                 if (warp == 0) {
-                    if (lane == 0) { fence_proxy_async_all(); cur = 0; produce_L(0); }
+                    fence_proxy_async_all(); cur = 0; produce_L(0);
                 } else if (warp == 1) {
-                    if (lane == 0) { cur = 0; mma_L(0); }
+                    cur = 0; mma_L(0);
                 }
             }
             ++step;
@@ -1095,13 +1096,13 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
             const int i0 = p.p_items <= G ? G - 1 - cta : cta;   // projection items start at the far end of the grid
             if constexpr (RES) {
                 if (warp == 0) {
-                    if (lane == 0 && res_p) {
+                    if (res_p) {
                         fence_proxy_async_all();
                         if (produce_one(&M.hb_p3[pin], r_qp * p.np, (uint32_t)p.np * (uint32_t)p.P * 2u))
                             mma_part(2, tm_p + (uint32_t)p.np, p.np, p.kb_p / 2, p.kb_p, false);
                     }
                 } else if (warp == 1) {
-                    if (lane == 0 && res_p) mma_part(2, tm_p, p.np, 0, p.kb_p / 2, false);
+                    if (res_p) mma_part(2, tm_p, p.np, 0, p.kb_p / 2, false);
                 } else {
                     if (e == 0) if constexpr (FULL) trace_event(p, 2, tr_n, step, TR_P, EV_START);
                     // rows still decoding, plus one while utterances wait for a row
@@ -1116,7 +1117,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                 }
                 early_res();
             } else if (warp == 0) {
-                if (lane == 0) {
+                {
                     fence_proxy_async_all();
                     cur = 0;
                     bool ok = true;
@@ -1125,16 +1126,16 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                         for (int kb = 0; kb < p.kb_p; ++kb) {
                             uint8_t* a_dst = acquire(sb_lp);
                             if (!a_dst) { ok = false; break; }
-                            mbar_expect_tx(&full_bar[cur], LOOP_A_BYTES + b_bytes);
-                            tma_load_2d(a_dst, &M.hb[pin][p.L - 1], kb * BK, mt * 128, &full_bar[cur]);
-                            tma_load_2d(a_dst + LOOP_A_BYTES, &M.w_pred, kb * BK, hg * p.np, &full_bar[cur]);
+                            mbar_expect_tx(&full_bar[cur], LOOP_A_BYTES + b_bytes, el);
+                            tma_load_2d(a_dst, &M.hb[pin][p.L - 1], kb * BK, mt * 128, &full_bar[cur], el);
+                            tma_load_2d(a_dst + LOOP_A_BYTES, &M.w_pred, kb * BK, hg * p.np, &full_bar[cur], el);
                             cur = cur + 1 == S_lp ? 0 : cur + 1;
                         }
                     }
                     if (ok && early) produce_L(0);
                 }
             } else if (warp == 1) {
-                if (lane == 0) {
+                {
                     const uint32_t idesc = idesc_bf16(128, n_tile);
                     cur = 0;
                     bool ok = true;
@@ -1147,11 +1148,11 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                             const uint64_t bdesc = smem_desc_sw128(a_addr + LOOP_A_BYTES);
 #pragma unroll
                             for (int k = 0; k < BK / 16; ++k)
-                                tc_mma_bf16(tm_p, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
-                            tc_commit(&empty_bar[cur]);
+                                tc_mma_bf16(tm_p, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
+                            tc_commit(&empty_bar[cur], el);
                             cur = cur + 1 == S_lp ? 0 : cur + 1;
                         }
-                        if (ok) { tc_commit(&acc_full[2]); ++acc_n[2]; }
+                        if (ok) { tc_commit(&acc_full[2], el); ++acc_n[2]; }
                     }
                     if (ok && early) mma_L(0);
                 }
@@ -1357,76 +1358,76 @@ joint_only_entry:
             unsigned long long* keys_cur = p.keys2 + (size_t)(step & 1) * p.rows_pad;
             if (RES && warp < 2) {
                 // one box for the whole z tile, then every MMA back to back (A = W_out tile in tensor memory)
-                if (lane == 0 && has_j) {
+                if (has_j) {
                     if (warp == 0) {
                         fence_proxy_async_all();
-                        if constexpr (FULL) trace_event(p, 0, tr_n, step, TR_J, EV_FIRST_ISSUE);
+                        if constexpr (FULL) if (el) trace_event(p, 0, tr_n, step, TR_J, EV_FIRST_ISSUE);
                         for (int rg = j_first; rg < p.rg_count; rg += p.rg_stride) {
                             const bool ok = produce_one(&M.z3, rg * n_tile, (uint32_t)n_tile * (uint32_t)p.H * 2u);
-                            if constexpr (FULL) trace_event(p, 0, tr_n, step, TR_J, EV_LAST_ISSUE);
+                            if constexpr (FULL) if (el) trace_event(p, 0, tr_n, step, TR_J, EV_LAST_ISSUE);
                             if (!ok || !mma_part(0, tm_j + (uint32_t)n_tile, n_tile, p.kb_h / 2, p.kb_h, true)) break;
                         }
-                        if constexpr (FULL) trace_event(p, 0, tr_n, step, TR_J, EV_COMMIT);
+                        if constexpr (FULL) if (el) trace_event(p, 0, tr_n, step, TR_J, EV_COMMIT);
                     } else {
                         for (int rg = j_first; rg < p.rg_count; rg += p.rg_stride)
                             if (!mma_part(0, tm_j, n_tile, 0, p.kb_h / 2, true)) break;
-                        if constexpr (FULL) trace_event(p, 1, tr_n, step, TR_J, EV_COMMIT);
+                        if constexpr (FULL) if (el) trace_event(p, 1, tr_n, step, TR_J, EV_COMMIT);
                     }
                 }
             } else if (!RES && warp == 0) {
-                if (lane == 0) {
+                {
                     fence_proxy_async_all();
                     cur = 0;
                     bool ok = true;
-                    if constexpr (FULL) trace_event(p, 0, tr_n, step, TR_J, EV_FIRST_ISSUE);
+                    if constexpr (FULL) if (el) trace_event(p, 0, tr_n, step, TR_J, EV_FIRST_ISSUE);
                     for (int i = cta; i < p.j_items && ok; i += G) {
                         const int rg = i / p.vt_count, vt = i - rg * p.vt_count;
                         for (int kb = 0; kb < p.kb_h; ++kb) {
                             uint8_t* dst = acquire(sb_j);
                             if (!dst) { ok = false; break; }
                             if (p.j_mode != J_STREAM) {
-                                mbar_expect_tx(&full_bar[cur], z_bytes);
-                                tma_load_2d(dst, &M.z, kb * BK, rg * n_tile, &full_bar[cur]);
+                                mbar_expect_tx(&full_bar[cur], z_bytes, el);
+                                tma_load_2d(dst, &M.z, kb * BK, rg * n_tile, &full_bar[cur], el);
                             } else {
-                                mbar_expect_tx(&full_bar[cur], LOOP_A_BYTES + z_bytes);
-                                tma_load_2d(dst, &M.w_out, kb * BK, vt * 128, &full_bar[cur]);
-                                tma_load_2d(dst + LOOP_A_BYTES, &M.z, kb * BK, rg * n_tile, &full_bar[cur]);
+                                mbar_expect_tx(&full_bar[cur], LOOP_A_BYTES + z_bytes, el);
+                                tma_load_2d(dst, &M.w_out, kb * BK, vt * 128, &full_bar[cur], el);
+                                tma_load_2d(dst + LOOP_A_BYTES, &M.z, kb * BK, rg * n_tile, &full_bar[cur], el);
                             }
                             cur = cur + 1 == S_j ? 0 : cur + 1;
                         }
                     }
-                    if constexpr (FULL) trace_event(p, 0, tr_n, step, TR_J, EV_LAST_ISSUE);
+                    if constexpr (FULL) if (el) trace_event(p, 0, tr_n, step, TR_J, EV_LAST_ISSUE);
                 }
             } else if (!RES && warp == 1) {
-                if (lane == 0) {
+                {
                     const uint32_t idesc = idesc_bf16(128, n_tile);
                     cur = 0;
                     bool ok = true;
-                    if (p.j_mode == J_SMEM && has_j) ok = mbar_wait(&stat_bar, 0, &s_abort);
+                    if (p.j_mode == J_SMEM && has_j) ok = mbar_wait_warp(&stat_bar, 0, &s_abort);
                     for (int i = cta; i < p.j_items && ok; i += G) {
                         if (!begin_acc(0)) { ok = false; break; }
                         for (int kb = 0; kb < p.kb_h; ++kb) {
                             if (!consume()) { ok = false; break; }
-                            if (kb == 0) if constexpr (FULL) trace_event(p, 1, tr_n, step, TR_J, EV_FIRST_DATA);
+                            if (kb == 0) if constexpr (FULL) if (el) trace_event(p, 1, tr_n, step, TR_J, EV_FIRST_DATA);
                             const uint32_t st_addr = smem_u32(ring + (size_t)cur * sb_j);
                             if (p.j_mode == J_TMEM) {
                                 const uint64_t bdesc = smem_desc_sw128(st_addr);
 #pragma unroll
                                 for (int k = 0; k < BK / 16; ++k)
                                     tc_mma_bf16_ts(tm_j, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
-                                                   (kb | k) != 0);
+                                                   (kb | k) != 0, el);
                             } else {
                                 const uint64_t adesc =
                                     smem_desc_sw128(p.j_mode == J_SMEM ? smem_u32(stat + (size_t)kb * LOOP_A_BYTES) : st_addr);
                                 const uint64_t bdesc = smem_desc_sw128(p.j_mode == J_SMEM ? st_addr : st_addr + LOOP_A_BYTES);
 #pragma unroll
                                 for (int k = 0; k < BK / 16; ++k)
-                                    tc_mma_bf16(tm_j, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
+                                    tc_mma_bf16(tm_j, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
                             }
-                            tc_commit(&empty_bar[cur]);
+                            tc_commit(&empty_bar[cur], el);
                             cur = cur + 1 == S_j ? 0 : cur + 1;
                         }
-                        if (ok) { tc_commit(&acc_full[0]); ++acc_n[0]; if constexpr (FULL) trace_event(p, 1, tr_n, step, TR_J, EV_COMMIT); }
+                        if (ok) { tc_commit(&acc_full[0], el); ++acc_n[0]; if constexpr (FULL) if (el) trace_event(p, 1, tr_n, step, TR_J, EV_COMMIT); }
                     }
                 }
             } else {

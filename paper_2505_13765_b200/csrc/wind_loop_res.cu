@@ -75,7 +75,8 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
     __shared__ unsigned long long win_key[FULL ? kMaxWindow : 1];
     __shared__ int s_jt[kGroupUtts], s_jrem[kGroupUtts];       // operand build: frame and frames left of the group's utterances
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
+    const uint32_t el = lane == 0;             // the lane that executes the CTA-level instructions of an issuing warp
     const int cta = blockIdx.x, G = gridDim.x;
     // a length outside [0, T] (found by the init kernel, which ran before this launch): the status is set, no CTA starts
     if (p.ctrl->bad_input) return;
@@ -277,6 +278,13 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
         return *vabort == 0;
     };
 
+    // the waits for a whole issuing warp, with one answer for all its lanes (lane 0 polls a counter)
+    auto mwait_warp = [&](uint64_t* bar, uint32_t parity, int site) -> bool { return __all_sync(0xffffffffu, mwait(bar, parity, site)); };
+    auto flag_wait_warp = [&](const uint32_t* ptr, uint32_t target, int site) -> bool {
+        bool ok = true;
+        if (el) ok = flag_wait(ptr, target, site);
+        return __all_sync(0xffffffffu, ok);
+    };
     // ----- one issuing thread's share of a GEMM: K blocks [kb_lo, kb_hi) into the accumulator at tm_d -----
     // Two threads call this for every GEMM (warp 1 and warp 0), with disjoint K ranges and separate accumulator
     // copies that the epilogue adds; an empty range only takes part in the commits.  sidx / use: which operand
@@ -284,10 +292,10 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
     auto mma_part = [&](int k_acc, uint32_t tm_d, int n_tile, int kb_lo, int kb_hi, bool a_tmem, int sidx, uint32_t use,
                         const uint8_t* b_smem) -> bool {
         const uint32_t idesc = idesc_bf16(a_tmem ? 128 : 64, n_tile);
-        if (!a_tmem && !mwait(&stat_bar, 0, 10)) return false;
-        if (!mwait(&acc_empty[k_acc], (acc_n[k_acc] & 1u) ^ 1u, 11 + k_acc)) return false;   // the epilogue has drained it
+        if (!a_tmem && !mwait_warp(&stat_bar, 0, 10)) return false;
+        if (!mwait_warp(&acc_empty[k_acc], (acc_n[k_acc] & 1u) ^ 1u, 11 + k_acc)) return false;   // the epilogue has drained it
         tc_fence_after();
-        if (!mwait(&full_bar[sidx], use & 1u, 14 + sidx)) return false;
+        if (!mwait_warp(&full_bar[sidx], use & 1u, 14 + sidx)) return false;
         tc_fence_after();
         const uint32_t b_addr = smem_u32(b_smem);
         const uint32_t b_block = (uint32_t)n_tile * BK * 2;
@@ -297,26 +305,26 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
                     tc_mma_bf16_ts(tm_d, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
-                                   kb != kb_lo || k != 0);
+                                   kb != kb_lo || k != 0, el);
             } else {
                 const uint64_t adesc = smem_desc_sw128(smem_u32(stat + (size_t)kb * RES_A_BYTES));
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0);
+                    tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0, el);
             }
         }
-        tc_commit(&empty_bar[sidx]);
-        tc_commit(&acc_full[k_acc]);
+        tc_commit(&empty_bar[sidx], el);
+        tc_commit(&acc_full[k_acc], el);
         ++acc_n[k_acc];
         return true;
     };
     // the state box of this step: ONE three-dimensional TMA box (64 columns, rows, all K blocks), once the MMAs
     // that read the buffer last have completed
     auto produce_box = [&](const CUtensorMap* map, int row0, uint32_t bytes) -> bool {
-        if (use0 > 0 && !mwait(&empty_bar[0], (use0 - 1) & 1u, 16)) return false;
-        if (z_sh && use1 > 0 && !mwait(&empty_bar[1], (use1 - 1) & 1u, 17)) return false;
-        mbar_expect_tx(&full_bar[0], bytes);
-        tma_load_3d(buf0, map, 0, row0, 0, &full_bar[0]);
+        if (use0 > 0 && !mwait_warp(&empty_bar[0], (use0 - 1) & 1u, 16)) return false;
+        if (z_sh && use1 > 0 && !mwait_warp(&empty_bar[1], (use1 - 1) & 1u, 17)) return false;
+        mbar_expect_tx(&full_bar[0], bytes, el);
+        tma_load_3d(buf0, map, 0, row0, 0, &full_bar[0], el);
         return true;
     };
 
@@ -732,19 +740,19 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
     auto early_res = [&]() {
         const bool mine = res_l || res_h1;
         if (warp == 0) {
-            if (lane == 0 && mine) {
+            if (mine) {
                 // the state of this CTA's utterance group as the last decoder-update slot left it
-                const bool ok = res_l ? flag_wait(f_h0 + r_ql, n_l * arr_h0(r_ql), 24) : flag_wait(f_h1 + r_ql, n_l * (uint32_t)p.ut_count, 25);
-                mark(TR_P, MK_E_FLAG);
+                const bool ok = res_l ? flag_wait_warp(f_h0 + r_ql, n_l * arr_h0(r_ql), 24) : flag_wait_warp(f_h1 + r_ql, n_l * (uint32_t)p.ut_count, 25);
+                if (el) mark(TR_P, MK_E_FLAG);
                 if (ok) {
                     fence_proxy_async_all();
                     if (produce_box(res_l ? &M.hb_l3[pin] : &M.hb_l3_1[pin], r_ql * p.nl, (uint32_t)p.nl * (uint32_t)p.P * 2u))
                         mma_part(1, tm_l, p.nl, p.kb_p, p.kb_p, false, 0, use0, buf0);   // one accumulator: warp 1 issues all of it
                 }
-                mark(TR_P, MK_E_ISSUED);
+                if (el) mark(TR_P, MK_E_ISSUED);
             }
         } else if (warp == 1) {
-            if (lane == 0 && mine) mma_part(1, tm_l, p.nl, 0, p.kb_p, false, 0, use0, buf0);
+            if (mine) mma_part(1, tm_l, p.nl, 0, p.kb_p, false, 0, use0, buf0);
         } else if (res_h1) {
             store_res_h1();
         }
@@ -954,15 +962,15 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
         if (p.L == 2) {
             // layer 1: W_ih[1] . (new layer-0 state) on the x1 CTAs, then their cell update
             if (warp == 0) {
-                if (lane == 0 && res_x1) {
-                    if (flag_wait(f_h0 + r_ql, n_l * arr_h0(r_ql), 26)) {
+                if (res_x1) {
+                    if (flag_wait_warp(f_h0 + r_ql, n_l * arr_h0(r_ql), 26)) {
                         fence_proxy_async_all();
                         if (produce_box(&M.hb_l3[pin ^ 1], r_ql * p.nl, (uint32_t)p.nl * (uint32_t)p.P * 2u))
                             mma_part(1, tm_l, p.nl, p.kb_p, p.kb_p, false, 0, use0, buf0);
                     }
                 }
             } else if (warp == 1) {
-                if (lane == 0 && res_x1) mma_part(1, tm_l, p.nl, 0, p.kb_p, false, 0, use0, buf0);
+                if (res_x1) mma_part(1, tm_l, p.nl, 0, p.kb_p, false, 0, use0, buf0);
             } else {
                 if (res_x1) epilogue_res_L(1, false);
                 if (e == 0) slot_done(TR_L);
@@ -985,24 +993,24 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
         // projection slot: pred_proj for every utterance; behind it, layer 0's GEMM of the next step
         // =====================================================================================
         if (warp == 0) {
-            if (lane == 0 && res_p) {
+            if (res_p) {
                 // the top layer's state of this CTA's utterances: every utterance group they belong to has arrived
                 const uint32_t* f = p.L == 2 ? f_h1 : f_h0;
                 const int b_lo = r_qp * p.np, b_hi = min(b_lo + p.np, p.B);
                 bool ok = true;
                 if (b_hi > b_lo)
                     for (int g = b_lo / p.nl; ok && g <= (b_hi - 1) / p.nl; ++g)
-                        ok = flag_wait(f + g, n_l * (p.L == 2 ? (uint32_t)p.ut_count : arr_h0(g)), 27);
-                mark(TR_P, MK_P_FLAG);
+                        ok = flag_wait_warp(f + g, n_l * (p.L == 2 ? (uint32_t)p.ut_count : arr_h0(g)), 27);
+                if (el) mark(TR_P, MK_P_FLAG);
                 if (ok) {
                     fence_proxy_async_all();
-                    if constexpr (FULL) trace_event(p, 0, tr_n, step, TR_P, EV_FIRST_ISSUE);
+                    if constexpr (FULL) if (el) trace_event(p, 0, tr_n, step, TR_P, EV_FIRST_ISSUE);
                     if (produce_box(&M.hb_p3[pin], r_qp * p.np, (uint32_t)p.np * (uint32_t)p.P * 2u))
                         mma_part(2, tm_p + (uint32_t)p.np, p.np, p.kb_p / 2, p.kb_p, false, 0, use0, buf0);
                 }
             }
         } else if (warp == 1) {
-            if (lane == 0 && res_p) mma_part(2, tm_p, p.np, 0, p.kb_p / 2, false, 0, use0, buf0);
+            if (res_p) mma_part(2, tm_p, p.np, 0, p.kb_p / 2, false, 0, use0, buf0);
         } else {
             if (e == 0) if constexpr (FULL) trace_event(p, 2, tr_n, step, TR_P, EV_START);
             if (res_p) epilogue_res_P(n_p + 1u);
@@ -1029,11 +1037,11 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
             const int32_t* t_cur = p.t2 + (size_t)(step & 1) * p.B;
             for (int rg = j_first; rg < p.rg_count; rg += p.rg_stride) {
                 if (warp < 2) {
-                    if (lane == 0) {
-                        if constexpr (FULL) trace_event(p, warp, tr_n, step, TR_J, EV_FIRST_ISSUE);
+                    {
+                        if constexpr (FULL) if (el) trace_event(p, warp, tr_n, step, TR_J, EV_FIRST_ISSUE);
                         if (warp == 0) mma_part(0, tm_j + (uint32_t)n_tile, n_tile, p.kb_h / 2, p.kb_h, true, 1, use1, zbuf);
                         else mma_part(0, tm_j, n_tile, 0, p.kb_h / 2, true, 1, use1, zbuf);
-                        if constexpr (FULL) trace_event(p, warp, tr_n, step, TR_J, EV_COMMIT);
+                        if constexpr (FULL) if (el) trace_event(p, warp, tr_n, step, TR_J, EV_COMMIT);
                     }
                 } else {
                     if (e == 0) if constexpr (FULL) trace_event(p, 2, tr_n, step, TR_J, EV_START);

@@ -113,7 +113,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     __shared__ int s_valid[BM];
 
     constexpr int GEMM_BN = GemmShape<MODE>::BN, GEMM_STAGES = GemmShape<MODE>::STAGES;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
+    const uint32_t el = lane == 0;   // the lane that executes the CTA-level instructions of an issuing warp
     constexpr uint32_t b_stage_bytes = GEMM_BN * BK * 2;
     constexpr uint32_t stage_bytes = A_STAGE_BYTES + b_stage_bytes;
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
@@ -152,24 +153,24 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const uint32_t tmem_base = tmem_slot;
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             for (int kb = 0; kb < p.k_blocks; ++kb) {
                 const int s = kb % GEMM_STAGES;
                 const uint32_t par = ((kb / GEMM_STAGES) & 1) ^ 1;
-                if (!mbar_wait(&empty_bar[s], par, &abort_flag)) break;
+                if (!mbar_wait_warp(&empty_bar[s], par, &abort_flag)) break;
                 uint8_t* a_dst = smem + (size_t)s * stage_bytes;
-                mbar_expect_tx(&full_bar[s], stage_bytes);
-                tma_load_2d(a_dst, &map_a, kb * BK, m_blk * BM, &full_bar[s]);
-                tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, kb * BK, n_tile_idx * GEMM_BN, &full_bar[s]);
+                mbar_expect_tx(&full_bar[s], stage_bytes, el);
+                tma_load_2d(a_dst, &map_a, kb * BK, m_blk * BM, &full_bar[s], el);
+                tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, kb * BK, n_tile_idx * GEMM_BN, &full_bar[s], el);
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             constexpr uint32_t idesc = idesc_bf16(BM, GEMM_BN);
             bool ok = true;
             for (int kb = 0; kb < p.k_blocks && ok; ++kb) {
                 const int s = kb % GEMM_STAGES;
-                ok = mbar_wait(&full_bar[s], (kb / GEMM_STAGES) & 1, &abort_flag);
+                ok = mbar_wait_warp(&full_bar[s], (kb / GEMM_STAGES) & 1, &abort_flag);
                 if (!ok) break;
                 tc_fence_after();
                 const uint32_t a_addr = smem_u32(smem + (size_t)s * stage_bytes);
@@ -177,10 +178,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
                 const uint64_t bdesc = smem_desc_sw128(a_addr + A_STAGE_BYTES);
 #pragma unroll
                 for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tmem_base, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
-                tc_commit(&empty_bar[s]);
+                    tc_mma_bf16(tmem_base, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
+                tc_commit(&empty_bar[s], el);
             }
-            if (ok) tc_commit(&accum_bar);
+            if (ok) tc_commit(&accum_bar, el);
         }
     } else {
         const int q = warp & 3;            // tensor-memory lane quadrant this warp may read
@@ -295,7 +296,8 @@ enc_proj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     __shared__ float s_bias[EP_MAX_H];
     __shared__ int s_scan[GEMM_THREADS / 32];
 
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
+    const uint32_t el = lane == 0;   // the lane that executes the CTA-level instructions of an issuing warp
     uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
     if (p.ctrl->bad_input) return;   // a length outside [0, T]: nothing is read through it
 
@@ -353,7 +355,7 @@ enc_proj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     };
 
     if (warp == 0) {
-        if (lane == 0) {
+        {
             uint32_t it = 0;
             bool ok = true;
             for (int k = blockIdx.x; k < n_tiles && ok; k += gridDim.x) {
@@ -362,16 +364,16 @@ enc_proj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 const int row0 = b * p.T + j * BM;
                 for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
                     const int s = it % EP_STAGES;
-                    if (!mbar_wait(&empty_bar[s], ((it / EP_STAGES) & 1) ^ 1, &abort_flag)) { ok = false; break; }
+                    if (!mbar_wait_warp(&empty_bar[s], ((it / EP_STAGES) & 1) ^ 1, &abort_flag)) { ok = false; break; }
                     uint8_t* a_dst = smem + (size_t)s * EP_STAGE_BYTES;
-                    mbar_expect_tx(&full_bar[s], EP_STAGE_BYTES);
-                    tma_load_2d(a_dst, &map_a, kb * BK, row0, &full_bar[s]);
-                    tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, kb * BK, nt * EP_BN, &full_bar[s]);
+                    mbar_expect_tx(&full_bar[s], EP_STAGE_BYTES, el);
+                    tma_load_2d(a_dst, &map_a, kb * BK, row0, &full_bar[s], el);
+                    tma_load_2d(a_dst + A_STAGE_BYTES, &map_b, kb * BK, nt * EP_BN, &full_bar[s], el);
                 }
             }
         }
     } else if (warp == 1) {
-        if (lane == 0) {
+        {
             uint32_t it = 0, n_acc = 0;
             bool ok = true;
             for (int k = blockIdx.x; k < n_tiles && ok; k += gridDim.x, ++n_acc) {
@@ -379,22 +381,22 @@ enc_proj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
                 const int n_cols = min(EP_BN, p.H - nt * EP_BN);            // a multiple of 64
                 const uint32_t idesc = idesc_bf16(BM, n_cols);
                 const uint32_t a = n_acc & 1u;
-                if (!mbar_wait(&acc_empty[a], ((n_acc >> 1) & 1u) ^ 1u, &abort_flag)) { ok = false; break; }
+                if (!mbar_wait_warp(&acc_empty[a], ((n_acc >> 1) & 1u) ^ 1u, &abort_flag)) { ok = false; break; }
                 tc_fence_after();
                 const uint32_t tm_d = tmem_base + a * EP_BN;
                 for (int kb = 0; kb < p.k_blocks; ++kb, ++it) {
                     const int s = it % EP_STAGES;
-                    if (!mbar_wait(&full_bar[s], (it / EP_STAGES) & 1, &abort_flag)) { ok = false; break; }
+                    if (!mbar_wait_warp(&full_bar[s], (it / EP_STAGES) & 1, &abort_flag)) { ok = false; break; }
                     tc_fence_after();
                     const uint32_t a_addr = smem_u32(smem + (size_t)s * EP_STAGE_BYTES);
                     const uint64_t adesc = smem_desc_sw128(a_addr);
                     const uint64_t bdesc = smem_desc_sw128(a_addr + A_STAGE_BYTES);
 #pragma unroll
                     for (int kk = 0; kk < BK / 16; ++kk)
-                        tc_mma_bf16(tm_d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (kb | kk) != 0);
-                    tc_commit(&empty_bar[s]);
+                        tc_mma_bf16(tm_d, adesc + (uint64_t)(kk * 2), bdesc + (uint64_t)(kk * 2), idesc, (kb | kk) != 0, el);
+                    tc_commit(&empty_bar[s], el);
                 }
-                if (ok) tc_commit(&acc_full[a]);
+                if (ok) tc_commit(&acc_full[a], el);
             }
         }
     } else {
