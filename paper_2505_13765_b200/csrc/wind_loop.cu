@@ -46,6 +46,7 @@
 #include <cstdlib>
 #include <mutex>
 
+#include "wind_loop_cl.cuh"
 #include "wind_loop_dev.cuh"
 
 namespace wind {
@@ -77,7 +78,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
     const int cta = blockIdx.x, G = gridDim.x;
     // a length outside [0, T] (found by the init kernel, which ran before this launch): the status is set, no CTA starts
     if (p.ctrl->bad_input) return;
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align_smem_1024(smem_raw);
     uint8_t* stat = smem;                       // W_out tile kept in shared memory (J_SMEM): kb_h blocks of 128 x 64 bf16
     uint8_t* ring = smem + p.stat_bytes;        // operand stages; geometry differs per phase, drained in between
 
@@ -1666,6 +1667,7 @@ static int g_attr_smem[64] = {};       // opt-in shared memory already granted t
 static int g_loop_extra_arrivals = 0;
 static LoopOptions g_loop_options = {1, -1, 4, -1};
 int loop_set_extra_arrivals(int n) { int prev = g_loop_extra_arrivals; g_loop_extra_arrivals = n > 0 ? n : 0; return prev; }
+int loop_extra_arrivals() { return g_loop_extra_arrivals; }
 void loop_set_options(const LoopOptions& o) { g_loop_options = o; }
 LoopOptions loop_get_options() { return g_loop_options; }
 
@@ -1719,7 +1721,7 @@ static cudaError_t loop_map(CUtensorMap* map, const void* base, uint64_t rows, u
 
 // the same matrix seen as (64 columns, rows, cols / 64 blocks): one box of (64, box_rows, all blocks) lands in shared
 // memory as cols / 64 consecutive K blocks of box_rows x 128 bytes, each with the 128-byte swizzle
-static cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
     cuuint64_t dims[3] = {(cuuint64_t)BK, rows, cols / BK};
     cuuint64_t strides[2] = {cols * 2, (cuuint64_t)BK * 2};
     cuuint32_t box[3] = {(cuuint32_t)BK, box_rows, (cuuint32_t)(cols / BK)};
@@ -1984,6 +1986,7 @@ cudaError_t loop_prepare(Call& c) {
 
 cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* prefix_len, float* logits_out,
                     int trace_step) {
+    if (!logits_out && trace_step < -1 && cl_supported(c)) return cl_loop(c);
     const LoopPlan& pl = t_loop_plan;
     LoopParams p{};
     p.ctrl = c.ctrl();

@@ -136,6 +136,10 @@ cudaError_t loop_plan_for(const wind_model_t& m, int B, int W, int sms, int smem
 cudaError_t loop_res_set_smem(int bytes);
 cudaError_t loop_res_launch(const LoopMaps& maps, const LoopParams& p, int grid, uint32_t smem_bytes, bool full, cudaStream_t stream);
 int loop_set_extra_arrivals(int n);  // returns the previous value
+int loop_extra_arrivals();
+// bf16 matrix [rows, cols] as (64 columns, rows, cols / 64): one box lands as K blocks of box_rows x 128 bytes, 128-byte swizzle
+// (needs a loop_prepare before it)
+cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
 cudaError_t loop_prepare(Call& c);   // plan + tensor maps + shared-memory opt-in (host only; not inside a capture)
 
 }  // namespace wind

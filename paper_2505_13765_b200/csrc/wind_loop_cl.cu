@@ -1,0 +1,769 @@
+// The decoding loop of the bf16 path for one-layer models whose decoder fits one thread-block cluster (sm_100a).
+//
+// A lock step is a chain of small dependent products, so what it costs is the latency of handing results from SM to SM.
+// Here every hand-over stays inside a cluster of 16 CTAs (st.async into distributed shared memory: about 0.25 us) instead of
+// going through L2 (a barrier over the chip alone is 1.3 us), and clusters share nothing but the queue of utterances.
+//
+// All weights of the loop stay on chip, cut over the 16 CTAs of a cluster (large model: 5.4 MB; a CTA holds 340 KB):
+//   tensor memory   W_hh rows of the CTA's first 32 hidden units (4 gates x 32 = the 128 lanes), operand A of the gates' MMA
+//   shared memory   W_out rows of its 1/16 of the vocabulary
+//   registers       W_pred rows of its 1/16 of the joint's hidden units and W_hh rows of its remaining hidden units, as
+//                   mma.sync fragments (no register may be spilled: next to 220 KB of shared memory there is no first-
+//                   level cache left, and a spilled value comes from L2)
+// A cluster decodes up to 8 utterances ("slots") at a time; a lock step of a cluster is
+//   keys    every CTA sends the best (logit, label) of its labels for each window row to the slot's owner (slot u: CTA u)
+//   control the owner takes Algorithm 2's decision and sends (token, next frame) to every CTA, then records it; the window's
+//           enc_proj rows start on their way (one TMA box per eight rows, in the layout of the joint's operand)
+//   gates   W_hh h was computed a step ahead; + the token's row of the gate table, cell update, new h to every CTA
+//   pred    W_pred h, pred_proj to every CTA
+//   joint   z = act(enc_proj rows + pred_proj) in place, times the CTA's W_out rows on tcgen05 (window rows on the M axis, so
+//           that an accumulator lane is a window row and its argmax needs no exchange between lanes)
+// W_pred h is 40 rows per CTA: as 40 dependent tcgen05.mma it would take 1000 cycles (24 each however small the tile), as
+// two chains of 20 mma.sync 420.  mma.sync and tcgen05.mma accumulate a K step of 16 identically (checked bit for bit), and
+// K halves, roundings and epilogue arithmetic are those of loop_kernel with resident weights: same transcripts, bit for bit.
+//
+// A slot whose utterance is finished takes the next one from the queue in the same lock step (its recurrent term and cell
+// state count as zero in the step that feeds start-of-sequence).
+//
+// Every wait is bounded.  A CTA that gives up sets WIND_ERR_TIMEOUT; the others of its cluster run out of their own waits;
+// all meet at the cluster barrier at the end, so no CTA leaves while another may still write into its shared memory.
+#include <cudaTypedefs.h>
+
+#include <mutex>
+#include <type_traits>
+
+#include "wind_loop_cl.cuh"
+#include "wind_loop_dev.cuh"
+
+namespace wind {
+
+struct ClDec { int tok; uint32_t flags, row, unused; };   // what an owner sends for its slot
+constexpr uint32_t CL_FRESH = 1u, CL_IDLE = 2u;
+
+// Warps: 0-3 gates and z (workers), 4-9 W_pred, 10-13 remainder units, 14 issuing thread, 15 control.  Warps 0-7 also
+// share the joint's epilogue.  NS: most slots in use (1, 2, 4, 8).
+template <int NS, int ACT>
+__global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant__ CUtensorMap enc_map, const ClParams p) {
+    extern __shared__ uint8_t smem_raw[];
+    __shared__ uint64_t bar_keys, bar_dec, bar_enc, bar_h, bar_pred, bar_z, bar_sync_mma, bar_acc_g, bar_acc_r, bar_acc_j;
+    __shared__ uint32_t tmem_slot;
+    __shared__ int s_abort;
+    __shared__ int s_hist[65];
+
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
+    if (p.ctrl->bad_input) return;             // a length outside [0, T]: the whole grid leaves before it does anything
+    const int r = (int)cl_rank();
+    const int cluster = blockIdx.x / CL_SIZE, n_clusters = gridDim.x / CL_SIZE;
+    const int NU = p.slots, U = p.P / CL_SIZE, HS = p.H / CL_SIZE;
+    const int kb_p = p.P / 64, kb_h = p.H / 64;
+    const int wp_shift = p.wp == 8 ? 3 : (p.wp == 16 ? 4 : 5);
+    const int n_groups = (NU << wp_shift) >> 3;
+    const int lab_base = cl_label_base(p.NV), lab_extra = cl_label_extra(p.NV);
+    const int lab0 = r * lab_base + 8 * min(r, lab_extra);              // this CTA's vocabulary entries [lab0, lab0 + labs)
+    const int lab_n = lab_base + (r < lab_extra ? 8 : 0);               // the MMA's N
+    const int labs = min(lab_n, max(0, p.NV - lab0));
+    const int lab_rows = lab_base + (lab_extra > 0 ? 8 : 0);            // rows of a K block of the W_out tile
+    const bool has_rem = U > 32;
+
+    uint8_t* smem = align_smem_1024(smem_raw);
+    const ClSmem L = cl_smem_layout(p.P, p.H, p.NV, NU, p.wp);
+    const uint32_t sbase = smem_u32(smem);
+    const ClDec* dec = reinterpret_cast<const ClDec*>(smem + L.dec);
+    float* s_bout = reinterpret_cast<float*>(smem + L.b_out);
+    float* s_bpred = reinterpret_cast<float*>(smem + L.b_pred);
+    float* gr = reinterpret_cast<float*>(smem + L.gr);
+
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        mbar_init(&bar_keys, 1);
+        mbar_init(&bar_dec, 1u + (uint32_t)p.extra_arrivals);   // extra_arrivals > 0: a test hook, the wait can then never end
+        mbar_init(&bar_enc, 1);
+        mbar_init(&bar_h, 1);
+        mbar_init(&bar_pred, 1);
+        mbar_init(&bar_z, 8);
+        mbar_init(&bar_sync_mma, 6u + (has_rem ? 4u : 0u));
+        mbar_init(&bar_acc_g, 1);
+        mbar_init(&bar_acc_r, 4);
+        mbar_init(&bar_acc_j, 1);
+        fence_barrier_init();
+        // armed for their first phase (later phases: by the warp that saw the previous one complete, and only then: a barrier must
+        // not be armed twice in a phase)
+        mbar_expect_tx(&bar_keys, (uint32_t)(2 * CL_SIZE * p.W) * 8u);
+        mbar_expect_tx(&bar_dec, (uint32_t)NU * 16u);
+        mbar_expect_tx(&bar_h, (uint32_t)(NU * p.P) * 2u);
+        mbar_expect_tx(&bar_pred, (uint32_t)(NU * p.H) * 2u);
+        prefetch_tmap(&enc_map);
+    }
+    if (warp == 14) tmem_alloc(&tmem_slot, LOOP_TMEM_COLS);
+    for (int i = threadIdx.x; i < 65; i += CL_THREADS) s_hist[i] = 0;
+    if (threadIdx.x < CL_SLOTS) *reinterpret_cast<uint4*>(smem + L.dec + threadIdx.x * 16) = make_uint4(0xFFFFFFFFu, CL_IDLE, 0u, 0u);
+    for (int i = threadIdx.x; i < CL_MAX_LABELS + 8; i += CL_THREADS) s_bout[i] = i < labs ? p.b_out[lab0 + i] : -INFINITY;
+    for (int i = threadIdx.x; i < 48; i += CL_THREADS) s_bpred[i] = i < HS ? p.b_pred[r * HS + i] : 0.f;
+    // ---- resident weights ----
+#pragma unroll 1
+    for (int row = warp; row < lab_rows; row += CL_THREADS / 32)                  // W_out: K blocks of lab_rows x 128 bytes, 128-byte swizzle
+        for (int c = lane; c < p.H / 8; c += 32) {
+            const uint4 v = row < labs ? *reinterpret_cast<const uint4*>(p.w_out + (size_t)(lab0 + row) * p.H + c * 8) : make_uint4(0, 0, 0, 0);
+            *reinterpret_cast<uint4*>(smem + L.w_out + (c >> 3) * (lab_rows * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)) = v;
+        }
+    for (uint32_t i = threadIdx.x; i < 2u * (uint32_t)p.P; i += CL_THREADS)       // h of slots nobody uses must be numbers
+        *reinterpret_cast<uint4*>(smem + L.h + i * 16) = make_uint4(0, 0, 0, 0);
+    fence_proxy_async();
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    const uint32_t tm_g = tmem + CL_MAX_DIM / 2, tm_j = tm_g + 32, tm_j2 = tm_j + 80;   // gates: 16 columns; joint: two copies of up to 72
+    const int q = warp & 3;                                                       // lane quadrant
+    const uint32_t lane_off = (uint32_t)(q * 32) << 16;
+    if (warp < 8) {                                                               // W_hh of units 0..31: lane 4 u + gate
+        const int u = 8 * q + (lane >> 2), g = lane & 3;
+        const bool in = u < U;
+        const uint4* src = reinterpret_cast<const uint4*>(p.w_hh + ((size_t)g * p.P + r * U + (in ? u : 0)) * p.P);
+#pragma unroll 1
+        for (int c0 = 16 * (warp >> 2); c0 < p.P / 2; c0 += 32) {
+            uint32_t v[16];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint4 x = in ? src[c0 / 4 + j] : make_uint4(0, 0, 0, 0);
+                v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
+            }
+            tmem_st16(tmem + lane_off + (uint32_t)c0, v);
+        }
+        tmem_st_wait();
+    }
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    cl_barrier();                                                                 // every CTA's barriers are ready for remote stores
+
+    bool ok = true;
+    // every slot idle: all warps of the cluster leave in the same step
+    auto all_idle = [&]() { return __all_sync(0xffffffffu, lane >= NU || (dec[min(lane, NU - 1)].flags & CL_IDLE) != 0u); };
+    // ldmatrix address of the state: two K steps of 16 at a time, matrix = 8 slots x 8 columns, lane = (column piece, slot)
+    const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
+    auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * 2048u + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
+
+    // The joint's operand z = act(enc_proj + pred_proj), in place, by warps 0..7 (it is bound by the shared memory's bandwidth:
+    // 30 KB per group of eight rows; four warps leave a third of that unused, 2830 against 2110 cycles for eight groups).
+    // Of a group the rows that count; threads per row: a multiple of eight, one per 16-byte piece of a K block.
+    const int z_rows = p.wp == 8 ? p.W : 8;
+    const int z_tpr = (256 / z_rows) & ~7;
+    const int z_r = (int)threadIdx.x / z_tpr, z_k0 = ((int)threadIdx.x % z_tpr) >> 3, z_kstep = z_tpr >> 3;   // z_kstep >= 4
+    auto build_z = [&](auto which) {
+        constexpr int AT_ONCE = decltype(which)::value;               // pieces in flight per thread (the W_pred warps have registers for one)
+        if (z_r < z_rows) {
+            uint8_t* zp = smem + L.z + (uint32_t)(z_r * 128 + (((lane & 7) ^ (z_r & 7)) << 4) + z_k0 * 1024);
+            const uint8_t* pp = smem + L.pred + (uint32_t)(z_k0 * 128 + (lane & 7) * 16);
+#pragma unroll 1
+            for (int gi = 0; gi < n_groups; ++gi, zp += p.H * 16) {
+                const uint8_t* py = pp + (uint32_t)(((gi << 3) >> wp_shift) * p.H * 2);
+#pragma unroll 1
+                for (int j0 = 0; j0 < 3; j0 += AT_ONCE) {
+                    uint4 x[AT_ONCE], y[AT_ONCE];
+#pragma unroll
+                    for (int j = 0; j < AT_ONCE; ++j)
+                        if (z_k0 + (j0 + j) * z_kstep < kb_h) {
+                            x[j] = *reinterpret_cast<const uint4*>(zp + (j0 + j) * z_kstep * 1024);
+                            y[j] = *reinterpret_cast<const uint4*>(py + (j0 + j) * z_kstep * 128);
+                        }
+#pragma unroll
+                    for (int j = 0; j < AT_ONCE; ++j)
+                        if (z_k0 + (j0 + j) * z_kstep < kb_h)
+                            *reinterpret_cast<uint4*>(zp + (j0 + j) * z_kstep * 1024) =
+                                make_uint4(act_add_bf16x2(x[j].x, y[j].x, ACT), act_add_bf16x2(x[j].y, y[j].y, ACT),
+                                           act_add_bf16x2(x[j].z, y[j].z, ACT), act_add_bf16x2(x[j].w, y[j].w, ACT));
+                }
+            }
+        }
+        fence_proxy_async();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&bar_z);
+    };
+
+    // Argmax of every window row over a share of this CTA's labels (HF), sent to the slots' owners.  With M = 64 accumulator row m
+    // lives in lane m % 16 of quadrant m / 16.
+    auto joint_argmax = [&](auto which) {
+        constexpr int HF = decltype(which)::value;
+        if (16 * q >= NU << wp_shift) return;                         // this warp's quadrant holds no window row
+        // CH columns at a time: their maximum, then the lowest label that has it (equal logits: the lower label)
+        constexpr int CH = HF ? 8 : 16;                                 // (the W_pred warps have registers for eight)
+        const int nh = (lab_n / 3) & ~7;                                // they take [0, nh), the workers [nh, lab_n)
+        float best = -INFINITY;
+        int lab = 0;
+#pragma unroll 1
+        for (int c = HF ? 0 : nh; c < (HF ? nh : lab_n); c += CH) {
+            float v[CH];
+            if constexpr (CH == 16) tmem_ld16_sum(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
+            else tmem_ld8_sum(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
+#pragma unroll
+            for (int j = 0; j < CH; j += 4) {
+                const float4 b4 = *reinterpret_cast<const float4*>(s_bout + c + j);  // -inf behind the last label
+                v[j] += b4.x; v[j + 1] += b4.y; v[j + 2] += b4.z; v[j + 3] += b4.w;
+            }
+            float m = v[0];
+#pragma unroll
+            for (int j = 1; j < CH; ++j) m = fmaxf(m, v[j]);
+            int at = CH;
+#pragma unroll
+            for (int j = CH - 1; j >= 0; --j) at = v[j] == m ? j : at;
+            if (m > best) { best = m; lab = c + at; }
+        }
+        const int row = 16 * q + (lane & 15);
+        const int s = row >> wp_shift, w = row & (p.wp - 1);
+        if (lane < 16 && s < NU && w < p.W) {
+            const unsigned long long key = best > -INFINITY ? pack_key(best, (uint32_t)(lab0 + lab)) : 0ull;
+            st_async_8(cl_map(sbase + L.kbuf + (uint32_t)(w * CL_KEY_PITCH + 2 * r + HF) * 8u, s), key, cl_map(smem_u32(&bar_keys), s));
+        }
+    };
+
+    if (warp < 4) {
+        // =====================================================================================
+        // workers: cell update, then the joint's operand
+        // =====================================================================================
+        const int e = threadIdx.x;                       // 0..127
+        const int g = lane & 3, u = 8 * q + (lane >> 2); // gate and hidden unit (of the CTA's first 32) of this thread's accumulator lane
+        const float sc = g == 2 ? 1.f : 0.5f, of = g == 2 ? 0.f : 0.5f;   // tanh, or the logistic function as 0.5 tanh(x / 2) + 0.5
+        const float* g0 = p.g0 + (size_t)g * p.P + r * U + u;
+        const float* g0r = p.g0 + r * U + 32 + (e & 7);
+        const bool rem_on = has_rem && e < 64 && 32 + (e & 7) < U && (e >> 3) < NU;
+        // h: 16-byte pieces of the CTA's part; a warp instruction serves 32 / lpd destinations with lpd lanes each
+        const int h_pieces = NU * (U / 8);
+        const int lpd_shift = h_pieces <= 8 ? 3 : (h_pieces <= 16 ? 4 : 5);
+        const int h_first = lane & ((1 << lpd_shift) - 1);
+        uint32_t h_src[2], h_dst[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int i = h_first + 32 * k;
+            const int uu = i / (U / 8), cc = i - uu * (U / 8), col = r * U + cc * 8;
+            h_src[k] = L.hst + (uint32_t)(uu * U + cc * 8) * 2u;
+            h_dst[k] = L.h + (uint32_t)((col >> 6) * 2048 + uu * 128 + ((((col >> 3) & 7) ^ (uu & 7)) << 4));
+        }
+        float c_st[2] = {0.f, 0.f}, c_rem = 0.f;         // cell state: (u, slots 2 g, 2 g + 1); (32 + (e & 7), slot e >> 3) for e < 64
+        __nv_bfloat16 h_st[2], h_rem = __float2bfloat16_rn(0.f);
+        h_st[0] = h_st[1] = h_rem;
+        __nv_bfloat16* hst = reinterpret_cast<__nv_bfloat16*>(smem + L.hst);
+        long long clk = 0, cyc[3] = {0, 0, 0};
+        const bool timed = blockIdx.x == 0 && e == 0;
+        unsigned long long ns0 = 0;
+        if (timed) { ns0 = globaltimer_ns(); clk = clock64(); }
+        auto lap = [&](int k) { if (timed) { const long long now = clock64(); cyc[k] += now - clk; clk = now; } };
+
+        for (uint32_t step = 0;; ++step) {
+            const uint32_t par = step & 1u;
+            // ---- decisions of the step; the gate table's rows are requested at once ----
+            if (ok) ok = cl_wait(&bar_dec, par);
+            if (ok && warp == 0 && lane == 0) mbar_expect_tx(&bar_dec, (uint32_t)NU * 16u);
+            lap(0);
+            const bool idle = all_idle();
+            float add[NS], add_r[4];
+            uint32_t fresh = 0u, live = 0u;
+            {
+                uint2 d[NS];                             // (token, flags); slots beyond NU never have a token
+#pragma unroll
+                for (int s = 0; s < NS; ++s) d[s] = *reinterpret_cast<const uint2*>(&dec[s]);
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    fresh |= (d[s].y & CL_FRESH) << s;
+                    live |= (uint32_t)((int)d[s].x >= 0) << s;
+                    add[s] = (int)d[s].x >= 0 && u < U ? g0[d[s].x * (uint32_t)(4 * p.P)] : 0.f;
+                }
+            }
+            if (rem_on) {
+                const int tok = dec[e >> 3].tok;
+#pragma unroll
+                for (int k = 0; k < 4; ++k) add_r[k] = tok >= 0 ? g0r[(uint32_t)tok * (uint32_t)(4 * p.P) + (uint32_t)(k * p.P)] : 0.f;
+            }
+            // ---- gates: recurrent term + gate table, cell update ----
+            if (step > 0) {
+                if (ok) ok = cl_wait(&bar_acc_g, (step - 1u) & 1u);
+                if (has_rem && ok) ok = cl_wait(&bar_acc_r, (step - 1u) & 1u);
+            }
+            tc_fence_after();
+            {
+                float x[8];
+                tmem_ld8(tm_g + lane_off, x);
+#pragma unroll
+                for (int s = 0; s < 8; ++s) {
+                    if (s < NS) x[s] = fmaf(tanh_fast((((fresh >> s) & 1u ? 0.f : x[s]) + add[s]) * sc), sc, of);
+                    else x[s] = 0.f;
+                }
+                // lane 4 u + g holds gate g of all slots; it is to hold the four gates of slots 2 g and 2 g + 1
+                const bool up2 = (g & 2) != 0, up1 = (g & 1) != 0;
+                float a[4], b[4];
+#pragma unroll
+                for (int j = 0; j < (NS < 4 ? NS : 4); ++j) {
+                    a[j] = up2 ? x[4 + j] : x[j];
+                    b[j] = __shfl_xor_sync(0xffffffffu, up2 ? x[j] : x[4 + j], 2);    // the same slots, gate g ^ 2
+                }
+#pragma unroll
+                for (int j = NS < 4 ? NS : 4; j < 4; ++j) a[j] = b[j] = 0.f;
+#pragma unroll
+                for (int k = 0; k < (NS < 2 ? NS : 2); ++k) {
+                    float own = up1 ? a[2 + k] : a[k], g2 = up1 ? b[2 + k] : b[k];
+                    float g1 = __shfl_xor_sync(0xffffffffu, up1 ? a[k] : a[2 + k], 1), g3 = __shfl_xor_sync(0xffffffffu, up1 ? b[k] : b[2 + k], 1);
+                    if (up1) { float t = own; own = g1; g1 = t; t = g2; g2 = g3; g3 = t; }
+                    if (up2) { float t = own; own = g2; g2 = t; t = g1; g1 = g3; g3 = t; }
+                    const float gi = own, gf = g1, gg = g2, go = g3;
+                    const int s = 2 * g + k;
+                    if (u < U && s < NU) {
+                        if ((live >> s) & 1u) {
+                            const float cold = (fresh >> s) & 1u ? 0.f : c_st[k];
+                            const float cc = gf * cold + gi * gg;
+                            c_st[k] = cc;
+                            h_st[k] = __float2bfloat16_rn(go * tanh_fast(cc));
+                        }
+                        hst[s * U + u] = h_st[k];
+                    }
+                }
+            }
+            if (rem_on) {
+                const int s = e >> 3;
+                if ((live >> s) & 1u) {
+                    float4 x = *reinterpret_cast<const float4*>(gr + s * CL_GR_PITCH + 4 * (e & 7));
+                    if ((fresh >> s) & 1u) x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    const float gi = fmaf(tanh_fast((x.x + add_r[0]) * 0.5f), 0.5f, 0.5f);
+                    const float gf = fmaf(tanh_fast((x.y + add_r[1]) * 0.5f), 0.5f, 0.5f);
+                    const float gg = fmaf(tanh_fast((x.z + add_r[2]) * 1.f), 1.f, 0.f);
+                    const float go = fmaf(tanh_fast((x.w + add_r[3]) * 0.5f), 0.5f, 0.5f);
+                    const float cold = (fresh >> s) & 1u ? 0.f : c_rem;
+                    const float cc = gf * cold + gi * gg;
+                    c_rem = cc;
+                    h_rem = __float2bfloat16_rn(go * tanh_fast(cc));
+                }
+                hst[s * U + 32 + (e & 7)] = h_rem;
+            }
+            tc_fence_before();
+            if (group_barrier_or<128>(1, !ok || idle)) break;
+            // h to all CTAs
+#pragma unroll
+            for (int k = 0; k < 2; ++k)
+                if (h_first + 32 * k < h_pieces) {
+                    const uint4 piece = *reinterpret_cast<const uint4*>(smem + h_src[k]);
+                    for (int d0 = warp * (32 >> lpd_shift) + (lane >> lpd_shift); d0 < CL_SIZE; d0 += 128 >> lpd_shift) {
+                        const uint32_t d = (uint32_t)(d0 + r) & (CL_SIZE - 1);
+                        st_async_16(cl_map(sbase, d) + h_dst[k], piece, cl_map(smem_u32(&bar_h), d));
+                    }
+                }
+            lap(1);
+            // ---- the joint's operand z = act(enc_proj + pred_proj), in place ----
+            if (ok) ok = cl_wait(&bar_enc, par);
+            if (ok) ok = cl_wait(&bar_pred, par);
+            if (ok && warp == 0 && lane == 0) mbar_expect_tx(&bar_pred, (uint32_t)(NU * p.H) * 2u);
+            lap(2);
+            build_z(std::integral_constant<int, 3>{});
+            if (ok) ok = cl_wait(&bar_acc_j, par);
+            tc_fence_after();
+            joint_argmax(std::integral_constant<int, 0>{});
+        }
+        if (timed) {
+            p.ctrl->active = 0;
+            for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = cyc[k];
+            p.ctrl->loop_ns = (long long)(globaltimer_ns() - ns0);
+        }
+    } else if (warp < 10) {
+        // =====================================================================================
+        // W_pred: (K half, 16 joint units) per warp, pred_proj[unit, slot] = W_pred h^T
+        // =====================================================================================
+        const int half = (warp - 4) / 3, mt = (warp - 4) % 3;
+        const int k16s = p.P / 32;                       // K steps of 16 in a half: at most 20
+        const bool mine = mt * 16 < HS;
+        uint32_t wf[20][4];                              // (rows behind the last one repeat it: their results go nowhere)
+        {
+            const uint32_t* r0 = reinterpret_cast<const uint32_t*>(p.w_pred + (size_t)(r * HS + min(16 * mt + (lane >> 2), HS - 1)) * p.P + half * (p.P / 2)) + (lane & 3);
+            const uint32_t* r1 = reinterpret_cast<const uint32_t*>(p.w_pred + (size_t)(r * HS + min(16 * mt + (lane >> 2) + 8, HS - 1)) * p.P + half * (p.P / 2)) + (lane & 3);
+#pragma unroll
+            for (int s0 = 0; s0 < 20; s0 += 4)
+                if (s0 < k16s)
+#pragma unroll
+                    for (int s = s0; s < s0 + 4; ++s) { wf[s][0] = r0[s * 8]; wf[s][1] = r1[s * 8]; wf[s][2] = r0[s * 8 + 4]; wf[s][3] = r1[s * 8 + 4]; }
+        }
+        float4* part = reinterpret_cast<float4*>(smem + L.part) + mt * 32 + lane;
+        __nv_bfloat16* pst = reinterpret_cast<__nv_bfloat16*>(smem + L.pst) + 16 * mt;     // [slot][48]
+        const int halves = min(2, (HS - 16 * mt) / 8);   // 16-byte pieces of a slot in this warp's 16 units
+        for (uint32_t step = 0;; ++step) {
+            const uint32_t par = step & 1u;
+            if (ok) ok = cl_wait(&bar_dec, par);
+            const bool idle = all_idle();
+            if (ok && !idle) ok = cl_wait(&bar_h, par);
+            if (ok && !idle && warp == 4 && lane == 0) mbar_expect_tx(&bar_h, (uint32_t)(NU * p.P) * 2u);
+            float acc[4] = {0.f, 0.f, 0.f, 0.f};
+            if (mine) {
+                uint32_t b[2][4];
+                ldmatrix_x4(b[0], h_at(half * (k16s / 2)));
+                // (the state rows of the next two steps are requested a turn early; at the end they are rows nobody uses)
+#pragma unroll
+                for (int s0 = 0; s0 < 20; s0 += 4)
+                    if (s0 < k16s)
+#pragma unroll
+                        for (int s = s0; s < s0 + 4; s += 2) {
+                            ldmatrix_x4(b[(s / 2 + 1) & 1], h_at(half * (k16s / 2) + s / 2 + 1));
+                            mma_16816(acc, wf[s][0], wf[s][1], wf[s][2], wf[s][3], b[(s / 2) & 1][0], b[(s / 2) & 1][1]);
+                            mma_16816(acc, wf[s + 1][0], wf[s + 1][1], wf[s + 1][2], wf[s + 1][3], b[(s / 2) & 1][2], b[(s / 2) & 1][3]);
+                        }
+                if (half) *part = make_float4(acc[0], acc[1], acc[2], acc[3]);
+            }
+            if (group_barrier_or<192>(2, !ok || idle)) break;
+            if (lane == 0) mbar_arrive(&bar_sync_mma);
+            if (half == 0 && mine) {
+                // the two K halves are added as loop_kernel adds its accumulators
+                const float4 o = *part;
+                const int m = lane >> 2, s = (lane & 3) * 2;
+                const float b0 = s_bpred[16 * mt + m], b1 = s_bpred[16 * mt + m + 8];
+                pst[s * 48 + m] = __float2bfloat16_rn(acc[0] + o.x + b0);
+                pst[(s + 1) * 48 + m] = __float2bfloat16_rn(acc[1] + o.y + b0);
+                pst[s * 48 + m + 8] = __float2bfloat16_rn(acc[2] + o.z + b1);
+                pst[(s + 1) * 48 + m + 8] = __float2bfloat16_rn(acc[3] + o.w + b1);
+                __syncwarp();
+                // 16-byte pieces of eight units of one slot: message i = (piece, destination)
+                for (int i = lane; i < NU * halves * CL_SIZE; i += 32) {
+                    const int pi = i >> 4, sl = halves == 2 ? pi >> 1 : pi, hh = halves == 2 ? pi & 1 : 0;
+                    const uint32_t d = (uint32_t)(i + r) & (CL_SIZE - 1);
+                    st_async_16(cl_map(sbase, d) + L.pred + (uint32_t)(sl * p.H + r * HS + 16 * mt + 8 * hh) * 2u,
+                                *reinterpret_cast<const uint4*>(pst + sl * 48 + 8 * hh), cl_map(smem_u32(&bar_pred), d));
+                }
+            }
+            if (warp < 8) {
+                if (ok) ok = cl_wait(&bar_enc, par);
+                if (ok) ok = cl_wait(&bar_pred, par);
+                build_z(std::integral_constant<int, 1>{});
+                if (ok) ok = cl_wait(&bar_acc_j, par);
+                tc_fence_after();
+                joint_argmax(std::integral_constant<int, 1>{});
+                tc_fence_before();
+            }
+        }
+    } else if (warp < 14) {
+        // =====================================================================================
+        // remainder units 32..: W_hh rows of units 32 + 2 k, + 1 (4 gates each: row 4 (u - 32) + gate) in warp 10 + k, one chain
+        // over all of K (as the gates' accumulator in loop_kernel), [slot, row] = h W_hh^T
+        // =====================================================================================
+        if (has_rem) {
+            const int row = 8 * (warp - 10) + (lane >> 2), u = 32 + (row >> 2), g = row & 3;
+            uint32_t wf[40][2];
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(p.w_hh + ((size_t)g * p.P + r * U + min(u, U - 1)) * p.P) + (lane & 3);
+#pragma unroll
+            for (int s0 = 0; s0 < 40; s0 += 8)
+                if (s0 < p.P / 16)
+#pragma unroll
+                    for (int s = s0; s < s0 + 8; ++s) { wf[s][0] = src[s * 8]; wf[s][1] = src[s * 8 + 4]; }
+            for (uint32_t step = 0;; ++step) {
+                const uint32_t par = step & 1u;
+                ok = cl_wait_warp(&bar_dec, par);
+                if (all_idle() || !ok) break;
+                ok = cl_wait_warp(&bar_h, par);
+                if (!ok) break;
+                float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                uint32_t a[2][4];
+                ldmatrix_x4(a[0], h_at(0));
+#pragma unroll
+                for (int s0 = 0; s0 < 40; s0 += 8)
+                    if (s0 < p.P / 16)
+#pragma unroll
+                        for (int s = s0; s < s0 + 8; s += 2) {
+                            ldmatrix_x4(a[(s / 2 + 1) & 1], h_at(s / 2 + 1));
+                            mma_16816(acc, a[(s / 2) & 1][0], 0u, a[(s / 2) & 1][1], 0u, wf[s][0], wf[s][1]);
+                            mma_16816(acc, a[(s / 2) & 1][2], 0u, a[(s / 2) & 1][3], 0u, wf[s + 1][0], wf[s + 1][1]);
+                        }
+                *reinterpret_cast<float2*>(gr + (lane >> 2) * CL_GR_PITCH + (warp - 10) * 8 + (lane & 3) * 2) = make_float2(acc[0], acc[1]);
+                __syncwarp();
+                if (lane == 0) { mbar_arrive(&bar_acc_r); mbar_arrive(&bar_sync_mma); }
+            }
+        }
+    } else if (warp == 14) {
+        // =====================================================================================
+        // issuing thread: the window's enc_proj rows, the gates' MMAs on the new state (a step ahead of their use), the joint's
+        // =====================================================================================
+        if (elect_one()) {
+            const uint32_t id_g = idesc_bf16(128, 16), id_j = idesc_bf16(64, lab_n);
+            // z: eight-row groups H * 16 bytes apart (each a TMA box: K blocks of 8 rows x 128 bytes)
+            const uint64_t ad0 = (smem_desc_sw128(sbase + L.z) & ~((uint64_t)0x3FFF << 32)) | ((uint64_t)(uint32_t)p.H << 32);
+            uint32_t n_g = 0u;
+            for (uint32_t step = 0;; ++step) {
+                const uint32_t par = step & 1u;
+                if (!(ok = cl_wait(&bar_dec, par))) break;
+                uint32_t idle = CL_IDLE;
+#pragma unroll 1
+                for (int s = 0; s < NU; ++s) idle &= dec[s].flags;
+                if (idle) break;
+                mbar_expect_tx(&bar_enc, (uint32_t)(n_groups * p.H * 16));
+#pragma unroll 1
+                for (int gi = 0; gi < n_groups; ++gi) {
+                    const int s = (gi << 3) >> wp_shift;
+                    tma_load_3d(smem + L.z + (uint32_t)(gi * p.H * 16), &enc_map, 0, (int)dec[s].row + ((gi << 3) & (p.wp - 1)), 0, &bar_enc);
+                }
+                // mma.sync and tcgen05.mma exclude each other on the tensor cores: the short chains go first (when they are
+                // done, all of h is there as well)
+                if (!(ok = cl_wait(&bar_sync_mma, par))) break;
+                fence_proxy_async_all();                 // h came in through remote generic stores
+                tc_fence_after();
+                uint64_t bd = smem_desc_sw128(sbase + L.h);
+#pragma unroll 1
+                for (int kb = 0; kb < kb_p; ++kb, bd += 2048 >> 4)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        tc_mma_bf16_ts(tm_g, tmem + (uint32_t)(kb * 32 + k * 8), bd + (uint64_t)(k * 2), id_g, (kb | k) != 0);
+                tc_commit(&bar_acc_g);
+                ++n_g;
+                if (!(ok = cl_wait(&bar_z, par))) break;
+                tc_fence_after();
+                bd = smem_desc_sw128(sbase + L.w_out);
+                uint64_t ad = ad0;
+#pragma unroll 1
+                for (int kb = 0; kb < kb_h; ++kb, bd += (uint64_t)(lab_rows * 8), ad += 1024 >> 4) {
+                    const bool second = kb >= kb_h / 2;  // K halves in two accumulator copies, as in loop_kernel
+                    const uint32_t d = second ? tm_j2 : tm_j;
+                    tc_mma_bf16(d, ad, bd, id_j, kb != (second ? kb_h / 2 : 0));
+#pragma unroll
+                    for (int k = 1; k < 4; ++k) tc_mma_bf16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), id_j, 1u);
+                }
+                tc_commit(&bar_acc_j);
+            }
+            // copies and MMAs in flight must have completed before the memory they use goes back
+            if (n_g > 0u) cl_wait(&bar_acc_g, (n_g - 1u) & 1u);
+            if (!ok) s_abort = 1;
+        }
+        __syncwarp();
+        ok = true;
+    } else if (r < NU) {
+        // =====================================================================================
+        // control: CTA u < NU owns slot u (every lane holds the same values)
+        // =====================================================================================
+        const bool dynamic = p.n_utt > NU * n_clusters;
+        int o_utt = -1, o_t = 0, o_len = 0, o_cnt = 0, o_pos = 0;
+        uint32_t o_row0 = 0u, n_steps = 0u;
+        unsigned long long n_rows = 0ull, n_tok = 0ull, n_forced = 0ull;
+        auto take = [&](int k) {                         // utterance k of the order, or, when it is empty or there is none, the next of the queue
+            for (;;) {
+                o_utt = -1; o_len = 0; o_t = 0; o_cnt = 0; o_pos = 0; o_row0 = 0u;
+                if (k >= 0 && k < p.n_utt) {
+                    o_utt = p.order ? p.order[k] : k;
+                    o_len = min(max(p.enc_len[o_utt], 0), p.T);
+                    o_row0 = (uint32_t)o_utt * (uint32_t)p.T;
+                    if (o_len > 0) return;
+                }
+                if (!dynamic || k >= p.n_utt) { o_utt = -1; return; }
+                int v = 0;
+                if (lane == 0) v = atomicAdd(&p.ctrl->next_utt, 1);
+                k = __shfl_sync(0xffffffffu, v, 0) - p.queue_base + NU * n_clusters;
+            }
+        };
+        auto announce = [&](int tok, bool fresh) {       // the slot's decision to every CTA
+            const bool idle = o_utt < 0;
+            const uint4 m = make_uint4((uint32_t)(idle ? -1 : tok), (fresh ? CL_FRESH : 0u) | (idle ? CL_IDLE : 0u),
+                                       idle ? 0u : o_row0 + (uint32_t)o_t, 0u);
+            if (lane < CL_SIZE) st_async_16(cl_map(sbase + L.dec + (uint32_t)r * 16u, lane), m, cl_map(smem_u32(&bar_dec), lane));
+        };
+        take(r * n_clusters + cluster);
+        announce(p.blank, true);
+        for (uint32_t step = 0;; ++step) {
+            const uint32_t par = step & 1u;
+            ok = cl_wait_warp(&bar_dec, par);
+            if (all_idle() || !ok) break;
+            ok = cl_wait_warp(&bar_keys, par);
+            if (!ok) break;
+            if (lane == 0) mbar_expect_tx(&bar_keys, (uint32_t)(2 * CL_SIZE * p.W) * 8u);
+            // lane = (window row, a share of the 32 keys of that row)
+            const ulonglong2* kp = reinterpret_cast<const ulonglong2*>(
+                smem + L.kbuf + (uint32_t)((lane & (p.wp - 1)) * CL_KEY_PITCH + (lane >> wp_shift) * p.wp) * 8u);
+            unsigned long long key = 0ull;
+#pragma unroll 1
+            for (int i = 0; i < p.wp / 2; i += 4) {
+                const ulonglong2 k0 = kp[i], k1 = kp[i + 1], k2 = kp[i + 2], k3 = kp[i + 3];
+                const unsigned long long m0 = max(max(k0.x, k0.y), max(k1.x, k1.y)), m1 = max(max(k2.x, k2.y), max(k3.x, k3.y));
+                key = max(key, max(m0, m1));
+            }
+            for (int o = p.wp; o < 32; o <<= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+            const int n = o_utt >= 0 ? min(p.W, o_len - o_t) : 0;        // an idle slot: no rows, nothing to record
+            uint32_t label = key_label(key);
+            const bool broken = key == 0ull || label >= (uint32_t)p.NV;
+            if (broken) label = (uint32_t)p.blank;
+            const uint32_t hit = __ballot_sync(0xffffffffu, lane < n && (int)label != p.blank);
+            const int first = hit ? __ffs((int)hit) - 1 : n;             // all blank: past the whole window
+            const int lab = (int)__shfl_sync(0xffffffffu, label, first & 31);
+            const int pos = o_pos, utt = o_utt;
+            const bool emit = hit && pos < p.max_out, overflow = hit && pos >= p.max_out;
+            int t = o_t + first;
+            const int t_emit = t;
+            if (first > 0) o_cnt = 0;
+            o_cnt += emit;
+            const bool forced = emit && o_cnt == p.S;
+            if (forced) { ++t; o_cnt = 0; }
+            o_pos += emit;
+            o_t = overflow ? o_len : t;                                  // no room for the token: this utterance stops here
+            n_steps += utt >= 0;
+            const bool stuck = n_steps >= (uint32_t)p.step_cap;
+            const bool done = utt >= 0 && (o_t >= o_len || stuck);
+            if (done) {
+                // finished: the slot takes the next utterance in this very step
+                if (lane == 0) {
+                    p.out_len[utt] = o_pos;
+                    if (o_t < o_len) set_status(p.ctrl, WIND_ERR_INTERNAL);
+                }
+                take(dynamic && !stuck ? -1 : p.n_utt);
+            }
+            announce(done ? p.blank : (emit ? lab : -1), done);          // what the step decided is recorded behind the answer
+            const uint32_t bad = __ballot_sync(0xffffffffu, lane < n && lane <= first && broken);   // rows after the first non-blank one do not count
+            n_rows += (unsigned)n; n_tok += emit; n_forced += forced;
+            if (lane == 0 && utt >= 0) {
+                s_hist[first] += 1;
+                if (emit) {
+                    p.out_tokens[(size_t)utt * p.max_out + pos] = lab;
+                    p.out_frames[(size_t)utt * p.max_out + pos] = t_emit;
+                }
+                if (overflow) set_status(p.ctrl, WIND_ERR_OUTPUT_OVERFLOW);
+                if (bad) set_status(p.ctrl, WIND_ERR_INTERNAL);
+            }
+        }
+        if (lane == 0 && n_steps > 0u) {
+            atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->joint_rows), n_rows);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->tokens), n_tok);
+            atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->forced), n_forced);
+            atomicMax(&p.ctrl->step, (int)n_steps);
+#pragma unroll 1
+            for (int k = 0; k < 65; ++k)
+                if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
+        }
+    }
+    if (!ok) s_abort = 1;
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 14) {
+        tc_fence_after();
+        tmem_dealloc(tmem, LOOP_TMEM_COLS);
+    }
+    if (threadIdx.x == 0 && s_abort) set_status(p.ctrl, WIND_ERR_TIMEOUT);
+    cl_barrier();                                        // no CTA leaves while another may still write into its shared memory
+}
+
+// ---------------------------------------------------------------------------
+// order of the utterances: longest first, so that the queue's tail is short (equal lengths keep their order)
+// ---------------------------------------------------------------------------
+constexpr int CL_ORDER_MAX = 4096;
+__global__ void __launch_bounds__(1024) cl_order_kernel(const int32_t* __restrict__ enc_len, int n, int32_t* __restrict__ order) {
+    __shared__ int32_t len[CL_ORDER_MAX];
+    for (int i = threadIdx.x; i < n; i += 1024) len[i] = enc_len[i];
+    __syncthreads();
+    for (int i = blockIdx.x * 1024 + threadIdx.x; i < n; i += gridDim.x * 1024) {
+        const int mine = len[i];
+        int rank = 0;
+        for (int j = 0; j < n; ++j) rank += len[j] > mine || (len[j] == mine && j < i);
+        order[rank] = i;
+    }
+}
+
+// ---------------------------------------------------------------------------
+// host side
+// ---------------------------------------------------------------------------
+static std::mutex g_cl_mutex;
+static int g_cl_clusters[64];          // per device: 0 not asked yet, -1 none, else clusters of 16 that are resident at a time
+
+template <int ACT>
+static const void* cl_fn_act(int ns) {
+    switch (ns) {
+        case 1: return (const void*)cl_kernel<1, ACT>;
+        case 2: return (const void*)cl_kernel<2, ACT>;
+        case 4: return (const void*)cl_kernel<4, ACT>;
+        default: return (const void*)cl_kernel<8, ACT>;
+    }
+}
+static const void* cl_fn(int ns, int act) { return act == WIND_ACT_RELU ? cl_fn_act<WIND_ACT_RELU>(ns) : cl_fn_act<WIND_ACT_TANH>(ns); }
+static uint32_t cl_smem_bytes(int P, int H, int NV, int slots, int wp) { return cl_smem_layout(P, H, NV, slots, wp).total + 1024u; }
+
+// clusters of 16 CTAs the current device holds at a time (one CTA per SM); 0: none
+static int cl_clusters() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 0;
+    std::lock_guard<std::mutex> lock(g_cl_mutex);
+    if (g_cl_clusters[dev] == 0) {
+        g_cl_clusters[dev] = -1;
+        int optin = 0;
+        if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
+        const int want = (int)cl_smem_bytes(CL_MAX_DIM, CL_MAX_DIM, 16 * CL_MAX_LABELS, 2, 32);
+        if (want > optin - 1024) return 0;
+        for (int k = 0; k < 8; ++k)
+            if (cudaFuncSetAttribute(cl_fn(1 << (k & 3), k >> 2), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                cudaFuncSetAttribute(cl_fn(1 << (k & 3), k >> 2), cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
+                cudaGetLastError();
+                return 0;
+            }
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(CL_SIZE);
+        cfg.blockDim = dim3(CL_THREADS);
+        cfg.dynamicSmemBytes = (size_t)want;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = CL_SIZE; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaOccupancyMaxActiveClusters(&n, cl_fn(8, WIND_ACT_RELU), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+        if (n > 0) g_cl_clusters[dev] = n;
+    }
+    return g_cl_clusters[dev] > 0 ? g_cl_clusters[dev] : 0;
+}
+
+// The shapes whose decoder fits one cluster: one LSTM layer, P and H multiples of 128 (a CTA's share is then whole 16-byte
+// pieces, and the K halves are equal) up to 640, at most 72 vocabulary entries per CTA, windows up to 32 rows.  Everything
+// else, and the FULL features (logits store, window-based decoding, timeline, forced loop modes), stays with loop_kernel.
+bool cl_supported(const Call& c) {
+    const wind_model_t& m = c.m;
+    const int nv = m.V + 1;
+    if (m.L != 1 || m.P % 128 || m.H % 128 || m.P > CL_MAX_DIM || m.H > CL_MAX_DIM || c.W > 32) return false;
+    if (cl_label_base(nv) + (cl_label_extra(nv) > 0 ? 8 : 0) > CL_MAX_LABELS) return false;
+    if (c.mode != WIND_MODE_FIRST_NONBLANK || c.joint_iters > 0) return false;
+    const LoopOptions o = loop_get_options();
+    if (!o.resident || o.dataflow >= 0 || o.joint_placement >= 0) return false;
+    return cl_clusters() > 0;
+}
+
+cudaError_t cl_loop(const Call& c) {
+    const wind_model_t& m = c.m;
+    const int n = c.N > 0 ? c.N : c.B;
+    ClParams p{};
+    p.ctrl = c.ctrl();
+    p.T = c.T; p.W = c.W; p.S = c.S; p.max_out = c.max_out; p.H = m.H; p.P = m.P; p.NV = m.V + 1; p.blank = m.blank_id;
+    p.n_utt = n;
+    p.wp = c.W <= 8 ? 8 : (c.W <= 16 ? 16 : 32);
+    // one slot per cluster as long as there are clusters, then more slots (a lock step of eight slots costs less than two of one)
+    const int most = 8 * CL_GROUPS / p.wp;
+    const int avail = cl_clusters();
+    const int clusters = n < avail ? n : avail;
+    if (clusters < 1) return cudaErrorNotSupported;
+    p.slots = (n + clusters - 1) / clusters < most ? (n + clusters - 1) / clusters : most;
+    const int ns = p.slots <= 1 ? 1 : (p.slots <= 2 ? 2 : (p.slots <= 4 ? 4 : 8));
+    p.queue_base = n < c.B ? n : c.B;
+    long long cap = (long long)c.T * (c.S + 1) + 2;
+    cap = (cap + 1) * n;                      // at worst one utterance after the other in one slot
+    p.step_cap = cap > 0x7fffffff ? 0x7fffffff : (int)cap;
+    p.extra_arrivals = loop_extra_arrivals();
+    p.enc_len = c.enc_len;
+    p.g0 = c.g0();
+    p.w_hh = (const __nv_bfloat16*)c.w_hh[0]; p.w_pred = (const __nv_bfloat16*)m.w_pred; p.w_out = (const __nv_bfloat16*)m.w_out;
+    p.b_pred = m.b_pred; p.b_out = m.b_out;
+    p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
+    if (n > p.slots * clusters && n <= CL_ORDER_MAX && sizeof(int32_t) * (size_t)n <= sizeof(float) * 2 * (size_t)c.B * m.P) {
+        int32_t* order = reinterpret_cast<int32_t*>(c.h(0));     // the plain-ALU path's state: not used by a bf16 tensor decode
+        cl_order_kernel<<<(n + 1023) / 1024, 1024, 0, c.stream>>>(c.enc_len, n, order);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
+        p.order = order;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(clusters * CL_SIZE));
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = cl_smem_bytes(m.P, m.H, p.NV, p.slots, p.wp);
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL_SIZE; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    CUtensorMap enc_map;
+    cudaError_t e = loop_map3(&enc_map, c.enc_proj(), (uint64_t)n * c.T, m.H, 8);
+    if (e != cudaSuccess) return e;
+    void* args[2] = {(void*)&enc_map, (void*)&p};
+    return cudaLaunchKernelExC(&cfg, cl_fn(ns, m.act), args);
+}
+
+}  // namespace wind

@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
     const int cta = blockIdx.x, G = gridDim.x;
     // a length outside [0, T] (found by the init kernel, which ran before this launch): the status is set, no CTA starts
     if (p.ctrl->bad_input) return;
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align_smem_1024(smem_raw);
     uint8_t* stat = smem;                       // this CTA's resident weight tile: kb_p blocks of 64 rows x 64 columns
     uint8_t* buf0 = smem + p.buf_off;           // the per-step state box
     float* stage_f = reinterpret_cast<float*>(smem + p.stage_off);   // epilogue staging

@@ -117,7 +117,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
     const uint32_t el = lane == 0;   // the lane that executes the CTA-level instructions of an issuing warp
     constexpr uint32_t b_stage_bytes = GEMM_BN * BK * 2;
     constexpr uint32_t stage_bytes = A_STAGE_BYTES + b_stage_bytes;
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align_smem_1024(smem_raw);
 
     // 1-D grid, column tile fastest so that the CTAs sharing a row tile run together
     const int n_tiles = (p.N + GEMM_BN - 1) / GEMM_BN;
@@ -298,7 +298,7 @@ enc_proj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
 
     const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
     const uint32_t el = lane == 0;   // the lane that executes the CTA-level instructions of an issuing warp
-    uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
+    uint8_t* smem = align_smem_1024(smem_raw);
     if (p.ctrl->bad_input) return;   // a length outside [0, T]: nothing is read through it
 
     if (threadIdx.x == 0) {

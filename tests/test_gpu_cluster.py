@@ -1,0 +1,38 @@
+"""The cluster kernel of the decoding loop (one-layer models whose decoder fits sixteen CTAs): edges of its tiles.
+
+Every case is decoded in the default mode, which picks the cluster kernel for these shapes, and with the grid-barrier
+kernel; the two use the same arithmetic, so the transcripts must be equal bit for bit, and the first is also checked
+against the oracle under the margin rule of the parity tests.
+"""
+import numpy as np
+import pytest
+
+from conftest import set_loop_mode
+from test_gpu_parity import check_against_oracle, pkg, ragged_case  # noqa: F401
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("N,T,P,H,V,act,W,S", [
+    (1, 40, 128, 128, 127, 0, 1, 3),       # smallest dimensions, eight vocabulary entries per CTA, one row
+    (3, 40, 640, 640, 1024, 0, 8, 10),     # the large model: remainder units, one CTA with eight more labels, one slot per cluster
+    (13, 30, 512, 640, 1151, 1, 8, 2),     # no remainder units; 72 labels in every CTA; two slots
+    (9, 30, 640, 128, 300, 0, 16, 2),      # padded window of 16
+    (25, 24, 256, 384, 1000, 1, 5, 3),     # four slots, six K blocks, odd window
+    (50, 24, 640, 512, 1030, 0, 4, 2),     # eight slots
+    (109, 20, 640, 640, 140, 0, 8, 3),     # sixteen slots; some CTAs without a label
+    (200, 16, 128, 640, 513, 1, 2, 2),     # more utterances than slots: the queue, longest first
+    (40, 20, 384, 256, 200, 0, 32, 3),     # widest window: four slots of 32 rows, refilled
+    (17, 20, 640, 640, 1024, 1, 11, 1),    # every emission forces an advance
+])
+def test_cluster_kernel_edges(pkg, N, T, P, H, V, act, W, S):  # noqa: F811
+    w, enc, lens = ragged_case(900 + N + W, B=N, T=T, D=64, E=64, P=P, L=1, H=H, V=V, act=act,
+                               blank_id=0 if N % 2 else None, bias=1.5, dtype="bf16")
+    rep, out = check_against_oracle(pkg, w, enc, lens, W, S, kernels=2)
+    set_loop_mode(pkg, "barriers")
+    model = pkg.WindModel(w)
+    tok, frm, olen, stats, st = pkg.decode(model, enc, lens, W, S)
+    assert st == 0 and stats["tokens"] == rep["stats"]["tokens"] and stats["jump_hist"] == rep["stats"]["jump_hist"]
+    for a, b in zip((tok, frm, olen), out):
+        assert np.array_equal(a, b)
