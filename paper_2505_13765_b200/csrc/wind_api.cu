@@ -179,6 +179,12 @@ static wind_status_t enqueue_decode(Call& c) {
         WIND_CUDA(tc_loop(c, nullptr, 0, nullptr, nullptr, g_trace_step));
         return WIND_OK;
     }
+    if (simt_loop_supported(c)) {
+        WIND_CUDA(launch_init(c, WIND_KERNELS_SIMT, 0, 3));
+        WIND_CUDA(simt_enc_proj(c));
+        WIND_CUDA(simt_loop(c));
+        return WIND_OK;
+    }
     const int per_step = 2 + simt_pred_launches(c);
     const int setup = 2 + simt_pred_launches(c);
     WIND_CUDA(launch_init(c, WIND_KERNELS_SIMT, per_step, setup));

@@ -69,6 +69,7 @@ struct Layout {
     size_t pred_proj;  // fp32 [B][H]        (plain-ALU path)
     size_t hb;         // bf16 [2][L][Bpad][P] LSTM hidden state as tensor-core operand rows (tensor path)
     size_t z;          // bf16 [rows_pad][H] joint activations act(enc_proj + pred_proj), the joint GEMM's operand (tensor path)
+    size_t zf;         // fp32 [rows_pad][H] joint activations of fp32 models
     size_t dh;         // fp32 [B][4P] layer 1's recurrent term, handed from its CTAs to the layer's update (tensor path, L >= 2)
     size_t g0;         // fp32 [V+1][4P] layer-0 gate pre-activations of every token: W_ih emb[tok] + b_ih + b_hh (tensor path)
     size_t trace;      // TraceEvent [kTraceRoles][kTraceEvents]: optional timeline of CTA 0 of the loop kernel
@@ -106,6 +107,7 @@ inline Layout make_layout(const wind_model_t& m, int B, int T, int W, int max_ou
     L.Bpad = (B + 127) / 128 * 128;
     L.hb = take(bf ? 2 * (size_t)m.L * L.Bpad * m.P * 2 : 0);
     L.z = take(bf ? (size_t)L.rows_pad * m.H * 2 : 0);
+    L.zf = take(bf ? 0 : sizeof(float) * (size_t)L.rows_pad * m.H);
     L.dh = take(bf && m.L >= 2 ? sizeof(float) * (size_t)B * 4 * m.P : 0);
     L.g0 = take(bf ? sizeof(float) * (size_t)(m.V + 1) * 4 * m.P : 0);
     L.trace = take(bf ? sizeof(TraceEvent) * kTraceRoles * kTraceEvents : 0);
@@ -161,6 +163,7 @@ struct Call {
     float* pred_proj() const { return reinterpret_cast<float*>(ws + lay.pred_proj); }
     void* enc_proj() const { return ws + lay.enc_proj; }
     __nv_bfloat16* z() const { return reinterpret_cast<__nv_bfloat16*>(ws + lay.z); }
+    float* zf() const { return reinterpret_cast<float*>(ws + lay.zf); }
     float* g0() const { return reinterpret_cast<float*>(ws + lay.g0); }
     float* dh() const { return reinterpret_cast<float*>(ws + lay.dh); }
     float2* jpart() const { return reinterpret_cast<float2*>(ws + lay.jpart); }
@@ -203,6 +206,8 @@ cudaError_t simt_pred_step(const Call& c, int parity_in);            // all laye
 cudaError_t simt_joint(const Call& c, float* logits_out /*nullable*/);
 cudaError_t simt_joint_shared(const Call& c, float* logits_out);   // every row's window comes from utterance 0 (beam search)
 int simt_pred_launches(const Call& c);
+bool simt_loop_supported(const Call& c);   // the decoding loop as one persistent kernel (wind_simt_loop.cu)
+cudaError_t simt_loop(const Call& c);
 
 // control
 cudaError_t launch_init(const Call& c, int kernels_used, int launches_per_step, int launches_setup);

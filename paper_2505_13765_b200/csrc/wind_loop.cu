@@ -275,10 +275,13 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                 const uint32_t a_addr = smem_u32(ring + (size_t)cur * sb_lp);
                 const uint64_t adesc = smem_desc_sw128(a_addr);
                 const uint64_t bdesc = smem_desc_sw128(a_addr + LOOP_A_BYTES);
+                if (elect_one()) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tm_l, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
-                tc_commit(&empty_bar[cur], el);
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_bf16(tm_l, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
+                    tc_commit(&empty_bar[cur]);
+                }
+                __syncwarp();
                 cur = cur + 1 == S_lp ? 0 : cur + 1;
             }
             tc_commit(&acc_full[1], el);
@@ -508,22 +511,25 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
         if (!consume()) return false;
         const uint32_t b_addr = smem_u32(ring);
         const uint32_t b_block = (uint32_t)n_tile * BK * 2;
-        for (int kb = kb_lo; kb < kb_hi; ++kb) {
-            const uint64_t bdesc = smem_desc_sw128(b_addr + (uint32_t)kb * b_block);
-            if (a_tmem) {
+        if (elect_one()) {
+            for (int kb = kb_lo; kb < kb_hi; ++kb) {
+                const uint64_t bdesc = smem_desc_sw128(b_addr + (uint32_t)kb * b_block);
+                if (a_tmem) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16_ts(tm_d, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
-                                   kb != kb_lo || k != 0, el);
-            } else {
-                const uint64_t adesc = smem_desc_sw128(smem_u32(stat + (size_t)kb * RES_A_BYTES));
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_bf16_ts(tm_d, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
+                                       kb != kb_lo || k != 0);
+                } else {
+                    const uint64_t adesc = smem_desc_sw128(smem_u32(stat + (size_t)kb * RES_A_BYTES));
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0, el);
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0);
+                }
             }
+            tc_commit(&empty_bar[0]);
+            tc_commit(&acc_full[k_acc]);
         }
-        tc_commit(&empty_bar[0], el);
-        tc_commit(&acc_full[k_acc], el);
+        __syncwarp();
         ++acc_n[k_acc];
         return true;
     };
@@ -1147,10 +1153,13 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                             const uint32_t a_addr = smem_u32(ring + (size_t)cur * sb_lp);
                             const uint64_t adesc = smem_desc_sw128(a_addr);
                             const uint64_t bdesc = smem_desc_sw128(a_addr + LOOP_A_BYTES);
+                            if (elect_one()) {
 #pragma unroll
-                            for (int k = 0; k < BK / 16; ++k)
-                                tc_mma_bf16(tm_p, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
-                            tc_commit(&empty_bar[cur], el);
+                                for (int k = 0; k < BK / 16; ++k)
+                                    tc_mma_bf16(tm_p, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
+                                tc_commit(&empty_bar[cur]);
+                            }
+                            __syncwarp();
                             cur = cur + 1 == S_lp ? 0 : cur + 1;
                         }
                         if (ok) { tc_commit(&acc_full[2], el); ++acc_n[2]; }
@@ -1411,21 +1420,24 @@ joint_only_entry:
                             if (!consume()) { ok = false; break; }
                             if (kb == 0) if constexpr (FULL) if (el) trace_event(p, 1, tr_n, step, TR_J, EV_FIRST_DATA);
                             const uint32_t st_addr = smem_u32(ring + (size_t)cur * sb_j);
-                            if (p.j_mode == J_TMEM) {
-                                const uint64_t bdesc = smem_desc_sw128(st_addr);
+                            if (elect_one()) {
+                                if (p.j_mode == J_TMEM) {
+                                    const uint64_t bdesc = smem_desc_sw128(st_addr);
 #pragma unroll
-                                for (int k = 0; k < BK / 16; ++k)
-                                    tc_mma_bf16_ts(tm_j, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
-                                                   (kb | k) != 0, el);
-                            } else {
-                                const uint64_t adesc =
-                                    smem_desc_sw128(p.j_mode == J_SMEM ? smem_u32(stat + (size_t)kb * LOOP_A_BYTES) : st_addr);
-                                const uint64_t bdesc = smem_desc_sw128(p.j_mode == J_SMEM ? st_addr : st_addr + LOOP_A_BYTES);
+                                    for (int k = 0; k < BK / 16; ++k)
+                                        tc_mma_bf16_ts(tm_j, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
+                                                       (kb | k) != 0);
+                                } else {
+                                    const uint64_t adesc =
+                                        smem_desc_sw128(p.j_mode == J_SMEM ? smem_u32(stat + (size_t)kb * LOOP_A_BYTES) : st_addr);
+                                    const uint64_t bdesc = smem_desc_sw128(p.j_mode == J_SMEM ? st_addr : st_addr + LOOP_A_BYTES);
 #pragma unroll
-                                for (int k = 0; k < BK / 16; ++k)
-                                    tc_mma_bf16(tm_j, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0, el);
+                                    for (int k = 0; k < BK / 16; ++k)
+                                        tc_mma_bf16(tm_j, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
+                                }
+                                tc_commit(&empty_bar[cur]);
                             }
-                            tc_commit(&empty_bar[cur], el);
+                            __syncwarp();
                             cur = cur + 1 == S_j ? 0 : cur + 1;
                         }
                         if (ok) { tc_commit(&acc_full[0], el); ++acc_n[0]; if constexpr (FULL) if (el) trace_event(p, 1, tr_n, step, TR_J, EV_COMMIT); }

@@ -299,22 +299,25 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
         tc_fence_after();
         const uint32_t b_addr = smem_u32(b_smem);
         const uint32_t b_block = (uint32_t)n_tile * BK * 2;
-        for (int kb = kb_lo; kb < kb_hi; ++kb) {
-            const uint64_t bdesc = smem_desc_sw128(b_addr + (uint32_t)kb * b_block);
-            if (a_tmem) {
+        if (elect_one()) {
+            for (int kb = kb_lo; kb < kb_hi; ++kb) {
+                const uint64_t bdesc = smem_desc_sw128(b_addr + (uint32_t)kb * b_block);
+                if (a_tmem) {
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16_ts(tm_d, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
-                                   kb != kb_lo || k != 0, el);
-            } else {
-                const uint64_t adesc = smem_desc_sw128(smem_u32(stat + (size_t)kb * RES_A_BYTES));
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_bf16_ts(tm_d, tmem_base + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc,
+                                       kb != kb_lo || k != 0);
+                } else {
+                    const uint64_t adesc = smem_desc_sw128(smem_u32(stat + (size_t)kb * RES_A_BYTES));
 #pragma unroll
-                for (int k = 0; k < BK / 16; ++k)
-                    tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0, el);
+                    for (int k = 0; k < BK / 16; ++k)
+                        tc_mma_bf16(tm_d, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, kb != kb_lo || k != 0);
+                }
             }
+            tc_commit(&empty_bar[sidx]);
+            tc_commit(&acc_full[k_acc]);
         }
-        tc_commit(&empty_bar[sidx], el);
-        tc_commit(&acc_full[k_acc], el);
+        __syncwarp();
         ++acc_n[k_acc];
         return true;
     };
