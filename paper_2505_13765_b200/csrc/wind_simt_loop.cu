@@ -2,7 +2,7 @@
 //
 // As separate kernels in a CUDA graph a lock step cost 20 us for a model of 64 units (launches) and 300 us for one of 640
 // units in fp32 (every weight read again by kernels with one block per output).  Here the weights stay in shared memory:
-//   LOCAL   the whole decoder fits one SM (64 units in fp32: 155 KB): a CTA decodes its utterances one after the other and
+//   one SM  the whole decoder fits one SM (64 units in fp32: 155 KB): a CTA decodes its utterances one after the other and
 //           nothing leaves the SM but the transcripts; the phases of a step are separated by block barriers.
 //   grid    otherwise: hidden units, joint units and labels are dealt out over all SMs (640 units in fp32: 117 KB each), and
 //           the phases are separated by grid barriers (1.3 us each).  Models whose weights do not fit on the chip run the
@@ -45,7 +45,7 @@ struct SimtLoopParams {
     const float* b_out;
     const void* enc_proj;
     const int32_t* enc_len;
-    float* h;                      // [2][L][B][P], a parity per utterance          (grid mode; LOCAL: shared memory)
+    float* h;                      // [2][L][B][P], a parity per utterance
     float* c;                      // [L][B][P]
     void* z;                       // [B * W][H]
     unsigned long long* keys;      // [2][B * W]
@@ -132,10 +132,10 @@ struct SlShare { int units, prows, labels; };
 __host__ __device__ inline SlShare sl_share(int P, int H, int NV, int G, int cta) {
     return SlShare{(P - cta + G - 1) / G, (H - cta + G - 1) / G, (NV - cta + G - 1) / G};
 }
-// Shared memory of a CTA in bytes: weights (resident), partial sums, per-utterance state, and in LOCAL mode the exchanged data.
+// Shared memory of a CTA in bytes: weights (resident), partial sums, per-utterance state, biases.
 struct SlSmem { size_t w_lstm0, w_lstm1, w_lstm_layer, w_pred,   // layer 0's rows, layer 1's, bytes of a further layer
-                        w_out, part, pred, key, ints, h, c, z, total; };
-__host__ __device__ inline SlSmem sl_smem(int es, int B, int W, int E, int P, int L, int H, int NV, int G, bool resident, bool local) {
+                        w_out, part, pred, key, ints, b_gate, b_pred, b_out, total; };
+__host__ __device__ inline SlSmem sl_smem(int es, int B, int W, int E, int P, int L, int H, int NV, int G, bool resident) {
     const SlShare s = sl_share(P, H, NV, G, 0);
     SlSmem m{};
     size_t off = 0;
@@ -151,32 +151,34 @@ __host__ __device__ inline SlSmem sl_smem(int es, int B, int W, int E, int P, in
     m.pred = take(sizeof(float) * (size_t)s.prows * B);
     m.key = take(sizeof(unsigned long long) * (size_t)B * W);
     m.ints = take(sizeof(int) * 7 * (size_t)B);
-    m.h = take(local ? sizeof(float) * 2 * (size_t)L * P : 0);
-    m.c = take(local ? sizeof(float) * (size_t)L * P : 0);
-    m.z = take(local ? (size_t)es * W * H : 0);
+    m.b_gate = take(sizeof(float) * (size_t)L * s.units * 4);
+    m.b_pred = take(sizeof(float) * (size_t)s.prows);
+    m.b_out = take(sizeof(float) * (size_t)s.labels);
     m.total = off;
     return m;
 }
 
-template <typename TW, bool LOCAL, bool VEC>
-__global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoopParams p) {
+template <typename TW, bool VEC>
+__global__ void __launch_bounds__(SL_THREADS, 1) simt_grid_kernel(const SimtLoopParams p) {
     extern __shared__ __align__(16) uint8_t sm[];
-    __shared__ int s_stop, s_n_emit, s_n_alive, s_red[2];
+    __shared__ int s_stop, s_n_emit, s_n_alive;
     __shared__ int s_hist[65];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int G = LOCAL ? 1 : gridDim.x, cta = LOCAL ? 0 : blockIdx.x;
+    const int G = gridDim.x, cta = blockIdx.x;
     if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
-    const int B = LOCAL ? 1 : p.B;
+    const int B = p.B;
     const SlShare own = sl_share(p.P, p.H, p.NV, G, cta);
-    const SlSmem M = sl_smem((int)sizeof(TW), B, p.W, p.E, p.P, p.L, p.H, p.NV, G, p.resident != 0, LOCAL);
+    const SlSmem M = sl_smem((int)sizeof(TW), B, p.W, p.E, p.P, p.L, p.H, p.NV, G, p.resident != 0);
     float* part = reinterpret_cast<float*>(sm + M.part);
     float* s_pred = reinterpret_cast<float*>(sm + M.pred);                     // [utterance][own joint unit]
     unsigned long long* s_key = reinterpret_cast<unsigned long long*>(sm + M.key);
     int* s_t = reinterpret_cast<int*>(sm + M.ints);
     int *s_len = s_t + B, *s_cnt = s_t + 2 * B, *s_pos = s_t + 3 * B, *s_tok = s_t + 4 * B, *s_hp = s_t + 5 * B, *s_list = s_t + 6 * B;
-    TW* z = LOCAL ? reinterpret_cast<TW*>(sm + M.z) : static_cast<TW*>(p.z);
-    float* h = LOCAL ? reinterpret_cast<float*>(sm + M.h) : p.h;
-    float* c = LOCAL ? reinterpret_cast<float*>(sm + M.c) : p.c;
+    TW* z = static_cast<TW*>(p.z);
+    float *h = p.h, *c = p.c;
+    float* s_bg = reinterpret_cast<float*>(sm + M.b_gate);                     // [layer][own unit][gate] b_ih + b_hh
+    float* s_bp = reinterpret_cast<float*>(sm + M.b_pred);
+    float* s_bo = reinterpret_cast<float*>(sm + M.b_out);
     const TW* emb = static_cast<const TW*>(p.emb);
     const TW* enc_proj = static_cast<const TW*>(p.enc_proj);
 
@@ -203,14 +205,19 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
         for (int i = warp; i < own.labels; i += SL_WARPS)
             copy_row(reinterpret_cast<TW*>(sm + M.w_out) + (size_t)i * p.H, static_cast<const TW*>(p.w_out) + ((size_t)i * G + cta) * p.H, p.H);
     }
+    for (int i = threadIdx.x; i < p.L * own.units * 4; i += SL_THREADS) {
+        const int l = i / (own.units * 4), j = (i / 4) % own.units, g = i & 3;
+        s_bg[i] = p.b_ih[l][g * p.P + j * G + cta] + p.b_hh[l][g * p.P + j * G + cta];
+    }
+    for (int i = threadIdx.x; i < own.prows; i += SL_THREADS) s_bp[i] = p.b_pred[i * G + cta];
+    for (int i = threadIdx.x; i < own.labels; i += SL_THREADS) s_bo[i] = p.b_out[i * G + cta];
     if (threadIdx.x == 0) s_stop = 0;
     for (int k = threadIdx.x; k < 65; k += SL_THREADS) s_hist[k] = 0;
 
-    // Barrier between phases: the block, or all CTAs.  False when the kernel is being abandoned (bounded wait).
+    // Barrier of all CTAs between phases.  False when the kernel is being abandoned (bounded wait).
     uint32_t epoch = 0;
     auto phase_sync = [&]() -> bool {
         __syncthreads();
-        if (LOCAL) return true;
         if (threadIdx.x == 0) {
             epoch += (uint32_t)(G + p.extra_arrivals);
             __threadfence();
@@ -230,10 +237,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
         __syncthreads();
         return s_stop == 0;
     };
-    auto fetch = [&](const auto* row, int k, int n) -> float4 {                 // data of this step from another warp or CTA
-        if constexpr (LOCAL) return sl_row4<VEC>(row, k, n);
-        else return sl_shared4<VEC>(row, k, n);
-    };
+    auto fetch = [&](const auto* row, int k, int n) -> float4 { return sl_shared4<VEC>(row, k, n); };   // data of this step from another CTA
     auto h_row = [&](int par, int l, int b) { return h + (((size_t)par * p.L + l) * B + b) * p.P; };
 
     // NB utterances s_list[i0 ..): partial sums of this CTA's hidden units in layer l
@@ -305,19 +309,14 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
         }
     };
 
-    // LOCAL: this CTA's utterances one after the other; grid: all utterances in one pass
-    for (int u0 = LOCAL ? (int)blockIdx.x : 0; u0 < (LOCAL ? p.B : 1); u0 += LOCAL ? (int)gridDim.x : 1) {
+    {
         // ---- start of sequence ----
         __syncthreads();
         for (int b = threadIdx.x; b < B; b += SL_THREADS) {
             s_t[b] = 0;
-            s_len[b] = min(max(p.enc_len[u0 + b], 0), p.T);
+            s_len[b] = min(max(p.enc_len[b], 0), p.T);
             s_cnt[b] = 0; s_pos[b] = 0; s_hp[b] = 0;
             s_tok[b] = s_len[b] > 0 ? p.blank : -1;
-        }
-        if (LOCAL) {
-            for (int i = threadIdx.x; i < 2 * p.L * p.P; i += SL_THREADS) h[i] = 0.f;
-            for (int i = threadIdx.x; i < p.L * p.P; i += SL_THREADS) c[i] = 0.f;
         }
         for (int i = threadIdx.x; i < B * p.W; i += SL_THREADS) s_key[i] = 0ull;
         __syncthreads();
@@ -328,7 +327,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
             // control: decisions for every utterance, in every CTA; lists of emitting and of live utterances
             // =============================================================================
             if (step >= 0) {
-                const unsigned long long* keys = LOCAL ? s_key : p.keys + (size_t)(step & 1) * B * p.W;
+                const unsigned long long* keys = p.keys + (size_t)(step & 1) * B * p.W;
                 for (int b = threadIdx.x; b < B; b += SL_THREADS) {
                     int t = s_t[b], tok = -1;
                     const int len = s_len[b];
@@ -342,9 +341,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                             for (int j = 0; j < 4; ++j) {
                                 kk[j] = 0ull;
                                 if (w0 + j < n) {
-                                    const unsigned long long* kp = keys + (size_t)b * p.W + w0 + j;
-                                    if constexpr (LOCAL) kk[j] = *kp;
-                                    else kk[j] = __ldcg(kp);
+                                    kk[j] = __ldcg(keys + (size_t)b * p.W + w0 + j);
                                 }
                             }
 #pragma unroll
@@ -373,11 +370,11 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                         }
                         s_t[b] = t;
                         s_cnt[b] = cnt;
-                        if (LOCAL || blockIdx.x == 0) {                           // recorded once
+                        if (blockIdx.x == 0) {                           // recorded once
                             if (tok >= 0) {
-                                p.out_tokens[(size_t)(u0 + b) * p.max_out + pos] = label;
-                                p.out_frames[(size_t)(u0 + b) * p.max_out + pos] = t_emit;
-                                p.out_len[u0 + b] = pos + 1;
+                                p.out_tokens[(size_t)b * p.max_out + pos] = label;
+                                p.out_frames[(size_t)b * p.max_out + pos] = t_emit;
+                                p.out_len[b] = pos + 1;
                             }
                             n_rows += n; n_tok += tok >= 0; n_forced += forced;
                             atomicAdd(&s_hist[jump < 64 ? jump : 64], 1);
@@ -406,7 +403,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
             __syncthreads();
             const int n_emit = s_n_emit;
             if (s_n_alive == 0) break;
-            if (steps >= p.step_cap) { if (threadIdx.x == 0 && (LOCAL || blockIdx.x == 0)) set_status(p.ctrl, WIND_ERR_INTERNAL); break; }
+            if (steps >= p.step_cap) { if (threadIdx.x == 0 && blockIdx.x == 0) set_status(p.ctrl, WIND_ERR_INTERNAL); break; }
             // =============================================================================
             // update and projection of the emitting utterances
             // =============================================================================
@@ -415,7 +412,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                     const int KS = own.units > 0 && own.units < SL_WARPS ? SL_WARPS / own.units : 1;
                     for (int i0 = 0; i0 < n_emit; i0 += SL_UTTS) {
                         const int n_here = min(SL_UTTS, n_emit - i0);
-                        if (LOCAL || n_here == 1) update_partials(std::integral_constant<int, 1>{}, l, i0, n_here, KS);
+                        if (n_here == 1) update_partials(std::integral_constant<int, 1>{}, l, i0, n_here, KS);
                         else update_partials(std::integral_constant<int, SL_UTTS>{}, l, i0, n_here, KS);
                         __syncthreads();
                         for (int i = threadIdx.x; i < own.units * n_here; i += SL_THREADS) {
@@ -425,7 +422,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                             for (int g = 0; g < 4; ++g) {
                                 float s = 0.f;
                                 for (int ks = 0; ks < KS; ++ks) s += part[(size_t)(ks * own.units + ui) * (4 * SL_UTTS) + g * SL_UTTS + u];
-                                a[g] = s + (p.b_ih[l][g * p.P + j] + p.b_hh[l][g * p.P + j]);
+                                a[g] = s + s_bg[(l * own.units + ui) * 4 + g];
                             }
                             const float gi = 1.f / (1.f + expf(-a[0])), gf = 1.f / (1.f + expf(-a[1])), gg = tanhf(a[2]), go = 1.f / (1.f + expf(-a[3]));
                             float* cs = c + ((size_t)l * B + b) * p.P + j;
@@ -440,14 +437,14 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                 const int KS = own.prows > 0 && own.prows < SL_WARPS ? SL_WARPS / own.prows : 1;
                 for (int i0 = 0; i0 < n_emit; i0 += SL_UTTS) {
                     const int n_here = min(SL_UTTS, n_emit - i0);
-                    if (LOCAL || n_here == 1) project_partials(std::integral_constant<int, 1>{}, i0, n_here, KS);
+                    if (n_here == 1) project_partials(std::integral_constant<int, 1>{}, i0, n_here, KS);
                     else project_partials(std::integral_constant<int, SL_UTTS>{}, i0, n_here, KS);
                     __syncthreads();
                     for (int i = threadIdx.x; i < own.prows * n_here; i += SL_THREADS) {
                         const int pi = i / n_here, u = i - pi * n_here;
                         float s = 0.f;
                         for (int ks = 0; ks < KS; ++ks) s += part[(size_t)(ks * own.prows + pi) * SL_UTTS + u];
-                        s_pred[(size_t)s_list[i0 + u] * own.prows + pi] = s + p.b_pred[pi * G + cta];
+                        s_pred[(size_t)s_list[i0 + u] * own.prows + pi] = s + s_bp[pi];
                     }
                     __syncthreads();
                 }
@@ -467,19 +464,19 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
             }
             __syncthreads();
             const int n_alive = s_n_alive;
-            unsigned long long* knext = LOCAL ? s_key : p.keys + (size_t)((step + 1) & 1) * B * p.W;
+            unsigned long long* knext = p.keys + (size_t)((step + 1) & 1) * B * p.W;
             for (int i = threadIdx.x; i < n_alive * p.W * own.prows; i += SL_THREADS) {
                 const int pi = i % own.prows, r = i / own.prows, b = s_list[r / p.W], w = r % p.W;
                 if (s_t[b] + w < s_len[b]) {
                     const int o = pi * G + cta;
-                    float v = (float)enc_proj[((size_t)(u0 + b) * p.T + s_t[b] + w) * p.H + o] + s_pred[(size_t)b * own.prows + pi];
+                    float v = (float)enc_proj[((size_t)b * p.T + s_t[b] + w) * p.H + o] + s_pred[(size_t)b * own.prows + pi];
                     v = p.act == WIND_ACT_RELU ? fmaxf(v, 0.f) : tanhf(v);
                     sl_store(z + ((size_t)b * p.W + w) * p.H + o, v);
                 }
             }
             for (int i = threadIdx.x; i < B * p.W; i += SL_THREADS) s_key[i] = 0ull;
             // (the other parity's keys were read by every CTA before the last barrier of the step before)
-            if (!LOCAL && blockIdx.x == 0)
+            if (blockIdx.x == 0)
                 for (int i = threadIdx.x; i < B * p.W; i += SL_THREADS) knext[i] = 0ull;
             if (!phase_sync()) goto done;
             // =============================================================================
@@ -524,7 +521,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                     unsigned long long key = 0ull;
                     if (lane < 16 && li < own.labels) {
                         const int v = li * G + cta;
-                        const float s = acc[0] + p.b_out[v];
+                        const float s = acc[0] + s_bo[li];
                         if (s > -INFINITY) key = pack_key(s, (uint32_t)v);
                     }
                     key = max(key, __shfl_xor_sync(0xffffffffu, key, 4));
@@ -535,14 +532,13 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
                     if (lane < SL_ROWS && sl >= 0 && key != 0ull) atomicMax(&s_key[sl], key);
                 }
                 __syncthreads();
-                if (!LOCAL)
-                    for (int i = threadIdx.x; i < B * p.W; i += SL_THREADS)
-                        if (s_key[i] != 0ull) atomicMax(&knext[i], s_key[i]);
+                for (int i = threadIdx.x; i < B * p.W; i += SL_THREADS)
+                    if (s_key[i] != 0ull) atomicMax(&knext[i], s_key[i]);
             }
             if (!phase_sync()) goto done;
         }
         // ---- counters ----
-        if (LOCAL || blockIdx.x == 0) {
+        if (blockIdx.x == 0) {
             if (threadIdx.x == 0) atomicMax(&p.ctrl->step, steps);
             if (n_rows) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->joint_rows), (unsigned long long)n_rows);
             if (n_tok) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->tokens), (unsigned long long)n_tok);
@@ -551,7 +547,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_loop_kernel(const SimtLoop
     }
 done:
     __syncthreads();
-    if (LOCAL || blockIdx.x == 0)
+    if (blockIdx.x == 0)
         for (int k = threadIdx.x; k < 65; k += SL_THREADS)
             if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
     if (threadIdx.x == 0) {
@@ -561,11 +557,246 @@ done:
 }
 
 // ---------------------------------------------------------------------------
+// The whole decoder inside one SM: a CTA decodes its utterances one after the other.  Everything is fp32 in shared memory
+// (bf16 operands converted once), rows padded with zeros to a multiple of four and behind that by four floats per thread of
+// a row, so that the 16-byte reads of neighbouring threads fall into different banks.  A row's dot product is cut over up to
+// eight neighbouring threads.  A step of the 64-unit fp32 model is bound by reading its 128 KB of gate weights (1000 cycles)
+// and by seven block barriers; in the grid form's code with one CTA it took 17000 cycles (8.6 us), 86 KB of instructions
+// against an instruction cache of 32 KB: 427 us for an utterance of 44 steps, here 234 us.
+// ---------------------------------------------------------------------------
+struct SlLocal {
+    int nin0, np, nh;                 // E, P, H rounded up to four
+    int lg_l, lg_p, lg_j;             // log2 of the threads per row: of the gates, of W_pred, of an output of the joint
+    int ld_l0, ld_l1, ld_p, ld_o;     // row pitches in floats
+    int w_l0, w_l1, w_l_layer, w_pred, w_out, emb, b_gate, b_pred, b_out, x, h, c, gates, pred, z, key;   // in floats
+    long long total;                  // in floats; the offsets mean something only where it fits shared memory
+};
+__host__ __device__ inline int sl_lg_tpr(int rows) { int l = 0; while (l < 3 && (rows << (l + 1)) <= SL_THREADS) ++l; return l; }
+__host__ __device__ inline SlLocal sl_local(int W, int E, int P, int L, int H, int NV, bool emb) {
+    SlLocal m{};
+    m.nin0 = (E + 3) & ~3; m.np = (P + 3) & ~3; m.nh = (H + 3) & ~3;
+    m.lg_l = sl_lg_tpr(4 * P); m.lg_p = sl_lg_tpr(H); m.lg_j = sl_lg_tpr(NV);
+    m.ld_l0 = m.nin0 + m.np + (4 << m.lg_l); m.ld_l1 = 2 * m.np + (4 << m.lg_l);
+    m.ld_p = m.np + (4 << m.lg_p); m.ld_o = m.nh + (4 << m.lg_j);
+    long long off = 0;
+    auto take = [&](long long n) { const long long o = off; off += (n + 3) & ~3ll; return (int)o; };
+    m.w_l0 = take(4ll * P * m.ld_l0);
+    m.w_l_layer = 4 * P * m.ld_l1;
+    m.w_l1 = take(4ll * P * m.ld_l1 * (L - 1));
+    m.w_pred = take((long long)H * m.ld_p);
+    m.w_out = take((long long)NV * m.ld_o);
+    m.emb = take(emb ? (long long)NV * m.nin0 : 0);
+    m.b_gate = take(4ll * L * P);
+    m.b_pred = take(H);
+    m.b_out = take(NV);
+    m.x = take(m.nin0);
+    m.h = take((long long)L * m.np);
+    m.c = take((long long)L * P);
+    m.gates = take(4ll * P);
+    m.pred = take(H);
+    m.z = take((long long)W * m.nh);
+    m.key = take(2ll * W);
+    m.total = off;
+    return m;
+}
+
+template <typename TW>
+__global__ void __launch_bounds__(SL_THREADS, 1) simt_local_kernel(const SimtLoopParams p, const int emb_here) {
+    extern __shared__ __align__(16) float sf[];
+    __shared__ int s_tok, s_t, s_more;
+    __shared__ int s_hist[65];
+    if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const SlLocal M = sl_local(p.W, p.E, p.P, p.L, p.H, p.NV, emb_here != 0);
+    // a matrix [rows][n] to column `at` of the padded rows at dst, with zeros up to the next multiple of four; a warp takes a row
+    auto load_rows = [&](float* dst, int ld, int at, const void* src_, int rows, int n) {
+        const TW* src = static_cast<const TW*>(src_);
+        const int n4 = (n + 3) & ~3;
+#pragma unroll 4
+        for (int row = warp; row < rows; row += SL_WARPS)
+            for (int k = lane; k < n4; k += 32) dst[row * ld + at + k] = k < n ? (float)src[(size_t)row * n + k] : 0.f;
+    };
+    for (int l = 0; l < p.L; ++l) {
+        float* dst = sf + (l == 0 ? M.w_l0 : M.w_l1 + (l - 1) * M.w_l_layer);
+        const int ld = l == 0 ? M.ld_l0 : M.ld_l1, nin = l == 0 ? p.E : p.P;
+        load_rows(dst, ld, 0, p.w_ih[l], 4 * p.P, nin);
+        load_rows(dst, ld, l == 0 ? M.nin0 : M.np, p.w_hh[l], 4 * p.P, p.P);
+        for (int i = tid; i < 4 * p.P; i += SL_THREADS) sf[M.b_gate + l * 4 * p.P + i] = p.b_ih[l][i] + p.b_hh[l][i];
+    }
+    load_rows(sf + M.w_pred, M.ld_p, 0, p.w_pred, p.H, p.P);
+    load_rows(sf + M.w_out, M.ld_o, 0, p.w_out, p.NV, p.H);
+    if (emb_here) load_rows(sf + M.emb, M.nin0, 0, p.emb, p.NV, p.E);
+    for (int i = tid; i < p.H; i += SL_THREADS) sf[M.b_pred + i] = p.b_pred[i];
+    for (int i = tid; i < p.NV; i += SL_THREADS) sf[M.b_out + i] = p.b_out[i];
+    for (int i = tid; i < 65; i += SL_THREADS) s_hist[i] = 0;
+    unsigned long long* s_key = reinterpret_cast<unsigned long long*>(sf + M.key);
+
+    // the share `part` of a dot product of two padded rows of n4 floats
+    auto dot = [&](const float* w, const float* x, int n4, int part, int lg, float acc) -> float {
+        float a1 = 0.f;
+#pragma unroll 4
+        for (int k = 4 * part; k < n4; k += 4 << lg) {
+            const float4 a = *reinterpret_cast<const float4*>(w + k), b = *reinterpret_cast<const float4*>(x + k);
+            acc = fmaf(a.y, b.y, fmaf(a.x, b.x, acc));
+            a1 = fmaf(a.w, b.w, fmaf(a.z, b.z, a1));
+        }
+        return acc + a1;
+    };
+    auto share_sum = [&](float v, int lg) {
+        for (int o = 1; o < 1 << lg; o <<= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        return v;
+    };
+    const TW* enc_proj = static_cast<const TW*>(p.enc_proj);
+    long long n_rows = 0, n_tok = 0, n_forced = 0;             // counts (the same in all lanes of warp 0)
+    int most_steps = 0;
+
+    for (int utt = blockIdx.x; utt < p.B; utt += gridDim.x) {
+        const int len = min(max(p.enc_len[utt], 0), p.T);
+        int cnt = 0, pos = 0, steps = 0, t = 0;                // the utterance's state (warp 0)
+        __syncthreads();
+        for (int i = tid; i < p.L * M.np; i += SL_THREADS) sf[M.h + i] = 0.f;
+        for (int i = tid; i < p.L * p.P; i += SL_THREADS) sf[M.c + i] = 0.f;
+        for (int i = tid; i < p.W; i += SL_THREADS) s_key[i] = 0ull;
+        if (tid == 0) { s_tok = p.blank; s_t = 0; s_more = len > 0; }
+        __syncthreads();
+        while (s_more) {
+            const int tok = s_tok, n = min(p.W, len - s_t);
+            const size_t row0 = (size_t)utt * p.T + s_t;
+            // this thread's first element of the window's enc_proj rows, requested before the decoder phases
+            const float z_enc = tid < n * p.H ? (float)enc_proj[row0 * p.H + tid] : 0.f;
+            if (tok >= 0) {
+                const float* x = sf + M.emb + tok * M.nin0;
+                if (!emb_here) {
+                    for (int k = tid; k < M.nin0; k += SL_THREADS) sf[M.x + k] = k < p.E ? (float)static_cast<const TW*>(p.emb)[(size_t)tok * p.E + k] : 0.f;
+                    x = sf + M.x;
+                    __syncthreads();
+                }
+                for (int l = 0; l < p.L; ++l) {
+                    const float* w = sf + (l == 0 ? M.w_l0 : M.w_l1 + (l - 1) * M.w_l_layer);
+                    const int ld = l == 0 ? M.ld_l0 : M.ld_l1, n_in = l == 0 ? M.nin0 : M.np, part = tid & ((1 << M.lg_l) - 1);
+                    const float* xl = l == 0 ? x : sf + M.h + (l - 1) * M.np;
+#pragma unroll 1
+                    for (int i = tid; i - lane < 4 * p.P << M.lg_l; i += SL_THREADS) {       // whole warps: threads past the end repeat the last row
+                        const int row = min(i >> M.lg_l, 4 * p.P - 1);
+                        const float* wr = w + row * ld;
+                        float v = dot(wr, xl, n_in, part, M.lg_l, 0.f);
+                        v = dot(wr + n_in, sf + M.h + l * M.np, M.np, part, M.lg_l, v);
+                        v = share_sum(v, M.lg_l);
+                        if (part == 0) sf[M.gates + row] = v + sf[M.b_gate + l * 4 * p.P + row];
+                    }
+                    __syncthreads();
+                    for (int j = tid; j < p.P; j += SL_THREADS) {
+                        const float* gt = sf + M.gates + j;
+                        const float gi = 1.f / (1.f + expf(-gt[0])), gf = 1.f / (1.f + expf(-gt[p.P])), gg = tanhf(gt[2 * p.P]), go = 1.f / (1.f + expf(-gt[3 * p.P]));
+                        float* cs = sf + M.c + l * p.P + j;
+                        const float cc = gf * *cs + gi * gg;
+                        *cs = cc;
+                        sf[M.h + l * M.np + j] = sl_round<TW>(go * tanhf(cc));
+                    }
+                    __syncthreads();
+                }
+                const int part = tid & ((1 << M.lg_p) - 1);
+#pragma unroll 1
+                for (int i = tid; i - lane < p.H << M.lg_p; i += SL_THREADS) {
+                    const int row = min(i >> M.lg_p, p.H - 1);
+                    const float v = share_sum(dot(sf + M.w_pred + row * M.ld_p, sf + M.h + (p.L - 1) * M.np, M.np, part, M.lg_p, 0.f), M.lg_p);
+                    if (part == 0) sf[M.pred + row] = v + sf[M.b_pred + row];
+                }
+                __syncthreads();
+            }
+#pragma unroll 1
+            for (int i = tid; i < n * M.nh; i += SL_THREADS) {
+                const int w = i / M.nh, k = i - w * M.nh;
+                float v = 0.f;
+                if (k < p.H) {
+                    v = (M.nh == p.H && i == tid ? z_enc : (float)enc_proj[(row0 + w) * p.H + k]) + sf[M.pred + k];
+                    v = sl_round<TW>(p.act == WIND_ACT_RELU ? fmaxf(v, 0.f) : tanhf(v));
+                }
+                sf[M.z + i] = v;
+            }
+            __syncthreads();
+            {
+                const int part = tid & ((1 << M.lg_j) - 1), outs = n * p.NV;
+#pragma unroll 1
+                for (int q = tid; q - lane < outs << M.lg_j; q += SL_THREADS) {
+                    const int i = min(q >> M.lg_j, outs - 1), w = i / p.NV, v = i - w * p.NV;
+                    const float s = share_sum(dot(sf + M.w_out + v * M.ld_o, sf + M.z + w * M.nh, M.nh, part, M.lg_j, 0.f), M.lg_j) + sf[M.b_out + v];
+                    unsigned long long key = s > -INFINITY ? pack_key(s, (uint32_t)v) : 0ull;
+                    if (__all_sync(0xffffffffu, w == __shfl_sync(0xffffffffu, w, 0))) {       // one row's outputs: one update for the warp
+#pragma unroll
+                        for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
+                        if (lane != 0) key = 0ull;
+                    } else if (part != 0) {
+                        key = 0ull;
+                    }
+                    if (key != 0ull) atomicMax(&s_key[w], key);
+                }
+            }
+            __syncthreads();
+            // control (Algorithm 2's branch) by warp 0: a lane looks at a window row and at the row 32 further on
+            if (warp == 0) {
+                const unsigned long long k0 = lane < n ? s_key[lane] : 0ull, k1 = lane + 32 < n ? s_key[lane + 32] : 0ull;
+                uint32_t l0 = key_label(k0), l1 = key_label(k1);
+                const bool bad0 = lane < n && (k0 == 0ull || l0 >= (uint32_t)p.NV), bad1 = lane + 32 < n && (k1 == 0ull || l1 >= (uint32_t)p.NV);
+                if (bad0 || lane >= n) l0 = (uint32_t)p.blank;
+                if (bad1 || lane + 32 >= n) l1 = (uint32_t)p.blank;
+                const uint32_t h0 = __ballot_sync(0xffffffffu, (int)l0 != p.blank), h1 = __ballot_sync(0xffffffffu, (int)l1 != p.blank);
+                const int first = h0 ? __ffs((int)h0) - 1 : (h1 ? 31 + __ffs((int)h1) : n);
+                const bool hit = (h0 | h1) != 0u;
+                const int label = (int)__shfl_sync(0xffffffffu, first < 32 ? l0 : l1, first & 31);
+                const bool bad = __any_sync(0xffffffffu, (bad0 && lane <= first) || (bad1 && lane + 32 <= first));
+                if (first > 0) cnt = 0;
+                t += first;
+                const int t_emit = t, at = pos;
+                const bool emit = hit && pos < p.max_out;
+                bool forced = false;
+                if (emit) {
+                    ++pos;
+                    if (++cnt == p.S) { ++t; cnt = 0; forced = true; }
+                } else if (hit) {
+                    t = len;                                                   // no room for the token: this utterance stops here
+                }
+                ++steps;
+                const bool stuck = steps >= p.step_cap && t < len;
+                n_rows += n; n_tok += emit; n_forced += forced;
+                if (lane == 0) {
+                    s_tok = emit ? label : -1;
+                    s_t = t;
+                    s_more = t < len && !stuck;
+                    s_hist[first] += 1;
+                    if (emit) {
+                        p.out_tokens[(size_t)utt * p.max_out + at] = label;
+                        p.out_frames[(size_t)utt * p.max_out + at] = t_emit;
+                    }
+                    if (hit && !emit) set_status(p.ctrl, WIND_ERR_OUTPUT_OVERFLOW);
+                    if (bad || stuck) set_status(p.ctrl, WIND_ERR_INTERNAL);
+                    if (t >= len || stuck) p.out_len[utt] = pos;
+                }
+                __syncwarp();
+                for (int w = lane; w < n; w += 32) s_key[w] = 0ull;
+            }
+            __syncthreads();
+        }
+        most_steps = max(most_steps, steps);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        atomicMax(&p.ctrl->step, most_steps);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->joint_rows), (unsigned long long)n_rows);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->tokens), (unsigned long long)n_tok);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->forced), (unsigned long long)n_forced);
+        if (blockIdx.x == 0) p.ctrl->active = 0;
+    }
+    for (int k = tid; k < 65; k += SL_THREADS)
+        if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-template <typename TW, bool LOCAL>
+template <typename TW>
 static const void* sl_fn(bool vec) {
-    return vec ? (const void*)simt_loop_kernel<TW, LOCAL, true> : (const void*)simt_loop_kernel<TW, LOCAL, false>;
+    return vec ? (const void*)simt_grid_kernel<TW, true> : (const void*)simt_grid_kernel<TW, false>;
 }
 
 static std::mutex g_sl_mutex;
@@ -582,9 +813,9 @@ static cudaError_t sl_device(int* optin) {
         int n = 0;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
         const int dyn = n - 1024;      // the kernels' static shared memory stays below 1 KB
-        for (bool vec : {false, true})
-            for (const void* fn : {sl_fn<float, true>(vec), sl_fn<float, false>(vec), sl_fn<__nv_bfloat16, true>(vec), sl_fn<__nv_bfloat16, false>(vec)})
-                if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)) != cudaSuccess) return e;
+        for (const void* fn : {sl_fn<float>(false), sl_fn<float>(true), sl_fn<__nv_bfloat16>(false), sl_fn<__nv_bfloat16>(true),
+                               (const void*)simt_local_kernel<float>, (const void*)simt_local_kernel<__nv_bfloat16>})
+            if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)) != cudaSuccess) return e;
         g_sl_optin[dev] = n;
     }
     *optin = g_sl_optin[dev];
@@ -592,41 +823,43 @@ static cudaError_t sl_device(int* optin) {
 }
 
 // Which form of the kernel a decode takes; false: none (window-based decoding, batches whose state does not fit)
-static bool sl_plan(const Call& c, bool* local, bool* resident, size_t* smem, int* grid) {
+static bool sl_plan(const Call& c, bool* local, bool* resident, bool* emb, size_t* smem, int* grid) {
     if (c.mode != WIND_MODE_FIRST_NONBLANK || c.B > SL_MAX_B) return false;
     int optin = 0, sms = 0;
     if (sl_device(&optin) != cudaSuccess || loop_sm_count(&sms) != cudaSuccess) { cudaGetLastError(); return false; }
     const wind_model_t& m = c.m;
     const int es = m.dtype == WIND_DT_BF16 ? 2 : 4;
     const size_t budget = (size_t)optin - 1024;
-    SlSmem s = sl_smem(es, 1, c.W, m.E, m.P, m.L, m.H, m.V + 1, 1, true, true);
-    if (s.total <= budget) {
+    const size_t one_sm = sizeof(float) * (size_t)sl_local(c.W, m.E, m.P, m.L, m.H, m.V + 1, false).total;
+    if (one_sm <= budget) {
         *local = *resident = true;
-        *smem = s.total;
+        *smem = sizeof(float) * (size_t)sl_local(c.W, m.E, m.P, m.L, m.H, m.V + 1, true).total;
+        *emb = *smem <= budget;        // the embedding table too where there is room, else its rows come from L2
+        if (!*emb) *smem = one_sm;
         *grid = c.B < sms ? c.B : sms;
         return true;
     }
-    *local = false;
+    *local = *emb = false;
     *grid = sms;
-    s = sl_smem(es, c.B, c.W, m.E, m.P, m.L, m.H, m.V + 1, sms, true, false);
+    SlSmem s = sl_smem(es, c.B, c.W, m.E, m.P, m.L, m.H, m.V + 1, sms, true);
     *resident = s.total <= budget;
-    if (!*resident) s = sl_smem(es, c.B, c.W, m.E, m.P, m.L, m.H, m.V + 1, sms, false, false);
+    if (!*resident) s = sl_smem(es, c.B, c.W, m.E, m.P, m.L, m.H, m.V + 1, sms, false);
     *smem = s.total;
     return s.total <= budget;
 }
 
 bool simt_loop_supported(const Call& c) {
-    bool local, resident;
+    bool local, resident, emb;
     size_t smem;
     int grid;
-    return sl_plan(c, &local, &resident, &smem, &grid);
+    return sl_plan(c, &local, &resident, &emb, &smem, &grid);
 }
 
 cudaError_t simt_loop(const Call& c) {
-    bool local, resident;
+    bool local, resident, emb;
     size_t smem;
     int grid;
-    if (!sl_plan(c, &local, &resident, &smem, &grid)) return cudaErrorNotSupported;
+    if (!sl_plan(c, &local, &resident, &emb, &smem, &grid)) return cudaErrorNotSupported;
     const wind_model_t& m = c.m;
     SimtLoopParams p{};
     p.ctrl = c.ctrl();
@@ -649,10 +882,14 @@ cudaError_t simt_loop(const Call& c) {
     p.enc_proj = c.enc_proj(); p.enc_len = c.enc_len;
     p.h = c.h(0); p.c = c.c(); p.z = m.dtype == WIND_DT_BF16 ? (void*)c.z() : (void*)c.zf(); p.keys = c.keys();
     p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
-    const void* fn = m.dtype == WIND_DT_BF16 ? (local ? sl_fn<__nv_bfloat16, true>(vec) : sl_fn<__nv_bfloat16, false>(vec))
-                                             : (local ? sl_fn<float, true>(vec) : sl_fn<float, false>(vec));
+    if (local) {
+        int emb_here = emb;
+        void* args[2] = {(void*)&p, (void*)&emb_here};
+        return cudaLaunchKernel(m.dtype == WIND_DT_BF16 ? (const void*)simt_local_kernel<__nv_bfloat16> : (const void*)simt_local_kernel<float>,
+                                dim3((unsigned)grid), dim3(SL_THREADS), args, smem, c.stream);
+    }
+    const void* fn = m.dtype == WIND_DT_BF16 ? sl_fn<__nv_bfloat16>(vec) : sl_fn<float>(vec);
     void* args[1] = {(void*)&p};
-    if (local) return cudaLaunchKernel(fn, dim3((unsigned)grid), dim3(SL_THREADS), args, smem, c.stream);
     return cudaLaunchCooperativeKernel(fn, dim3((unsigned)grid), dim3(SL_THREADS), args, smem, c.stream);
 }
 

@@ -13,6 +13,8 @@ pytestmark = pytest.mark.gpu
     ("f32", 1, 60, 64, 64, 64, 1, 64, 32, 0, 4, 5),        # one SM, one utterance
     ("f32", 150, 20, 20, 24, 24, 2, 40, 30, 1, 3, 2),      # one SM, more utterances than SMs, two layers
     ("f32", 5, 30, 17, 19, 21, 1, 33, 29, 0, 9, 3),        # one SM, element-wise rows, window of more than eight rows
+    ("f32", 3, 20, 20, 64, 32, 1, 16, 900, 0, 4, 3),       # one SM, embedding table in L2, more labels than threads
+    ("f32", 2, 90, 16, 16, 16, 1, 16, 20, 0, 40, 3),       # one SM, window of more than 32 rows
     ("f32", 9, 24, 32, 160, 320, 1, 300, 500, 0, 8, 4),    # grid: units in some CTAs only, three passes of utterances
     ("f32", 3, 24, 32, 130, 333, 2, 301, 449, 1, 5, 2),    # grid, element-wise rows, two layers, tanh
     ("f32", 2, 10, 32, 640, 1024, 3, 1024, 4000, 0, 8, 2), # grid, weights too large for the chip
