@@ -562,7 +562,7 @@ static wind_status_t check_beam_args(const wind_model_t* m, int32_t T, int32_t W
     wind_status_t s = check_model(m);
     if (s != WIND_OK) return s;
     if (K < 1 || S < 1) return WIND_ERR_INVALID_ARG;
-    if (K > 16) return WIND_ERR_UNSUPPORTED;
+    if (K > kMaxBeam) return WIND_ERR_UNSUPPORTED;
     return check_shape(m, K, T, W);
 }
 

@@ -4,15 +4,20 @@
 // the host; everything that touches the model runs in kernels on the caller's stream: the encoder projection once,
 // and per iteration (one frame t taken from the map) the decoder update of the hypotheses that survived pruning
 // (batched over the beam), the windowed joint for every hypothesis, Eq. (1) and its K best entries per hypothesis.
-// Only K x K (label, offset, log-probability) triples cross to the host per iteration.
+// Only K x K (label, offset, log-probability) triples cross to the host per iteration.  An iteration is one kernel
+// (wind_beam_step.cu) whose result the host polls for, or, for shapes that kernel does not take, a sequence of kernels.
 //
 // Decoder states live in a pool of slots in the workspace.  A hypothesis created by a label is evaluated lazily: it
 // carries (parent slot, label) until it survives the pruning of its frame, so at most K decoder updates are made per
 // iteration although K x K hypotheses are created.  Slots are reference-counted (a hypothesis created by the blank
 // entry shares its parent's slot).
+#include <immintrin.h>
+
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstring>
+#include <mutex>
 #include <vector>
 
 #include "wind_internal.cuh"
@@ -84,6 +89,63 @@ struct Hyp {
     int count = 0;
     int slot = -1;          // decoder state after tok (-1: not evaluated yet)
     int parent = -1;        // slot of the state before the last token, while slot == -1
+};
+
+// What an iteration's kernel writes to the host.  Page-locked blocks are kept for later searches, at most eight of them.
+struct Mailbox {
+    uint32_t done[kMaxBeam];
+    BeamTop top[kMaxBeam * kMaxBeam];
+};
+std::mutex g_mail_mutex;
+std::vector<Mailbox*> g_mail;
+constexpr size_t kMailKept = 8;
+
+struct MailboxLease {
+    Mailbox* box = nullptr;
+    cudaStream_t stream;
+    explicit MailboxLease(cudaStream_t s) : stream(s) {}
+    cudaError_t take() {
+        {
+            std::lock_guard<std::mutex> lock(g_mail_mutex);
+            if (!g_mail.empty()) { box = g_mail.back(); g_mail.pop_back(); }
+        }
+        if (!box) {
+            void* q = nullptr;
+            const cudaError_t e = cudaHostAlloc(&q, sizeof(Mailbox), cudaHostAllocPortable);
+            if (e != cudaSuccess) return e;
+            box = static_cast<Mailbox*>(q);
+        }
+        std::memset(box, 0, sizeof(Mailbox));
+        return cudaSuccess;
+    }
+    // the search's last kernel may still be running: neither the block nor the caller's workspace is given back before its end
+    ~MailboxLease() {
+        if (!box) return;
+        cudaStreamSynchronize(stream);
+        std::lock_guard<std::mutex> lock(g_mail_mutex);
+        if (g_mail.size() < kMailKept) { g_mail.push_back(box); return; }
+        cudaFreeHost(box);
+    }
+    // until the kernel has written `n` hypotheses' entries; false: it ended without writing them
+    cudaError_t wait(uint32_t seq, int n, bool* written) {
+        *written = false;
+        auto all = [&] {
+            for (int b = 0; b < n; ++b)
+                if (*const_cast<volatile uint32_t*>(&box->done[b]) != seq) return false;
+            std::atomic_thread_fence(std::memory_order_acquire);
+            return true;
+        };
+        for (uint32_t spins = 1;; ++spins) {
+            if (all()) { *written = true; return cudaSuccess; }
+            _mm_pause();
+            if ((spins & 4095u) == 0u) {          // a kernel that gave up, or an error on the stream, writes nothing
+                const cudaError_t e = cudaStreamQuery(stream);
+                if (e == cudaErrorNotReady) continue;
+                if (e == cudaSuccess) *written = all();
+                return e;
+            }
+        }
+    }
 };
 
 double log_add(double a, double b) {
@@ -159,6 +221,10 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
         refs[0]++;
         t2hyps[0].push_back(std::move(h0));
     }
+    MailboxLease mail(st);
+    const bool one_kernel = beam_step_supported(cb);
+    if (one_kernel) BEAM_CUDA(mail.take());
+    uint32_t bar_base = 0;
     std::vector<int32_t> host_ints(4 * (size_t)K), top(3 * (size_t)K * K);
     const int32_t* top_label = top.data();
     const int32_t* top_jump = top.data() + (size_t)K * K;
@@ -352,18 +418,38 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
                 }
             }
             for (int b = 0; b < nh; ++b) host_ints[3 * K + b] = hyps[b].slot;
-            BEAM_CUDA(cudaMemcpyAsync(d_exp, host_ints.data() + 3 * K, sizeof(int32_t) * K, cudaMemcpyHostToDevice, st));
-            beam_gather_g_kernel<<<K, 128, 0, st>>>(g_pool, d_exp, cb.pred_proj(), d_t, t, T, m.H);   // sets the frames first
-            BEAM_CUDA(launch_set_t(cb, d_t));   // frames of the rows, and the control block's "active" word
-            if (nu > 0) {
-                BEAM_CUDA(run_update(nu));   // (the parents are no longer needed by these hypotheses)
-                beam_gather_g_kernel<<<K, 128, 0, st>>>(g_pool, d_exp, cb.pred_proj(), d_t, t, T, m.H);
+            if (one_kernel) {
+                BeamStep io{};
+                io.K = K; io.n_update = nu; io.n_hyps = nh; io.n_rows = n; io.t = t;
+                io.seq = (uint32_t)steps;
+                io.top = mail.box->top;
+                io.done = mail.box->done;
+                for (int u = 0; u < nu; ++u) { io.src[u] = host_ints[u]; io.tok[u] = host_ints[K + u]; io.dst[u] = host_ints[2 * K + u]; }
+                for (int b = 0; b < nh; ++b) io.slot[b] = hyps[b].slot;
+                BEAM_CUDA(beam_step(cb, io, h_pool, c_pool, g_pool, logits, &bar_base));
+                for (int u = 0; u < nu; ++u) release(host_ints[u]);
+                bool written = false;
+                BEAM_CUDA(mail.wait(io.seq, nh, &written));
+                if (!written) return WIND_ERR_TIMEOUT;
+                for (int i = 0; i < nh * K; ++i) {
+                    top[(size_t)i] = mail.box->top[i].label;
+                    top[(size_t)K * K + i] = mail.box->top[i].jump;
+                    std::memcpy(&top[2 * (size_t)K * K + i], &mail.box->top[i].logp, sizeof(float));
+                }
+            } else {
+                BEAM_CUDA(cudaMemcpyAsync(d_exp, host_ints.data() + 3 * K, sizeof(int32_t) * K, cudaMemcpyHostToDevice, st));
+                beam_gather_g_kernel<<<K, 128, 0, st>>>(g_pool, d_exp, cb.pred_proj(), d_t, t, T, m.H);   // sets the frames first
+                BEAM_CUDA(launch_set_t(cb, d_t));   // frames of the rows, and the control block's "active" word
+                if (nu > 0) {
+                    BEAM_CUDA(run_update(nu));   // (the parents are no longer needed by these hypotheses)
+                    beam_gather_g_kernel<<<K, 128, 0, st>>>(g_pool, d_exp, cb.pred_proj(), d_t, t, T, m.H);
+                }
+                // ---- window logits of every hypothesis, Eq. (1), the K best entries each ----
+                BEAM_CUDA(simt_joint_shared(cb, logits));
+                BEAM_CUDA(launch_first_output(logits, d_len, d_t, K, W, NV, m.blank_id, K, d_top_label, d_top_jump, d_top_logp, st));
+                BEAM_CUDA(cudaMemcpyAsync(top.data(), d_top_label, sizeof(int32_t) * 3 * K * K, cudaMemcpyDeviceToHost, st));
+                BEAM_CUDA(cudaStreamSynchronize(st));
             }
-            // ---- window logits of every hypothesis, Eq. (1), the K best entries each ----
-            BEAM_CUDA(simt_joint_shared(cb, logits));
-            BEAM_CUDA(launch_first_output(logits, d_len, d_t, K, W, NV, m.blank_id, K, d_top_label, d_top_jump, d_top_logp, st));
-            BEAM_CUDA(cudaMemcpyAsync(top.data(), d_top_label, sizeof(int32_t) * 3 * K * K, cudaMemcpyDeviceToHost, st));
-            BEAM_CUDA(cudaStreamSynchronize(st));
             // ---- expansions ----
             for (int b = 0; b < nh; ++b) {
                 const Hyp& h = hyps[b];

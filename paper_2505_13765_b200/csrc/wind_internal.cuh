@@ -226,6 +226,19 @@ struct BeamLayout {
     size_t total;
     int slots;
 };
+// One iteration on the device (wind_beam_step.cu): decoder updates, window logits, Eq. (1), the K best entries per hypothesis.
+constexpr int kMaxBeam = 16;
+struct BeamTop { int32_t label, jump; float logp; int32_t pad; };
+struct BeamStep {
+    int32_t K, n_update, n_hyps, n_rows, t;   // n_rows: the window, cut short by the end of the utterance
+    uint32_t seq;                             // written to done[b] behind hypothesis b's entries
+    BeamTop* top;                             // [K][K]  host memory
+    uint32_t* done;                           // [K]     host memory
+    int32_t src[kMaxBeam], tok[kMaxBeam], dst[kMaxBeam];   // n_update decoder updates: slot before, token, slot after
+    int32_t slot[kMaxBeam];                                // n_hyps hypotheses: their states
+};
+bool beam_step_supported(const Call& c);
+cudaError_t beam_step(const Call& c, const BeamStep& io, float* h_pool, float* c_pool, float* g_pool, float* logits, uint32_t* bar_base);
 BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, size_t base);
 wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_search, int max_hyps, int max_out, int32_t* out_tokens,
                               int32_t* out_frames, int32_t* out_len, double* out_score, int32_t* n_hyps, int64_t* n_steps,
