@@ -4,8 +4,8 @@
 // the host; everything that touches the model runs in kernels on the caller's stream: the encoder projection once,
 // and per iteration (one frame t taken from the map) the decoder update of the hypotheses that survived pruning
 // (batched over the beam), the windowed joint for every hypothesis, Eq. (1) and its K best entries per hypothesis.
-// Only K x K (label, offset, log-probability) triples cross to the host per iteration.  An iteration is one kernel
-// (wind_beam_step.cu) whose result the host polls for, or, for shapes that kernel does not take, a sequence of kernels.
+// Only K x K (label, offset, log-probability) triples cross to the host per iteration.  An iteration goes to one resident kernel
+// (wind_beam_step.cu) that takes it as a command, or, for shapes that kernel does not take, a sequence of kernels.
 //
 // Decoder states live in a pool of slots in the workspace.  A hypothesis created by a label is evaluated lazily: it
 // carries (parent slot, label) until it survives the pruning of its frame, so at most K decoder updates are made per
@@ -91,60 +91,85 @@ struct Hyp {
     int parent = -1;        // slot of the state before the last token, while slot == -1
 };
 
-// What an iteration's kernel writes to the host.  Page-locked blocks are kept for later searches, at most eight of them.
-struct Mailbox {
-    uint32_t done[kMaxBeam];
-    BeamTop top[kMaxBeam * kMaxBeam];
-};
+// Page-locked mailboxes are kept for later searches, at most eight of them.
 std::mutex g_mail_mutex;
-std::vector<Mailbox*> g_mail;
+std::vector<BeamMail*> g_mail;
 constexpr size_t kMailKept = 8;
 
-struct MailboxLease {
-    Mailbox* box = nullptr;
-    cudaStream_t stream;
-    explicit MailboxLease(cudaStream_t s) : stream(s) {}
-    cudaError_t take() {
+// The resident kernel of one search, as the host sees it.
+struct BeamDevice {
+    const Call& c;
+    float *h_pool, *c_pool, *g_pool, *logits;
+    unsigned long long* relay;
+    bool single;                 // other kernels run on the stream between the iterations: one launch per command
+    BeamMail* mail = nullptr;
+    uint32_t seq = 0, bar_base = 0;
+    bool running = false;
+
+    cudaError_t open() {
         {
             std::lock_guard<std::mutex> lock(g_mail_mutex);
-            if (!g_mail.empty()) { box = g_mail.back(); g_mail.pop_back(); }
+            if (!g_mail.empty()) { mail = g_mail.back(); g_mail.pop_back(); }
         }
-        if (!box) {
+        if (!mail) {
             void* q = nullptr;
-            const cudaError_t e = cudaHostAlloc(&q, sizeof(Mailbox), cudaHostAllocPortable);
+            const cudaError_t e = cudaHostAlloc(&q, sizeof(BeamMail), cudaHostAllocPortable);
             if (e != cudaSuccess) return e;
-            box = static_cast<Mailbox*>(q);
+            mail = static_cast<BeamMail*>(q);
         }
-        std::memset(box, 0, sizeof(Mailbox));
-        return cudaSuccess;
+        std::memset(mail, 0, sizeof(BeamMail));
+        return cudaMemsetAsync(relay, 0, sizeof(unsigned long long) * kBeamWords, c.stream);
     }
-    // the search's last kernel may still be running: neither the block nor the caller's workspace is given back before its end
-    ~MailboxLease() {
-        if (!box) return;
-        cudaStreamSynchronize(stream);
-        std::lock_guard<std::mutex> lock(g_mail_mutex);
-        if (g_mail.size() < kMailKept) { g_mail.push_back(box); return; }
-        cudaFreeHost(box);
+    void post(const int32_t* words) {        // 4 + 4 K values
+        ++seq;
+        volatile unsigned long long* out = mail->cmd;
+        for (int i = 0; i < 4 + 4 * c.B; ++i) out[i] = (unsigned long long)seq << 32 | (uint32_t)words[i];
     }
-    // until the kernel has written `n` hypotheses' entries; false: it ended without writing them
-    cudaError_t wait(uint32_t seq, int n, bool* written) {
-        *written = false;
-        auto all = [&] {
-            for (int b = 0; b < n; ++b)
-                if (*const_cast<volatile uint32_t*>(&box->done[b]) != seq) return false;
-            std::atomic_thread_fence(std::memory_order_acquire);
-            return true;
-        };
-        for (uint32_t spins = 1;; ++spins) {
-            if (all()) { *written = true; return cudaSuccess; }
-            _mm_pause();
-            if ((spins & 4095u) == 0u) {          // a kernel that gave up, or an error on the stream, writes nothing
-                const cudaError_t e = cudaStreamQuery(stream);
-                if (e == cudaErrorNotReady) continue;
-                if (e == cudaSuccess) *written = all();
-                return e;
+    // one command, until its result (nh * K entries) is there
+    wind_status_t run(const int32_t* words, cudaError_t* err) {
+        const int n_out = 2 * words[1] * c.B;
+        post(words);
+        for (int launches = 0;;) {
+            if (!running) {
+                // (a kernel that ends for want of commands took every CTA with it, between two commands)
+                if (++launches > 8) return WIND_ERR_TIMEOUT;
+                if ((*err = beam_step(c, mail, relay, seq, bar_base, single, h_pool, c_pool, g_pool, logits)) != cudaSuccess) return WIND_ERR_CUDA;
+                running = true;
             }
+            bool there = false;
+            for (uint32_t spins = 1; !there; ++spins) {
+                there = true;
+                for (int i = n_out - 1; i >= 0 && there; --i)
+                    there = (uint32_t)(static_cast<volatile unsigned long long*>(mail->top)[i] >> 32) == seq;
+                if (there) break;
+                _mm_pause();
+                if ((spins & 4095u) == 0u && (*err = cudaStreamQuery(c.stream)) != cudaErrorNotReady) {
+                    if (*err != cudaSuccess) return WIND_ERR_CUDA;
+                    running = false;
+                    if (*static_cast<volatile uint32_t*>(&mail->failed)) return WIND_ERR_TIMEOUT;
+                    break;
+                }
+            }
+            if (!there) {                // it ended before it saw the command, or with the result just written
+                std::atomic_thread_fence(std::memory_order_acquire);
+                there = true;
+                for (int i = 0; i < n_out && there; ++i) there = (uint32_t)(mail->top[i] >> 32) == seq;
+                if (!there) { post(words); continue; }
+            }
+            if (single) running = false;
+            bar_base += beam_step_arrivals(c, words[0]);
+            return WIND_OK;
         }
+    }
+    // Neither the mailbox nor the caller's workspace is given back before the kernel's end.
+    ~BeamDevice() {
+        if (!mail) return;
+        std::vector<int32_t> end(4 + 4 * (size_t)c.B, -1);
+        post(end.data());
+        cudaStreamSynchronize(c.stream);
+        std::lock_guard<std::mutex> lock(g_mail_mutex);
+        if (g_mail.size() < kMailKept) g_mail.push_back(mail);
+        else cudaFreeHost(mail);
     }
 };
 
@@ -171,6 +196,7 @@ BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, s
     L.top_label = take(sizeof(int32_t) * 3 * (size_t)K * K);   // labels, offsets, log-probabilities: one block, one copy
     L.top_jump = L.top_label + sizeof(int32_t) * (size_t)K * K;
     L.top_logp = L.top_jump + sizeof(int32_t) * (size_t)K * K;
+    L.relay = take(sizeof(uint64_t) * kBeamWords);
     L.total = off;
     return L;
 }
@@ -221,10 +247,10 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
         refs[0]++;
         t2hyps[0].push_back(std::move(h0));
     }
-    MailboxLease mail(st);
-    const bool one_kernel = beam_step_supported(cb);
-    if (one_kernel) BEAM_CUDA(mail.take());
-    uint32_t bar_base = 0;
+    BeamDevice dev{cb, h_pool, c_pool, g_pool, logits, reinterpret_cast<unsigned long long*>(ws + bl.relay), prefix_search != 0};
+    const bool resident = beam_step_supported(cb);
+    if (resident) BEAM_CUDA(dev.open());
+    std::vector<int32_t> words(4 + 4 * (size_t)K);
     std::vector<int32_t> host_ints(4 * (size_t)K), top(3 * (size_t)K * K);
     const int32_t* top_label = top.data();
     const int32_t* top_jump = top.data() + (size_t)K * K;
@@ -418,23 +444,17 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
                 }
             }
             for (int b = 0; b < nh; ++b) host_ints[3 * K + b] = hyps[b].slot;
-            if (one_kernel) {
-                BeamStep io{};
-                io.K = K; io.n_update = nu; io.n_hyps = nh; io.n_rows = n; io.t = t;
-                io.seq = (uint32_t)steps;
-                io.top = mail.box->top;
-                io.done = mail.box->done;
-                for (int u = 0; u < nu; ++u) { io.src[u] = host_ints[u]; io.tok[u] = host_ints[K + u]; io.dst[u] = host_ints[2 * K + u]; }
-                for (int b = 0; b < nh; ++b) io.slot[b] = hyps[b].slot;
-                BEAM_CUDA(beam_step(cb, io, h_pool, c_pool, g_pool, logits, &bar_base));
+            if (resident) {
+                words[0] = nu; words[1] = nh; words[2] = n; words[3] = t;
+                std::copy(host_ints.begin(), host_ints.end(), words.begin() + 4);
+                const wind_status_t rs = dev.run(words.data(), cuda_err);
+                if (rs != WIND_OK) return rs;
                 for (int u = 0; u < nu; ++u) release(host_ints[u]);
-                bool written = false;
-                BEAM_CUDA(mail.wait(io.seq, nh, &written));
-                if (!written) return WIND_ERR_TIMEOUT;
                 for (int i = 0; i < nh * K; ++i) {
-                    top[(size_t)i] = mail.box->top[i].label;
-                    top[(size_t)K * K + i] = mail.box->top[i].jump;
-                    std::memcpy(&top[2 * (size_t)K * K + i], &mail.box->top[i].logp, sizeof(float));
+                    const uint32_t at = (uint32_t)dev.mail->top[2 * i], bits = (uint32_t)dev.mail->top[2 * i + 1];
+                    top[(size_t)i] = at == 0xffffffffu ? -1 : (int32_t)(at % (uint32_t)NV);
+                    top[(size_t)K * K + i] = at == 0xffffffffu ? -1 : (int32_t)(at / (uint32_t)NV);
+                    std::memcpy(&top[2 * (size_t)K * K + i], &bits, sizeof(float));
                 }
             } else {
                 BEAM_CUDA(cudaMemcpyAsync(d_exp, host_ints.data() + 3 * K, sizeof(int32_t) * K, cudaMemcpyHostToDevice, st));

@@ -1,14 +1,25 @@
-// One iteration of the beam search (Algorithm 3) as one kernel: decoder update of the hypotheses that have no state yet,
-// their projection, the window's logits under every hypothesis, Eq. (1) and the K best entries each, written to host memory.
+// The beam search's iterations (Algorithm 3) on the device: decoder update of the hypotheses that have no state yet, their
+// projection, the window's logits under every hypothesis, Eq. (1) and the K best entries of each.
 //
 // As separate kernels an iteration of the 640-unit model with beam 4 took 85 us, of which 51 us were eleven kernels and copies
 // (a block per hidden unit or per sixteen labels loads its weights, waits for them, and uses them once) and the rest gaps and
-// the synchronisation.  Here hidden units, joint units and labels are dealt out over all SMs, every CTA requests all its
-// weights (67 KB) at the start, the phases follow one another behind grid barriers, and the host polls for the result.
+// the synchronisation.  Here hidden units, joint units and labels are dealt out over all SMs with their weights (67 KB each) in
+// shared memory, the phases follow one another behind grid barriers, and the kernel stays for the whole search: the host
+// writes each iteration's command to page-locked memory and reads the result there: 24 us an iteration.  One launch per iteration
+// took 42 us: 6 us of launch, the weights again, and every instruction fetched from L2 because it runs once.  What is left: 2 us
+// from host to host, three grid barriers (1.5 us each with their skew), and phases of 1 to 3 us that are chains of a few L2 and
+// shared-memory latencies each.
+//
+// The kernel never depends on the host's pace: without a command for 200 us it ends, and the host launches it again with the
+// next one (all state is in global memory).  So another stream's work, a debugger or a descheduled host thread cost time only.
+//
+// A command or result word carries its 32 bits and the command's number in one 8-byte store, so no fence or flag is needed on
+// either side of the bus.
 //
 // A dot product is summed as the per-phase kernels sum it, so that both give the same bits: 32 chains, chain r over
-// k = r, r + 32, ..., then a butterfly.  A thread carries four neighbouring chains, so eight threads make a row, and a warp
-// four rows with 8-byte reads of the weights.
+// k = r, r + 32, ..., then a butterfly.  A lane carries one chain of four weight rows times four operand rows.  Rows are kept
+// interleaved by four ([k][4]), so that a step is two loads for sixteen products: with rows kept apart the eight loads of a step
+// took 135 cycles.
 #include "wind_internal.cuh"
 #include "wind_loop.cuh"
 #include "wind_ptx.cuh"
@@ -22,57 +33,57 @@ constexpr int BS_WARPS = BS_THREADS / 32;
 constexpr int BS_UTTS = 4;            // updates of a pass
 constexpr int BS_ROWS = 4;            // window rows of a joint item
 
+constexpr unsigned long long BS_IDLE_NS = 200000ull;
+
 // dimensions shared by the host's plan and the kernel; all sizes in elements, offsets in bytes
 struct BsPlan {
-    int G, units, prows, labels;      // grid, and the most a CTA owns of each
-    int ld_l, ld_p, ld_o;             // row pitches: gates (any layer), W_pred, W_out
-    int k_l, k_p;                     // floats of a staged x row of the gates / of h
-    int zrows, ld_z;                  // window rows of a joint pass
-    uint32_t w_pred, w_out, area, x, total;   // area: the gates' weights, then x behind them; later z, then the window's logits
+    int units, prows, labels;         // the most a CTA owns of each
+    int k_l, k_p;                     // row lengths, rounded up to 32: of the gates (any layer), of W_pred
+    int zrows, k_z;                   // window rows of a joint pass; row length of the joint, rounded up to 32
+    int resident;                     // the gates' weights of all layers stay; else a layer's are loaded in front of its use
+    uint32_t layer, w_l, w_pred, w_out, bias, enc, x, z, total;   // layer: bytes of one layer's weights; z: later the window's logits
 };
-template <typename TW> __host__ __device__ inline int bs_pitch(int k) {
-    // eight threads read a row's 32 elements and four rows are read at a time: rows shifted by half the banks
-    const int p = (k + 31) / 32 * 32;
-    return sizeof(TW) == 2 ? (p % 64 == 32 ? p : p + 32) : p + 4;
-}
-template <typename TW> __host__ __device__ inline BsPlan bs_plan(int G, int W, int K, int E, int P, int L, int H, int NV, uint32_t budget) {
+template <typename TW> static BsPlan bs_plan(int G, int W, int K, int E, int P, int L, int H, int NV, uint32_t budget) {
     BsPlan s{};
-    s.G = G;
     s.units = (P + G - 1) / G; s.prows = (H + G - 1) / G; s.labels = (NV + G - 1) / G;
     const int k0 = E + P, k1 = L > 1 ? 2 * P : 0, kmax = k0 > k1 ? k0 : k1;
-    s.ld_l = bs_pitch<TW>(kmax); s.ld_p = bs_pitch<TW>(P); s.ld_o = bs_pitch<TW>(H);
     s.k_l = (kmax + 31) / 32 * 32; s.k_p = (P + 31) / 32 * 32;
-    s.ld_z = (H + 31) / 32 * 32;
-    unsigned long long off = 0;
-    auto take = [&](unsigned long long bytes) { const unsigned long long o = off; off += (bytes + 15) / 16 * 16; return (uint32_t)o; };
-    s.w_pred = take((unsigned long long)sizeof(TW) * s.prows * s.ld_p);
-    s.w_out = take((unsigned long long)sizeof(TW) * s.labels * s.ld_o);
-    s.area = (uint32_t)off;
-    unsigned long long gates = (unsigned long long)sizeof(TW) * s.units * 4 * s.ld_l;
-    s.x = (uint32_t)(s.area + gates);
-    gates += 4ull * BS_UTTS * s.k_l;
-    const unsigned long long window = 4ull * W * NV;
-    unsigned long long area = gates > window ? gates : window;
-    const unsigned long long row = 4ull * s.ld_z;
-    int rows = (K * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
-    if (off + row * BS_ROWS <= budget) {
-        const unsigned long long fit = (budget - off) / row / BS_ROWS * BS_ROWS;
-        if ((unsigned long long)rows > fit) rows = (int)fit;
-    } else {
-        rows = BS_ROWS;
+    s.k_z = (H + 31) / 32 * 32;
+    const int all = (K * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
+    for (s.resident = 1; s.resident >= 0; --s.resident) {
+        unsigned long long off = 0;
+        auto take = [&](unsigned long long bytes) { const unsigned long long o = off; off += (bytes + 15) / 16 * 16; return (uint32_t)o; };
+        const unsigned long long layer = (unsigned long long)sizeof(TW) * s.units * 4 * s.k_l;
+        s.layer = (uint32_t)layer;
+        s.w_l = take(layer * (s.resident ? L : 1));
+        s.w_pred = take((unsigned long long)sizeof(TW) * ((s.prows + 3) / 4 * 4) * s.k_p);
+        s.w_out = take((unsigned long long)sizeof(TW) * ((s.labels + 3) / 4 * 4) * s.k_z);
+        s.bias = take(4ull * (4 * L * s.units + s.prows + s.labels));
+        s.enc = take((unsigned long long)sizeof(TW) * W * H);
+        const unsigned long long xa = 4ull * BS_UTTS * s.k_l, xb = 4ull * K * H;
+        s.x = take(xa > xb ? xa : xb);
+        s.z = (uint32_t)off;
+        const unsigned long long row = 4ull * s.k_z, window = 4ull * W * NV;
+        const unsigned long long fit = off < budget ? (budget - off) / row / BS_ROWS * BS_ROWS : 0;
+        s.zrows = fit < (unsigned long long)all ? (int)fit : all;
+        off += row * s.zrows > window ? row * s.zrows : window;
+        s.total = s.zrows == 0 || off > budget ? 0xffffffffu : (uint32_t)off;
+        if (s.total <= budget && s.zrows >= (s.resident && all > 16 ? 16 : BS_ROWS)) break;
     }
-    s.zrows = rows;
-    if (row * rows > area) area = row * rows;
-    off += area;
-    s.total = off > 0xffffffffull ? 0xffffffffu : (uint32_t)off;
+    if (s.resident < 0) s.resident = 0;
     return s;
 }
 
 struct BsParams {
-    BeamStep io;
     Ctrl* ctrl;
+    BeamMail* mail;                    // page-locked host memory
+    unsigned long long* relay;         // the command in device memory, read by every CTA
+    uint32_t first_seq;                // number of the first command
     uint32_t bar_base;                 // arrivals at the grid barrier before this launch
-    uint32_t extra_arrivals, budget;
+    uint32_t extra_arrivals;
+    BsPlan plan;
+    int single;                        // end after one command
+    int K;
     int E, P, L, H, NV, blank, act, W;
     const void* emb;
     const void* w_ih[kMaxLayers];
@@ -90,42 +101,44 @@ struct BsParams {
 template <typename TW> __device__ __forceinline__ float bs_round(float x);
 template <> __device__ __forceinline__ float bs_round<float>(float x) { return x; }
 template <> __device__ __forceinline__ float bs_round<__nv_bfloat16>(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-__device__ __forceinline__ float4 bs_load4(const float* p) { return *reinterpret_cast<const float4*>(p); }
-__device__ __forceinline__ float4 bs_load4(const __nv_bfloat16* p) {
-    const uint2 v = *reinterpret_cast<const uint2*>(p);
-    const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.x)), b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&v.y));
-    return make_float4(a.x, a.y, b.x, b.y);
-}
 
-// N dot products of this lane group's weight row with N rows of x; w and x point at the thread's first element.  All eight
-// threads of the group get the sums.
-template <int N, typename TW>
-__device__ __forceinline__ void bs_dots(const TW* w, const float* x, int x_pitch, int steps, float* sum) {
-    float a[N][4];
+// Dot products of four rows of weights with four rows of x, both [k][4] in shared memory; the addresses are the lane's first
+// element (k = lane).  Afterwards lane l holds the one of weight row l >> 3 and x row (l >> 1) & 3.
+// (One function for the three phases, and few unrolled loops elsewhere: an iteration runs its code once, and what does not stay
+// in the 32 KB instruction cache is fetched at three cycles an instruction.)
+template <typename TW>
+__device__ __noinline__ float bs_dots(uint32_t w, uint32_t x, int steps) {
+    float a[16];
 #pragma unroll
-    for (int n = 0; n < N; ++n)
-#pragma unroll
-        for (int j = 0; j < 4; ++j) a[n][j] = 0.f;
+    for (int i = 0; i < 16; ++i) a[i] = 0.f;
 #pragma unroll 4
     for (int i = 0; i < steps; ++i) {
-        const float4 wv = bs_load4(w + 32 * i);
+        float wv[4], xv[4];
+        if constexpr (sizeof(TW) == 2) {
+            uint32_t v0, v1;
+            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(w + 256u * i));
+            wv[0] = __uint_as_float(v0 << 16); wv[1] = __uint_as_float(v0 & 0xffff0000u);
+            wv[2] = __uint_as_float(v1 << 16); wv[3] = __uint_as_float(v1 & 0xffff0000u);
+        } else {
+            asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(wv[0]), "=f"(wv[1]), "=f"(wv[2]), "=f"(wv[3]) : "r"(w + 512u * i));
+        }
+        asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(xv[0]), "=f"(xv[1]), "=f"(xv[2]), "=f"(xv[3]) : "r"(x + 512u * i));
 #pragma unroll
-        for (int n = 0; n < N; ++n) {
-            const float4 xv = *reinterpret_cast<const float4*>(x + n * x_pitch + 32 * i);
-            a[n][0] = fmaf(wv.x, xv.x, a[n][0]);
-            a[n][1] = fmaf(wv.y, xv.y, a[n][1]);
-            a[n][2] = fmaf(wv.z, xv.z, a[n][2]);
-            a[n][3] = fmaf(wv.w, xv.w, a[n][3]);
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int n = 0; n < 4; ++n) a[4 * j + n] = fmaf(wv[j], xv[n], a[4 * j + n]);
+    }
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int half = 8; half >= 1; half >>= 1) {
+        const bool up = (lane & (2 * half)) != 0;
+#pragma unroll
+        for (int c = 0; c < half; ++c) {
+            const float send = up ? a[c] : a[c + half], keep = up ? a[c + half] : a[c];
+            a[c] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * half);
         }
     }
-#pragma unroll
-    for (int n = 0; n < N; ++n) {
-#pragma unroll
-        for (int o = 4; o > 0; o >>= 1)
-#pragma unroll
-            for (int j = 0; j < 4; ++j) a[n][j] += __shfl_xor_sync(0xffffffffu, a[n][j], o);
-        sum[n] = (a[n][0] + a[n][2]) + (a[n][1] + a[n][3]);
-    }
+    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
 }
 
 __device__ __forceinline__ float bs_warp_max(float v) {
@@ -138,57 +151,86 @@ __device__ __forceinline__ float bs_warp_sum(float v) {
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
 }
-// (value, index) as one integer: larger values first, then smaller indices; 0 where there is none
-__device__ __forceinline__ unsigned long long bs_pair(float v, int i) { return v > -INFINITY ? pack_key(v, (uint32_t)i) : 0ull; }
 __device__ __forceinline__ unsigned long long bs_best_of_warp(unsigned long long key) {
     const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(key >> 32));
     const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(key >> 32) == hi ? (uint32_t)key : 0u);
     return ((unsigned long long)hi << 32) | lo;
 }
+__device__ __forceinline__ unsigned long long bs_word(uint32_t value, uint32_t seq) { return ((unsigned long long)seq << 32) | value; }
 
-// KL: entries of a thread's own list of best entries (at least K)
-template <typename TW, int KL>
+template <typename TW>
 __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams p) {
     extern __shared__ __align__(16) uint8_t sm[];
     __shared__ int s_stop;
-    __shared__ float s_lse[kMaxWindow], s_before[kMaxWindow];
-    __shared__ unsigned long long s_cand[BS_WARPS * KL];
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = lane >> 3, q = lane & 7;
+    __shared__ int s_cmd[kBeamWords];
+    __shared__ float s_lse[kMaxWindow], s_blank[kMaxWindow];     // of a row: log-sum-exp, blank's log-probability
+    __shared__ unsigned long long s_cand[BS_WARPS * kMaxBeam];
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, grp = lane >> 3, col = (lane >> 1) & 3;   // the dot product a lane ends up with
     const int G = gridDim.x, cta = blockIdx.x;
-    const int P = p.P, H = p.H, NV = p.NV, K = p.io.K, LP = p.L * P;
-    const BsPlan M = bs_plan<TW>(G, p.W, K, p.E, P, p.L, H, NV, p.budget);
+    const int P = p.P, H = p.H, NV = p.NV, K = p.K, LP = p.L * P;
+    const BsPlan& M = p.plan;
     const int units = (P - cta + G - 1) / G, prows = (H - cta + G - 1) / G, labels = (NV - cta + G - 1) / G;
     TW* w_pred = reinterpret_cast<TW*>(sm + M.w_pred);
     TW* w_out = reinterpret_cast<TW*>(sm + M.w_out);
-    TW* w_l = reinterpret_cast<TW*>(sm + M.area);
+    TW* encs = reinterpret_cast<TW*>(sm + M.enc);
+    float* b_gate = reinterpret_cast<float*>(sm + M.bias);                     // [layer][own unit][gate]
+    float *b_pred = b_gate + 4 * p.L * M.units, *b_out = b_pred + M.prows;
     float* xs = reinterpret_cast<float*>(sm + M.x);
-    float* area = reinterpret_cast<float*>(sm + M.area);
-    const int nu = p.io.n_update, nh = p.io.n_hyps;
+    float* zs = reinterpret_cast<float*>(sm + M.z);
     if (tid == 0) s_stop = 0;
 
-    // n elements (whole 16-byte pieces) by one warp, asynchronously, and zeros up to a multiple of 32
-    auto copy_row = [&](TW* dst, const TW* src, int n, int n32) {
+    // n elements (whole 16-byte pieces) by one warp, asynchronously
+    auto copy_row = [&](TW* dst, const TW* src, int n) {
         constexpr int PIECE = 16 / (int)sizeof(TW);
+#pragma unroll 1
         for (int k = lane * PIECE; k < n; k += 32 * PIECE)
             asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst + k)), "l"(src + k) : "memory");
-        for (int k = n + lane; k < n32; k += 32) dst[k] = (TW)0.f;
+    };
+    auto layer_at = [&](int l) { return reinterpret_cast<TW*>(sm + M.w_l + (size_t)(M.resident ? l : 0) * M.layer); };
+    // element k of four rows (rows past the end: zeros) into [k][4]
+    auto interleave = [&](TW* dst, const TW* r0, const TW* r1, const TW* r2, const TW* r3, int n, int n32) {
+#pragma unroll 2
+        for (int k = lane; k < n32; k += 32) {
+            const TW zero = (TW)0.f;
+            TW* d = dst + 4 * k;
+            d[0] = r0 && k < n ? r0[k] : zero;
+            d[1] = r1 && k < n ? r1[k] : zero;
+            d[2] = r2 && k < n ? r2[k] : zero;
+            d[3] = r3 && k < n ? r3[k] : zero;
+        }
     };
     auto load_layer = [&](int l) {
         const int nin = l == 0 ? p.E : P, K32 = (nin + P + 31) / 32 * 32;
-        for (int i = warp; i < units * 4; i += BS_WARPS) {
-            const size_t row = (size_t)(i & 3) * P + (size_t)(i >> 2) * G + cta;
-            copy_row(w_l + i * M.ld_l, static_cast<const TW*>(p.w_ih[l]) + row * nin, nin, nin);
-            copy_row(w_l + i * M.ld_l + nin, static_cast<const TW*>(p.w_hh[l]) + row * P, P, K32 - nin);
+        const TW *wi = static_cast<const TW*>(p.w_ih[l]), *wh = static_cast<const TW*>(p.w_hh[l]);
+#pragma unroll 1
+        for (int i = warp; i < units; i += BS_WARPS) {
+            const size_t j = (size_t)i * G + cta;
+            TW* dst = layer_at(l) + 4 * i * M.k_l;
+            interleave(dst, wi + j * nin, wi + (P + j) * nin, wi + (2 * P + j) * nin, wi + (3 * P + j) * nin, nin, nin);
+            interleave(dst + 4 * nin, wh + j * P, wh + (P + j) * P, wh + (2 * P + j) * P, wh + (3 * P + j) * P, P, K32 - nin);
         }
-        asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    if (nu > 0) load_layer(0);
-    if (nu > 0)
-        for (int i = warp; i < prows; i += BS_WARPS)
-            copy_row(w_pred + i * M.ld_p, static_cast<const TW*>(p.w_pred) + ((size_t)i * G + cta) * P, P, M.k_p);
-    for (int i = warp; i < labels; i += BS_WARPS)
-        copy_row(w_out + i * M.ld_o, static_cast<const TW*>(p.w_out) + ((size_t)i * G + cta) * H, H, M.ld_z);
-    asm volatile("cp.async.commit_group;" ::: "memory");
+    auto load_rows = [&](TW* dst, const void* src_, int rows, int n, int n32) {      // this CTA's rows of W_pred or W_out
+        const TW* src = static_cast<const TW*>(src_);
+#pragma unroll 1
+        for (int i = 4 * warp; i < rows; i += 4 * BS_WARPS) {
+            auto row = [&](int j) { return i + j < rows ? src + ((size_t)(i + j) * G + cta) * n : nullptr; };
+            interleave(dst + i * n32, row(0), row(1), row(2), row(3), n, n32);
+        }
+    };
+    if (M.resident)
+#pragma unroll 1
+        for (int l = 0; l < p.L; ++l) load_layer(l);
+    load_rows(w_pred, p.w_pred, prows, P, M.k_p);
+    load_rows(w_out, p.w_out, labels, H, M.k_z);
+
+#pragma unroll 1
+    for (int i = tid; i < 4 * p.L * units; i += BS_THREADS) {
+        const int l = i / (4 * units), r = i - l * 4 * units, at = (r & 3) * P + (r >> 2) * G + cta;
+        b_gate[4 * l * M.units + r] = p.b_ih[l][at] + p.b_hh[l][at];
+    }
+    for (int i = tid; i < prows; i += BS_THREADS) b_pred[i] = p.b_pred[i * G + cta];
+    for (int i = tid; i < labels; i += BS_THREADS) b_out[i] = p.b_out[i * G + cta];
 
     uint32_t epoch = p.bar_base;
     auto arrive = [&] {
@@ -196,6 +238,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
         epoch += (uint32_t)G;
         if (tid == 0) { __threadfence(); atomicAdd(&p.ctrl->bar, 1u); }
     };
+    auto give_up = [&] { s_stop = 1; set_status(p.ctrl, WIND_ERR_TIMEOUT); *const_cast<volatile uint32_t*>(&p.mail->failed) = 1u; };
     auto wait = [&]() -> bool {        // bounded; false: given up
         if (tid == 0) {
             const uint32_t target = epoch + p.extra_arrivals;
@@ -207,205 +250,295 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                 if ((it & 63u) == 0u) {
                     const unsigned long long now = globaltimer_ns();
                     if (t0 == 0) t0 = now;
-                    else if (now - t0 > kWaitLimitNs) { s_stop = 1; set_status(p.ctrl, WIND_ERR_TIMEOUT); break; }
+                    else if (now - t0 > kWaitLimitNs) { give_up(); break; }
                 }
             }
         }
         __syncthreads();
         return s_stop == 0;
     };
+    // Command `seq` into s_cmd: warp 0 of CTA 0 takes it from the host and passes it on in device memory.
+    auto take_command = [&](uint32_t seq) {
+        __syncthreads();
+        if (warp == 0) {
+            const int words = 4 + 4 * K;
+            const volatile unsigned long long* from = cta == 0 ? p.mail->cmd : p.relay;
+            const unsigned long long limit = cta == 0 ? BS_IDLE_NS : kWaitLimitNs;
+            unsigned long long v[(kBeamWords + 31) / 32], t0 = 0;
+            for (uint32_t it = 1;; ++it) {
+                bool ok = true;
+#pragma unroll
+                for (int j = 0; j < (kBeamWords + 31) / 32; ++j) {
+                    v[j] = 0ull;
+                    if (lane + 32 * j < words) {
+                        v[j] = from[lane + 32 * j];
+                        ok = ok && (uint32_t)(v[j] >> 32) == seq;
+                    }
+                }
+                if (__all_sync(0xffffffffu, ok)) break;
+                if ((it & 15u) == 0u) {
+                    const unsigned long long now = __shfl_sync(0xffffffffu, globaltimer_ns(), 0);
+                    if (t0 == 0) {
+                        t0 = now;
+                    } else if (now - t0 > limit) {
+                        if (cta != 0 && lane == 0) give_up();
+#pragma unroll
+                        for (int j = 0; j < (kBeamWords + 31) / 32; ++j) v[j] = bs_word(0xffffffffu, seq);
+                        break;
+                    }
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < (kBeamWords + 31) / 32; ++j)
+                if (lane + 32 * j < words) {
+                    if (cta == 0) const_cast<volatile unsigned long long*>(p.relay)[lane + 32 * j] = v[j];
+                    s_cmd[lane + 32 * j] = (int)(uint32_t)v[j];
+                }
+        }
+        __syncthreads();
+    };
 
-    // ---- decoder update: per layer the gates of this CTA's hidden units, then h and c into the new hypotheses' slots ----
-    if (nu > 0) {
-        for (int l = 0; l < p.L; ++l) {
-            const int nin = l == 0 ? p.E : P, K32 = (nin + P + 31) / 32 * 32;
+    for (uint32_t seq = p.first_seq;; ++seq) {
+        take_command(seq);
+        const int nu = s_cmd[0], nh = s_cmd[1], n = s_cmd[2], t = s_cmd[3];
+        if (nu < 0) return;                                  // the end of the search, or no command for too long
+        const int *c_src = s_cmd + 4, *c_tok = c_src + K, *c_dst = c_tok + K, *c_slot = c_dst + K;
+        if (nu > 0 && !M.resident) load_layer(0);
+#pragma unroll 1
+        for (int w = warp; w < n; w += BS_WARPS) copy_row(encs + w * H, static_cast<const TW*>(p.enc_proj) + (size_t)(t + w) * H, H);
+
+        // ---- decoder update: per layer the gates of this CTA's hidden units, then h and c into the new hypotheses' slots ----
+        if (nu > 0) {
+#pragma unroll 1
+            for (int l = 0; l < p.L; ++l) {
+                const int nin = l == 0 ? p.E : P, K32 = (nin + P + 31) / 32 * 32;
+#pragma unroll 1
+                for (int u0 = 0; u0 < nu; u0 += BS_UTTS) {
+                    const int n_here = min(BS_UTTS, nu - u0);
+                    if (u0 > 0) __syncthreads();
+                    // x and the state before it of four updates (those behind the last repeat it)
+                    int src[BS_UTTS], dst[BS_UTTS], tok[BS_UTTS];
+#pragma unroll
+                    for (int u = 0; u < BS_UTTS; ++u) { const int uu = u0 + min(u, n_here - 1); src[u] = c_src[uu]; dst[u] = c_dst[uu]; tok[u] = c_tok[uu]; }
+                    const int me = u0 + min(col, n_here - 1);
+                    auto c_of = [&](int ui) { return p.c_pool + (size_t)c_src[me] * LP + l * P + ui * G + cta; };
+                    float c_in = warp < units ? __ldcg(c_of(warp)) : 0.f;          // requested ahead of everything else
+#pragma unroll 1
+                    for (int k = tid; k < K32; k += BS_THREADS) {
+                        float x[BS_UTTS] = {0.f, 0.f, 0.f, 0.f};
+                        if (k < nin && l == 0) {
+#pragma unroll
+                            for (int u = 0; u < BS_UTTS; ++u) x[u] = (float)static_cast<const TW*>(p.emb)[(size_t)tok[u] * p.E + k];
+                        } else if (k < nin + P) {
+                            const int at = k < nin ? (l - 1) * P + k : l * P + k - nin;
+#pragma unroll
+                            for (int u = 0; u < BS_UTTS; ++u) x[u] = bs_round<TW>(__ldcg(p.h_pool + (size_t)(k < nin ? dst[u] : src[u]) * LP + at));
+                        }
+                        *reinterpret_cast<float4*>(xs + 4 * k) = make_float4(x[0], x[1], x[2], x[3]);
+                    }
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncthreads();
+#pragma unroll 1
+                    for (int ui = warp; ui < units; ui += BS_WARPS) {
+                        const int j = ui * G + cta;
+                        const float mine = bs_dots<TW>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * lane), K32 / 32) + b_gate[4 * (l * M.units + ui) + grp];
+                        const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
+                                    ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
+                        const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
+                        const float cc = gf * c_in + gi * gg;
+                        if ((lane & 25) == 0 && col < n_here) {
+                            p.c_pool[(size_t)c_dst[me] * LP + l * P + j] = cc;
+                            p.h_pool[(size_t)c_dst[me] * LP + l * P + j] = go * tanhf(cc);
+                        }
+                        if (ui + BS_WARPS < units) c_in = __ldcg(c_of(ui + BS_WARPS));
+                    }
+                }
+                arrive();
+                if (!M.resident && l + 1 < p.L) load_layer(l + 1);
+                if (!wait()) return;
+            }
+            // ---- pred_proj of this CTA's joint units ----
+#pragma unroll 1
             for (int u0 = 0; u0 < nu; u0 += BS_UTTS) {
                 const int n_here = min(BS_UTTS, nu - u0);
                 if (u0 > 0) __syncthreads();
-                // x and the state before it, one row per update
-                for (int u = 0; u < BS_UTTS; ++u) {
-                    const int uu = u0 + min(u, n_here - 1);
-                    for (int k = tid; k < K32; k += BS_THREADS) {
-                        float x = 0.f;
-                        if (k < nin) x = l == 0 ? (float)static_cast<const TW*>(p.emb)[(size_t)p.io.tok[uu] * p.E + k]
-                                                : bs_round<TW>(__ldcg(p.h_pool + (size_t)p.io.dst[uu] * LP + (l - 1) * P + k));
-                        else if (k < nin + P) x = bs_round<TW>(__ldcg(p.h_pool + (size_t)p.io.src[uu] * LP + l * P + k - nin));
-                        xs[u * M.k_l + k] = x;
+                int dst[BS_UTTS];
+#pragma unroll
+                for (int u = 0; u < BS_UTTS; ++u) dst[u] = c_dst[u0 + min(u, n_here - 1)];
+#pragma unroll 1
+                for (int k = tid; k < M.k_p; k += BS_THREADS) {
+                    float x[BS_UTTS] = {0.f, 0.f, 0.f, 0.f};
+                    if (k < P) {
+#pragma unroll
+                        for (int u = 0; u < BS_UTTS; ++u) x[u] = bs_round<TW>(__ldcg(p.h_pool + (size_t)dst[u] * LP + (p.L - 1) * P + k));
                     }
+                    *reinterpret_cast<float4*>(xs + 4 * k) = make_float4(x[0], x[1], x[2], x[3]);
                 }
-                if (u0 == 0 && l == 0) asm volatile("cp.async.wait_group 1;" ::: "memory");   // the gates' weights; the others may still come
-                else asm volatile("cp.async.wait_all;" ::: "memory");
                 __syncthreads();
-                for (int item = warp; item < units * 2; item += BS_WARPS) {
-                    const int ui = item >> 1, u = (item & 1) * 2, j = ui * G + cta;
-                    if (u >= n_here) continue;
-                    // c and the biases are requested ahead of the sums
-                    const int me = u0 + min(u + (lane & 1), n_here - 1);
-                    const float c_in = __ldcg(p.c_pool + (size_t)p.io.src[me] * LP + l * P + j);
-                    const float bias = p.b_ih[l][grp * P + j] + p.b_hh[l][grp * P + j];
-                    float s[2];
-                    bs_dots<2>(w_l + (ui * 4 + grp) * M.ld_l + 4 * q, xs + u * M.k_l + 4 * q, M.k_l, K32 / 32, s);
-                    const float mine = ((lane & 1) ? s[1] : s[0]) + bias;
-                    const float ai = __shfl_sync(0xffffffffu, mine, lane & 1), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 1)),
-                                ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 1)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 1));
-                    const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
-                    const float cc = gf * c_in + gi * gg;
-                    if (lane < 2 && u + lane < n_here) {
-                        p.c_pool[(size_t)p.io.dst[me] * LP + l * P + j] = cc;
-                        p.h_pool[(size_t)p.io.dst[me] * LP + l * P + j] = go * tanhf(cc);
-                    }
+#pragma unroll 1
+                for (int pg = warp; pg * 4 < prows; pg += BS_WARPS) {
+                    const int pi = pg * 4 + grp, o = min(pi, prows - 1) * G + cta;
+                    const float mine = bs_dots<TW>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * lane), M.k_p / 32) + b_pred[min(pi, prows - 1)];
+                    if ((lane & 1) == 0 && pi < prows && col < n_here) p.g_pool[(size_t)c_dst[u0 + col] * H + o] = mine;
                 }
             }
             arrive();
-            if (l + 1 < p.L) load_layer(l + 1);
             if (!wait()) return;
         }
-        // ---- pred_proj of this CTA's joint units ----
-        for (int u0 = 0; u0 < nu; u0 += BS_UTTS) {
-            const int n_here = min(BS_UTTS, nu - u0);
-            if (u0 > 0) __syncthreads();
-            for (int u = 0; u < n_here; ++u)
-                for (int k = tid; k < M.k_p; k += BS_THREADS)
-                    xs[u * M.k_l + k] = k < P ? bs_round<TW>(__ldcg(p.h_pool + (size_t)p.io.dst[u0 + u] * LP + (p.L - 1) * P + k)) : 0.f;
-            asm volatile("cp.async.wait_all;" ::: "memory");
+
+        // ---- logits of this CTA's labels for every row of the window under every hypothesis ----
+        const int rows = nh * n;
+#pragma unroll 1
+        for (int b = warp >> 2; b < nh; b += BS_WARPS / 4)
+#pragma unroll 2
+            for (int k = (tid & 127) * 4; k < H; k += 512)
+                *reinterpret_cast<float4*>(xs + b * H + k) = __ldcg(reinterpret_cast<const float4*>(p.g_pool + (size_t)c_slot[b] * H + k));
+        asm volatile("cp.async.wait_all;" ::: "memory");
+#pragma unroll 1
+        for (int r0 = 0; r0 < rows; r0 += M.zrows) {
+            const int nr = min(M.zrows, rows - r0), nr4 = (nr + BS_ROWS - 1) / BS_ROWS;
             __syncthreads();
-            for (int item = warp; item < (prows + 3) / 4 * n_here; item += BS_WARPS) {
-                const int u = item % n_here, pi = item / n_here * 4 + grp, pr = min(pi, prows - 1), o = pr * G + cta;
-                const float bias = p.b_pred[o];
-                float s;
-                bs_dots<1>(w_pred + pr * M.ld_p + 4 * q, xs + u * M.k_l + 4 * q, M.k_l, M.k_p / 32, &s);
-                if (q == 0 && pi < prows) p.g_pool[(size_t)p.io.dst[u0 + u] * H + o] = s + bias;
+            // a warp takes four rows and a share of k
+            const int cut = nr4 < BS_WARPS ? BS_WARPS / nr4 : 1;
+#pragma unroll 1
+            for (int item = warp; item < nr4 * cut; item += BS_WARPS) {
+                const int rg = item / cut;
+                const TW* e4[4];
+                const float* g4[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    const int row = min(r0 + rg * BS_ROWS + j, rows - 1), b = row / n;
+                    e4[j] = encs + (row - b * n) * H;
+                    g4[j] = xs + b * H;
+                }
+#pragma unroll 2
+                for (int k = lane + 32 * (item - rg * cut); k < M.k_z; k += 32 * cut) {
+                    float z[4] = {0.f, 0.f, 0.f, 0.f};
+                    if (k < H) {
+#pragma unroll
+                        for (int j = 0; j < 4; ++j) z[j] = (float)e4[j][k] + g4[j][k];
+                        if (p.act == WIND_ACT_RELU) {
+#pragma unroll
+                            for (int j = 0; j < 4; ++j) z[j] = fmaxf(z[j], 0.f);
+                        } else {
+#pragma unroll 1
+                            for (int j = 0; j < 4; ++j) {              // one tanh in the code
+                                const float v = tanhf(z[0]);
+                                z[0] = z[1]; z[1] = z[2]; z[2] = z[3]; z[3] = v;
+                            }
+                        }
+                    }
+                    *reinterpret_cast<float4*>(zs + 4 * (rg * M.k_z + k)) =
+                        make_float4(bs_round<TW>(z[0]), bs_round<TW>(z[1]), bs_round<TW>(z[2]), bs_round<TW>(z[3]));
+                }
+            }
+            __syncthreads();
+            const int lgs = (labels + 3) / 4;
+#pragma unroll 1
+            for (int item = warp; item < lgs * nr4; item += BS_WARPS) {
+                const int rg = item / lgs, lg = item - rg * lgs, li = lg * 4 + grp, v = min(li, labels - 1) * G + cta;
+                const float mine = bs_dots<TW>(smem_u32(w_out + 4 * (lg * M.k_z + lane)), smem_u32(zs + 4 * (rg * M.k_z + lane)), M.k_z / 32) + b_out[min(li, labels - 1)];
+                const int row = r0 + rg * BS_ROWS + col, b = row / n;
+                if ((lane & 1) == 0 && rg * BS_ROWS + col < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = mine;
             }
         }
         arrive();
-        if (!wait()) return;
-    }
-
-    // ---- logits of this CTA's labels for every row of the window under every hypothesis ----
-    const int n = p.io.n_rows, rows = nh * n;
-    asm volatile("cp.async.wait_all;" ::: "memory");
-    for (int r0 = 0; r0 < rows; r0 += M.zrows) {
-        const int nr = min(M.zrows, rows - r0), nr4 = (nr + BS_ROWS - 1) / BS_ROWS;
-        const int h4 = M.ld_z / 4;
-        __syncthreads();
-#pragma unroll 2
-        for (int i = tid; i < nr4 * BS_ROWS * h4; i += BS_THREADS) {
-            const int r = i / h4, k = (i - r * h4) * 4, row = r0 + r, b = row / n, w = row - b * n;
-            float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
-            if (row < rows && k < H) {
-                const float4 e = bs_load4(static_cast<const TW*>(p.enc_proj) + (size_t)(p.io.t + w) * H + k);
-                const float4 g = __ldcg(reinterpret_cast<const float4*>(p.g_pool + (size_t)p.io.slot[b] * H + k));
-                z = make_float4(e.x + g.x, e.y + g.y, e.z + g.z, e.w + g.w);
-                if (p.act == WIND_ACT_RELU) z = make_float4(fmaxf(z.x, 0.f), fmaxf(z.y, 0.f), fmaxf(z.z, 0.f), fmaxf(z.w, 0.f));
-                else z = make_float4(tanhf(z.x), tanhf(z.y), tanhf(z.z), tanhf(z.w));
-                z = make_float4(bs_round<TW>(z.x), bs_round<TW>(z.y), bs_round<TW>(z.z), bs_round<TW>(z.w));
-            }
-            *reinterpret_cast<float4*>(area + r * M.ld_z + k) = z;
-        }
-        __syncthreads();
-        const int lgs = (labels + 3) / 4;
-        for (int item = warp; item < lgs * nr4; item += BS_WARPS) {
-            const int rg = item / lgs, li = (item - rg * lgs) * 4 + grp, lr = min(li, labels - 1), v = lr * G + cta;
-            const float bias = p.b_out[v];
-            float s[BS_ROWS];
-            bs_dots<BS_ROWS>(w_out + lr * M.ld_o + 4 * q, area + rg * BS_ROWS * M.ld_z + 4 * q, M.ld_z, M.ld_z / 32, s);
-            float mine = s[0];
-#pragma unroll
-            for (int i = 1; i < BS_ROWS; ++i) mine = q == i ? s[i] : mine;
-            const int row = r0 + rg * BS_ROWS + q, b = row / n;
-            if (q < BS_ROWS && rg * BS_ROWS + q < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = mine + bias;
-        }
-    }
-    arrive();
-    if (cta >= nh) return;
-    if (!wait()) return;
-
-    // ---- Eq. (1) for hypothesis `cta`, the window's logits in shared memory ----
-    const float* src = p.logits + (size_t)cta * p.W * NV;
-    const int total = n * NV;
+        if (cta < nh) {
+            if (!wait()) return;
+            // ---- Eq. (1) for hypothesis `cta`, the window's logits in shared memory ----
+            const float* src = p.logits + (size_t)cta * p.W * NV;
+            const int total = n * NV;
+#pragma unroll 16
+            for (int i = tid; i < total; i += BS_THREADS) zs[i] = __ldcg(src + i);
+            __syncthreads();
+#pragma unroll 1
+            for (int w = warp; w < n; w += BS_WARPS) {
+                const float* row = zs + w * NV;
+                float mx = -INFINITY;
 #pragma unroll 8
-    for (int i = tid; i < total; i += BS_THREADS) area[i] = __ldcg(src + i);
-    __syncthreads();
-    for (int w = warp; w < n; w += BS_WARPS) {
-        const float* row = area + w * NV;
-        float mx = -INFINITY;
+                for (int v = lane; v < NV; v += 32) mx = fmaxf(mx, row[v]);
+                mx = bs_warp_max(mx);
+                float se = 0.f;
+#pragma unroll 8
+                for (int v = lane; v < NV; v += 32) se += expf(row[v] - mx);
+                se = bs_warp_sum(se);
+                if (lane == 0) {
+                    const float lse = mx + logf(se);
+                    s_lse[w] = lse;
+                    s_blank[w] = row[p.blank] - lse;
+                }
+            }
+            __syncthreads();
+            // log P'(v, w) = logit + shift: all blanks before, then v
+            auto shift_of = [&](int w) {
+                float before = 0.f;
+#pragma unroll 8
+                for (int i = 0; i < w; ++i) before += s_blank[i];
+                return before - s_lse[w];
+            };
+            // ---- the K best entries, best first; equal values in order of (offset, label) ----
+            // A lane finds the best entry of its share, the warp takes out the best of its lanes K times, and all its lanes
+            // together look through the share that lost its entry.  (Sorted lists per thread took 9000 cycles for a window of
+            // 8 x 1025, a rescan by the one lane 10700.)
+            const int parts = n < BS_WARPS ? BS_WARPS / n : 1, stride = 32 * parts;      // warps of a row
+            unsigned long long mine = 0ull;
+#pragma unroll 1
+            for (int item = warp; item < n * parts; item += BS_WARPS) {
+                const int w = item / parts;
+                const float shift = shift_of(w);
+                const float* row = zs + w * NV;
+                const int skip = w != n - 1 ? p.blank : -1;
+                float bv = -INFINITY;
+                int at = -1;
 #pragma unroll 4
-        for (int v = lane; v < NV; v += 32) mx = fmaxf(mx, row[v]);
-        mx = bs_warp_max(mx);
-        float se = 0.f;
-#pragma unroll 4
-        for (int v = lane; v < NV; v += 32) se += expf(row[v] - mx);
-        se = bs_warp_sum(se);
-        if (lane == 0) s_lse[w] = mx + logf(se);
-    }
-    __syncthreads();
-    if (tid == 0) {
-        float before = 0.f;
-        for (int w = 0; w < n; ++w) {
-            s_before[w] = before;
-            before += area[w * NV + p.blank] - s_lse[w];
-        }
-    }
-    __syncthreads();
-    // ---- the K best entries, best first; equal values in order of (offset, label): a thread's own, a warp's, the block's ----
-    unsigned long long best[KL];
-#pragma unroll
-    for (int j = 0; j < KL; ++j) best[j] = 0ull;
-    for (int w = warp; w < n; w += BS_WARPS) {
-        const float shift = s_before[w] - s_lse[w];
-        for (int v = lane; v < NV; v += 32) {
-            const float x = area[w * NV + v] + shift;
-            unsigned long long key = (v == p.blank && w != n - 1) ? 0ull : bs_pair(x, w * NV + v);
-            if (key > best[KL - 1]) {
-#pragma unroll
-                for (int j = 0; j < KL; ++j) {
-                    const unsigned long long hi = key > best[j] ? key : best[j], lo = key > best[j] ? best[j] : key;
-                    best[j] = hi; key = lo;
+                for (int v = lane + 32 * (item - w * parts); v < NV; v += stride) {
+                    const float x = row[v] + shift;
+                    if (x > bv && v != skip) { bv = x; at = v; }                        // v ascends: the first of equals stays
+                }
+                if (at >= 0) mine = max(mine, pack_key(bv, (uint32_t)(w * NV + at)));
+            }
+#pragma unroll 1
+            for (int k = 0; k < K; ++k) {
+                const unsigned long long top = bs_best_of_warp(mine);
+                if (lane == 0) s_cand[warp * K + k] = top;
+                if (top == 0ull || k + 1 == K) continue;
+                const int owner = __ffs((int)__ballot_sync(0xffffffffu, mine == top)) - 1;
+                unsigned long long next = 0ull;
+#pragma unroll 1
+                for (int item = warp; item < n * parts; item += BS_WARPS) {
+                    const int w = item / parts;
+                    const float shift = shift_of(w);
+                    const int skip = w != n - 1 ? p.blank : -1;
+#pragma unroll 1
+                    for (int v = owner + 32 * (item - w * parts) + lane * stride; v < NV; v += 32 * stride) {
+                        const float x = zs[w * NV + v] + shift;
+                        const unsigned long long key = x > -INFINITY && v != skip ? pack_key(x, (uint32_t)(w * NV + v)) : 0ull;
+                        if (key < top) next = max(next, key);
+                    }
+                }
+                next = bs_best_of_warp(next);
+                if (lane == owner) mine = next;
+            }
+            __syncthreads();
+            if (warp == 0) {
+                int pos = 0;                                        // lanes 0..15 take one warp's list each
+#pragma unroll 1
+                for (int k = 0; k < K; ++k) {
+                    const unsigned long long mine = lane < BS_WARPS && pos < K ? s_cand[lane * K + pos] : 0ull, top = bs_best_of_warp(mine);
+                    if (mine == top) ++pos;
+                    if (lane == 0) {
+                        volatile unsigned long long* out = p.mail->top + 2 * (cta * K + k);
+                        out[0] = bs_word(top != 0ull ? key_label(top) : 0xffffffffu, seq);
+                        out[1] = bs_word(__float_as_uint(top != 0ull ? key_logit(top) : -INFINITY), seq);
+                    }
                 }
             }
         }
-    }
-    auto pop_best = [&]() -> unsigned long long {       // the warp's best entry, taken out of its owner's list
-        const unsigned long long top = bs_best_of_warp(best[0]);
-        if (top != 0ull && best[0] == top) {
-#pragma unroll
-            for (int j = 0; j + 1 < KL; ++j) best[j] = best[j + 1];
-            best[KL - 1] = 0ull;
-        }
-        return top;
-    };
-#pragma unroll 1
-    for (int k = 0; k < KL; ++k) {
-        const unsigned long long top = pop_best();
-        if (lane == 0) s_cand[warp * KL + k] = top;
-    }
-    __syncthreads();
-    if (warp != 0) return;
-    // lanes 0..15 take one warp's list each
-#pragma unroll
-    for (int j = 0; j < KL; ++j) best[j] = lane < BS_WARPS ? s_cand[lane * KL + j] : 0ull;
-#pragma unroll 1
-    for (int k = 0; k < K; ++k) {
-        const unsigned long long top = pop_best();
-        if (lane == 0) {
-            const int i = (int)key_label(top), off = top != 0ull ? i / NV : -1;
-            BeamTop r;
-            r.label = top != 0ull ? i - off * NV : -1;
-            r.jump = off;
-            r.logp = top != 0ull ? key_logit(top) : -INFINITY;
-            r.pad = 0;
-            p.io.top[cta * K + k] = r;
-        }
-    }
-    if (lane == 0) {
-        __threadfence_system();
-        *const_cast<volatile uint32_t*>(p.io.done + cta) = p.io.seq;
+        if (p.single) return;
     }
 }
 
-template <typename TW> static const void* bs_fn(int K) {
-    return K <= 4 ? (const void*)beam_step_kernel<TW, 4> : (K <= 8 ? (const void*)beam_step_kernel<TW, 8> : (const void*)beam_step_kernel<TW, 16>);
-}
+template <typename TW> static const void* bs_fn() { return (const void*)beam_step_kernel<TW>; }
 
 static std::mutex g_bs_mutex;
 static int g_bs_optin[64] = {};        // opt-in shared memory per block, 0: not asked yet
@@ -419,9 +552,8 @@ static cudaError_t bs_device(int* optin) {
     if (!g_bs_optin[dev]) {
         int n = 0;
         if ((e = cudaDeviceGetAttribute(&n, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev)) != cudaSuccess) return e;
-        for (int K : {4, 8, 16})
-            for (const void* fn : {bs_fn<float>(K), bs_fn<__nv_bfloat16>(K)})
-                if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, n - 4096)) != cudaSuccess) return e;   // static: below 4 KB
+        for (const void* fn : {bs_fn<float>(), bs_fn<__nv_bfloat16>()})
+            if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, n - 4096)) != cudaSuccess) return e;   // static: below 4 KB
         g_bs_optin[dev] = n;
     }
     *optin = g_bs_optin[dev];
@@ -435,7 +567,7 @@ static BsPlan bs_plan_of(const Call& c, int sms, uint32_t budget) {
 }
 
 // Rows in whole 16-byte pieces (8 bf16; fp32 models take the same rule), a CTA's weights and one window's logits in shared
-// memory, every CTA the owner of something, and a CTA for every hypothesis.  Else the per-phase kernels.
+// memory, and a CTA for every hypothesis.  Else the per-phase kernels.
 bool beam_step_supported(const Call& c) {
     const wind_model_t& m = c.m;
     if (m.E % 8 || m.P % 8 || m.H % 8) return false;
@@ -448,27 +580,32 @@ bool beam_step_supported(const Call& c) {
     return c.B <= sms && bs_plan_of(c, sms, (uint32_t)optin - 4096u).total <= (uint32_t)optin - 4096u;
 }
 
-cudaError_t beam_step(const Call& c, const BeamStep& io, float* h_pool, float* c_pool, float* g_pool, float* logits, uint32_t* bar_base) {
+cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base, bool single,
+                      float* h_pool, float* c_pool, float* g_pool, float* logits) {
     int optin = 0, sms = 0;
     cudaError_t e = bs_device(&optin);
     if (e == cudaSuccess) e = loop_sm_count(&sms);
     if (e != cudaSuccess) return e;
     const wind_model_t& m = c.m;
     BsParams p{};
-    p.io = io;
-    p.ctrl = c.ctrl();
-    p.bar_base = *bar_base;
+    p.ctrl = c.ctrl(); p.mail = mail; p.relay = relay;
+    p.first_seq = first_seq; p.bar_base = bar_base; p.single = single; p.K = c.B;
     p.extra_arrivals = (uint32_t)loop_extra_arrivals();
-    p.budget = (uint32_t)optin - 4096u;
+    p.plan = bs_plan_of(c, sms, (uint32_t)optin - 4096u);
     p.E = m.E; p.P = m.P; p.L = m.L; p.H = m.H; p.NV = m.V + 1; p.blank = m.blank_id; p.act = m.act; p.W = c.W;
     p.emb = m.emb; p.w_pred = m.w_pred; p.b_pred = m.b_pred; p.w_out = m.w_out; p.b_out = m.b_out;
     for (int l = 0; l < m.L; ++l) { p.w_ih[l] = c.w_ih[l]; p.w_hh[l] = c.w_hh[l]; p.b_ih[l] = c.b_ih[l]; p.b_hh[l] = c.b_hh[l]; }
     p.enc_proj = c.enc_proj();
     p.h_pool = h_pool; p.c_pool = c_pool; p.g_pool = g_pool; p.logits = logits;
-    *bar_base += (uint32_t)sms * (uint32_t)((io.n_update > 0 ? m.L + 1 : 0) + 1);
-    const void* fn = m.dtype == WIND_DT_BF16 ? bs_fn<__nv_bfloat16>(io.K) : bs_fn<float>(io.K);
+    const void* fn = m.dtype == WIND_DT_BF16 ? bs_fn<__nv_bfloat16>() : bs_fn<float>();
     void* args[1] = {(void*)&p};
-    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)sms), dim3(BS_THREADS), args, bs_plan_of(c, sms, p.budget).total, c.stream);
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)sms), dim3(BS_THREADS), args, p.plan.total, c.stream);
+}
+// arrivals at the grid barrier during one command
+uint32_t beam_step_arrivals(const Call& c, int n_update) {
+    int sms = 0;
+    loop_sm_count(&sms);
+    return (uint32_t)sms * (uint32_t)((n_update > 0 ? c.m.L + 1 : 0) + 1);
 }
 
 }  // namespace wind

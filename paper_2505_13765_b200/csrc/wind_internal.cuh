@@ -223,22 +223,25 @@ struct BeamLayout {
     size_t ints;                     // int32 [8][K] per-iteration index arrays
     size_t logits;                   // fp32 [K][W][V+1]
     size_t top_label, top_jump, top_logp;   // [K][K]
+    size_t relay;                    // uint64 [kBeamWords]
     size_t total;
     int slots;
 };
-// One iteration on the device (wind_beam_step.cu): decoder updates, window logits, Eq. (1), the K best entries per hypothesis.
+// Iterations on the device (wind_beam_step.cu): a kernel that takes commands from page-locked host memory and leaves each
+// hypothesis's K best entries there.  A word is (number of the command) << 32 | value.
 constexpr int kMaxBeam = 16;
-struct BeamTop { int32_t label, jump; float logp; int32_t pad; };
-struct BeamStep {
-    int32_t K, n_update, n_hyps, n_rows, t;   // n_rows: the window, cut short by the end of the utterance
-    uint32_t seq;                             // written to done[b] behind hypothesis b's entries
-    BeamTop* top;                             // [K][K]  host memory
-    uint32_t* done;                           // [K]     host memory
-    int32_t src[kMaxBeam], tok[kMaxBeam], dst[kMaxBeam];   // n_update decoder updates: slot before, token, slot after
-    int32_t slot[kMaxBeam];                                // n_hyps hypotheses: their states
+constexpr int kBeamWords = 4 + 4 * kMaxBeam;
+struct BeamMail {
+    // n_update (-1: end), n_hyps, n_rows (the window, cut short by the end of the utterance), t; then for K updates each the
+    // slot of the state before, the token, the slot of the state after; then the states of K hypotheses
+    alignas(128) unsigned long long cmd[kBeamWords];
+    alignas(128) unsigned long long top[2 * kMaxBeam * kMaxBeam];   // per entry: offset * (V + 1) + label (all ones: none), fp32 bits of log P'
+    alignas(128) uint32_t failed;                                   // a wait inside the kernel ran out
 };
 bool beam_step_supported(const Call& c);
-cudaError_t beam_step(const Call& c, const BeamStep& io, float* h_pool, float* c_pool, float* g_pool, float* logits, uint32_t* bar_base);
+cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base, bool single,
+                      float* h_pool, float* c_pool, float* g_pool, float* logits);
+uint32_t beam_step_arrivals(const Call& c, int n_update);
 BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, size_t base);
 wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_search, int max_hyps, int max_out, int32_t* out_tokens,
                               int32_t* out_frames, int32_t* out_len, double* out_score, int32_t* n_hyps, int64_t* n_steps,
