@@ -1731,12 +1731,24 @@ static cudaError_t loop_map(CUtensorMap* map, const void* base, uint64_t rows, u
     return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// the same matrix seen as (64 columns, rows, cols / 64 blocks): one box of (64, box_rows, all blocks) lands in shared
-// memory as cols / 64 consecutive K blocks of box_rows x 128 bytes, each with the 128-byte swizzle
-cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows) {
+// the same matrix seen as (64 columns, rows, cols / 64 blocks): one box of (64, box_rows, box_blocks; 0: all) lands in shared
+// memory as that many consecutive K blocks of box_rows x 128 bytes, each with the 128-byte swizzle
+cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks) {
     cuuint64_t dims[3] = {(cuuint64_t)BK, rows, cols / BK};
     cuuint64_t strides[2] = {cols * 2, (cuuint64_t)BK * 2};
-    cuuint32_t box[3] = {(cuuint32_t)BK, box_rows, (cuuint32_t)(cols / BK)};
+    cuuint32_t box[3] = {(cuuint32_t)BK, box_rows, box_blocks ? box_blocks : (cuuint32_t)(cols / BK)};
+    cuuint32_t estr[3] = {1, 1, 1};
+    CUresult r = g_encode_loop(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
+                               CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
+}
+
+// [blocks][rows][64] bf16, box box_blocks x box_rows x 64, 128-byte swizzle
+cudaError_t loop_map_blocks(CUtensorMap* map, const void* base, uint64_t blocks, uint64_t rows, uint32_t box_rows, uint32_t box_blocks) {
+    cuuint64_t dims[3] = {(cuuint64_t)BK, rows, blocks};
+    cuuint64_t strides[2] = {(cuuint64_t)BK * 2, rows * BK * 2};
+    cuuint32_t box[3] = {(cuuint32_t)BK, box_rows, box_blocks};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = g_encode_loop(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, const_cast<void*>(base), dims, strides, box, estr,
                                CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
@@ -1998,8 +2010,11 @@ cudaError_t loop_prepare(Call& c) {
 
 cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* prefix_len, float* logits_out,
                     int trace_step) {
-    if (!logits_out && trace_step < -1 && cl_supported(c)) return cl_loop(c);
     const LoopPlan& pl = t_loop_plan;
+    if (!logits_out && trace_step < -1) {
+        if (cl_supported(c)) return cl_loop(c);
+        if (!pl.resident && wide_supported(c)) return wide_loop(c);
+    }
     LoopParams p{};
     p.ctrl = c.ctrl();
     p.B = c.B; p.T = c.T; p.W = c.W; p.S = c.S; p.max_out = c.max_out;

@@ -137,9 +137,14 @@ cudaError_t loop_res_set_smem(int bytes);
 cudaError_t loop_res_launch(const LoopMaps& maps, const LoopParams& p, int grid, uint32_t smem_bytes, bool full, cudaStream_t stream);
 int loop_set_extra_arrivals(int n);  // returns the previous value
 int loop_extra_arrivals();
-// bf16 matrix [rows, cols] as (64 columns, rows, cols / 64): one box lands as K blocks of box_rows x 128 bytes, 128-byte swizzle
-// (needs a loop_prepare before it)
-cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows);
+// bf16 matrix [rows, cols] as (64 columns, rows, cols / 64): one box lands as box_blocks (0: all) K blocks of box_rows x 128
+// bytes, 128-byte swizzle (needs a loop_prepare before it)
+cudaError_t loop_map3(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint32_t box_rows, uint32_t box_blocks = 0);
+// [blocks][rows][64] bf16: one box lands as box_blocks K blocks of box_rows x 128 bytes
+cudaError_t loop_map_blocks(CUtensorMap* map, const void* base, uint64_t blocks, uint64_t rows, uint32_t box_rows, uint32_t box_blocks);
+// the kernel for large vocabularies (wind_loop_wide.cu)
+bool wide_supported(const Call& c);
+cudaError_t wide_loop(const Call& c);
 cudaError_t loop_prepare(Call& c);   // plan + tensor maps + shared-memory opt-in (host only; not inside a capture)
 
 }  // namespace wind
