@@ -330,14 +330,23 @@ wind_status_t wind_decode_greedy_host(const wind_model_t* m, const void* enc_hos
     for (int b = 0; b < B; ++b)
         if (enc_len_host[b] < 0 || enc_len_host[b] > T) return WIND_ERR_INVALID_ARG;   // before anything is enqueued
     // only the valid frames of every utterance cross the bus (padding frames are never read for a decision)
-    for (int b = 0; b < B; ++b) {
-        const int len = enc_len_host[b];
-        if (len > 0)
-            WIND_CUDA(cudaMemcpyAsync(static_cast<uint8_t*>(d_enc) + es * (size_t)b * T * m->D,
-                                      static_cast<const uint8_t*>(enc_host) + es * (size_t)b * T * m->D, es * (size_t)len * m->D,
-                                      cudaMemcpyHostToDevice, st));
-    }
     WIND_CUDA(cudaMemcpyAsync(d_len, enc_len_host, sizeof(int32_t) * B, cudaMemcpyHostToDevice, st));
+    const size_t frame = es * (size_t)m->D;
+    int longest_enc = 0;
+    for (int b = 0; b < B; ++b) longest_enc = enc_len_host[b] > longest_enc ? enc_len_host[b] : longest_enc;
+    // page-locked memory in whole 16-byte pieces: one kernel fetches all of it.  Pageable memory, odd frames, and batches of more
+    // utterances than a grid has rows: a copy per utterance.
+    cudaPointerAttributes at{};
+    const bool known = cudaPointerGetAttributes(&at, enc_host) == cudaSuccess;
+    if (!known) cudaGetLastError();
+    if (known && at.type == cudaMemoryTypeHost && at.devicePointer && frame % 16 == 0 && reinterpret_cast<uintptr_t>(at.devicePointer) % 16 == 0 && B <= 65535) {
+        WIND_CUDA(launch_gather_frames(at.devicePointer, d_enc, d_len, B, longest_enc, frame, frame * (size_t)T, st));
+    } else {
+        for (int b = 0; b < B; ++b)
+            if (enc_len_host[b] > 0)
+                WIND_CUDA(cudaMemcpyAsync(static_cast<uint8_t*>(d_enc) + frame * (size_t)b * T, static_cast<const uint8_t*>(enc_host) + frame * (size_t)b * T,
+                                          frame * (size_t)enc_len_host[b], cudaMemcpyHostToDevice, st));
+    }
     Call c;
     fill_call(c, m, d_enc, d_len, B, T, W, max_symbols, d_tok, d_frm, d_olen, max_out, workspace, st);
     s = enqueue_decode(c);

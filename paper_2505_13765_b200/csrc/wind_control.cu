@@ -249,4 +249,29 @@ cudaError_t launch_fill_z(const Call& c) {
     return cudaGetLastError();
 }
 
+// The valid frames of every utterance from page-locked host memory, in 16-byte pieces: block (x, b) copies 32 KB of utterance b.
+// One cudaMemcpyAsync per utterance left the bus idle between copies (24 utterances, 12.3 MB: 390 us).
+constexpr size_t GATHER_BYTES = 32768;
+__global__ void __launch_bounds__(256) gather_frames_kernel(const uint8_t* __restrict__ src, uint8_t* __restrict__ dst, const int32_t* __restrict__ enc_len,
+                                                            size_t frame_bytes, size_t utt_bytes) {
+    const size_t bytes = (size_t)max(enc_len[blockIdx.y], 0) * frame_bytes, at = (size_t)blockIdx.x * GATHER_BYTES;
+    if (at >= bytes) return;
+    const uint4* s = reinterpret_cast<const uint4*>(src + blockIdx.y * utt_bytes + at);
+    uint4* d = reinterpret_cast<uint4*>(dst + blockIdx.y * utt_bytes + at);
+    const int n = (int)((bytes - at < GATHER_BYTES ? bytes - at : GATHER_BYTES) / 16);
+    uint4 v[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if ((int)threadIdx.x + 256 * i < n) v[i] = __ldg(s + threadIdx.x + 256 * i);
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        if ((int)threadIdx.x + 256 * i < n) d[threadIdx.x + 256 * i] = v[i];
+}
+cudaError_t launch_gather_frames(const void* src, void* dst, const int32_t* enc_len, int B, int longest, size_t frame_bytes, size_t utt_bytes, cudaStream_t stream) {
+    const size_t chunks = ((size_t)longest * frame_bytes + GATHER_BYTES - 1) / GATHER_BYTES;
+    if (chunks == 0) return cudaSuccess;
+    gather_frames_kernel<<<dim3((unsigned)chunks, (unsigned)B), 256, 0, stream>>>((const uint8_t*)src, (uint8_t*)dst, enc_len, frame_bytes, utt_bytes);
+    return cudaGetLastError();
+}
+
 }  // namespace wind

@@ -211,6 +211,8 @@ cudaError_t launch_init(const Call& c, int kernels_used, int launches_per_step, 
 cudaError_t launch_control(const Call& c, cudaGraphConditionalHandle handle, int use_handle);
 cudaError_t launch_force_tokens(const Call& c, const int32_t* prefix, int U, const int32_t* prefix_len, int u);
 cudaError_t launch_set_t(const Call& c, const int32_t* t0);
+cudaError_t launch_gather_frames(const void* src, void* dst, const int32_t* enc_len, int B, int longest, size_t frame_bytes, size_t utt_bytes,
+                                 cudaStream_t stream);   // src: device address of page-locked host memory
 cudaError_t launch_fill_z(const Call& c);   // measurement aid: fixed joint activations
 
 // first-output distribution of a window (Eq. 1), in place on the window's logits
