@@ -14,6 +14,8 @@
 //   keys    every CTA sends the best (logit, label) of its labels for each window row to the slot's owner (slot u: CTA u)
 //   control the owner takes Algorithm 2's decision and sends (token, next frame) to every CTA, then records it; the window's
 //           enc_proj rows start on their way (one TMA box per eight rows, in the layout of the joint's operand)
+//   (a step in which no slot feeds a token to its decoder goes from here to the joint, and only slots that do send anything in
+//   the next two phases: most steps of narrow windows emit nothing)
 //   gates   W_hh h was computed a step ahead; + the token's row of the gate table, cell update, new h to every CTA
 //   pred    W_pred h, pred_proj to every CTA
 //   joint   z = act(enc_proj rows + pred_proj) in place, times the CTA's W_out rows on tcgen05 (window rows on the M axis, so
@@ -80,18 +82,16 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         mbar_init(&bar_enc, 1);
         mbar_init(&bar_h, 1);
         mbar_init(&bar_pred, 1);
-        mbar_init(&bar_z, 8);
+        mbar_init(&bar_z, 10u + (has_rem ? 4u : 0u));
         mbar_init(&bar_sync_mma, 6u + (has_rem ? 4u : 0u));
         mbar_init(&bar_acc_g, 1);
         mbar_init(&bar_acc_r, 4);
         mbar_init(&bar_acc_j, 1);
         fence_barrier_init();
         // armed for their first phase (later phases: by the warp that saw the previous one complete, and only then: a barrier must
-        // not be armed twice in a phase)
+        // not be armed twice in a phase).  bar_h and bar_pred are armed in the steps that update a decoder, once it is known how many.
         mbar_expect_tx(&bar_keys, (uint32_t)(2 * CL_SIZE * p.W) * 8u);
         mbar_expect_tx(&bar_dec, (uint32_t)NU * 16u);
-        mbar_expect_tx(&bar_h, (uint32_t)(NU * p.P) * 2u);
-        mbar_expect_tx(&bar_pred, (uint32_t)(NU * p.H) * 2u);
         prefetch_tmap(&enc_map);
     }
     if (warp == 14) tmem_alloc(&tmem_slot, LOOP_TMEM_COLS);
@@ -140,26 +140,32 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     bool ok = true;
     // every slot idle: all warps of the cluster leave in the same step
     auto all_idle = [&]() { return __all_sync(0xffffffffu, lane >= NU || (dec[min(lane, NU - 1)].flags & CL_IDLE) != 0u); };
+    // slots that feed a token to their decoder in this step
+    auto live_slots = [&]() { return __ballot_sync(0xffffffffu, lane < NU && dec[min(lane, NU - 1)].tok >= 0); };
     // ldmatrix address of the state: two K steps of 16 at a time, matrix = 8 slots x 8 columns, lane = (column piece, slot)
     const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
     auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * 2048u + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
 
-    // The joint's operand z = act(enc_proj + pred_proj), in place, by warps 0..7 (it is bound by the shared memory's bandwidth:
-    // 30 KB per group of eight rows; four warps leave a third of that unused, 2830 against 2110 cycles for eight groups).
-    // Of a group the rows that count; threads per row: a multiple of eight, one per 16-byte piece of a K block.
-    const int z_rows = p.wp == 8 ? p.W : 8;
-    const int z_tpr = (256 / z_rows) & ~7;
-    const int z_r = (int)threadIdx.x / z_tpr, z_k0 = ((int)threadIdx.x % z_tpr) >> 3, z_kstep = z_tpr >> 3;   // z_kstep >= 4
+    // The joint's operand z = act(enc_proj + pred_proj), in place, by every warp that computes (0..13; it is bound by the shared
+    // memory's bandwidth: 30 KB per group of eight rows, 2110 cycles for eight groups).  Of a group the rows that count: three
+    // eighths of them to the four workers, the others to the W_pred and remainder warps, which have registers for one 16-byte piece
+    // at a time.  (Half to the workers, half to four W_pred warps: these took 4250 cycles for eight groups.)  Threads per row: a
+    // multiple of eight, one per 16-byte piece of a K block.
+    const int z_rows = p.wp == 8 ? p.W : 8, z_mine = warp < 4 ? (3 * z_rows + 4) / 8 : z_rows - (3 * z_rows + 4) / 8;
+    const int z_threads = warp < 4 ? 128 : (has_rem ? 320 : 192), z_tid = warp < 4 ? (int)threadIdx.x : (int)threadIdx.x - 128;
+    const int z_tpr = (z_threads / max(z_mine, 1)) & ~7, z_at = z_tid / z_tpr;
+    const bool z_on = z_at < z_mine;
+    const int z_r = (warp < 4 ? 0 : z_rows - z_mine) + z_at, z_k0 = (z_tid % z_tpr) >> 3, z_kstep = z_tpr >> 3;
     auto build_z = [&](auto which) {
         constexpr int AT_ONCE = decltype(which)::value;               // pieces in flight per thread (the W_pred warps have registers for one)
-        if (z_r < z_rows) {
+        if (z_on) {
             uint8_t* zp = smem + L.z + (uint32_t)(z_r * 128 + (((lane & 7) ^ (z_r & 7)) << 4) + z_k0 * 1024);
             const uint8_t* pp = smem + L.pred + (uint32_t)(z_k0 * 128 + (lane & 7) * 16);
 #pragma unroll 1
             for (int gi = 0; gi < n_groups; ++gi, zp += p.H * 16) {
                 const uint8_t* py = pp + (uint32_t)(((gi << 3) >> wp_shift) * p.H * 2);
 #pragma unroll 1
-                for (int j0 = 0; j0 < 3; j0 += AT_ONCE) {
+                for (int j0 = 0; z_k0 + j0 * z_kstep < kb_h; j0 += AT_ONCE) {
                     uint4 x[AT_ONCE], y[AT_ONCE];
 #pragma unroll
                     for (int j = 0; j < AT_ONCE; ++j)
@@ -231,12 +237,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         const int h_pieces = NU * (U / 8);
         const int lpd_shift = h_pieces <= 8 ? 3 : (h_pieces <= 16 ? 4 : 5);
         const int h_first = lane & ((1 << lpd_shift) - 1);
-        uint32_t h_src[2], h_dst[2];
+        uint32_t h_src[2], h_dst[2];                     // h_src: slot in the top byte
 #pragma unroll
         for (int k = 0; k < 2; ++k) {
             const int i = h_first + 32 * k;
             const int uu = i / (U / 8), cc = i - uu * (U / 8), col = r * U + cc * 8;
-            h_src[k] = L.hst + (uint32_t)(uu * U + cc * 8) * 2u;
+            h_src[k] = (L.hst + (uint32_t)(uu * U + cc * 8) * 2u) | (uint32_t)uu << 24;
             h_dst[k] = L.h + (uint32_t)((col >> 6) * 2048 + uu * 128 + ((((col >> 3) & 7) ^ (uu & 7)) << 4));
         }
         float c_st[2] = {0.f, 0.f}, c_rem = 0.f;         // cell state: (u, slots 2 g, 2 g + 1); (32 + (e & 7), slot e >> 3) for e < 64
@@ -249,8 +255,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         if (timed) { ns0 = globaltimer_ns(); clk = clock64(); }
         auto lap = [&](int k) { if (timed) { const long long now = clock64(); cyc[k] += now - clk; clk = now; } };
 
-        for (uint32_t step = 0;; ++step) {
-            const uint32_t par = step & 1u;
+        // parities in one word (registers are short): bit 0 of the step, bit 1 of the updates so far, bit 2: there was one
+        for (uint32_t st = 0u;; st ^= 1u) {
+            const uint32_t par = st & 1u;
             // ---- decisions of the step; the gate table's rows are requested at once ----
             if (ok) ok = cl_wait(&bar_dec, par);
             if (ok && warp == 0 && lane == 0) mbar_expect_tx(&bar_dec, (uint32_t)NU * 16u);
@@ -275,10 +282,13 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 for (int k = 0; k < 4; ++k) add_r[k] = tok >= 0 ? g0r[(uint32_t)tok * (uint32_t)(4 * p.P) + (uint32_t)(k * p.P)] : 0.f;
             }
             // ---- gates: recurrent term + gate table, cell update ----
-            if (step > 0) {
-                if (ok) ok = cl_wait(&bar_acc_g, (step - 1u) & 1u);
-                if (has_rem && ok) ok = cl_wait(&bar_acc_r, (step - 1u) & 1u);
+            if (live != 0u) {
+            if (ok && warp == 0 && lane == 0) mbar_expect_tx(&bar_pred, (uint32_t)(__popc(live) * p.H) * 2u);
+            if (st & 4u) {
+                if (ok) ok = cl_wait(&bar_acc_g, (~st >> 1) & 1u);
+                if (has_rem && ok) ok = cl_wait(&bar_acc_r, (~st >> 1) & 1u);
             }
+            st = (st ^ 2u) | 4u;
             tc_fence_after();
             {
                 float x[8];
@@ -334,12 +344,13 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 hst[s * U + 32 + (e & 7)] = h_rem;
             }
             tc_fence_before();
+            }
             if (group_barrier_or<128>(1, !ok || idle)) break;
             // h to all CTAs
 #pragma unroll
             for (int k = 0; k < 2; ++k)
-                if (h_first + 32 * k < h_pieces) {
-                    const uint4 piece = *reinterpret_cast<const uint4*>(smem + h_src[k]);
+                if (h_first + 32 * k < h_pieces && ((live >> (h_src[k] >> 24)) & 1u)) {
+                    const uint4 piece = *reinterpret_cast<const uint4*>(smem + (h_src[k] & 0xFFFFFFu));
                     for (int d0 = warp * (32 >> lpd_shift) + (lane >> lpd_shift); d0 < CL_SIZE; d0 += 128 >> lpd_shift) {
                         const uint32_t d = (uint32_t)(d0 + r) & (CL_SIZE - 1);
                         st_async_16(cl_map(sbase, d) + h_dst[k], piece, cl_map(smem_u32(&bar_h), d));
@@ -348,10 +359,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             lap(1);
             // ---- the joint's operand z = act(enc_proj + pred_proj), in place ----
             if (ok) ok = cl_wait(&bar_enc, par);
-            if (ok) ok = cl_wait(&bar_pred, par);
-            if (ok && warp == 0 && lane == 0) mbar_expect_tx(&bar_pred, (uint32_t)(NU * p.H) * 2u);
+            if (ok) ok = cl_wait(&bar_pred, (~st >> 1) & 1u);        // of the last update: this step's, or long there
             lap(2);
-            build_z(std::integral_constant<int, 3>{});
+            build_z(std::integral_constant<int, 2>{});
             if (ok) ok = cl_wait(&bar_acc_j, par);
             tc_fence_after();
             joint_argmax(std::integral_constant<int, 0>{});
@@ -381,14 +391,16 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         float4* part = reinterpret_cast<float4*>(smem + L.part) + mt * 32 + lane;
         __nv_bfloat16* pst = reinterpret_cast<__nv_bfloat16*>(smem + L.pst) + 16 * mt;     // [slot][48]
         const int halves = min(2, (HS - 16 * mt) / 8);   // 16-byte pieces of a slot in this warp's 16 units
-        for (uint32_t step = 0;; ++step) {
-            const uint32_t par = step & 1u;
+        for (uint32_t st = 0u;; st ^= 1u) {              // bit 0: parity of the step, bit 1: of the updates so far
+            const uint32_t par = st & 1u;
             if (ok) ok = cl_wait(&bar_dec, par);
             const bool idle = all_idle();
-            if (ok && !idle) ok = cl_wait(&bar_h, par);
-            if (ok && !idle && warp == 4 && lane == 0) mbar_expect_tx(&bar_h, (uint32_t)(NU * p.P) * 2u);
+            const uint32_t live = live_slots();
+            if (ok && live != 0u && warp == 4 && lane == 0) mbar_expect_tx(&bar_h, (uint32_t)(__popc(live) * p.P) * 2u);
+            if (live != 0u) st ^= 2u;
+            if (ok) ok = cl_wait(&bar_h, (~st >> 1) & 1u);           // of the last update: this step's, or long there
             float acc[4] = {0.f, 0.f, 0.f, 0.f};
-            if (mine) {
+            if (mine && live != 0u) {
                 uint32_t b[2][4];
                 ldmatrix_x4(b[0], h_at(half * (k16s / 2)));
                 // (the state rows of the next two steps are requested a turn early; at the end they are rows nobody uses)
@@ -404,8 +416,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (half) *part = make_float4(acc[0], acc[1], acc[2], acc[3]);
             }
             if (group_barrier_or<192>(2, !ok || idle)) break;
-            if (lane == 0) mbar_arrive(&bar_sync_mma);
-            if (half == 0 && mine) {
+            if (lane == 0 && live != 0u) mbar_arrive(&bar_sync_mma);
+            if (half == 0 && mine && live != 0u) {
                 // the two K halves are added as loop_kernel adds its accumulators
                 const float4 o = *part;
                 const int m = lane >> 2, s = (lane & 3) * 2;
@@ -419,14 +431,14 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 for (int i = lane; i < NU * halves * CL_SIZE; i += 32) {
                     const int pi = i >> 4, sl = halves == 2 ? pi >> 1 : pi, hh = halves == 2 ? pi & 1 : 0;
                     const uint32_t d = (uint32_t)(i + r) & (CL_SIZE - 1);
-                    st_async_16(cl_map(sbase, d) + L.pred + (uint32_t)(sl * p.H + r * HS + 16 * mt + 8 * hh) * 2u,
+                    if ((live >> sl) & 1u) st_async_16(cl_map(sbase, d) + L.pred + (uint32_t)(sl * p.H + r * HS + 16 * mt + 8 * hh) * 2u,
                                 *reinterpret_cast<const uint4*>(pst + sl * 48 + 8 * hh), cl_map(smem_u32(&bar_pred), d));
                 }
             }
+            if (ok) ok = cl_wait(&bar_enc, par);
+            if (ok) ok = cl_wait(&bar_pred, (~st >> 1) & 1u);
+            build_z(std::integral_constant<int, 1>{});
             if (warp < 8) {
-                if (ok) ok = cl_wait(&bar_enc, par);
-                if (ok) ok = cl_wait(&bar_pred, par);
-                build_z(std::integral_constant<int, 1>{});
                 if (ok) ok = cl_wait(&bar_acc_j, par);
                 tc_fence_after();
                 joint_argmax(std::integral_constant<int, 1>{});
@@ -447,11 +459,13 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (s0 < p.P / 16)
 #pragma unroll
                     for (int s = s0; s < s0 + 8; ++s) { wf[s][0] = src[s * 8]; wf[s][1] = src[s * 8 + 4]; }
-            for (uint32_t step = 0;; ++step) {
-                const uint32_t par = step & 1u;
+            for (uint32_t st = 0u;; st ^= 1u) {          // bit 0: parity of the step, bit 1: of the updates so far
+                const uint32_t par = st & 1u;
                 ok = cl_wait_warp(&bar_dec, par);
                 if (all_idle() || !ok) break;
-                ok = cl_wait_warp(&bar_h, par);
+                if (live_slots() != 0u) {
+                st ^= 2u;
+                ok = cl_wait_warp(&bar_h, (~st >> 1) & 1u);
                 if (!ok) break;
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
                 uint32_t a[2][4];
@@ -468,6 +482,10 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 *reinterpret_cast<float2*>(gr + (lane >> 2) * CL_GR_PITCH + (warp - 10) * 8 + (lane & 3) * 2) = make_float2(acc[0], acc[1]);
                 __syncwarp();
                 if (lane == 0) { mbar_arrive(&bar_acc_r); mbar_arrive(&bar_sync_mma); }
+                }
+                ok = cl_wait_warp(&bar_enc, par) && cl_wait_warp(&bar_pred, (~st >> 1) & 1u);
+                if (!ok) break;
+                build_z(std::integral_constant<int, 1>{});
             }
         }
     } else if (warp == 14) {
@@ -483,8 +501,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 const uint32_t par = step & 1u;
                 if (!(ok = cl_wait(&bar_dec, par))) break;
                 uint32_t idle = CL_IDLE;
+                bool update = false;
 #pragma unroll 1
-                for (int s = 0; s < NU; ++s) idle &= dec[s].flags;
+                for (int s = 0; s < NU; ++s) { idle &= dec[s].flags; update = update || dec[s].tok >= 0; }
                 if (idle) break;
                 mbar_expect_tx(&bar_enc, (uint32_t)(n_groups * p.H * 16));
 #pragma unroll 1
@@ -492,23 +511,24 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                     const int s = (gi << 3) >> wp_shift;
                     tma_load_3d(smem + L.z + (uint32_t)(gi * p.H * 16), &enc_map, 0, (int)dec[s].row + ((gi << 3) & (p.wp - 1)), 0, &bar_enc);
                 }
-                // mma.sync and tcgen05.mma exclude each other on the tensor cores: the short chains go first (when they are
-                // done, all of h is there as well)
-                if (!(ok = cl_wait(&bar_sync_mma, par))) break;
-                fence_proxy_async_all();                 // h came in through remote generic stores
-                tc_fence_after();
-                uint64_t bd = smem_desc_sw128(sbase + L.h);
+                if (update) {
+                    // mma.sync and tcgen05.mma exclude each other on the tensor cores: the short chains go first (when they are
+                    // done, all of h is there as well)
+                    if (!(ok = cl_wait(&bar_sync_mma, n_g & 1u))) break;
+                    fence_proxy_async_all();             // h came in through remote generic stores
+                    tc_fence_after();
+                    uint64_t hd = smem_desc_sw128(sbase + L.h);
 #pragma unroll 1
-                for (int kb = 0; kb < kb_p; ++kb, bd += 2048 >> 4)
+                    for (int kb = 0; kb < kb_p; ++kb, hd += 2048 >> 4)
 #pragma unroll
-                    for (int k = 0; k < 4; ++k)
-                        tc_mma_bf16_ts(tm_g, tmem + (uint32_t)(kb * 32 + k * 8), bd + (uint64_t)(k * 2), id_g, (kb | k) != 0);
-                tc_commit(&bar_acc_g);
-                ++n_g;
+                        for (int k = 0; k < 4; ++k)
+                            tc_mma_bf16_ts(tm_g, tmem + (uint32_t)(kb * 32 + k * 8), hd + (uint64_t)(k * 2), id_g, (kb | k) != 0);
+                    tc_commit(&bar_acc_g);
+                    ++n_g;
+                }
                 if (!(ok = cl_wait(&bar_z, par))) break;
                 tc_fence_after();
-                bd = smem_desc_sw128(sbase + L.w_out);
-                uint64_t ad = ad0;
+                uint64_t bd = smem_desc_sw128(sbase + L.w_out), ad = ad0;
 #pragma unroll 1
                 for (int kb = 0; kb < kb_h; ++kb, bd += (uint64_t)(lab_rows * 8), ad += 1024 >> 4) {
                     const bool second = kb >= kb_h / 2;  // K halves in two accumulator copies, as in loop_kernel
