@@ -428,11 +428,30 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 pst[(s + 1) * 48 + m + 8] = __float2bfloat16_rn(acc[3] + o.w + b1);
                 __syncwarp();
                 // 16-byte pieces of eight units of one slot: message i = (piece, destination)
+                if constexpr (NS <= 2)
                 for (int i = lane; i < NU * halves * CL_SIZE; i += 32) {
                     const int pi = i >> 4, sl = halves == 2 ? pi >> 1 : pi, hh = halves == 2 ? pi & 1 : 0;
                     const uint32_t d = (uint32_t)(i + r) & (CL_SIZE - 1);
                     if ((live >> sl) & 1u) st_async_16(cl_map(sbase, d) + L.pred + (uint32_t)(sl * p.H + r * HS + 16 * mt + 8 * hh) * 2u,
                                 *reinterpret_cast<const uint4*>(pst + sl * 48 + 8 * hh), cl_map(smem_u32(&bar_pred), d));
+                }
+            }
+            if constexpr (NS > 2) {
+                // many slots: all six warps send, a destination at a time each, a piece per lane
+                if (live != 0u) {
+                    asm volatile("bar.sync 2, 192;" ::: "memory");
+                    const int per_slot = HS / 8;
+#pragma unroll 1
+                    for (int i = lane; i < NU * per_slot; i += 32) {
+                        const int sl = i / per_slot, c = i - sl * per_slot;
+                        if ((live >> sl) & 1u) {
+                            const uint4 piece = *reinterpret_cast<const uint4*>(smem + L.pst + (uint32_t)(sl * 48 + 8 * c) * 2u);
+                            for (int d0 = warp - 4; d0 < CL_SIZE; d0 += 6) {
+                                const uint32_t d = (uint32_t)(d0 + r) & (CL_SIZE - 1);
+                                st_async_16(cl_map(sbase, d) + L.pred + (uint32_t)(sl * p.H + r * HS + 8 * c) * 2u, piece, cl_map(smem_u32(&bar_pred), d));
+                            }
+                        }
+                    }
                 }
             }
             if (ok) ok = cl_wait(&bar_enc, par);
