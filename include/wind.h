@@ -412,8 +412,8 @@ wind_status_t wind_bench_joint(const wind_model_t* m, int32_t B, int32_t W, int3
                                void* stream, wind_joint_bench_t* host_out);
 
 /*
- * Test hook for the failure path of the persistent loop kernel: with extra_arrivals > 0 its grid barrier waits
- * for that many arrivals more than there are CTAs, so the first barrier of the next decode can never fill.  Every
+ * Test hook for the failure path of the persistent kernels: with extra_arrivals > 0 their first cross-CTA wait asks
+ * for that many arrivals more than there will be, so the first barrier of the next decode can never fill.  Every
  * wait in the kernel is bounded (about two seconds), so the decode then ends by itself: the CTAs give up, free
  * their tensor memory and return, and the call reports WIND_ERR_TIMEOUT with undefined outputs; the CUDA context
  * stays usable.  0 restores normal operation.  Returns the previous value.  The paper has no counterpart (its only
@@ -424,6 +424,8 @@ int32_t wind_debug_stall_barrier(int32_t extra_arrivals);
 /*
  * Options of the tensor-core loop's tile planner, process-wide (defaults: 1, -1, 4, -1).  Meant for tests and
  * measurements, which use them to reach every mode of the loop kernels on one shape; results do not depend on them.
+ * (With the defaults, plain greedy decoding of the shapes they take runs in the cluster kernel or in the kernel for
+ * large vocabularies instead; resident = 0, a forced placement or a forced dataflow reach the kernels below.)
  *   resident         0: never choose the resident-weights mode (weights then stream through shared memory every
  *                    step, as for shapes whose tiles do not fit on chip)
  *   joint_placement  streaming mode only: where a CTA keeps its W_out tile when it owns one joint item: -1 the
