@@ -614,7 +614,7 @@ done:
 // a row, so that the 16-byte reads of neighbouring threads fall into different banks.  A row's dot product is cut over up to
 // eight neighbouring threads.  A step of the 64-unit fp32 model is bound by reading its 128 KB of gate weights (1000 cycles)
 // and by seven block barriers; in the grid form's code with one CTA it took 17000 cycles (8.6 us), 86 KB of instructions
-// against an instruction cache of 32 KB: 427 us for an utterance of 44 steps, here 230 us.
+// against an instruction cache of 32 KB: 427 us for an utterance of 44 steps, here 170 us.
 // ---------------------------------------------------------------------------
 struct SlLocal {
     int nin0, np, nh;                 // E, P, H rounded up to four
@@ -627,7 +627,7 @@ __host__ __device__ inline int sl_lg_tpr(int rows) { int l = 0; while (l < 3 && 
 __host__ __device__ inline SlLocal sl_local(int W, int E, int P, int L, int H, int NV, bool emb) {
     SlLocal m{};
     m.nin0 = (E + 3) & ~3; m.np = (P + 3) & ~3; m.nh = (H + 3) & ~3;
-    m.lg_l = sl_lg_tpr(4 * P); m.lg_p = sl_lg_tpr(H); m.lg_j = sl_lg_tpr(NV);
+    m.lg_l = sl_lg_tpr(4 * P); m.lg_p = sl_lg_tpr(H); m.lg_j = sl_lg_tpr(W * NV);   // (one round over the threads where that is possible)
     m.ld_l0 = m.nin0 + m.np + (4 << m.lg_l); m.ld_l1 = 2 * m.np + (4 << m.lg_l);
     m.ld_p = m.np + (4 << m.lg_p); m.ld_o = m.nh + (4 << m.lg_j);
     long long off = 0;
@@ -678,13 +678,18 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_local_kernel(const SimtLoo
     if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const SlLocal M = sl_local(p.W, p.E, p.P, p.L, p.H, p.NV, emb_here != 0);
-    // a matrix [rows][n] to column `at` of the padded rows at dst, with zeros up to the next multiple of four; a warp takes a row
+    // a matrix [rows][n] to column `at` of the padded rows at dst, with zeros up to the next multiple of four; a warp takes 32
+    // elements at a time
+    // (eight loads under way: a row per warp and no loads ahead took 14 us for 186 KB)
     auto load_rows = [&](float* dst, int ld, int at, const void* src_, int rows, int n) {
         const TW* src = static_cast<const TW*>(src_);
-        const int n4 = (n + 3) & ~3;
-#pragma unroll 4
-        for (int row = warp; row < rows; row += SL_WARPS)
-            for (int k = lane; k < n4; k += 32) dst[row * ld + at + k] = k < n ? (float)__ldg(src + (size_t)row * n + k) : 0.f;
+        const int n4 = (n + 3) & ~3, chunks = (n4 + 31) / 32;
+#pragma unroll 8
+        for (int i = warp; i < rows * chunks; i += SL_WARPS) {
+            const int row = i / chunks, k = (i - row * chunks) * 32 + lane;
+            const float v = k < n ? (float)__ldg(src + (size_t)row * n + k) : 0.f;
+            if (k < n4) dst[row * ld + at + k] = v;
+        }
     };
 #pragma unroll 1
     for (int l = 0; l < p.L; ++l) {
@@ -794,14 +799,15 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_local_kernel(const SimtLoo
                     const int i = min(q >> M.lg_j, outs - 1), w = i / p.NV, v = i - w * p.NV;
                     const float s = share_sum(sl_local_dot(smem_u32(sf + M.w_out + v * M.ld_o), smem_u32(sf + M.z + w * M.nh), M.nh, part, M.lg_j, 0.f), M.lg_j) + sf[M.b_out + v];
                     unsigned long long key = s > -INFINITY ? pack_key(s, (uint32_t)v) : 0ull;
-                    if (__all_sync(0xffffffffu, w == __shfl_sync(0xffffffffu, w, 0))) {       // one row's outputs: one update for the warp
-#pragma unroll
-                        for (int o = 16; o > 0; o >>= 1) key = max(key, __shfl_xor_sync(0xffffffffu, key, o));
-                        if (lane != 0) key = 0ull;
-                    } else if (part != 0) {
-                        key = 0ull;
+                    // one update of s_key for each window row among the warp's outputs (one or two of them)
+                    for (uint32_t left = __ballot_sync(0xffffffffu, key != 0ull); left != 0u; left = __ballot_sync(0xffffffffu, key != 0ull)) {
+                        const int wr = __shfl_sync(0xffffffffu, w, __ffs((int)left) - 1);
+                        const unsigned long long mine = w == wr ? key : 0ull;
+                        const uint32_t hi = __reduce_max_sync(0xffffffffu, (uint32_t)(mine >> 32));
+                        const uint32_t lo = __reduce_max_sync(0xffffffffu, (uint32_t)(mine >> 32) == hi ? (uint32_t)mine : 0u);
+                        if (lane == 0) atomicMax(&s_key[wr], ((unsigned long long)hi << 32) | lo);
+                        if (w == wr) key = 0ull;
                     }
-                    if (key != 0ull) atomicMax(&s_key[w], key);
                 }
             }
             __syncthreads();
