@@ -77,7 +77,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
     const uint32_t el = lane == 0;             // the lane that executes the CTA-level instructions of an issuing warp
     const int cta = blockIdx.x, G = gridDim.x;
     // a length outside [0, T] (found by the init kernel, which ran before this launch): the status is set, no CTA starts
-    if (p.ctrl->bad_input) return;
+    if (p.ctrl->bad_input || (p.choose && p.ctrl->use_grid == 0)) return;
     uint8_t* smem = align_smem_1024(smem_raw);
     uint8_t* stat = smem;                       // W_out tile kept in shared memory (J_SMEM): kb_h blocks of 128 x 64 bf16
     uint8_t* ring = smem + p.stat_bytes;        // operand stages; geometry differs per phase, drained in between
@@ -2011,9 +2011,15 @@ cudaError_t loop_prepare(Call& c) {
 cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* prefix_len, float* logits_out,
                     int trace_step) {
     const LoopPlan& pl = t_loop_plan;
+    bool choose = false;
     if (!logits_out && trace_step < -1) {
-        if (cl_supported(c)) return cl_loop(c);
-        if (!pl.resident && wide_supported(c)) return wide_loop(c);
+        if (cl_supported(c)) {
+            // (the kernel with grid barriers follows it only where the lengths may favour it)
+            const cudaError_t e = cl_loop(c, pl.resident && !pl.dataflow, &choose);
+            if (e != cudaSuccess || !choose) return e;
+        } else if (!pl.resident && wide_supported(c)) {
+            return wide_loop(c);
+        }
     }
     LoopParams p{};
     p.ctrl = c.ctrl();
@@ -2048,7 +2054,7 @@ cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* 
     p.window = c.mode == WIND_MODE_WINDOW && !logits_out;
     p.nbkeys = c.keys() + 2 * (size_t)c.lay.rows_pad; p.jpart = c.jpart(); p.jblank = c.jblank(); p.parts = 4 * pl.vt_count;
     p.flags = c.flags(); p.pred_pub = c.pred_pub(); p.kslot = c.kslot();
-    p.joint_iters = c.joint_iters;
+    p.joint_iters = c.joint_iters; p.choose = choose;
     const bool full = p.forced || p.window || p.trace || p.joint_iters > 0;
     if (pl.resident && pl.dataflow) return loop_res_launch(t_loop_maps, p, pl.grid, pl.smem_bytes, full, c.stream);
     void* args[2] = {(void*)&t_loop_maps, (void*)&p};

@@ -53,7 +53,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     __shared__ int s_hist[65];
 
     const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
-    if (p.ctrl->bad_input) return;             // a length outside [0, T]: the whole grid leaves before it does anything
+    if (p.ctrl->bad_input || (p.choose && p.ctrl->use_grid != 0)) return;   // a length outside [0, T], or another kernel's turn: the whole grid leaves before it does anything
     const int r = (int)cl_rank();
     const int cluster = blockIdx.x / CL_SIZE, n_clusters = gridDim.x / CL_SIZE;
     const int NU = p.slots, U = p.P / CL_SIZE, HS = p.H / CL_SIZE;
@@ -691,6 +691,37 @@ __global__ void __launch_bounds__(1024) cl_order_kernel(const int32_t* __restric
     }
 }
 
+// Whether the kernel with grid barriers is the better one for these lengths.  The clusters decode `slots` utterances at a time and
+// take the next from the queue, the other kernel all `rows` at a time, in steps that cost `ratio` times as much.  Compared are
+// bounds on the frames of the busiest slot: the longest utterance, the mean load, and q utterances of at least the length of
+// number (q - 1) slots + 1, of which some slot has to take q; for refilled rows (in the caller's order) the mean load and half an
+// utterance.  (128 utterances of 2400 to 2500 frames, W = 8: 19.9 ms in clusters, three rounds of 56 slots, against 15.0; of 125
+// to 2500 frames: 8.3 against 13.4.)
+__global__ void __launch_bounds__(1024) cl_choose_kernel(Ctrl* ctrl, const int32_t* __restrict__ enc_len, int n, int slots, int rows, float ratio) {
+    __shared__ int32_t len[CL_ORDER_MAX];
+    __shared__ int s_longest, s_bound;
+    __shared__ unsigned long long s_total;
+    if (threadIdx.x == 0) { s_longest = 0; s_bound = 0; s_total = 0ull; }
+    for (int i = threadIdx.x; i < n; i += 1024) len[i] = max(enc_len[i], 0);
+    __syncthreads();
+    unsigned long long total = 0ull;
+    for (int i = threadIdx.x; i < n; i += 1024) {
+        const int mine = len[i];
+        int rank = 0;
+        for (int j = 0; j < n; ++j) rank += len[j] > mine || (len[j] == mine && j < i);
+        if (rank == 0) s_longest = mine;
+        if (rank % slots == 0) atomicMax(&s_bound, (rank / slots + 1) * mine);
+        total += (unsigned)mine;
+    }
+    atomicAdd(&s_total, total);
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        const float mean = (float)s_total / slots, clusters = fmaxf(mean, (float)s_bound);
+        const float grid = n > rows ? (float)s_total / rows + 0.5f * s_longest : (float)s_longest;
+        ctrl->use_grid = clusters > ratio * grid;
+    }
+}
+
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
@@ -756,7 +787,7 @@ bool cl_supported(const Call& c) {
     return cl_clusters() > 0;
 }
 
-cudaError_t cl_loop(const Call& c) {
+cudaError_t cl_loop(const Call& c, bool grid_too, bool* choose) {
     const wind_model_t& m = c.m;
     const int n = c.N > 0 ? c.N : c.B;
     ClParams p{};
@@ -787,6 +818,16 @@ cudaError_t cl_loop(const Call& c) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         p.order = order;
+    }
+    // Cost of a step of all rows in the other kernel, in steps of a cluster with all its slots (measured at 100 to 128 rows of 1, 4, 8
+    // and 16 window rows); a cluster has half the slots when a window takes 16 rows.
+    const float ratio = p.wp == 8 ? 2.15f : 3.4f;
+    *choose = grid_too && p.wp <= 16 && n <= CL_ORDER_MAX && (float)((n + p.slots * clusters - 1) / (p.slots * clusters)) > ratio;
+    p.choose = *choose;
+    if (*choose) {
+        cl_choose_kernel<<<1, 1024, 0, c.stream>>>(c.ctrl(), c.enc_len, n, p.slots * clusters, c.B, ratio);
+        cudaError_t e = cudaGetLastError();
+        if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg{};
     cfg.gridDim = dim3((unsigned)(clusters * CL_SIZE));

@@ -24,7 +24,7 @@ struct ClParams {
     int slots;                         // utterances a cluster decodes at a time (NU)
     int wp;                            // window rows of a slot, padded: 8, 16 or 32
     int queue_base;                    // value of ctrl->next_utt before the first utterance is taken from the queue
-    int step_cap, extra_arrivals;
+    int step_cap, extra_arrivals, choose;
     const int32_t* order;              // [n_utt] order in which utterances are taken; null: 0, 1, ...
     const int32_t* enc_len;
     const float* g0;                   // [NV][4P]
@@ -147,6 +147,8 @@ __device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, ui
 
 // host side (wind_loop_cl.cu)
 bool cl_supported(const Call& c);              // shapes, device and options allow the cluster kernel for this decode
-cudaError_t cl_loop(const Call& c);
+// grid_too: the kernel with grid barriers could take this decode as well; *choose: it has to be launched behind this one, and
+// ctrl->use_grid tells either of them whether it is to run
+cudaError_t cl_loop(const Call& c, bool grid_too, bool* choose);
 
 }  // namespace wind
