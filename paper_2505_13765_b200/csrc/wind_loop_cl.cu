@@ -692,34 +692,36 @@ __global__ void __launch_bounds__(1024) cl_order_kernel(const int32_t* __restric
 }
 
 // Whether the kernel with grid barriers is the better one for these lengths.  The clusters decode `slots` utterances at a time and
-// take the next from the queue, the other kernel all `rows` at a time, in steps that cost `ratio` times as much.  Compared are
-// bounds on the frames of the busiest slot: the longest utterance, the mean load, and q utterances of at least the length of
-// number (q - 1) slots + 1, of which some slot has to take q; for refilled rows (in the caller's order) the mean load and half an
-// utterance.  (128 utterances of 2400 to 2500 frames, W = 8: 19.9 ms in clusters, three rounds of 56 slots, against 15.0; of 125
-// to 2500 frames: 8.3 against 13.4.)
-__global__ void __launch_bounds__(1024) cl_choose_kernel(Ctrl* ctrl, const int32_t* __restrict__ enc_len, int n, int slots, int rows, float ratio) {
-    __shared__ int32_t len[CL_ORDER_MAX];
-    __shared__ int s_longest, s_bound;
-    __shared__ unsigned long long s_total;
-    if (threadIdx.x == 0) { s_longest = 0; s_bound = 0; s_total = 0ull; }
-    for (int i = threadIdx.x; i < n; i += 1024) len[i] = max(enc_len[i], 0);
-    __syncthreads();
-    unsigned long long total = 0ull;
-    for (int i = threadIdx.x; i < n; i += 1024) {
-        const int mine = len[i];
-        int rank = 0;
-        for (int j = 0; j < n; ++j) rank += len[j] > mine || (len[j] == mine && j < i);
-        if (rank == 0) s_longest = mine;
-        if (rank % slots == 0) atomicMax(&s_bound, (rank / slots + 1) * mine);
-        total += (unsigned)mine;
+// take the next from the queue, the other kernel all `rows` at a time (refilled in the caller's order), in steps that cost
+// `ratio` times as much.  A warp each plays either schedule through: every utterance goes to the place that is free first.
+// (128 utterances of 2400 to 2500 frames, W = 8: 19.9 ms in clusters, three rounds of 56 slots, against 15.0; of 125 to 2500
+// frames: 8.3 against 13.4.)
+constexpr int CL_CHOOSE_ROWS = 512;
+__global__ void __launch_bounds__(64) cl_choose_kernel(Ctrl* ctrl, const int32_t* __restrict__ enc_len, const int32_t* __restrict__ order, int n, int slots,
+                                                       int rows, float ratio) {
+    __shared__ uint32_t free_at[2][CL_CHOOSE_ROWS];      // frames until the place is free << 9 | place
+    __shared__ uint32_t s_span[2];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, places = w == 0 ? slots : rows;
+    uint32_t* f = free_at[w];
+    for (int i = lane; i < CL_CHOOSE_ROWS; i += 32) f[i] = i < places ? (uint32_t)i : 0xffffffffu;
+    uint32_t span = 0u, mine_free = lane < places ? (uint32_t)lane : 0xffffffffu;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane, u = j < n ? (w == 0 && order ? order[j] : j) : 0;
+        const uint32_t mine = j < n ? (uint32_t)max(enc_len[u], 0) : 0u;
+        for (int k = 0; k < 32 && j0 + k < n; ++k) {
+            const uint32_t best = __reduce_min_sync(0xffffffffu, mine_free);
+            const uint32_t end = min((best >> 9) + __shfl_sync(0xffffffffu, mine, k), 0x7ffffeu);
+            span = max(span, end);
+            if (best == mine_free) {                     // the place's lane: its places are lane, lane + 32, ...
+                f[best & 511u] = end << 9 | (best & 511u);
+                mine_free = 0xffffffffu;
+                for (int i = lane; i < places; i += 32) mine_free = min(mine_free, f[i]);
+            }
+        }
     }
-    atomicAdd(&s_total, total);
+    if (lane == 0) s_span[w] = span;
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const float mean = (float)s_total / slots, clusters = fmaxf(mean, (float)s_bound);
-        const float grid = n > rows ? (float)s_total / rows + 0.5f * s_longest : (float)s_longest;
-        ctrl->use_grid = clusters > ratio * grid;
-    }
+    if (threadIdx.x == 0) ctrl->use_grid = (float)s_span[0] > ratio * (float)s_span[1];
 }
 
 // ---------------------------------------------------------------------------
@@ -820,12 +822,14 @@ cudaError_t cl_loop(const Call& c, bool grid_too, bool* choose) {
         p.order = order;
     }
     // Cost of a step of all rows in the other kernel, in steps of a cluster with all its slots (measured at 100 to 128 rows of 1, 4, 8
-    // and 16 window rows); a cluster has half the slots when a window takes 16 rows.
-    const float ratio = p.wp == 8 ? 2.15f : 3.4f;
-    *choose = grid_too && p.wp <= 16 && n <= CL_ORDER_MAX && (float)((n + p.slots * clusters - 1) / (p.slots * clusters)) > ratio;
+    // and 16 window rows: 1.9 to 2.3, and 3.0 to 3.5 where a window takes 16 rows and a cluster has half the slots).
+    const float ratio = p.wp == 8 ? 2.1f : 3.2f;
+    // (its rows have to be that many times the slots, in whole rounds, or no lengths can favour it)
+    const int rows = c.B < n ? c.B : n;
+    *choose = grid_too && p.wp <= 16 && n <= CL_ORDER_MAX && rows <= CL_CHOOSE_ROWS && (float)((rows + p.slots * clusters - 1) / (p.slots * clusters)) > ratio;
     p.choose = *choose;
     if (*choose) {
-        cl_choose_kernel<<<1, 1024, 0, c.stream>>>(c.ctrl(), c.enc_len, n, p.slots * clusters, c.B, ratio);
+        cl_choose_kernel<<<1, 64, 0, c.stream>>>(c.ctrl(), c.enc_len, p.order, n, p.slots * clusters, rows, ratio);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
