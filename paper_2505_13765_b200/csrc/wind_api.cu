@@ -1,5 +1,7 @@
 // C ABI entry points: argument checks, workspace carving, launch sequence, and the
 // device-resident decoding loop (a CUDA-graph WHILE node whose body is two lock steps).
+#include <cudaTypedefs.h>
+
 #include <algorithm>
 #include <cstdio>
 #include <cstdlib>
@@ -164,6 +166,39 @@ static wind_status_t get_loop_graph(const Call& c, bool tensor, cudaGraphExec_t*
     g_graphs.push_back(g);
     *exec_out = g.exec;
     return WIND_OK;
+}
+
+// Device address of `bytes` of page-locked host memory at `host`; null where the GPU cannot reach all of them.  What is known of
+// the first byte says nothing about the rest: a caller may have page-locked the head of an array only, so the allocations (or
+// registered ranges) that hold it are followed to the last byte, and have to lie side by side for the GPU too.
+static const void* gpu_address_of_host(const void* host, size_t bytes) {
+    static const PFN_cuPointerGetAttribute_v4000 attribute = [] {
+        void* fn = nullptr;
+        cudaDriverEntryPointQueryResult found;
+        if (cudaGetDriverEntryPoint("cuPointerGetAttribute", &fn, cudaEnableDefault, &found) != cudaSuccess || found != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            fn = nullptr;
+        }
+        return reinterpret_cast<PFN_cuPointerGetAttribute_v4000>(fn);
+    }();
+    if (!attribute) return nullptr;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, host) != cudaSuccess) { cudaGetLastError(); return nullptr; }
+    if (at.type != cudaMemoryTypeHost || !at.devicePointer) return nullptr;
+    const CUdeviceptr first = reinterpret_cast<CUdeviceptr>(at.devicePointer);
+    for (size_t seen = 0; seen < bytes;) {
+        const CUdeviceptr p = reinterpret_cast<CUdeviceptr>(host) + seen;
+        CUmemorytype type{};
+        CUdeviceptr start = 0, dev = 0;
+        size_t size = 0;
+        if (attribute(&type, CU_POINTER_ATTRIBUTE_MEMORY_TYPE, p) != CUDA_SUCCESS || type != CU_MEMORYTYPE_HOST ||
+            attribute(&dev, CU_POINTER_ATTRIBUTE_DEVICE_POINTER, p) != CUDA_SUCCESS || dev != first + seen ||
+            attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, p) != CUDA_SUCCESS ||
+            attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, p) != CUDA_SUCCESS || dev < start || dev - start >= size)
+            return nullptr;
+        seen += size - (size_t)(dev - start);
+    }
+    return at.devicePointer;
 }
 
 // Enqueue the whole decode on c.stream (no synchronisation).
@@ -334,13 +369,14 @@ wind_status_t wind_decode_greedy_host(const wind_model_t* m, const void* enc_hos
     const size_t frame = es * (size_t)m->D;
     int longest_enc = 0;
     for (int b = 0; b < B; ++b) longest_enc = enc_len_host[b] > longest_enc ? enc_len_host[b] : longest_enc;
-    // page-locked memory in whole 16-byte pieces: one kernel fetches all of it.  Pageable memory, odd frames, and batches of more
-    // utterances than a grid has rows: a copy per utterance.
-    cudaPointerAttributes at{};
-    const bool known = cudaPointerGetAttributes(&at, enc_host) == cudaSuccess;
-    if (!known) cudaGetLastError();
-    if (known && at.type == cudaMemoryTypeHost && at.devicePointer && frame % 16 == 0 && reinterpret_cast<uintptr_t>(at.devicePointer) % 16 == 0 && B <= 65535) {
-        WIND_CUDA(launch_gather_frames(at.devicePointer, d_enc, d_len, B, longest_enc, frame, frame * (size_t)T, st));
+    // page-locked memory in whole 16-byte pieces: one kernel fetches all of it.  Memory that is not page-locked up to the last
+    // valid frame, odd frames, and batches of more utterances than a grid has rows: a copy per utterance.
+    size_t reach = 0;
+    for (int b = 0; b < B; ++b)
+        if (enc_len_host[b] > 0) reach = frame * ((size_t)b * T + (size_t)enc_len_host[b]);
+    const void* src = frame % 16 == 0 && B <= 65535 && reach > 0 ? gpu_address_of_host(enc_host, reach) : nullptr;
+    if (src && reinterpret_cast<uintptr_t>(src) % 16 == 0) {
+        WIND_CUDA(launch_gather_frames(src, d_enc, d_len, B, longest_enc, frame, frame * (size_t)T, st));
     } else {
         for (int b = 0; b < B; ++b)
             if (enc_len_host[b] > 0)
