@@ -40,7 +40,7 @@
 namespace wind {
 
 struct ClDec { int tok; uint32_t flags, row, unused; };   // what an owner sends for its slot
-constexpr uint32_t CL_FRESH = 1u, CL_IDLE = 2u;
+constexpr uint32_t CL_FRESH = 1u, CL_IDLE = 2u, CL_ODD = 4u;   // CL_ODD: parity of the step it is for
 
 // Warps: 0-3 gates and z (workers), 4-9 W_pred, 10-13 remainder units, 14 issuing thread, 15 control.  Warps 0-7 also
 // share the joint's epilogue.  NS: most slots in use (1, 2, 4, 8).
@@ -587,18 +587,22 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 k = __shfl_sync(0xffffffffu, v, 0) - p.queue_base + NU * n_clusters;
             }
         };
-        auto announce = [&](int tok, bool fresh) {       // the slot's decision to every CTA
+        auto announce = [&](int tok, bool fresh, uint32_t odd) {       // the slot's decision to every CTA
             const bool idle = o_utt < 0;
-            const uint4 m = make_uint4((uint32_t)(idle ? -1 : tok), (fresh ? CL_FRESH : 0u) | (idle ? CL_IDLE : 0u),
+            const uint4 m = make_uint4((uint32_t)(idle ? -1 : tok), (fresh ? CL_FRESH : 0u) | (idle ? CL_IDLE : 0u) | odd * CL_ODD,
                                        idle ? 0u : o_row0 + (uint32_t)o_t, 0u);
             if (lane < CL_SIZE) st_async_16(cl_map(sbase + L.dec + (uint32_t)r * 16u, lane), m, cl_map(smem_u32(&bar_dec), lane));
         };
         take(r * n_clusters + cluster);
-        announce(p.blank, true);
+        announce(p.blank, true, 0u);
         for (uint32_t step = 0;; ++step) {
             const uint32_t par = step & 1u;
             ok = cl_wait_warp(&bar_dec, par);
-            if (all_idle() || !ok) break;
+            // Every slot idle, as all_idle, but of this step's decisions alone: nothing waits for this warp's look at dec, so the
+            // owners of the other slots may have overwritten theirs with the next step's (this slot's comes from this warp).  Where
+            // there is a next step, this one is not the last.
+            const bool last = __all_sync(0xffffffffu, lane >= NU || (dec[min(lane, NU - 1)].flags & (CL_IDLE | CL_ODD)) == (CL_IDLE | par * CL_ODD));
+            if (last || !ok) break;
             ok = cl_wait_warp(&bar_keys, par);
             if (!ok) break;
             if (lane == 0) mbar_expect_tx(&bar_keys, (uint32_t)(2 * CL_SIZE * p.W) * 8u);
@@ -641,7 +645,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 }
                 take(dynamic && !stuck ? -1 : p.n_utt);
             }
-            announce(done ? p.blank : (emit ? lab : -1), done);          // what the step decided is recorded behind the answer
+            announce(done ? p.blank : (emit ? lab : -1), done, par ^ 1u);          // what the step decided is recorded behind the answer
             const uint32_t bad = __ballot_sync(0xffffffffu, lane < n && lane <= first && broken);   // rows after the first non-blank one do not count
             n_rows += (unsigned)n; n_tok += emit; n_forced += forced;
             if (lane == 0 && utt >= 0) {
