@@ -155,6 +155,7 @@ struct BeamDevice {
                 there = true;
                 for (int i = 0; i < n_out && there; ++i) there = (uint32_t)(mail->top[i] >> 32) == seq;
                 if (!there) { post(words); continue; }
+                ++seq;               // it may have left word that no command of the next number came: that number is not used
             }
             if (single) running = false;
             bar_base += beam_step_arrivals(c, words[0]);
