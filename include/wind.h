@@ -325,8 +325,14 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
  * Entries of P' are ranked by probability, then offset, then label.  Scores are natural-log probabilities; the
  * window's log-softmax is fp32, sums over steps are fp64.  K = 1 gives wind_decode_window_greedy's result.
  * The map, recombination and pruning run on the host; the model arithmetic (encoder projection, decoder updates of
- * surviving hypotheses, windowed joint, Eq. (1) and its K best entries) runs in kernels on `stream`, which the call
- * synchronises once per iteration to read K x K (label, offset, log-probability) triples.
+ * surviving hypotheses, windowed joint, Eq. (1) and its K best entries) runs in kernels on `stream`.  For most shapes (E, P, H
+ * multiples of 8, weights 16-byte aligned, one window's logits in shared memory) that is one kernel which stays for many
+ * iterations: it takes each from page-locked host memory and leaves the K x K (label, offset, log-probability) triples there,
+ * and the calling thread spins on them.  It has a block of 512 threads on every SM while it stays, so kernels of other
+ * streams that do not fit beside it (most that use shared memory or many registers) wait for it; it ends every 5 ms (with prefix_search: after every iteration) and is launched again behind them.  Other shapes launch
+ * kernels per iteration and synchronise `stream` to read the triples.  The call synchronises `stream` before it returns.
+ * The call takes 5 KB of page-locked host memory from the driver (cudaHostAlloc) unless an earlier search left its own
+ * behind: up to eight such blocks are kept until the process ends, more are freed when their search returns.
  *   enc        DEVICE [T, D], element type m->dtype.    T >= 1, 1 <= W <= 64, 1 <= K <= 16.
  *   out_*      HOST: tokens/frames [max_hyps, max_out], lengths and scores [max_hyps], *n_hyps = hypotheses written
  *              (at most max_hyps, best first); a hypothesis longer than max_out is cut in the token arrays, its

@@ -11,10 +11,13 @@
 // carries (parent slot, label) until it survives the pruning of its frame, so at most K decoder updates are made per
 // iteration although K x K hypotheses are created.  Slots are reference-counted (a hypothesis created by the blank
 // entry shares its parent's slot).
+#if defined(__x86_64__)
 #include <immintrin.h>
+#endif
 
 #include <algorithm>
 #include <atomic>
+#include <chrono>
 #include <cmath>
 #include <cstring>
 #include <mutex>
@@ -96,7 +99,19 @@ std::mutex g_mail_mutex;
 std::vector<BeamMail*> g_mail;
 constexpr size_t kMailKept = 8;
 
-// The resident kernel of one search, as the host sees it.
+// between two looks at the mailbox
+inline void cpu_relax() {
+#if defined(__x86_64__)
+    _mm_pause();
+#elif defined(__aarch64__)
+    asm volatile("yield" ::: "memory");
+#endif
+}
+
+// The resident kernel of one search, as the host sees it.  It holds every SM, so little of another stream fits beside it: after
+// kTurn it ends with the command in hand, what waits on other streams goes first, and the next command launches it again (25 us,
+// mostly its weights: half a percent of the search).
+constexpr std::chrono::milliseconds kTurn(5);
 struct BeamDevice {
     const Call& c;
     float *h_pool, *c_pool, *g_pool, *logits;
@@ -105,6 +120,7 @@ struct BeamDevice {
     BeamMail* mail = nullptr;
     uint32_t seq = 0, bar_base = 0;
     bool running = false;
+    std::chrono::steady_clock::time_point launched{};
 
     cudaError_t open() {
         {
@@ -120,21 +136,26 @@ struct BeamDevice {
         std::memset(mail, 0, sizeof(BeamMail));
         return cudaMemsetAsync(relay, 0, sizeof(unsigned long long) * kBeamWords, c.stream);
     }
-    void post(const int32_t* words) {        // 4 + 4 K values
+    void post(const int32_t* words, bool last) {        // 4 + 4 K values
         ++seq;
         volatile unsigned long long* out = mail->cmd;
-        for (int i = 0; i < 4 + 4 * c.B; ++i) out[i] = (unsigned long long)seq << 32 | (uint32_t)words[i];
+        for (int i = 0; i < 4 + 4 * c.B; ++i) {
+            const uint32_t flag = last && i == 1 ? kBeamLast : 0u;
+            out[i] = (unsigned long long)seq << 32 | ((uint32_t)words[i] | flag);
+        }
     }
     // one command, until its result (nh * K entries) is there
     wind_status_t run(const int32_t* words, cudaError_t* err) {
         const int n_out = 2 * words[1] * c.B;
-        post(words);
+        bool last = single || (running && std::chrono::steady_clock::now() - launched > kTurn);
+        post(words, last);
         for (int launches = 0;;) {
             if (!running) {
                 // (a kernel that ends for want of commands took every CTA with it, between two commands)
                 if (++launches > 8) return WIND_ERR_TIMEOUT;
-                if ((*err = beam_step(c, mail, relay, seq, bar_base, single, h_pool, c_pool, g_pool, logits)) != cudaSuccess) return WIND_ERR_CUDA;
+                if ((*err = beam_step(c, mail, relay, seq, bar_base, h_pool, c_pool, g_pool, logits)) != cudaSuccess) return WIND_ERR_CUDA;
                 running = true;
+                launched = std::chrono::steady_clock::now();
             }
             bool there = false;
             for (uint32_t spins = 1; !there; ++spins) {
@@ -142,7 +163,7 @@ struct BeamDevice {
                 for (int i = n_out - 1; i >= 0 && there; --i)
                     there = (uint32_t)(static_cast<volatile unsigned long long*>(mail->top)[i] >> 32) == seq;
                 if (there) break;
-                _mm_pause();
+                cpu_relax();
                 if ((spins & 4095u) == 0u && (*err = cudaStreamQuery(c.stream)) != cudaErrorNotReady) {
                     if (*err != cudaSuccess) return WIND_ERR_CUDA;
                     running = false;
@@ -154,10 +175,10 @@ struct BeamDevice {
                 std::atomic_thread_fence(std::memory_order_acquire);
                 there = true;
                 for (int i = 0; i < n_out && there; ++i) there = (uint32_t)(mail->top[i] >> 32) == seq;
-                if (!there) { post(words); continue; }
+                if (!there) { last = single; post(words, last); continue; }
                 ++seq;               // it may have left word that no command of the next number came: that number is not used
             }
-            if (single) running = false;
+            if (last) running = false;
             bar_base += beam_step_arrivals(c, words[0]);
             return WIND_OK;
         }
@@ -166,7 +187,7 @@ struct BeamDevice {
     ~BeamDevice() {
         if (!mail) return;
         std::vector<int32_t> end(4 + 4 * (size_t)c.B, -1);
-        post(end.data());
+        post(end.data(), false);
         cudaStreamSynchronize(c.stream);
         std::lock_guard<std::mutex> lock(g_mail_mutex);
         if (g_mail.size() < kMailKept) g_mail.push_back(mail);

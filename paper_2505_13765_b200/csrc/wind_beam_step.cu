@@ -11,7 +11,8 @@
 // shared-memory latencies each.
 //
 // The kernel never depends on the host's pace: without a command for 200 us it ends, and the host launches it again with the
-// next one (all state is in global memory).  So another stream's work, a debugger or a descheduled host thread cost time only.
+// next one (all state is in global memory).  So a debugger or a descheduled host thread cost the search time only.  On every SM
+// it leaves 8 of 64 thousand registers, so most kernels of other streams wait for its end: the host has it end every 5 ms.
 //
 // A command or result word carries its 32 bits and the command's number in one 8-byte store, so no fence or flag is needed on
 // either side of the bus.
@@ -82,7 +83,6 @@ struct BsParams {
     uint32_t bar_base;                 // arrivals at the grid barrier before this launch
     uint32_t extra_arrivals;
     BsPlan plan;
-    int single;                        // end after one command
     int K;
     int E, P, L, H, NV, blank, act, W;
     const void* emb;
@@ -300,7 +300,8 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
 
     for (uint32_t seq = p.first_seq;; ++seq) {
         take_command(seq);
-        const int nu = s_cmd[0], nh = s_cmd[1], n = s_cmd[2], t = s_cmd[3];
+        const int nu = s_cmd[0], nh = s_cmd[1] & (int)(kBeamLast - 1u), n = s_cmd[2], t = s_cmd[3];
+        const bool last = (s_cmd[1] & (int)kBeamLast) != 0;
         if (nu < 0) return;                                  // the end of the search, or no command for too long
         const int *c_src = s_cmd + 4, *c_tok = c_src + K, *c_dst = c_tok + K, *c_slot = c_dst + K;
         if (nu > 0 && !M.resident) load_layer(0);
@@ -534,7 +535,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                 }
             }
         }
-        if (p.single) return;
+        if (last) return;
     }
 }
 
@@ -580,7 +581,7 @@ bool beam_step_supported(const Call& c) {
     return c.B <= sms && bs_plan_of(c, sms, (uint32_t)optin - 4096u).total <= (uint32_t)optin - 4096u;
 }
 
-cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base, bool single,
+cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
                       float* h_pool, float* c_pool, float* g_pool, float* logits) {
     int optin = 0, sms = 0;
     cudaError_t e = bs_device(&optin);
@@ -589,7 +590,7 @@ cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, 
     const wind_model_t& m = c.m;
     BsParams p{};
     p.ctrl = c.ctrl(); p.mail = mail; p.relay = relay;
-    p.first_seq = first_seq; p.bar_base = bar_base; p.single = single; p.K = c.B;
+    p.first_seq = first_seq; p.bar_base = bar_base; p.K = c.B;
     p.extra_arrivals = (uint32_t)loop_extra_arrivals();
     p.plan = bs_plan_of(c, sms, (uint32_t)optin - 4096u);
     p.E = m.E; p.P = m.P; p.L = m.L; p.H = m.H; p.NV = m.V + 1; p.blank = m.blank_id; p.act = m.act; p.W = c.W;

@@ -231,15 +231,16 @@ struct BeamLayout {
 // hypothesis's K best entries there.  A word is (number of the command) << 32 | value.
 constexpr int kMaxBeam = 16;
 constexpr int kBeamWords = 4 + 4 * kMaxBeam;
+constexpr uint32_t kBeamLast = 0x10000u;
 struct BeamMail {
-    // n_update (-1: end), n_hyps, n_rows (the window, cut short by the end of the utterance), t; then for K updates each the
+    // n_update (-1: end), n_hyps (and kBeamLast: the kernel ends behind this command), n_rows (the window, cut short by the end of the utterance), t; then for K updates each the
     // slot of the state before, the token, the slot of the state after; then the states of K hypotheses
     alignas(128) unsigned long long cmd[kBeamWords];
     alignas(128) unsigned long long top[2 * kMaxBeam * kMaxBeam];   // per entry: offset * (V + 1) + label (all ones: none), fp32 bits of log P'
     alignas(128) uint32_t failed;                                   // a wait inside the kernel ran out
 };
 bool beam_step_supported(const Call& c);
-cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base, bool single,
+cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
                       float* h_pool, float* c_pool, float* g_pool, float* logits);
 uint32_t beam_step_arrivals(const Call& c, int n_update);
 BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, size_t base);

@@ -39,3 +39,47 @@ def test_beam_iteration_kernel(pkg, E, P, L, H, V, act, W, K, S):  # noqa: F811
         assert all(abs(a[k][2] - b[k][2]) < 1e-4 and list(a[k][1]) == list(b[k][1]) for k in a)
     print(f"[beam iteration] K={K} W={W}: {decided}/6 cases decidable and equal to the oracle")
     assert decided >= (1 if K < 8 else 0)
+
+
+def test_other_streams_get_their_turn_during_a_search(pkg):  # noqa: F811
+    # The resident kernel holds every SM (57 of 64 thousand registers each).  A search of a few hundred milliseconds in one
+    # thread, matrix products one after the other on another stream in this one: several of them have to end while the search is
+    # still under way.
+    import threading
+    import time
+
+    w = random_weights(np.random.default_rng(9500), 16, 64, 64, 1, 64, 200, act=0, blank_bias=6.0, bias_scale=0.1)
+    w["dtype"] = "f32"
+    model = pkg.WindModel(w)
+    T, W, K, S = 16000, 1, 4, 2
+    enc = np.random.default_rng(9501).standard_normal((T, 16)).astype(np.float32)
+    alone = pkg.wind_beam_search(model, enc, W, K, S, max_hyps=K)
+    x = torch.zeros(1024, 1024, device="cuda", dtype=torch.bfloat16)
+    side, own = torch.cuda.Stream(), torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        torch.mm(x, x)
+    torch.cuda.synchronize()
+    took, result = [], []
+
+    def search():
+        with torch.cuda.stream(own):
+            t0 = time.perf_counter()
+            result.append(pkg.wind_beam_search(model, enc, W, K, S, max_hyps=K))
+            took.append((t0, time.perf_counter()))
+
+    thread = threading.Thread(target=search)
+    thread.start()
+    done = []
+    while thread.is_alive():
+        with torch.cuda.stream(side):
+            torch.mm(x, x)
+        side.synchronize()
+        done.append(time.perf_counter())
+        time.sleep(0.002)
+    thread.join()
+    t0, t1 = took[0]
+    inside = [t for t in done if t0 + 0.3 * (t1 - t0) < t < t0 + 0.9 * (t1 - t0)]
+    print(f"[beam turns] search {1e3 * (t1 - t0):.0f} ms, {len(inside)} kernels of another stream in its middle part")
+    assert t1 - t0 > 0.1 and len(inside) >= 5
+    for a, b in zip(alone[0], result[0][0]):
+        assert list(a[0]) == list(b[0]) and list(a[1]) == list(b[1]) and a[2] == b[2]
