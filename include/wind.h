@@ -329,8 +329,9 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
  * multiples of 8, weights 16-byte aligned, one window's logits in shared memory) that is one kernel which stays for many
  * iterations: it takes each from page-locked host memory and leaves the K x K (label, offset, log-probability) triples there,
  * and the calling thread spins on them.  It has a block of 512 threads on every SM while it stays, so kernels of other
- * streams that do not fit beside it (most that use shared memory or many registers) wait for it; it ends every 5 ms (with prefix_search: after every iteration) and is launched again behind them.  Other shapes launch
- * kernels per iteration and synchronise `stream` to read the triples.  The call synchronises `stream` before it returns.
+ * streams that do not fit beside it (most that use shared memory or many registers) wait for it; it ends every 5 ms
+ * (with prefix_search: after every iteration) and is launched again behind them.  Other shapes launch kernels per iteration
+ * and synchronise `stream` to read the triples.  The call synchronises `stream` before it returns.
  * The call takes 5 KB of page-locked host memory from the driver (cudaHostAlloc) unless an earlier search left its own
  * behind: up to eight such blocks are kept until the process ends, more are freed when their search returns.
  *   enc        DEVICE [T, D], element type m->dtype.    T >= 1, 1 <= W <= 64, 1 <= K <= 16.
@@ -466,6 +467,22 @@ typedef struct {
     int32_t slots, ul, ug_count, mt_count, hg_count, stages_lp, stages_j, stage_lp, stage_j;
 } wind_plan_t;
 wind_status_t wind_debug_plan(const wind_model_t* m, int32_t B, int32_t W, int32_t sms, int32_t smem_optin, wind_plan_t* out);
+
+/*
+ * Which kernel ran the decoding loop of the last decode that used `workspace` (for tests and measurements; synchronises
+ * `stream`).  Where two kernels are launched and the lengths decide between them on the device, it is the one that decoded.
+ */
+typedef enum {
+    WIND_LOOP_NONE = 0,        /* kernels per phase (a CUDA graph), or no loop: nothing decoded, a length out of range */
+    WIND_LOOP_ONE_SM = 1,      /* plain ALUs, the decoder inside one SM */
+    WIND_LOOP_GRID = 2,        /* plain ALUs, the decoder spread over the chip */
+    WIND_LOOP_BARRIERS = 3,    /* tensor cores, weights on chip, grid barriers between the phases */
+    WIND_LOOP_COUNTERS = 4,    /* tensor cores, weights on chip, arrival counters */
+    WIND_LOOP_STREAMING = 5,   /* tensor cores, weights streamed every step */
+    WIND_LOOP_CLUSTERS = 6,    /* tensor cores, thread-block clusters */
+    WIND_LOOP_WIDE = 7         /* tensor cores, large vocabularies: one role per CTA */
+} wind_loop_kernel_t;
+wind_status_t wind_debug_loop_kernel(const void* workspace, void* stream, int32_t* host_out);
 
 /* Process-wide choice of kernels for the bf16 path (default AUTO).  Returns the previous value. */
 int32_t wind_set_kernels(int32_t kernels);

@@ -27,11 +27,13 @@ WIND_ERR_WORKSPACE = 7
 WIND_ACT_RELU, WIND_ACT_TANH = 0, 1
 WIND_DT_F32, WIND_DT_BF16 = 0, 1
 WIND_KERNELS_AUTO, WIND_KERNELS_SIMT, WIND_KERNELS_TENSOR = 0, 1, 2
+(WIND_LOOP_NONE, WIND_LOOP_ONE_SM, WIND_LOOP_GRID, WIND_LOOP_BARRIERS, WIND_LOOP_COUNTERS, WIND_LOOP_STREAMING, WIND_LOOP_CLUSTERS,
+ WIND_LOOP_WIDE) = range(8)
 
 EXPORTS = [
     "wind_workspace_bytes", "wind_decode_greedy", "wind_decode_window_greedy", "wind_host_staging_bytes", "wind_decode_greedy_host",
     "wind_eval_joint_window", "wind_window_first_output", "wind_eval_joint_window_static", "wind_profile_decode", "wind_beam_workspace_bytes", "wind_beam_search", "wind_plan_batches", "wind_read_stats", "wind_set_trace", "wind_read_trace", "wind_debug_stall_barrier", "wind_set_kernels", "wind_status_string", "wind_last_cuda_error",
-    "wind_set_loop_options", "wind_debug_plan", "wind_bench_joint", "wind_refill_workspace_bytes", "wind_decode_greedy_refill",
+    "wind_set_loop_options", "wind_debug_plan", "wind_bench_joint", "wind_refill_workspace_bytes", "wind_decode_greedy_refill", "wind_debug_loop_kernel",
 ]
 
 _vp = C.c_void_p
@@ -137,6 +139,8 @@ def load_library():
     L.wind_plan_batches.restype = i32
     L.wind_read_stats.argtypes = [_vp, _vp, C.POINTER(wind_stats_t)]
     L.wind_read_stats.restype = i32
+    L.wind_debug_loop_kernel.argtypes = [_vp, _vp, C.POINTER(i32)]
+    L.wind_debug_loop_kernel.restype = i32
     L.wind_set_trace.argtypes = [i32]
     L.wind_set_trace.restype = i32
     L.wind_read_trace.argtypes = [mp, i32, i32, i32, _vp, _vp, C.POINTER(wind_trace_event_t), i32, C.POINTER(i32)]
@@ -469,6 +473,15 @@ def wind_read_stats(workspace, stream=None) -> Dict[str, object]:
     if st != WIND_OK:
         raise WindError(st)
     return s.as_dict()
+
+
+def wind_debug_loop_kernel(workspace, stream=None) -> int:
+    """Which kernel ran the decoding loop of the last decode that used `workspace` (WIND_LOOP_*)."""
+    which = C.c_int32(-1)
+    st = load_library().wind_debug_loop_kernel(_ws_ptr(workspace), _stream_ptr(stream), C.byref(which))
+    if st != WIND_OK:
+        raise WindError(st)
+    return int(which.value)
 
 
 # ---------------------------------------------------------------------------

@@ -678,6 +678,15 @@ wind_status_t wind_read_stats(const void* workspace, void* stream, wind_stats_t*
     return WIND_OK;
 }
 
+wind_status_t wind_debug_loop_kernel(const void* workspace, void* stream, int32_t* host_out) {
+    if (!workspace || !host_out) return WIND_ERR_INVALID_ARG;
+    Ctrl hc;
+    WIND_CUDA(cudaMemcpyAsync(&hc, workspace, sizeof(Ctrl), cudaMemcpyDeviceToHost, (cudaStream_t)stream));
+    WIND_CUDA(cudaStreamSynchronize((cudaStream_t)stream));
+    *host_out = hc.loop_kernel;
+    return WIND_OK;
+}
+
 wind_status_t wind_bench_joint(const wind_model_t* m, int32_t B, int32_t W, int32_t iters, void* workspace, size_t workspace_bytes,
                                void* stream, wind_joint_bench_t* host_out) {
     wind_status_t s = check_model(m);

@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(256) init_kernel(Ctrl* ctrl, int32_t* t, unsig
             ctrl->timeout_cta = 0;
             ctrl->next_utt = N < B ? N : B;
             ctrl->n_utt = N;
+            ctrl->loop_kernel = WIND_LOOP_NONE;
         }
     }
 }

@@ -1661,6 +1661,7 @@ done:
         if (cta == 0) {
             if (exit_status) set_status(p.ctrl, exit_status);
             p.ctrl->active = s_active;
+            p.ctrl->loop_kernel = RES ? WIND_LOOP_BARRIERS : WIND_LOOP_STREAMING;
             for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = cyc[k];
             p.ctrl->loop_ns = (long long)(globaltimer_ns() - ns0);
         }

@@ -368,6 +368,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         }
         if (timed) {
             p.ctrl->active = 0;
+            p.ctrl->loop_kernel = WIND_LOOP_CLUSTERS;
             for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = cyc[k];
             p.ctrl->loop_ns = (long long)(globaltimer_ns() - ns0);
         }

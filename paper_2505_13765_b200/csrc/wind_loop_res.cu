@@ -1129,6 +1129,7 @@ done:
     if (cta == 0 && e == 0) {
         if (exit_status) set_status(p.ctrl, exit_status);
         p.ctrl->active = s_active;
+        p.ctrl->loop_kernel = WIND_LOOP_COUNTERS;
         for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = cyc[k];
         p.ctrl->loop_ns = (long long)(globaltimer_ns() - ns0);
     }

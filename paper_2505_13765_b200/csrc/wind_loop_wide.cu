@@ -562,6 +562,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
         if (cta == 0) {
             if (exit_status) set_status(p.ctrl, exit_status);
             p.ctrl->active = 0;
+            p.ctrl->loop_kernel = WIND_LOOP_WIDE;
             for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = cyc[k];
             p.ctrl->loop_ns = (long long)(globaltimer_ns() - ns0);
         }

@@ -604,7 +604,7 @@ done:
             if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
     if (tid == 0) {
         if (s_stop) set_status(p.ctrl, WIND_ERR_TIMEOUT);
-        if (cta == 0) p.ctrl->active = 0;
+        if (cta == 0) { p.ctrl->active = 0; p.ctrl->loop_kernel = WIND_LOOP_GRID; }
     }
 }
 
@@ -864,7 +864,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_local_kernel(const SimtLoo
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->joint_rows), (unsigned long long)n_rows);
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->tokens), (unsigned long long)n_tok);
         atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->forced), (unsigned long long)n_forced);
-        if (blockIdx.x == 0) p.ctrl->active = 0;
+        if (blockIdx.x == 0) { p.ctrl->active = 0; p.ctrl->loop_kernel = WIND_LOOP_ONE_SM; }
     }
 #pragma unroll 1
     for (int k = tid; k < 65; k += SL_THREADS)

@@ -3,6 +3,7 @@ barriers takes over from the clusters.  Either way the transcripts and counters 
 import numpy as np
 import pytest
 
+from conftest import set_loop_mode
 from test_gpu_parity import pkg, ragged_case  # noqa: F401
 
 torch = pytest.importorskip("torch")
@@ -44,4 +45,37 @@ def test_refilled_rows_either_way(pkg, N, B, W):  # noqa: F811
     finally:
         pkg.binding.wind_set_loop_options()
     for a, b in zip(got[:3], want[:3]):
+        assert np.array_equal(a, b)
+
+
+def loop_kernel_of(pkg, model, enc, lens, W, S):  # noqa: F811
+    """Transcripts on device buffers of this test's own, and which kernel's they are."""
+    B, T, _ = enc.shape
+    d = model.device
+    tok, frm = torch.full((B, T * S), -1, dtype=torch.int32, device=d), torch.full((B, T * S), -1, dtype=torch.int32, device=d)
+    olen = torch.zeros(B, dtype=torch.int32, device=d)
+    ws = pkg.alloc_workspace(model, B, T, W)
+    st = pkg.wind_decode_greedy(model, pkg.to_device_enc(model, enc), torch.from_numpy(lens).to(d), W, S, tok, frm, olen, ws)
+    assert st == 0
+    return pkg.binding.wind_debug_loop_kernel(ws), [x.cpu().numpy() for x in (tok, frm, olen)]
+
+
+@pytest.mark.parametrize("B,W,T,lo,want", [
+    (128, 8, 60, 60, "BARRIERS"),      # equal lengths: three rounds of slots
+    (128, 8, 60, 2, "CLUSTERS"),       # ragged ones
+    (112, 8, 60, 60, "CLUSTERS"),      # two rounds
+    (16, 8, 60, 60, "CLUSTERS"),       # one round
+])
+def test_which_kernel_decodes(pkg, B, W, T, lo, want):  # noqa: F811
+    S = 3
+    w, enc, _ = ragged_case(1980 + B + W + lo, B=B, T=T, D=64, E=64, P=128, L=1, H=128, V=200, bias=3.0, dtype="bf16")
+    lens = np.random.default_rng(B + lo).integers(lo, T + 1, size=B).astype(np.int32)
+    enc = np.nan_to_num(enc)
+    model = pkg.WindModel(w)
+    kernel, got = loop_kernel_of(pkg, model, enc, lens, W, S)
+    assert kernel == getattr(pkg.binding, "WIND_LOOP_" + want)
+    set_loop_mode(pkg, "barriers")
+    kernel, ref = loop_kernel_of(pkg, model, enc, lens, W, S)
+    assert kernel == pkg.binding.WIND_LOOP_BARRIERS
+    for a, b in zip(got, ref):
         assert np.array_equal(a, b)
