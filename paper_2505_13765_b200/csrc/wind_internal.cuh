@@ -50,7 +50,7 @@ struct Ctrl {
     int32_t timeout_cta;
     int32_t next_utt;         // first utterance that has not been given a batch row yet (more utterances than rows)
     int32_t n_utt;
-    int32_t use_grid;         // which of two launched loop kernels decodes: 0 the cluster kernel, 1 the one with grid barriers
+    int32_t use_grid;         // which of two launched loop kernels decodes: 0 the cluster kernel, 1 the other one
     int32_t loop_kernel;      // wind_loop_kernel_t: set by the kernel that decodes
 };
 

@@ -2014,10 +2014,12 @@ cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* 
     const LoopPlan& pl = t_loop_plan;
     bool choose = false;
     if (!logits_out && trace_step < -1) {
-        if (cl_supported(c)) {
-            // (the kernel with grid barriers follows it only where the lengths may favour it)
-            const cudaError_t e = cl_loop(c, pl.resident && !pl.dataflow, &choose);
-            if (e != cudaSuccess || !choose) return e;
+        ClPlan q;
+        if (cl_plan(c, pl, &q)) {
+            // (the kernel of the plan follows it only where the lengths may favour it)
+            const cudaError_t e = cl_loop(c, q);
+            if (e != cudaSuccess || !q.choose) return e;
+            choose = true;
         } else if (!pl.resident && wide_supported(c)) {
             return wide_loop(c);
         }

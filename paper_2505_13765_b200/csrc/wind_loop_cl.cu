@@ -31,6 +31,7 @@
 // all meet at the cluster barrier at the end, so no CTA leaves while another may still write into its shared memory.
 #include <cudaTypedefs.h>
 
+#include <cmath>
 #include <mutex>
 #include <type_traits>
 
@@ -696,37 +697,64 @@ __global__ void __launch_bounds__(1024) cl_order_kernel(const int32_t* __restric
     }
 }
 
-// Whether the kernel with grid barriers is the better one for these lengths.  The clusters decode `slots` utterances at a time and
-// take the next from the queue, the other kernel all `rows` at a time (refilled in the caller's order), in steps that cost
-// `ratio` times as much.  A warp each plays either schedule through: every utterance goes to the place that is free first.
-// (128 utterances of 2400 to 2500 frames, W = 8: 19.9 ms in clusters, three rounds of 56 slots, against 15.0; of 125 to 2500
-// frames: 8.3 against 13.4.)
+// Whether the other kernel that could take this decode (grid barriers, arrival counters or streamed weights, as the planner has it)
+// is the better one for these lengths.  The clusters decode `slots` utterances at a time and take the next from the queue, longest
+// first, in steps of cl_us; the other kernel decodes all `rows` at a time (refilled in the caller's order) in steps of other_us.
+// Bounds of what either schedule takes mostly decide; where they overlap, a warp each plays them through: every utterance goes to
+// the place that is free first.  (128 utterances of 2400 to 2500 frames, W = 8: 19.9 ms in clusters, three rounds of 56 slots,
+// against 15.0; of 125 to 2500 frames: 8.3 against 13.4.)
 constexpr int CL_CHOOSE_ROWS = 512;
-__global__ void __launch_bounds__(64) cl_choose_kernel(Ctrl* ctrl, const int32_t* __restrict__ enc_len, const int32_t* __restrict__ order, int n, int slots,
-                                                       int rows, float ratio) {
+__global__ void __launch_bounds__(256) cl_choose_kernel(Ctrl* ctrl, const int32_t* __restrict__ enc_len, const int32_t* __restrict__ order, int n, int T,
+                                                        int slots, int rows, float cl_us, float other_us) {
     __shared__ uint32_t free_at[2][CL_CHOOSE_ROWS];      // frames until the place is free << 9 | place
     __shared__ uint32_t s_span[2];
+    __shared__ unsigned long long s_sum;
+    __shared__ int s_longest;
+    if (threadIdx.x == 0) { s_sum = 0ull; s_longest = 0; }
+    __syncthreads();
+    auto length = [&](int u) { return min(max(enc_len[u], 0), T); };
+    unsigned long long mine_sum = 0ull;
+    int mine_longest = 0;
+    for (int i = threadIdx.x; i < n; i += 256) { const int l = length(i); mine_sum += (unsigned long long)l; mine_longest = max(mine_longest, l); }
+    atomicAdd(&s_sum, mine_sum);
+    atomicMax(&s_longest, mine_longest);
+    __syncthreads();
+    // all rows of the other kernel wait for the slowest, a slot averages over its utterances: 1.14 times the mean number of steps
+    // at 200 frames, 1.28 at 120 (128 utterances of equal length)
+    auto other_cost = [&](float span) { return other_us * span * (1.f + 2.5f * rsqrtf(fmaxf(span, 1.f))); };
+    const bool queue = n > rows;
+    const float longest = (float)s_longest, sum = (float)s_sum, next = (float)(order && n > slots ? length(order[slots]) : s_longest);
+    const float cl_lo = fmaxf(longest, sum / (float)slots), cl_hi = fmaxf(longest, sum / (float)slots + next);
+    const float other_lo = queue ? fmaxf(longest, sum / (float)rows) : longest, other_hi = queue ? longest + sum / (float)rows : longest;
+    const bool clusters = cl_us * cl_hi <= other_cost(other_lo), other = cl_us * cl_lo > other_cost(other_hi);
+    if (clusters || other || n > CL_ORDER_MAX || (queue && rows > CL_CHOOSE_ROWS)) {
+        if (threadIdx.x == 0) ctrl->use_grid = clusters ? 0 : (other ? 1 : cl_us * (cl_lo + cl_hi) > 2.f * other_cost(0.5f * (other_lo + other_hi)));
+        return;
+    }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, places = w == 0 ? slots : rows;
-    uint32_t* f = free_at[w];
-    for (int i = lane; i < CL_CHOOSE_ROWS; i += 32) f[i] = i < places ? (uint32_t)i : 0xffffffffu;
-    uint32_t span = 0u, mine_free = lane < places ? (uint32_t)lane : 0xffffffffu;
-    for (int j0 = 0; j0 < n; j0 += 32) {
-        const int j = j0 + lane, u = j < n ? (w == 0 && order ? order[j] : j) : 0;
-        const uint32_t mine = j < n ? (uint32_t)max(enc_len[u], 0) : 0u;
-        for (int k = 0; k < 32 && j0 + k < n; ++k) {
-            const uint32_t best = __reduce_min_sync(0xffffffffu, mine_free);
-            const uint32_t end = min((best >> 9) + __shfl_sync(0xffffffffu, mine, k), 0x7ffffeu);
-            span = max(span, end);
-            if (best == mine_free) {                     // the place's lane: its places are lane, lane + 32, ...
-                f[best & 511u] = end << 9 | (best & 511u);
-                mine_free = 0xffffffffu;
-                for (int i = lane; i < places; i += 32) mine_free = min(mine_free, f[i]);
+    if (w == 0 || (w == 1 && queue)) {
+        uint32_t* f = free_at[w];
+        for (int i = lane; i < CL_CHOOSE_ROWS; i += 32) f[i] = i < places ? (uint32_t)i : 0xffffffffu;
+        uint32_t span = 0u, mine_free = lane < places ? (uint32_t)lane : 0xffffffffu;
+        for (int j0 = 0; j0 < n; j0 += 32) {
+            const int j = j0 + lane;
+            const uint32_t mine = j < n ? (uint32_t)length(w == 0 && order ? order[j] : j) : 0u;
+            for (int k = 0; k < 32 && j0 + k < n; ++k) {
+                const uint32_t best = __reduce_min_sync(0xffffffffu, mine_free);
+                const uint32_t end = min((best >> 9) + __shfl_sync(0xffffffffu, mine, k), 0x7ffffeu);
+                span = max(span, end);
+                if (best == mine_free) {                 // the place's lane: its places are lane, lane + 32, ...
+                    f[best & 511u] = end << 9 | (best & 511u);
+                    mine_free = 0xffffffffu;
+                    for (int i = lane; i < places; i += 32) mine_free = min(mine_free, f[i]);
+                }
             }
         }
+        if (lane == 0) s_span[w] = span;
     }
-    if (lane == 0) s_span[w] = span;
+    if (!queue && threadIdx.x == 32) s_span[1] = (uint32_t)s_longest;
     __syncthreads();
-    if (threadIdx.x == 0) ctrl->use_grid = (float)s_span[0] > ratio * (float)s_span[1];
+    if (threadIdx.x == 0) ctrl->use_grid = cl_us * (float)s_span[0] > other_cost((float)s_span[1]);
 }
 
 // ---------------------------------------------------------------------------
@@ -780,10 +808,26 @@ static int cl_clusters() {
     return g_cl_clusters[dev] > 0 ? g_cl_clusters[dev] : 0;
 }
 
+// What a lock step costs, in us: of a cluster with all its slots, and of the other kernel with all its rows.  Fitted to 430 measured
+// pairs (P and H 128 to 640, 501 and 1025 labels, ReLU and tanh, W = 1 to 32, 29 to 600 utterances of equal and of ragged lengths):
+// 3, 8 and 8 % rms.  Chosen by these, a decode takes 0.7 % longer than by the better kernel of each pair on the average; with a
+// constant ratio, 2.1 and 3.2 for windows of 8 and 16 rows, and clusters alone beyond that or for up to 64 utterances, it took 11 %
+// (64 utterances of 120 frames at W = 32: 1.53 ms against 1.32; 128: 2.84 against 1.79; 64 at W = 24, P = H = 384: 1.31 against 0.89).
+static float cl_step_us(const wind_model_t& m, int W, int wp) {
+    const float P = (float)m.P, H = (float)m.H, z = m.act == WIND_ACT_RELU ? 0.f : 0.0018f * H;
+    return z + (wp == 8 ? 4.3f + 0.0013f * P + (0.0009f + 0.0026f * (float)W / 8.f) * H : 4.25f + 0.0009f * P + 0.0028f * H);
+}
+static float other_step_us(const wind_model_t& m, const LoopPlan& pl, int B, int W) {
+    const float P = (float)m.P, H = (float)m.H, rows = (float)B * (float)W;
+    if (!pl.resident) return -2.5f + 3.8f * (float)pl.mt_count + 0.0053f * rows + 0.0177f * P + 0.0145f * H;
+    const int waves = (pl.rg_count + pl.rg_stride - 1) / pl.rg_stride;
+    return 10.1f + 0.005f * H + 0.002f * rows + (pl.dataflow ? 6.5f : 3.f) * (float)(waves - 1);
+}
+
 // The shapes whose decoder fits one cluster: one LSTM layer, P and H multiples of 128 (a CTA's share is then whole 16-byte
 // pieces, and the K halves are equal) up to 640, at most 72 vocabulary entries per CTA, windows up to 32 rows.  Everything
 // else, and the FULL features (logits store, window-based decoding, timeline, forced loop modes), stays with loop_kernel.
-bool cl_supported(const Call& c) {
+static bool cl_supported(const Call& c) {
     const wind_model_t& m = c.m;
     const int nv = m.V + 1;
     if (m.L != 1 || m.P % 128 || m.H % 128 || m.P > CL_MAX_DIM || m.H > CL_MAX_DIM || c.W > 32) return false;
@@ -794,20 +838,44 @@ bool cl_supported(const Call& c) {
     return cl_clusters() > 0;
 }
 
-cudaError_t cl_loop(const Call& c, bool grid_too, bool* choose) {
+// How a decode runs in clusters; false: it does not.  `other` is the plan by which another kernel could take it.
+// Where that has the weights on the chip its transcripts are the same bit for bit, and where any lengths could favour it (the
+// clusters may need as many rounds as its rows make of their slots) both are launched and the lengths decide on the device.
+// Streamed weights go with other roundings; which of the two decodes must not depend on the lengths of a batch, so the shapes
+// alone decide, for lengths whose mean is 0.6 of the longest, or rows that are refilled throughout.
+bool cl_plan(const Call& c, const LoopPlan& other, ClPlan* out) {
+    if (!cl_supported(c)) return false;
+    const int n = c.N > 0 ? c.N : c.B, avail = cl_clusters();
+    ClPlan q{};
+    q.wp = c.W <= 8 ? 8 : (c.W <= 16 ? 16 : 32);
+    // one slot per cluster as long as there are clusters, then more slots (a lock step of eight slots costs less than two of one)
+    const int most = 8 * CL_GROUPS / q.wp;
+    q.clusters = n < avail ? n : avail;
+    q.slots = (n + q.clusters - 1) / q.clusters < most ? (n + q.clusters - 1) / q.clusters : most;
+    const int slots = q.slots * q.clusters;
+    q.rows = c.B < n ? c.B : n;
+    q.cl_us = cl_step_us(c.m, c.W, q.wp);
+    q.other_us = other_step_us(c.m, other, c.B, c.W);
+    q.order = n > slots && n <= CL_ORDER_MAX && sizeof(int32_t) * (size_t)n <= sizeof(float) * 2 * (size_t)c.B * c.m.P;
+    const float rounds = (float)((q.rows + slots - 1) / slots), cost = q.other_us * (1.f + 2.5f / sqrtf((float)c.T));
+    if (rounds > 1.f) {
+        if (!other.resident && (n > q.rows ? (float)q.rows / (float)slots : 0.6f * rounds) * q.cl_us > cost) return false;
+        q.choose = other.resident && rounds * q.cl_us > cost;
+    }
+    *out = q;
+    return true;
+}
+
+cudaError_t cl_loop(const Call& c, const ClPlan& q) {
     const wind_model_t& m = c.m;
     const int n = c.N > 0 ? c.N : c.B;
     ClParams p{};
     p.ctrl = c.ctrl();
     p.T = c.T; p.W = c.W; p.S = c.S; p.max_out = c.max_out; p.H = m.H; p.P = m.P; p.NV = m.V + 1; p.blank = m.blank_id;
     p.n_utt = n;
-    p.wp = c.W <= 8 ? 8 : (c.W <= 16 ? 16 : 32);
-    // one slot per cluster as long as there are clusters, then more slots (a lock step of eight slots costs less than two of one)
-    const int most = 8 * CL_GROUPS / p.wp;
-    const int avail = cl_clusters();
-    const int clusters = n < avail ? n : avail;
-    if (clusters < 1) return cudaErrorNotSupported;
-    p.slots = (n + clusters - 1) / clusters < most ? (n + clusters - 1) / clusters : most;
+    p.wp = q.wp;
+    p.slots = q.slots;
+    p.choose = q.choose;
     const int ns = p.slots <= 1 ? 1 : (p.slots <= 2 ? 2 : (p.slots <= 4 ? 4 : 8));
     p.queue_base = n < c.B ? n : c.B;
     long long cap = (long long)c.T * (c.S + 1) + 2;
@@ -819,27 +887,20 @@ cudaError_t cl_loop(const Call& c, bool grid_too, bool* choose) {
     p.w_hh = (const __nv_bfloat16*)c.w_hh[0]; p.w_pred = (const __nv_bfloat16*)m.w_pred; p.w_out = (const __nv_bfloat16*)m.w_out;
     p.b_pred = m.b_pred; p.b_out = m.b_out;
     p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
-    if (n > p.slots * clusters && n <= CL_ORDER_MAX && sizeof(int32_t) * (size_t)n <= sizeof(float) * 2 * (size_t)c.B * m.P) {
+    if (q.order) {
         int32_t* order = reinterpret_cast<int32_t*>(c.h(0));     // the plain-ALU path's state: not used by a bf16 tensor decode
         cl_order_kernel<<<(n + 1023) / 1024, 1024, 0, c.stream>>>(c.enc_len, n, order);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
         p.order = order;
     }
-    // Cost of a step of all rows in the other kernel, in steps of a cluster with all its slots (measured at 100 to 128 rows of 1, 4, 8
-    // and 16 window rows: 1.9 to 2.3, and 3.0 to 3.5 where a window takes 16 rows and a cluster has half the slots).
-    const float ratio = p.wp == 8 ? 2.1f : 3.2f;
-    // (its rows have to be that many times the slots, in whole rounds, or no lengths can favour it)
-    const int rows = c.B < n ? c.B : n;
-    *choose = grid_too && p.wp <= 16 && n <= CL_ORDER_MAX && rows <= CL_CHOOSE_ROWS && (float)((rows + p.slots * clusters - 1) / (p.slots * clusters)) > ratio;
-    p.choose = *choose;
-    if (*choose) {
-        cl_choose_kernel<<<1, 64, 0, c.stream>>>(c.ctrl(), c.enc_len, p.order, n, p.slots * clusters, rows, ratio);
+    if (q.choose) {
+        cl_choose_kernel<<<1, 256, 0, c.stream>>>(c.ctrl(), c.enc_len, p.order, n, c.T, q.slots * q.clusters, q.rows, q.cl_us, q.other_us);
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(clusters * CL_SIZE));
+    cfg.gridDim = dim3((unsigned)(q.clusters * CL_SIZE));
     cfg.blockDim = dim3(CL_THREADS);
     cfg.dynamicSmemBytes = cl_smem_bytes(m.P, m.H, p.NV, p.slots, p.wp);
     cfg.stream = c.stream;

@@ -6,6 +6,7 @@
 #include <stdint.h>
 
 #include "wind_internal.cuh"
+#include "wind_loop.cuh"
 #include "wind_ptx.cuh"
 
 namespace wind {
@@ -146,9 +147,14 @@ __device__ __forceinline__ void mma_16816(float* c, uint32_t a0, uint32_t a1, ui
 }
 
 // host side (wind_loop_cl.cu)
-bool cl_supported(const Call& c);              // shapes, device and options allow the cluster kernel for this decode
-// grid_too: the kernel with grid barriers could take this decode as well; *choose: it has to be launched behind this one, and
-// ctrl->use_grid tells either of them whether it is to run
-cudaError_t cl_loop(const Call& c, bool grid_too, bool* choose);
+struct ClPlan {
+    int clusters, slots, wp;           // as in ClParams
+    int rows;                          // utterances the other kernel decodes at a time
+    bool order;                        // the utterances are taken longest first
+    bool choose;                       // the other kernel has to be launched behind this one, and ctrl->use_grid tells either whether it is to run
+    float cl_us, other_us;             // what a lock step of either costs
+};
+bool cl_plan(const Call& c, const LoopPlan& other, ClPlan* out);
+cudaError_t cl_loop(const Call& c, const ClPlan& q);
 
 }  // namespace wind

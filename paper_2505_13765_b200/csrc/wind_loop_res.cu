@@ -79,7 +79,7 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
     const uint32_t el = lane == 0;             // the lane that executes the CTA-level instructions of an issuing warp
     const int cta = blockIdx.x, G = gridDim.x;
     // a length outside [0, T] (found by the init kernel, which ran before this launch): the status is set, no CTA starts
-    if (p.ctrl->bad_input) return;
+    if (p.ctrl->bad_input || (p.choose && p.ctrl->use_grid == 0)) return;
     uint8_t* smem = align_smem_1024(smem_raw);
     uint8_t* stat = smem;                       // this CTA's resident weight tile: kb_p blocks of 64 rows x 64 columns
     uint8_t* buf0 = smem + p.buf_off;           // the per-step state box

@@ -60,15 +60,23 @@ def loop_kernel_of(pkg, model, enc, lens, W, S):  # noqa: F811
     return pkg.binding.wind_debug_loop_kernel(ws), [x.cpu().numpy() for x in (tok, frm, olen)]
 
 
-@pytest.mark.parametrize("B,W,T,lo,want", [
-    (128, 8, 60, 60, "BARRIERS"),      # equal lengths: three rounds of slots
-    (128, 8, 60, 2, "CLUSTERS"),       # ragged ones
-    (112, 8, 60, 60, "CLUSTERS"),      # two rounds
-    (16, 8, 60, 60, "CLUSTERS"),       # one round
+@pytest.mark.parametrize("B,W,T,lo,dim,want", [
+    (128, 8, 60, 60, 640, "BARRIERS"),      # equal lengths: three rounds of slots
+    (128, 8, 60, 2, 640, "CLUSTERS"),       # ragged ones
+    (112, 8, 60, 60, 128, "CLUSTERS"),      # two rounds
+    (16, 8, 60, 60, 128, "CLUSTERS"),       # one round
+    (128, 32, 60, 60, 128, "BARRIERS"),     # widest window: ten rounds
+    (128, 17, 60, 60, 640, "BARRIERS"),
+    (64, 32, 60, 60, 128, "COUNTERS"),      # up to 64 rows the other kernel is the one with arrival counters
+    (64, 32, 60, 2, 128, "CLUSTERS"),
+    (57, 16, 300, 290, 640, "COUNTERS"),
+    (28, 16, 60, 60, 640, "CLUSTERS"),
+    (400, 24, 100, 100, 640, "STREAMING"),  # more rows than the resident kernels take: the shapes decide
+    (400, 24, 100, 10, 640, "STREAMING"),
 ])
-def test_which_kernel_decodes(pkg, B, W, T, lo, want):  # noqa: F811
+def test_which_kernel_decodes(pkg, B, W, T, lo, dim, want):  # noqa: F811
     S = 3
-    w, enc, _ = ragged_case(1980 + B + W + lo, B=B, T=T, D=64, E=64, P=128, L=1, H=128, V=200, bias=3.0, dtype="bf16")
+    w, enc, _ = ragged_case(1980 + B + W + lo, B=B, T=T, D=64, E=64, P=dim, L=1, H=dim, V=200, bias=3.0, dtype="bf16")
     lens = np.random.default_rng(B + lo).integers(lo, T + 1, size=B).astype(np.int32)
     enc = np.nan_to_num(enc)
     model = pkg.WindModel(w)
@@ -76,6 +84,29 @@ def test_which_kernel_decodes(pkg, B, W, T, lo, want):  # noqa: F811
     assert kernel == getattr(pkg.binding, "WIND_LOOP_" + want)
     set_loop_mode(pkg, "barriers")
     kernel, ref = loop_kernel_of(pkg, model, enc, lens, W, S)
-    assert kernel == pkg.binding.WIND_LOOP_BARRIERS
+    assert kernel == (pkg.binding.WIND_LOOP_STREAMING if want == "STREAMING" else pkg.binding.WIND_LOOP_BARRIERS)
     for a, b in zip(got, ref):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("N,B,W,lo,want", [
+    (384, 128, 16, 100, "BARRIERS"),        # rows refilled in the other kernel as well
+    (300, 64, 8, 1, "CLUSTERS"),
+    (4200, 128, 32, 1, "BARRIERS"),         # more utterances than are put in order or played through
+])
+def test_which_kernel_refills(pkg, N, B, W, lo, want):  # noqa: F811
+    T, S = (100, 3) if N < 1000 else (4, 3)
+    w, enc, _ = ragged_case(1990 + N, B=N, T=T, D=64, E=64, P=128, L=1, H=128, V=200, bias=3.0, dtype="bf16")
+    lens = np.random.default_rng(N).integers(lo, T + 1, size=N).astype(np.int32)
+    enc = np.nan_to_num(enc)
+    model = pkg.WindModel(w)
+    d = model.device
+    tok, frm = torch.full((N, T * S), -1, dtype=torch.int32, device=d), torch.full((N, T * S), -1, dtype=torch.int32, device=d)
+    olen = torch.zeros(N, dtype=torch.int32, device=d)
+    ws = torch.empty(pkg.binding.wind_refill_workspace_bytes(model, N, T, B, W) + 256, dtype=torch.uint8, device=d)
+    st = pkg.binding.wind_decode_greedy_refill(model, pkg.to_device_enc(model, enc), torch.from_numpy(lens).to(d), B, W, S, tok, frm, olen, ws)
+    assert st == 0 and pkg.binding.wind_debug_loop_kernel(ws) == getattr(pkg.binding, "WIND_LOOP_" + want)
+    set_loop_mode(pkg, "barriers")
+    want_out = pkg.decode_refill(model, enc, lens, B, W, S)
+    for a, b in zip((tok, frm, olen), want_out[:3]):
+        assert np.array_equal(a.cpu().numpy(), b)
