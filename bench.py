@@ -612,13 +612,15 @@ def dataset_op(args, cfg, W):
 
     def run(batches, k):
         def once():
-            steps = 0
+            steps = launches = 0
             for enc_d, len_d, tok, frm, ol, wsb in batches:
                 pkg.wind_decode_greedy(model, enc_d, len_d, W, cfg.S, tok, frm, ol, wsb, stream=stream)
-                steps += pkg.wind_read_stats(wsb, stream)["steps"]
-            return steps
+                st = pkg.wind_read_stats(wsb, stream)
+                steps += st["steps"]
+                launches += st["launches_setup"] + st["steps"] * st["launches_per_step"]
+            return steps, launches
         for _ in range(max(3, args.warmup)):
-            steps = once()
+            steps, launches = once()
         torch.cuda.synchronize()
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         e0.record(stream)
@@ -626,7 +628,7 @@ def dataset_op(args, cfg, W):
             once()
         e1.record(stream)
         torch.cuda.synchronize()
-        return e0.elapsed_time(e1) / k, steps
+        return e0.elapsed_time(e1) / k, steps, launches
 
     def run_refill(idx_order, k):
         # all utterances resident at the set's T, decoded on B batch rows that are refilled inside the loop
@@ -651,9 +653,9 @@ def dataset_op(args, cfg, W):
         torch.cuda.synchronize()
         return e0.elapsed_time(e1) / k, steps
 
-    ms_a, steps_a = run(pack(np.arange(N)), args.steps)
+    ms_a, steps_a, _ = run(pack(np.arange(N)), args.steps)
     torch.cuda.empty_cache()
-    ms_p, steps_p = run(pack(order), args.steps)
+    ms_p, steps_p, launches_p = run(pack(order), args.steps)
     torch.cuda.empty_cache()
     refill = {}
     try:
@@ -672,7 +674,7 @@ def dataset_op(args, cfg, W):
         "length_aware": {"ms": ms_p, "lock_steps": steps_p, "batch_T": [int(t) for t in batch_T]},
         "arrival_order": {"ms": ms_a, "lock_steps": steps_a, "value": audio_s / (ms_a * 1e-3)},
         "speedup_vs_arrival_order": ms_a / ms_p, "refilled_rows": refill,
-        "gpu_launches": 4 * len(batch_T) * args.steps,
+        "gpu_launches": launches_p * args.steps,
     }))
 
 

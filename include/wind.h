@@ -109,7 +109,8 @@ typedef struct {
     int64_t jump_hist[65]; /* jump sizes 0..min(W,64): i on an emission, n on an all-blank window */
     int32_t status;        /* device status word (wind_status_t) */
     int32_t launches_per_step; /* kernel nodes in one loop iteration */
-    int32_t launches_setup;    /* kernel launches outside the loop (projection, init, first decoder update) */
+    int32_t launches_setup;    /* kernel launches outside such iterations: projection, init, first decoder update, and the loop
+                                  itself where it is one kernel (two where the lengths decide between two of them) */
     int32_t kernels;           /* wind_kernels_t actually used */
     int32_t timeout_site;      /* after WIND_ERR_TIMEOUT from the resident-weights loop kernel: a code for the wait that ran
                                   out first (a diagnostic: grep the code in the kernel source) and the CTA it ran out in */

@@ -201,27 +201,27 @@ static const void* gpu_address_of_host(const void* host, size_t bytes) {
     return at.devicePointer;
 }
 
-// Enqueue the whole decode on c.stream (no synchronisation).
-static wind_status_t enqueue_decode(Call& c) {
+// Enqueue the whole decode on c.stream (no synchronisation).  before: kernels the call has launched already.
+static wind_status_t enqueue_decode(Call& c, int before = 0) {
     const bool tensor = use_tensor(c);
     if (c.m.dtype == WIND_DT_BF16 && g_kernels == WIND_KERNELS_TENSOR && !tensor) return WIND_ERR_UNSUPPORTED;
     if (tensor) {
         // projection and gate table once, then the whole loop as one persistent kernel
         WIND_CUDA(tc_prepare(c));
-        WIND_CUDA(launch_init(c, WIND_KERNELS_TENSOR, 0, tc_setup_launches(c)));
+        WIND_CUDA(launch_init(c, WIND_KERNELS_TENSOR, 0, before + tc_setup_launches(c, g_trace_step)));
         WIND_CUDA(tc_enc_proj(c));
         WIND_CUDA(tc_gate_table(c));
         WIND_CUDA(tc_loop(c, nullptr, 0, nullptr, nullptr, g_trace_step));
         return WIND_OK;
     }
     if (simt_loop_supported(c)) {
-        WIND_CUDA(launch_init(c, WIND_KERNELS_SIMT, 0, 3));
+        WIND_CUDA(launch_init(c, WIND_KERNELS_SIMT, 0, before + 3));
         WIND_CUDA(simt_enc_proj(c));
         WIND_CUDA(simt_loop(c));
         return WIND_OK;
     }
     const int per_step = 2 + simt_pred_launches(c);
-    const int setup = 2 + simt_pred_launches(c);
+    const int setup = before + 2 + simt_pred_launches(c);
     WIND_CUDA(launch_init(c, WIND_KERNELS_SIMT, per_step, setup));
     WIND_CUDA(simt_enc_proj(c));
     WIND_CUDA(simt_pred_step(c, 0));  // start of sequence: h[0] (zeros) -> h[1]
@@ -338,7 +338,7 @@ wind_status_t wind_decode_greedy_refill(const wind_model_t* m, const void* enc, 
     // rows are refilled inside the persistent loop kernel of the tensor-core set only
     if (!use_tensor(c)) return WIND_ERR_UNSUPPORTED;
     WIND_CUDA(tc_prepare(c));
-    WIND_CUDA(launch_init(c, WIND_KERNELS_TENSOR, 0, tc_setup_launches(c)));
+    WIND_CUDA(launch_init(c, WIND_KERNELS_TENSOR, 0, tc_setup_launches(c, g_trace_step)));
     WIND_CUDA(tc_enc_proj(c));
     WIND_CUDA(tc_gate_table(c));
     WIND_CUDA(tc_loop(c, nullptr, 0, nullptr, nullptr, g_trace_step));
@@ -375,7 +375,8 @@ wind_status_t wind_decode_greedy_host(const wind_model_t* m, const void* enc_hos
     for (int b = 0; b < B; ++b)
         if (enc_len_host[b] > 0) reach = frame * ((size_t)b * T + (size_t)enc_len_host[b]);
     const void* src = frame % 16 == 0 && B <= 65535 && reach > 0 ? gpu_address_of_host(enc_host, reach) : nullptr;
-    if (src && reinterpret_cast<uintptr_t>(src) % 16 == 0) {
+    const bool gathered = src && reinterpret_cast<uintptr_t>(src) % 16 == 0;
+    if (gathered) {
         WIND_CUDA(launch_gather_frames(src, d_enc, d_len, B, longest_enc, frame, frame * (size_t)T, st));
     } else {
         for (int b = 0; b < B; ++b)
@@ -385,7 +386,7 @@ wind_status_t wind_decode_greedy_host(const wind_model_t* m, const void* enc_hos
     }
     Call c;
     fill_call(c, m, d_enc, d_len, B, T, W, max_symbols, d_tok, d_frm, d_olen, max_out, workspace, st);
-    s = enqueue_decode(c);
+    s = enqueue_decode(c, gathered ? 1 : 0);
     if (s != WIND_OK) return s;
     // lengths first, then the columns of the two output arrays that hold tokens (up to the longest transcript)
     WIND_CUDA(cudaMemcpyAsync(out_len_host, d_olen, sizeof(int32_t) * B, cudaMemcpyDeviceToHost, st));
@@ -521,7 +522,7 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
         cudaEvent_t ev[4];
         for (auto& e : ev) WIND_CUDA(cudaEventCreate(&e));
         WIND_CUDA(tc_prepare(c));
-        WIND_CUDA(launch_init(c, WIND_KERNELS_TENSOR, 0, tc_setup_launches(c)));
+        WIND_CUDA(launch_init(c, WIND_KERNELS_TENSOR, 0, tc_setup_launches(c, g_trace_step)));
         WIND_CUDA(cudaEventRecord(ev[0], c.stream));
         WIND_CUDA(tc_enc_proj(c));
         WIND_CUDA(cudaEventRecord(ev[1], c.stream));

@@ -262,6 +262,6 @@ cudaError_t tc_gate_table(const Call& c);  // g0[tok] = W_ih[0] emb[tok] + b_ih[
 // store the window logits at t (set beforehand in both t buffers) to logits_out.
 cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* prefix_len, float* logits_out,
                     int trace_step);
-int tc_setup_launches(const Call& c);
+int tc_setup_launches(const Call& c, int trace_step);   // kernels a decode launches in all (after tc_prepare)
 
 }  // namespace wind

@@ -2009,6 +2009,12 @@ cudaError_t loop_prepare(Call& c) {
     return cudaSuccess;
 }
 
+int loop_launches(const Call& c, int trace_step) {
+    ClPlan q;
+    if (trace_step >= -1 || !cl_plan(c, t_loop_plan, &q)) return 1;
+    return 1 + q.order + 2 * q.choose;      // the order, the choice and the other kernel
+}
+
 cudaError_t tc_loop(const Call& c, const int32_t* prefix, int U, const int32_t* prefix_len, float* logits_out,
                     int trace_step) {
     const LoopPlan& pl = t_loop_plan;

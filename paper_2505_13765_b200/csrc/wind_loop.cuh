@@ -146,6 +146,7 @@ cudaError_t loop_map_blocks(CUtensorMap* map, const void* base, uint64_t blocks,
 // the kernel for large vocabularies (wind_loop_wide.cu)
 bool wide_supported(const Call& c);
 cudaError_t wide_loop(const Call& c);
+int loop_launches(const Call& c, int trace_step);   // kernels tc_loop launches for a decode (after loop_prepare)
 cudaError_t loop_prepare(Call& c);   // plan + tensor maps + shared-memory opt-in (host only; not inside a capture)
 
 }  // namespace wind

@@ -507,6 +507,6 @@ cudaError_t tc_gate_table(const Call& c) {
     return cudaGetLastError();
 }
 
-int tc_setup_launches(const Call& c) { (void)c; return 4; }  // init, projection, gate table, loop
+int tc_setup_launches(const Call& c, int trace_step) { return 3 + loop_launches(c, trace_step); }  // init, projection, gate table; the loop's
 
 }  // namespace wind

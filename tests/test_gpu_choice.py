@@ -110,3 +110,22 @@ def test_which_kernel_refills(pkg, N, B, W, lo, want):  # noqa: F811
     want_out = pkg.decode_refill(model, enc, lens, B, W, S)
     for a, b in zip((tok, frm, olen), want_out[:3]):
         assert np.array_equal(a.cpu().numpy(), b)
+
+
+@pytest.mark.parametrize("B,W,dim,want", [(7, 8, 128, 4), (60, 8, 128, 5), (128, 8, 640, 7), (400, 24, 640, 4)])
+def test_launch_count(pkg, B, W, dim, want):  # noqa: F811
+    # init, projection, gate table, loop; with more utterances than slots their order; where the lengths decide, the choice and the
+    # other kernel; from the host, the kernel that fetches the frames
+    T, S = 100, 3
+    w, enc, lens = ragged_case(2100 + B, B=B, T=T, D=64, E=64, P=dim, L=1, H=dim, V=200, bias=3.0, dtype="bf16")
+    enc = np.nan_to_num(enc)
+    model = pkg.WindModel(w)
+    assert pkg.decode(model, enc, lens, W, S)[3]["launches_setup"] == want
+    max_out = T * S
+    enc_h, len_h = torch.from_numpy(enc).to(torch.bfloat16).pin_memory(), torch.from_numpy(lens).pin_memory()
+    tok = torch.full((B, max_out), -1, dtype=torch.int32)
+    ws = pkg.alloc_workspace(model, B, T, W, host_staging_max_out=max_out)
+    assert pkg.wind_decode_greedy_host(model, enc_h, len_h, W, S, tok, tok.clone(), torch.zeros(B, dtype=torch.int32), ws) == 0
+    assert pkg.wind_read_stats(ws)["launches_setup"] == want + 1
+    set_loop_mode(pkg, "barriers")
+    assert pkg.decode(model, enc, lens, W, S)[3]["launches_setup"] == 4
