@@ -112,8 +112,8 @@ typedef struct {
     int32_t launches_setup;    /* kernel launches outside such iterations: projection, init, first decoder update, and the loop
                                   itself where it is one kernel (two where the lengths decide between two of them) */
     int32_t kernels;           /* wind_kernels_t actually used */
-    int32_t timeout_site;      /* after WIND_ERR_TIMEOUT from the resident-weights loop kernel: a code for the wait that ran
-                                  out first (a diagnostic: grep the code in the kernel source) and the CTA it ran out in */
+    int32_t timeout_site;      /* after WIND_ERR_TIMEOUT from a persistent kernel: a code for the wait that ran out first (a
+                                  diagnostic: note_timeout in the sources lists them) and the CTA it ran out in */
     int32_t timeout_cta;
 } wind_stats_t;
 
@@ -421,10 +421,10 @@ wind_status_t wind_bench_joint(const wind_model_t* m, int32_t B, int32_t W, int3
 
 /*
  * Test hook for the failure path of the persistent kernels: with extra_arrivals > 0 their first cross-CTA wait asks
- * for that many arrivals more than there will be, so the first barrier of the next decode can never fill.  Every
- * wait in the kernel is bounded (about two seconds), so the decode then ends by itself: the CTAs give up, free
- * their tensor memory and return, and the call reports WIND_ERR_TIMEOUT with undefined outputs; the CUDA context
- * stays usable.  0 restores normal operation.  Returns the previous value.  The paper has no counterpart (its only
+ * for that many arrivals more than there will be, so the first barrier of the next decode (or beam search) can never
+ * fill.  (The kernel that decodes inside one SM has no such wait.)  Every wait in the kernels is bounded (two to three
+ * seconds), so the call then ends by itself: the CTAs give up, free their tensor memory and return, and it reports
+ * WIND_ERR_TIMEOUT with undefined outputs; the CUDA context stays usable.  0 restores normal operation.  Returns the previous value.  The paper has no counterpart (its only
  * mention of a safeguard is the beam-search footnote about not staying on one frame forever).
  */
 int32_t wind_debug_stall_barrier(int32_t extra_arrivals);

@@ -238,7 +238,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
         epoch += (uint32_t)G;
         if (tid == 0) { __threadfence(); atomicAdd(&p.ctrl->bar, 1u); }
     };
-    auto give_up = [&] { s_stop = 1; set_status(p.ctrl, WIND_ERR_TIMEOUT); *const_cast<volatile uint32_t*>(&p.mail->failed) = 1u; };
+    auto give_up = [&](int site) { s_stop = 1; note_timeout(p.ctrl, site, cta); set_status(p.ctrl, WIND_ERR_TIMEOUT); *const_cast<volatile uint32_t*>(&p.mail->failed) = 1u; };
     auto wait = [&]() -> bool {        // bounded; false: given up
         if (tid == 0) {
             const uint32_t target = epoch + p.extra_arrivals;
@@ -250,7 +250,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                 if ((it & 63u) == 0u) {
                     const unsigned long long now = globaltimer_ns();
                     if (t0 == 0) t0 = now;
-                    else if (now - t0 > kWaitLimitNs) { give_up(); break; }
+                    else if (now - t0 > kWaitLimitNs) { give_up(6); break; }
                 }
             }
         }
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                     if (t0 == 0) {
                         t0 = now;
                     } else if (now - t0 > limit) {
-                        if (cta != 0 && lane == 0) give_up();
+                        if (cta != 0 && lane == 0) give_up(7);
 #pragma unroll
                         for (int j = 0; j < (kBeamWords + 31) / 32; ++j) v[j] = bs_word(0xffffffffu, seq);
                         break;

@@ -46,7 +46,7 @@ struct Ctrl {
     int32_t abort;            // some CTA gave up: everybody leaves
     long long phase_cycles[4];  // SM cycles spent in the joint / decoder-update / projection phases (CTA 0), [3] unused
     long long loop_ns;        // wall time of the loop kernel (CTA 0, global timer)
-    int32_t timeout_site;     // which wait ran out first (resident-weights loop kernel; 0 = none), and in which CTA
+    int32_t timeout_site;     // which wait ran out first (note_timeout; 0 = none), and in which CTA
     int32_t timeout_cta;
     int32_t next_utt;         // first utterance that has not been given a batch row yet (more utterances than rows)
     int32_t n_utt;
@@ -195,6 +195,12 @@ __device__ inline float key_logit(unsigned long long key) {
 }
 
 __device__ inline void set_status(Ctrl* ctrl, int32_t s) { atomicCAS(&ctrl->status, 0, s); }
+// A wait of CTA `cta` ran out: the first one of the call stays.  Sites: 1 loop_kernel; 3 grid barrier of
+// wide_kernel, 4 another wait in it; 5 grid barrier of simt_grid_kernel; 6 grid barrier of beam_step_kernel, 7 its wait for a command; 20 to 43 in
+// loop_res_kernel, 50 + the warp in cl_kernel (its roles stand there)
+__device__ inline void note_timeout(Ctrl* ctrl, int site, int cta) {
+    if (atomicCAS(&ctrl->timeout_site, 0, site) == 0) ctrl->timeout_cta = cta;
+}
 
 // ---------------------------------------------------------------------------
 // launchers (each enqueues on call.stream; returns cudaGetLastError())

@@ -1657,7 +1657,7 @@ done:
         tmem_dealloc(tmem_base, LOOP_TMEM_COLS);
     }
     if (threadIdx.x == 0) {
-        if (s_abort == 1) set_status(p.ctrl, WIND_ERR_TIMEOUT);
+        if (s_abort == 1) { note_timeout(p.ctrl, 1, cta); set_status(p.ctrl, WIND_ERR_TIMEOUT); }
         if (cta == 0) {
             if (exit_status) set_status(p.ctrl, exit_status);
             p.ctrl->active = s_active;

@@ -562,7 +562,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             }
             // copies and MMAs in flight must have completed before the memory they use goes back
             if (n_g > 0u) cl_wait(&bar_acc_g, (n_g - 1u) & 1u);
-            if (!ok) s_abort = 1;
+            if (!ok) s_abort = 1 + 14;
         }
         __syncwarp();
         ok = true;
@@ -670,14 +670,15 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
         }
     }
-    if (!ok) s_abort = 1;
+    if (!ok) s_abort = 1 + warp;
     tc_fence_before();
     __syncthreads();
     if (warp == 14) {
         tc_fence_after();
         tmem_dealloc(tmem, LOOP_TMEM_COLS);
     }
-    if (threadIdx.x == 0 && s_abort) set_status(p.ctrl, WIND_ERR_TIMEOUT);
+    if (threadIdx.x == 0 && s_abort) { note_timeout(p.ctrl, 49 + s_abort, blockIdx.x); set_status(p.ctrl, WIND_ERR_TIMEOUT); }
+    __syncwarp();
     cl_barrier();                                        // no CTA leaves while another may still write into its shared memory
 }
 

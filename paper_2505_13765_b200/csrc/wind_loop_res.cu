@@ -184,7 +184,7 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
     };
     // a wait of this CTA ran out: note which one (the first in the grid stays), flag the CTA and everybody else
     auto give_up = [&](int site) {
-        if (atomicCAS(&p.ctrl->timeout_site, 0, site) == 0) p.ctrl->timeout_cta = cta;
+        note_timeout(p.ctrl, site, cta);
         *vabort = 1;
         atomicExch(&p.ctrl->abort, 1);
     };

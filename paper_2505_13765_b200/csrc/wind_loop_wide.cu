@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
                         if (ld_volatile_i32(&p.ctrl->abort)) { s_abort = 2; break; }
                         const unsigned long long now = globaltimer_ns();
                         if (t0 == 0) t0 = now;
-                        else if (now - t0 > kWaitLimitNs) { s_abort = 1; atomicExch(&p.ctrl->abort, 1); break; }
+                        else if (now - t0 > kWaitLimitNs) { s_abort = 1; note_timeout(p.ctrl, 3, cta); atomicExch(&p.ctrl->abort, 1); break; }
                     }
                 }
             }
@@ -558,7 +558,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
         for (int k = threadIdx.x; k < 65; k += WD_THREADS)
             if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
     if (threadIdx.x == 0) {
-        if (s_abort == 1) set_status(p.ctrl, WIND_ERR_TIMEOUT);
+        if (s_abort == 1) { note_timeout(p.ctrl, 4, cta); set_status(p.ctrl, WIND_ERR_TIMEOUT); }
         if (cta == 0) {
             if (exit_status) set_status(p.ctrl, exit_status);
             p.ctrl->active = 0;

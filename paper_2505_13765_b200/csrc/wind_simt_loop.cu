@@ -603,7 +603,7 @@ done:
         for (int k = tid; k < 65; k += SL_THREADS)
             if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
     if (tid == 0) {
-        if (s_stop) set_status(p.ctrl, WIND_ERR_TIMEOUT);
+        if (s_stop) { note_timeout(p.ctrl, 5, cta); set_status(p.ctrl, WIND_ERR_TIMEOUT); }
         if (cta == 0) { p.ctrl->active = 0; p.ctrl->loop_kernel = WIND_LOOP_GRID; }
     }
 }
