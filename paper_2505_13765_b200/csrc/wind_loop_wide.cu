@@ -36,8 +36,10 @@ constexpr uint32_t WD_Z_STAGE = WD_NJ * BK * 2;
 
 // Window rows of a slot in the coming step.  `blanks` and `labels` are recent sums over all utterances: rows found blank, and
 // rows with a label.  With blank probability q a window of w rows takes an utterance (1 - q^w) / (1 - q) rows further; a step of
-// 256 rows costs 1.25 times one of 128, and it has to bring half as much again (32 utterances, W = 16, 40 % of the frames with a
-// label: 128 rows throughout 23.1 ms, 256 rows 25.5 ms, this rule with 1.25 in place of 1.5 23.8 ms; without labels 256 rows win).
+// 256 rows costs 1.25 times one of 128, and q is an estimate, so it has to bring a little more: 1.35 times.  Measured with 5, 10,
+// 15, 20, 30, 40 and 60 % of the frames carrying a label, 12 to 32 utterances, W = 8 to 16 (42 batches): 1.35 is within 1.7 % of the
+// best of 1.25, 1.35, 1.5 and 1.7 but for one (12 utterances, 10 %: 4.1 %), 0.4 % on the average; 1.25 0.6 % (40 %, 32 x 16: 6.19 ms
+// against 5.98), 1.5 1.2 % (5 %, 32 x 8: 2.59 against 2.45), 256 rows throughout 5 % (most at 60 %: 24 %), 128 throughout 4 % (5 %: 23 %).
 __device__ __forceinline__ int wide_rows(int W, int live, float blanks, float labels) {
     const int n = max(live, 1), narrow = min(W, WD_NJ / n), wide = min(W, WD_ROWS / n);
     if (narrow == wide) return narrow;
@@ -47,7 +49,7 @@ __device__ __forceinline__ int wide_rows(int W, int live, float blanks, float la
         reach *= q;
         if (w == narrow) reach_narrow = reach;
     }
-    return 1.f - reach > 1.5f * (1.f - reach_narrow) ? wide : narrow;
+    return 1.f - reach > 1.35f * (1.f - reach_narrow) ? wide : narrow;
 }
 
 struct WdMaps {
