@@ -120,7 +120,8 @@ struct BeamDevice {
     BeamMail* mail = nullptr;
     uint32_t seq = 0, bar_base = 0;
     bool running = false;
-    std::chrono::steady_clock::time_point launched{};
+    bool on_chip = false;        // it has given a result since its launch (which may have waited for other streams)
+    std::chrono::steady_clock::time_point since{};      // the first of them
 
     cudaError_t open() {
         {
@@ -147,7 +148,7 @@ struct BeamDevice {
     // one command, until its result (nh * K entries) is there
     wind_status_t run(const int32_t* words, cudaError_t* err) {
         const int n_out = 2 * words[1] * c.B;
-        bool last = single || (running && std::chrono::steady_clock::now() - launched > kTurn);
+        bool last = single || (running && std::chrono::steady_clock::now() - since > kTurn);
         post(words, last);
         for (int launches = 0;;) {
             if (!running) {
@@ -155,7 +156,7 @@ struct BeamDevice {
                 if (++launches > 8) return WIND_ERR_TIMEOUT;
                 if ((*err = beam_step(c, mail, relay, seq, bar_base, h_pool, c_pool, g_pool, logits)) != cudaSuccess) return WIND_ERR_CUDA;
                 running = true;
-                launched = std::chrono::steady_clock::now();
+                on_chip = false;
             }
             bool there = false;
             for (uint32_t spins = 1; !there; ++spins) {
@@ -178,6 +179,7 @@ struct BeamDevice {
                 if (!there) { last = single; post(words, last); continue; }
                 ++seq;               // it may have left word that no command of the next number came: that number is not used
             }
+            if (!on_chip) { on_chip = true; since = std::chrono::steady_clock::now(); }
             if (last) running = false;
             bar_base += beam_step_arrivals(c, words[0]);
             return WIND_OK;
