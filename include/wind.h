@@ -37,15 +37,18 @@
  *     tensor-core operands: enc_proj (stored once per call), the LSTM hidden state h wherever it
  *     is consumed (the recurrent term of the next update, the input of the layer above and
  *     pred_proj -- the recurrence therefore feeds back a bf16 h), and the joint's activations
- *     act(enc_proj + pred_proj).  Both kernel sets (wind_kernels_t) round in the same places; the
- *     tensor-core kernels with on-chip weights also round pred_proj to bf16 before that sum.
- *     The tensor-core kernels evaluate the gate nonlinearities (and tanh activations) with the
- *     hardware tanh approximation (absolute error about 5e-4, below the bf16 rounding of h) when
- *     the weights are resident on chip; the plain-ALU kernels use tanhf / expf.  Joint logits
+ *     act(enc_proj + pred_proj).  Both kernel sets (wind_kernels_t) round in these places.  The
+ *     tensor-core kernels fall into two groups.  Clusters, grid barriers and arrival counters
+ *     (wind_loop_kernel_t) also round pred_proj to bf16 before that sum and evaluate the gate
+ *     nonlinearities with the hardware tanh approximation (absolute error about 5e-4, below the
+ *     bf16 rounding of h).  Streamed weights and the kernel for large vocabularies do neither:
+ *     pred_proj stays fp32, the gates use tanhf / expf.  Tanh activations of the joint are the
+ *     hardware's in both; the plain-ALU kernels use tanhf / expf throughout.  Joint logits
  *     agree with an fp64 evaluation of the same bf16 weights within 2e-2, also after hundreds
  *     of decoder updates; decisions whose top-two margin is smaller than such differences can
- *     come out differently between kernel sets (AUTO picks the set by shape), never between two
- *     runs of one set, and never between window sizes.
+ *     come out differently between kernel sets and between the two groups (picked by the
+ *     model's dimensions and the sizes of the call, never by the lengths), never between two
+ *     runs of one call, the kernels of a group, or window sizes that one group decodes.
  *   - Calls enqueue work on `stream`, synchronise that stream once at the end to read the
  *     device status word, and return it.  Errors detectable on the host return before
  *     any launch.  Every device-side wait is bounded; a wait that runs out sets
