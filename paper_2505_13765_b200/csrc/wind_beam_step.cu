@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                         const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
                                     ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
                         const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
-                        const float cc = gf * c_in + gi * gg;
+                        const float cc = cell_update_fc(gf, c_in, gi, gg);
                         if ((lane & 25) == 0 && col < n_here) {
                             p.c_pool[(size_t)c_dst[me] * LP + l * P + j] = cc;
                             p.h_pool[(size_t)c_dst[me] * LP + l * P + j] = go * tanhf(cc);

@@ -194,6 +194,12 @@ __device__ inline float key_logit(unsigned long long key) {
     return __uint_as_float((hi & 0x80000000u) ? (hi & 0x7FFFFFFFu) : ~hi);
 }
 
+// The cell update f c + i g.  Kernels that are to give the same transcripts have to round it alike, and left to the compiler the
+// product that goes into the fused multiply-add differs from place to place (one ulp of c, now and then one of a bf16 h).
+// cell_update: clusters, grid barriers, arrival counters; cell_update_fc: every other kernel.
+__device__ __forceinline__ float cell_update(float f, float c, float i, float g) { return __fmaf_rn(i, g, __fmul_rn(f, c)); }
+__device__ __forceinline__ float cell_update_fc(float f, float c, float i, float g) { return __fmaf_rn(f, c, __fmul_rn(i, g)); }
+
 __device__ inline void set_status(Ctrl* ctrl, int32_t s) { atomicCAS(&ctrl->status, 0, s); }
 // A wait of CTA `cta` ran out: the first one of the call stays.  Sites: 1 loop_kernel; 3 grid barrier of
 // wide_kernel, 4 another wait in it; 5 grid barrier of simt_grid_kernel; 6 grid barrier of beam_step_kernel, 7 its wait for a command; 20 to 43 in

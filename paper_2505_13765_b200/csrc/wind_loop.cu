@@ -457,7 +457,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                                     const float gf = sigmoid_f(pre[1][j] + add[1][j]);
                                     const float gg = tanhf(pre[2][j] + add[2][j]);
                                     const float go = sigmoid_f(pre[3][j] + add[3][j]);
-                                    const float cc = gf * cold[j] + gi * gg;
+                                    const float cc = cell_update_fc(gf, cold[j], gi, gg);
                                     cst[unit] = cc;
                                     hout[unit] = __float2bfloat16_rn(go * tanhf(cc));
                                 } else if (tok == -2) {
@@ -768,7 +768,7 @@ __global__ void __launch_bounds__(RES ? LOOP_THREADS_RES : LOOP_THREADS, 1) loop
                         if (tok_s[j] >= 0) {
                             const float gi = stage_f[(0 * 64 + j) * 16 + u16], gf = stage_f[(1 * 64 + j) * 16 + u16];
                             const float gg = stage_f[(2 * 64 + j) * 16 + u16], go = stage_f[(3 * 64 + j) * 16 + u16];
-                            const float cc = gf * cold[jj] + gi * gg;
+                            const float cc = cell_update(gf, cold[jj], gi, gg);
                             cst[(size_t)bj * p.P] = cc;
                             hout[(size_t)bj * p.P] = __float2bfloat16_rn(go * tanh_fast(cc));
                         } else if (tok_s[j] == -2) {

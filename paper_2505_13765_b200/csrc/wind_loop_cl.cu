@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                     if (u < U && s < NU) {
                         if ((live >> s) & 1u) {
                             const float cold = (fresh >> s) & 1u ? 0.f : c_st[k];
-                            const float cc = gf * cold + gi * gg;
+                            const float cc = cell_update(gf, cold, gi, gg);
                             c_st[k] = cc;
                             h_st[k] = __float2bfloat16_rn(go * tanh_fast(cc));
                         }
@@ -338,7 +338,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                     const float gg = fmaf(tanh_fast((x.z + add_r[2]) * 1.f), 1.f, 0.f);
                     const float go = fmaf(tanh_fast((x.w + add_r[3]) * 0.5f), 0.5f, 0.5f);
                     const float cold = (fresh >> s) & 1u ? 0.f : c_rem;
-                    const float cc = gf * cold + gi * gg;
+                    const float cc = cell_update(gf, cold, gi, gg);
                     c_rem = cc;
                     h_rem = __float2bfloat16_rn(go * tanh_fast(cc));
                 }

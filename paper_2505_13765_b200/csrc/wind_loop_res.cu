@@ -621,7 +621,7 @@ __global__ void __launch_bounds__(LOOP_THREADS_RES, 1) loop_res_kernel(const __g
                         if (tok_s[j] >= 0) {
                             const float gi = stage_f[(0 * 64 + j) * 16 + u16], gf = stage_f[(1 * 64 + j) * 16 + u16];
                             const float gg = stage_f[(2 * 64 + j) * 16 + u16], go = stage_f[(3 * 64 + j) * 16 + u16];
-                            const float cc = gf * cold[jj] + gi * gg;
+                            const float cc = cell_update(gf, cold[jj], gi, gg);
                             cst[(size_t)bj * p.P] = cc;
                             hout[(size_t)bj * p.P] = __float2bfloat16_rn(go * tanh_fast(cc));
                         } else {

@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
                         if (s_tok[b] >= 0) {
                             const float gi = stage[(0 * p.nl + b) * 16 + un], gf = stage[(1 * p.nl + b) * 16 + un];
                             const float gg = stage[(2 * p.nl + b) * 16 + un], go = stage[(3 * p.nl + b) * 16 + un];
-                            cell[jj] = gf * cell[jj] + gi * gg;
+                            cell[jj] = cell_update_fc(gf, cell[jj], gi, gg);
                             hid[jj] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(go * tanhf(cell[jj])));
                         }
                         out[b * BK + un] = __ushort_as_bfloat16((unsigned short)hid[jj]);

@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(128) lstm_layer_simt_kernel(const Ctrl* __rest
             float gf = 1.f / (1.f + expf(-(a[1] + bias[1])));
             float gg = tanhf(a[2] + bias[2]);
             float go = 1.f / (1.f + expf(-(a[3] + bias[3])));
-            float cc = gf * c_state[(size_t)b * P + j] + gi * gg;
+            float cc = cell_update_fc(gf, c_state[(size_t)b * P + j], gi, gg);
             c_state[(size_t)b * P + j] = cc;
             h_out[(size_t)b * P + j] = go * tanhf(cc);
         }

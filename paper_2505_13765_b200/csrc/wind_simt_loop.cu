@@ -451,7 +451,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_grid_kernel(const SimtLoop
                             a[g] = s + b_gate[4 * (l * M.units + ui) + g];
                         }
                         const float gi = 1.f / (1.f + expf(-a[0])), gf = 1.f / (1.f + expf(-a[1])), gg = tanhf(a[2]), go = 1.f / (1.f + expf(-a[3]));
-                        const float cc = gf * c_old + gi * gg;
+                        const float cc = cell_update_fc(gf, c_old, gi, gg);
                         *cs = cc;
                         h_row(s_hp[b] ^ 1, l, b)[j] = go * tanhf(cc);
                     }
@@ -766,7 +766,7 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_local_kernel(const SimtLoo
                         const float* gt = sf + M.gates + j;
                         const float gi = 1.f / (1.f + expf(-gt[0])), gf = 1.f / (1.f + expf(-gt[p.P])), gg = tanhf(gt[2 * p.P]), go = 1.f / (1.f + expf(-gt[3 * p.P]));
                         float* cs = sf + M.c + l * p.P + j;
-                        const float cc = gf * *cs + gi * gg;
+                        const float cc = cell_update_fc(gf, *cs, gi, gg);
                         *cs = cc;
                         sf[M.h + l * M.np + j] = sl_round<TW>(go * tanhf(cc));
                     }
