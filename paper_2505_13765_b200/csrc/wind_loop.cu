@@ -1932,6 +1932,10 @@ cudaError_t loop_plan_for(const wind_model_t& m, int B, int W, int sms, int smem
         r.w_first = l_sets * r.l_items;
         r.w_count = (B + 63) / 64;
         if (r.w_first + r.w_count + r.p_items > G) r.w_count = 0;
+        // Arrival counters sum over the slots, which is sound only while nobody who arrives can be a slot ahead of the others.  A
+        // recording CTA whose 64 utterances are all finished can (it waits for no pred_proj any more): where a group of utterances
+        // spans two of them, the group's first decoder CTA records instead.
+        if (r.dataflow && r.nl > 64 && r.w_count > 1) r.w_count = 0;
         r.l_early = 1;
         const int acc_cols = r.nl > 2 * r.np ? r.nl : 2 * r.np;
         if ((long long)r.smem_bytes <= (long long)budget + 1024 && r.tm_l + acc_cols <= (int)LOOP_TMEM_COLS) {

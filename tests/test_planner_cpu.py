@@ -161,3 +161,18 @@ def test_the_shapes_that_once_went_wrong_and_the_configured_ones():
     pkg.wind_set_loop_options()
     assert pkg.wind_debug_plan(dict(large, P=100), 8, 4)[0] == bd.WIND_ERR_UNSUPPORTED
     assert pkg.wind_debug_plan(dict(large, V=50), 8, 4)[0] == bd.WIND_ERR_UNSUPPORTED
+
+
+def test_no_utterance_group_spans_two_recording_ctas():
+    # Arrival counters sum over lock steps: a recording CTA with nothing left to record could be a step ahead of the others that
+    # arrive on the same group's counter.
+    pkg.wind_set_loop_options(dataflow=1)
+    wide = 0
+    for P in (64, 128, 256, 384, 512, 640):
+        for L in (1, 2):
+            for B in range(1, 257, 3):
+                st, pl = pkg.wind_debug_plan(dict(D=64, E=64, P=P, L=L, H=128, V=300), B, 4)
+                if st == bd.WIND_OK and pl["resident"] and pl["dataflow"]:
+                    wide += pl["nl"] > 64 and B > 64
+                    assert pl["nl"] <= 64 or pl["w_count"] <= 1, (P, L, B, pl)
+    assert wide > 0
