@@ -333,7 +333,7 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
  * multiples of 8, weights 16-byte aligned, one window's logits in shared memory) that is one kernel which stays for many
  * iterations: it takes each from page-locked host memory and leaves the K x K (label, offset, log-probability) triples there,
  * and the calling thread spins on them.  It has a block of 512 threads on every SM while it stays, so kernels of other
- * streams that do not fit beside it (most that use shared memory or many registers) wait for it; it ends every 5 ms
+ * streams that do not fit beside it (most that use shared memory or many registers) wait for it; it ends every 10 ms
  * (with prefix_search: after every iteration) and is launched again behind them.  Other shapes launch kernels per iteration
  * and synchronise `stream` to read the triples.  The call synchronises `stream` before it returns.
  * The call takes 5 KB of page-locked host memory from the driver (cudaHostAlloc) unless an earlier search left its own

@@ -109,9 +109,9 @@ inline void cpu_relax() {
 }
 
 // The resident kernel of one search, as the host sees it.  It holds every SM, so little of another stream fits beside it: after
-// kTurn it ends with the command in hand, what waits on other streams goes first, and the next command launches it again (25 us,
-// mostly its weights: half a percent of the search).
-constexpr std::chrono::milliseconds kTurn(5);
+// kTurn it ends with the command in hand, what waits on other streams goes first, and the next command launches it again (30 us,
+// mostly its weights: 0.3 % of the search; 0.6 % with 5 ms).
+constexpr std::chrono::milliseconds kTurn(10);
 struct BeamDevice {
     const Call& c;
     float *h_pool, *c_pool, *g_pool, *logits;

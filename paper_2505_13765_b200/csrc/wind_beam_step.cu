@@ -12,7 +12,7 @@
 //
 // The kernel never depends on the host's pace: without a command for 200 us it ends, and the host launches it again with the
 // next one (all state is in global memory).  So a debugger or a descheduled host thread cost the search time only.  On every SM
-// it leaves 8 of 64 thousand registers, so most kernels of other streams wait for its end: the host has it end every 5 ms.
+// it leaves 8 of 64 thousand registers, so most kernels of other streams wait for its end: the host has it end every 10 ms.
 //
 // A command or result word carries its 32 bits and the command's number in one 8-byte store, so no fence or flag is needed on
 // either side of the bus.
