@@ -1967,7 +1967,8 @@ static thread_local LoopMaps t_loop_maps;
 static thread_local LoopPlan t_loop_plan;
 
 cudaError_t loop_prepare(Call& c) {
-    cudaError_t e = get_encode_loop();
+    cudaError_t e = bind_context(c.stream);
+    if (e == cudaSuccess) e = get_encode_loop();
     if (e != cudaSuccess) return e;
     LoopPlan& pl = t_loop_plan;
     if ((e = loop_plan(c, &pl)) != cudaSuccess) return e;

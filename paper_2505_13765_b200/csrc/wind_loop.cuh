@@ -147,6 +147,12 @@ cudaError_t loop_map_blocks(CUtensorMap* map, const void* base, uint64_t blocks,
 bool wide_supported(const Call& c);
 cudaError_t wide_loop(const Call& c);
 int loop_launches(const Call& c, int trace_step);   // kernels tc_loop launches for a decode (after loop_prepare)
+// Makes the device's context current in this thread, if none is: tensor maps are built by the driver, which does not, and a
+// decode may be the first thing a thread does on the GPU.  (The runtime does with any call on a stream.)
+inline cudaError_t bind_context(cudaStream_t stream) {
+    unsigned flags = 0;
+    return cudaStreamGetFlags(stream, &flags);
+}
 cudaError_t loop_prepare(Call& c);   // plan + tensor maps + shared-memory opt-in (host only; not inside a capture)
 
 }  // namespace wind

@@ -64,7 +64,8 @@ static thread_local TcMaps t_maps;
 static cudaError_t tc_set_attributes();
 
 cudaError_t tc_prepare(Call& c) {
-    cudaError_t e = get_encode();
+    cudaError_t e = bind_context(c.stream);
+    if (e == cudaSuccess) e = get_encode();
     if (e != cudaSuccess) return e;
     TcMaps& M = t_maps;
     const wind_model_t& m = c.m;
