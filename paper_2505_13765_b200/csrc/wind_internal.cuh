@@ -203,7 +203,7 @@ __device__ __forceinline__ float cell_update_fc(float f, float c, float i, float
 __device__ inline void set_status(Ctrl* ctrl, int32_t s) { atomicCAS(&ctrl->status, 0, s); }
 // A wait of CTA `cta` ran out: the first one of the call stays.  Sites: 1 loop_kernel; 3 grid barrier of
 // wide_kernel, 4 another wait in it; 5 grid barrier of simt_grid_kernel; 6 grid barrier of beam_step_kernel, 7 its wait for a command; 20 to 43 in
-// loop_res_kernel, 50 + the warp in cl_kernel (its roles stand there)
+// loop_res_kernel, 50 + the warp in cl_kernel (its roles stand there), 70 + the layer in its cl_recurrent
 __device__ inline void note_timeout(Ctrl* ctrl, int site, int cta) {
     if (atomicCAS(&ctrl->timeout_site, 0, site) == 0) ctrl->timeout_cta = cta;
 }

@@ -43,20 +43,242 @@ namespace wind {
 struct ClDec { int tok; uint32_t flags, row, unused; };   // what an owner sends for its slot
 constexpr uint32_t CL_FRESH = 1u, CL_IDLE = 2u, CL_ODD = 4u;   // CL_ODD: parity of the step it is for
 
+// W_hh (or the second layer's W_ih) rows of the CTA's hidden units 0..31 into tensor memory: lane 4 u + gate.  Warps 0-7.
+__device__ __forceinline__ void cl_gate_rows_to_tmem(const __nv_bfloat16* w, int P, int r, int warp, int lane, uint32_t tmem) {
+    const int q = warp & 3, U = P / CL_SIZE, u = 8 * q + (lane >> 2), g = lane & 3;
+    const bool in = u < U;
+    const uint4* src = reinterpret_cast<const uint4*>(w + ((size_t)g * P + r * U + (in ? u : 0)) * P);
+#pragma unroll 1
+    for (int c0 = 16 * (warp >> 2); c0 < P / 2; c0 += 32) {
+        uint32_t v[16];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint4 x = in ? src[c0 / 4 + j] : make_uint4(0, 0, 0, 0);
+            v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
+        }
+        tmem_st16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
+    }
+    tmem_st_wait();
+}
+
+// The recurrent terms of two-layer models.  Such a decoder (large dimensions: 12 MB) does not fit a cluster, but W_hh h of either
+// layer is not needed before the next step's update, so a cluster per layer keeps that layer's W_hh and computes it for all decoding
+// clusters while these go on: CTA r of a decoding cluster leaves its units of the new state in hx and adds one to req; CTA r here
+// fetches the state of all units once 16 CTAs have, multiplies its rows (the units of CTA r there) and leaves the result where CTA r
+// reads it (rx), every value with the number of the update: value and "ready" arrive in one load, and no write has to be waited for
+// (a counter behind the writes, a copy into shared memory and their fences took 3500 cycles).  hx has two copies by parity of the
+// updates: a CTA writes a copy again only two updates later, when every CTA of its cluster has had the answer to the update between;
+// nothing else here needs more than one, since a CTA's next request follows its answer.  The round trip through L2 takes most of a
+// step, so requests should not queue: the states of all clusters lie one behind the other as row groups of one operand, and a chain
+// of MMAs serves every request that is there when it starts (its other columns go nowhere).
+// Warps: 0-3 results, 4-11 remainder units (mma.sync; 4-7 for even clusters), 14 issues MMAs, 15 fetches states.
+constexpr int CL_REC_SETS = 3;                            // accumulators: the results of one chain leave under the next ones
+__device__ __noinline__ void cl_recurrent(const CUtensorMap& hx_map, const ClParams& p, const int layer, const int r, uint8_t* smem) {
+    __shared__ uint64_t bar_full[CL_DECODERS], bar_acc[CL_REC_SETS], bar_free[CL_REC_SETS];
+    __shared__ uint32_t tmem_slot;
+    __shared__ volatile uint32_t s_total[CL_DECODERS];    // updates of a decoding cluster that has left (before that: all ones)
+    __shared__ volatile uint32_t s_mask[CL_REC_SETS];     // decoding clusters whose results an accumulator holds; 0: no more of them
+    __shared__ volatile int s_abort;
+    const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
+    const int n_dec = (int)gridDim.x / CL_SIZE - 2, U = p.P / CL_SIZE, NU = p.slots;
+    const bool has_rem = U > 32;
+    const uint32_t state = (uint32_t)p.P * 16u;           // bytes of a cluster's state: K blocks of 8 slots x 128 bytes
+    const uint32_t acc_cols = (uint32_t)(8 * n_dec + 15) & ~15u;
+    if (threadIdx.x == 0) {
+        s_abort = 0;
+        for (int c = 0; c < CL_DECODERS; ++c) { s_total[c] = 0xFFFFFFFFu; mbar_init(&bar_full[c], 1); }
+        for (int c = 0; c < CL_REC_SETS; ++c) { mbar_init(&bar_acc[c], 2); mbar_init(&bar_free[c], 4); }
+        fence_barrier_init();
+        prefetch_tmap(&hx_map);
+    }
+    if (warp == 14) tmem_alloc(&tmem_slot, LOOP_TMEM_COLS);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    if (warp < 8) cl_gate_rows_to_tmem(p.w_rec[layer], p.P, r, warp, lane, tmem);
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tm_acc = tmem + CL_MAX_DIM / 2;
+    auto answer = [&](int c) { return p.rx + ((size_t)(c * 2 + layer) * CL_SIZE + r) * (size_t)(NU * 4 * U); };
+    uint32_t n = 0u;                                      // of cluster `lane`: updates this warp has dealt with
+    // work(mask) for those of the clusters `mine` whose state is there, until all of them have left
+    auto serve = [&](uint32_t mine, auto work) {
+        const int c = min(lane, n_dec - 1);
+        const bool on = lane < n_dec && ((mine >> lane) & 1u);
+        for (;;) {
+            const uint32_t total = s_total[c];
+            const uint32_t ready = __ballot_sync(0xffffffffu, on && n != total && mbar_test(&bar_full[c], n & 1u));
+            if (__any_sync(0xffffffffu, s_abort) || __all_sync(0xffffffffu, !on || n == total)) break;
+            if (ready) {
+                work(ready);
+                n += (ready >> lane) & 1u;
+            }
+        }
+    };
+    if (warp < 4) {
+        const int e = threadIdx.x, u = 8 * warp + (lane >> 2);
+        for (uint32_t set = 0u, turn = 0u;;) {
+            // (the warp that issues leaves a mask of 0 behind its last chain)
+            bool there = false;
+            while (!(there = __all_sync(0xffffffffu, mbar_test(&bar_acc[set], turn & 1u))) && !__any_sync(0xffffffffu, s_abort)) {}
+            const uint32_t mask = there ? s_mask[set] : 0u;
+            if (mask == 0u) break;
+            tc_fence_after();
+            n += (mask >> lane) & 1u;
+            const bool alone = (mask & (mask - 1u)) == 0u;
+            for (uint32_t left = mask; left; left &= left - 1u) {
+                const int c = __ffs((int)left) - 1;
+                const uint32_t stamp = __shfl_sync(0xffffffffu, n, c);
+                float x[8];
+                tmem_ld8(tm_acc + set * acc_cols + (alone ? 0u : 8u * (uint32_t)c) + ((uint32_t)(warp * 32) << 16), x);
+                unsigned long long* dst = answer(c) + e;
+                if (u < U)
+#pragma unroll
+                    for (int s = 0; s < 8; ++s)
+                        if (s < NU) st_relaxed_u64(dst + s * 4 * U, (unsigned long long)stamp << 32 | __float_as_uint(x[s]));
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive(&bar_free[set]);
+            if (++set == CL_REC_SETS) { set = 0u; ++turn; }
+        }
+    } else if (warp < 12) {
+        if (has_rem) {
+            const int k = (warp - 4) & 3, row = 8 * k + (lane >> 2), u = 32 + (row >> 2), g = row & 3;
+            uint32_t wf[40][2];
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(p.w_rec[layer] + ((size_t)g * p.P + r * U + min(u, U - 1)) * p.P) + (lane & 3);
+#pragma unroll
+            for (int s0 = 0; s0 < 40; s0 += 8)
+                if (s0 < p.P / 16)
+#pragma unroll
+                    for (int s = s0; s < s0 + 8; ++s) { wf[s][0] = src[s * 8]; wf[s][1] = src[s * 8 + 4]; }
+            serve(warp < 8 ? 0x55555555u : 0xAAAAAAAAu, [&](uint32_t mask) {
+                for (uint32_t left = mask; left; left &= left - 1u) {
+                    const int c = __ffs((int)left) - 1;
+                    const uint32_t h_row = smem_u32(smem) + (uint32_t)c * state + (uint32_t)((lane & 7) * 128);
+                    auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * 1024u + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
+                    float acc[4] = {0.f, 0.f, 0.f, 0.f};
+                    uint32_t a[2][4];
+                    ldmatrix_x4(a[0], h_at(0));
+#pragma unroll
+                    for (int s0 = 0; s0 < 40; s0 += 8)
+                        if (s0 < p.P / 16)
+#pragma unroll
+                            for (int s = s0; s < s0 + 8; s += 2) {
+                                ldmatrix_x4(a[(s / 2 + 1) & 1], h_at(s / 2 + 1));       // (the last turn: rows nobody uses)
+                                mma_16816(acc, a[(s / 2) & 1][0], 0u, a[(s / 2) & 1][1], 0u, wf[s][0], wf[s][1]);
+                                mma_16816(acc, a[(s / 2) & 1][2], 0u, a[(s / 2) & 1][3], 0u, wf[s + 1][0], wf[s + 1][1]);
+                            }
+                    const unsigned long long stamp = (unsigned long long)(__shfl_sync(0xffffffffu, n, c) + 1u) << 32;
+                    unsigned long long* dst = answer(c) + (lane >> 2) * 4 * U + 128 + k * 8 + (lane & 3) * 2;
+                    if ((lane >> 2) < NU) {
+                        st_relaxed_u64(dst, stamp | __float_as_uint(acc[0]));
+                        st_relaxed_u64(dst + 1, stamp | __float_as_uint(acc[1]));
+                    }
+                }
+            });
+        }
+    } else if (warp == 14) {
+        const uint32_t id_all = idesc_bf16(128, (int)acc_cols), id_one = idesc_bf16(128, 16);
+        uint32_t set = 0u, turn = 0u;                     // chains so far: turn * CL_REC_SETS + set
+        auto next = [&](uint32_t mask) {                  // an accumulator for the next chain
+            if (turn > 0u && !cl_wait_warp(&bar_free[set], (turn - 1u) & 1u)) { s_abort = 1; return false; }
+            if (lane == 0) { s_mask[set] = mask; mbar_arrive(&bar_acc[set]); }
+            __syncwarp();
+            return true;
+        };
+        serve(0xFFFFFFFFu, [&](uint32_t mask) {
+            if (!next(mask)) return;
+            tc_fence_after();
+            if (elect_one()) {
+                // row groups (the clusters' states) `state` bytes apart.  One request alone: its state and the rows behind it (an MMA
+                // has 16 columns at the least, and with 48 the chain takes half as long again)
+                const bool alone = (mask & (mask - 1u)) == 0u;
+                const uint32_t first = alone ? (uint32_t)(__ffs((int)mask) - 1) * state : 0u, id = alone ? id_one : id_all;
+                uint64_t hd = (smem_desc_sw128(smem_u32(smem) + first) & ~((uint64_t)0x3FFF << 32)) | ((uint64_t)(state >> 4) << 32);
+#pragma unroll 1
+                for (int kb = 0; kb < p.P / 64; ++kb, hd += 1024 >> 4)
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        tc_mma_bf16_ts(tm_acc + set * acc_cols, tmem + (uint32_t)(kb * 32 + k * 8), hd + (uint64_t)(k * 2), id, (kb | k) != 0);
+                tc_commit(&bar_acc[set]);
+            }
+            __syncwarp();
+            if (++set == CL_REC_SETS) { set = 0u; ++turn; }
+        });
+        // MMAs in flight use tensor memory
+        if (set > 0u || turn > 0u) cl_wait_warp(&bar_acc[set > 0u ? set - 1u : CL_REC_SETS - 1], (set > 0u ? turn : turn - 1u) & 1u);
+        if (!s_abort && next(0u) && lane == 0) mbar_arrive(&bar_acc[set]);
+        __syncwarp();
+    } else if (warp == 15) {
+        const int c = min(lane, n_dec - 1);
+        bool left = lane >= n_dec;
+        uint32_t beat = 0u;
+        unsigned long long since = globaltimer_ns();
+        for (uint32_t it = 1u;; ++it) {
+            // (whether a cluster has left is asked now and then, and before what it has asked for: nothing may come after that)
+            const uint32_t gone = (it & 63u) == 0u && !left ? ld_acquire_u32(p.done + c) : 0u;
+            if (!left) {
+                const uint32_t there = ld_acquire_u32(p.req + layer * CL_DECODERS + c) - (uint32_t)CL_SIZE * n;
+                if (there >= (uint32_t)CL_SIZE) {
+                    fence_proxy_async_all();              // written by generic stores
+                    mbar_expect_tx(&bar_full[c], state);
+                    tma_load_3d(smem + (uint32_t)c * state, &hx_map, 0, ((c * 2 + layer) * 2 + (int)(n & 1u)) * 8, 0, &bar_full[c]);
+                    ++n;
+                } else if (gone == (uint32_t)CL_SIZE) {
+                    left = true;
+                    s_total[c] = n;
+                }
+            }
+            if (__all_sync(0xffffffffu, left)) break;
+            if ((it & 1023u) == 0u) {
+                // a decoding cluster may have nothing to ask for long (blanks), but it counts its steps
+                const uint32_t b = left ? 0u : ld_acquire_u32(p.beat + c) + n;
+                const unsigned long long now = globaltimer_ns();
+                if (__any_sync(0xffffffffu, b != beat)) since = now;
+                beat = b;
+                if (__any_sync(0xffffffffu, now - since > 2 * kWaitLimitNs || ld_acquire_u32(reinterpret_cast<const uint32_t*>(&p.ctrl->abort)) != 0u)) { s_abort = 1; break; }
+            }
+        }
+        if (lane < n_dec && n > 0u) cl_wait(&bar_full[lane], (n - 1u) & 1u);     // copies in flight
+        __syncwarp();
+    }
+    tc_fence_before();
+    __syncthreads();
+    if (warp == 14) {
+        tc_fence_after();
+        tmem_dealloc(tmem, LOOP_TMEM_COLS);
+    }
+    if (threadIdx.x == 0 && s_abort) {
+        atomicExch(&p.ctrl->abort, 1);
+        note_timeout(p.ctrl, 70 + layer, blockIdx.x);
+        set_status(p.ctrl, WIND_ERR_TIMEOUT);
+    }
+}
+
 // Warps: 0-3 gates and z (workers), 4-9 W_pred, 10-13 remainder units, 14 issuing thread, 15 control.  Warps 0-7 also
 // share the joint's epilogue.  NS: most slots in use (1, 2, 4, 8).
-template <int NS, int ACT>
-__global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant__ CUtensorMap enc_map, const ClParams p) {
+template <int NS, int ACT, int NL>
+__global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant__ CUtensorMap enc_map, const __grid_constant__ CUtensorMap hx_map, const __grid_constant__ ClParams p) {
     extern __shared__ uint8_t smem_raw[];
-    __shared__ uint64_t bar_keys, bar_dec, bar_enc, bar_h, bar_pred, bar_z, bar_sync_mma, bar_acc_g, bar_acc_r, bar_acc_j;
+    __shared__ uint64_t bar_keys, bar_dec, bar_enc, bar_h, bar_pred, bar_z, bar_sync_mma, bar_acc_g, bar_acc_r, bar_acc_j, bar_h0, bar_rec;
     __shared__ uint32_t tmem_slot;
     __shared__ int s_abort;
     __shared__ int s_hist[65];
+    __shared__ long long s_lap[4];
 
     const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
     if (p.ctrl->bad_input || (p.choose && p.ctrl->use_grid != 0)) return;   // a length outside [0, T], or another kernel's turn: the whole grid leaves before it does anything
     const int r = (int)cl_rank();
-    const int cluster = blockIdx.x / CL_SIZE, n_clusters = gridDim.x / CL_SIZE;
+    if constexpr (NL == 2) {
+        if (blockIdx.x / CL_SIZE < 2) {                  // (these come first: nobody waits for CTAs that are not resident yet)
+            cl_recurrent(hx_map, p, (int)blockIdx.x / CL_SIZE, r, align_smem_1024(smem_raw));
+            return;
+        }
+    }
+    const int cluster = (int)blockIdx.x / CL_SIZE - (NL == 2 ? 2 : 0), n_clusters = (int)gridDim.x / CL_SIZE - (NL == 2 ? 2 : 0);
     const int NU = p.slots, U = p.P / CL_SIZE, HS = p.H / CL_SIZE;
     const int kb_p = p.P / 64, kb_h = p.H / 64;
     const int wp_shift = p.wp == 8 ? 3 : (p.wp == 16 ? 4 : 5);
@@ -67,9 +289,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     const int labs = min(lab_n, max(0, p.NV - lab0));
     const int lab_rows = lab_base + (lab_extra > 0 ? 8 : 0);            // rows of a K block of the W_out tile
     const bool has_rem = U > 32;
+    // Whether warps 10-13 have a part in the steps.  They then build z in every one of them: a warp that nobody waits for could fall two
+    // steps behind and take one decision for another.
+    const bool rem_warps = has_rem || NL == 2;
 
     uint8_t* smem = align_smem_1024(smem_raw);
-    const ClSmem L = cl_smem_layout(p.P, p.H, p.NV, NU, p.wp);
+    const ClSmem& L = p.smem;                            // (worked out on the host: there is no register to spare)
     const uint32_t sbase = smem_u32(smem);
     const ClDec* dec = reinterpret_cast<const ClDec*>(smem + L.dec);
     float* s_bout = reinterpret_cast<float*>(smem + L.b_out);
@@ -78,16 +303,19 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
 
     if (threadIdx.x == 0) {
         s_abort = 0;
+        s_lap[0] = s_lap[1] = s_lap[2] = 0;
         mbar_init(&bar_keys, 1);
         mbar_init(&bar_dec, 1u + (uint32_t)p.extra_arrivals);   // extra_arrivals > 0: a test hook, the wait can then never end
         mbar_init(&bar_enc, 1);
         mbar_init(&bar_h, 1);
         mbar_init(&bar_pred, 1);
-        mbar_init(&bar_z, 10u + (has_rem ? 4u : 0u));
+        mbar_init(&bar_z, 10u + (rem_warps ? 4u : 0u));
         mbar_init(&bar_sync_mma, 6u + (has_rem ? 4u : 0u));
         mbar_init(&bar_acc_g, 1);
         mbar_init(&bar_acc_r, 4);
         mbar_init(&bar_acc_j, 1);
+        mbar_init(&bar_h0, 1);
+        mbar_init(&bar_rec, 4);
         fence_barrier_init();
         // armed for their first phase (later phases: by the warp that saw the previous one complete, and only then: a barrier must
         // not be armed twice in a phase).  bar_h and bar_pred are armed in the steps that update a decoder, once it is known how many.
@@ -107,8 +335,18 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             const uint4 v = row < labs ? *reinterpret_cast<const uint4*>(p.w_out + (size_t)(lab0 + row) * p.H + c * 8) : make_uint4(0, 0, 0, 0);
             *reinterpret_cast<uint4*>(smem + L.w_out + (c >> 3) * (lab_rows * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)) = v;
         }
-    for (uint32_t i = threadIdx.x; i < 2u * (uint32_t)p.P; i += CL_THREADS)       // h of slots nobody uses must be numbers
-        *reinterpret_cast<uint4*>(smem + L.h + i * 16) = make_uint4(0, 0, 0, 0);
+    for (uint32_t i = threadIdx.x; i < (L.pred - L.h0) / 16u; i += CL_THREADS)    // h of slots nobody uses must be numbers
+        *reinterpret_cast<uint4*>(smem + L.h0 + i * 16) = make_uint4(0, 0, 0, 0);
+    for (int i = threadIdx.x; i < NL * CL_SLOTS * U / 8; i += CL_THREADS) *reinterpret_cast<uint4*>(smem + L.hst + i * 16) = make_uint4(0, 0, 0, 0);
+    if constexpr (NL == 2)
+        for (int i = threadIdx.x; i < 4 * U; i += CL_THREADS) {
+            const int at = (i & 3) * p.P + r * U + (i >> 2);
+            reinterpret_cast<float*>(smem + L.b_gate)[i] = p.b_gate[0][at] + p.b_gate[1][at];
+        }
+    // the recurrent term of layer l (two layers)
+    auto rec_at = [&](int l) { return p.rx + ((size_t)(cluster * 2 + l) * CL_SIZE + r) * (size_t)(NU * 4 * U); };
+    if constexpr (NL == 2)
+        for (int i = threadIdx.x; i < NU * 4 * U; i += CL_THREADS) rec_at(0)[i] = rec_at(1)[i] = 0ull;   // no update has number 0
     fence_proxy_async();
     tc_fence_before();
     __syncthreads();
@@ -117,22 +355,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     const uint32_t tm_g = tmem + CL_MAX_DIM / 2, tm_j = tm_g + 32, tm_j2 = tm_j + 80;   // gates: 16 columns; joint: two copies of up to 72
     const int q = warp & 3;                                                       // lane quadrant
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    if (warp < 8) {                                                               // W_hh of units 0..31: lane 4 u + gate
-        const int u = 8 * q + (lane >> 2), g = lane & 3;
-        const bool in = u < U;
-        const uint4* src = reinterpret_cast<const uint4*>(p.w_hh + ((size_t)g * p.P + r * U + (in ? u : 0)) * p.P);
-#pragma unroll 1
-        for (int c0 = 16 * (warp >> 2); c0 < p.P / 2; c0 += 32) {
-            uint32_t v[16];
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint4 x = in ? src[c0 / 4 + j] : make_uint4(0, 0, 0, 0);
-                v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
-            }
-            tmem_st16(tmem + lane_off + (uint32_t)c0, v);
-        }
-        tmem_st_wait();
-    }
+    if (warp < 8) cl_gate_rows_to_tmem(p.w_gate, p.P, r, warp, lane, tmem);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -144,8 +367,9 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     // slots that feed a token to their decoder in this step
     auto live_slots = [&]() { return __ballot_sync(0xffffffffu, lane < NU && dec[min(lane, NU - 1)].tok >= 0); };
     // ldmatrix address of the state: two K steps of 16 at a time, matrix = 8 slots x 8 columns, lane = (column piece, slot)
+    constexpr uint32_t H_BLOCK = NL == 2 ? 1024u : 2048u;
     const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
-    auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * 2048u + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
+    auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * H_BLOCK + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
 
     // The joint's operand z = act(enc_proj + pred_proj), in place, by every warp that computes (0..13; it is bound by the shared
     // memory's bandwidth: 30 KB per group of eight rows, 2110 cycles for eight groups).  Of a group the rows that count: three
@@ -153,7 +377,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     // at a time.  (Half to the workers, half to four W_pred warps: these took 4250 cycles for eight groups.)  Threads per row: a
     // multiple of eight, one per 16-byte piece of a K block.
     const int z_rows = p.wp == 8 ? p.W : 8, z_mine = warp < 4 ? (3 * z_rows + 4) / 8 : z_rows - (3 * z_rows + 4) / 8;
-    const int z_threads = warp < 4 ? 128 : (has_rem ? 320 : 192), z_tid = warp < 4 ? (int)threadIdx.x : (int)threadIdx.x - 128;
+    const int z_threads = warp < 4 ? 128 : (rem_warps ? 320 : 192), z_tid = warp < 4 ? (int)threadIdx.x : (int)threadIdx.x - 128;
     const int z_tpr = (z_threads / max(z_mine, 1)) & ~7, z_at = z_tid / z_tpr;
     const bool z_on = z_at < z_mine;
     const int z_r = (warp < 4 ? 0 : z_rows - z_mine) + z_at, z_k0 = (z_tid % z_tpr) >> 3, z_kstep = z_tpr >> 3;
@@ -244,17 +468,15 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             const int i = h_first + 32 * k;
             const int uu = i / (U / 8), cc = i - uu * (U / 8), col = r * U + cc * 8;
             h_src[k] = (L.hst + (uint32_t)(uu * U + cc * 8) * 2u) | (uint32_t)uu << 24;
-            h_dst[k] = L.h + (uint32_t)((col >> 6) * 2048 + uu * 128 + ((((col >> 3) & 7) ^ (uu & 7)) << 4));
+            h_dst[k] = L.h + (uint32_t)(col >> 6) * H_BLOCK + (uint32_t)(uu * 128 + ((((col >> 3) & 7) ^ (uu & 7)) << 4));
         }
-        float c_st[2] = {0.f, 0.f}, c_rem = 0.f;         // cell state: (u, slots 2 g, 2 g + 1); (32 + (e & 7), slot e >> 3) for e < 64
-        __nv_bfloat16 h_st[2], h_rem = __float2bfloat16_rn(0.f);
-        h_st[0] = h_st[1] = h_rem;
-        __nv_bfloat16* hst = reinterpret_cast<__nv_bfloat16*>(smem + L.hst);
-        long long clk = 0, cyc[3] = {0, 0, 0};
-        const bool timed = blockIdx.x == 0 && e == 0;
+        // cell state: (u, slots 2 g, 2 g + 1); (32 + (e & 7), slot e >> 3) for e < 64.  Two layers: kept in shared memory, [layer][3][e]
+        float c_st[2] = {0.f, 0.f}, c_rem = 0.f;
+        uint32_t updates = 0u;                           // (two layers)
+        const bool timed = cluster == 0 && r == 0 && e == 0;
         unsigned long long ns0 = 0;
-        if (timed) { ns0 = globaltimer_ns(); clk = clock64(); }
-        auto lap = [&](int k) { if (timed) { const long long now = clock64(); cyc[k] += now - clk; clk = now; } };
+        if (timed) { ns0 = globaltimer_ns(); s_lap[3] = clock64(); }
+        auto lap = [&](int k) { if (timed) { const long long now = clock64(); s_lap[k] += now - s_lap[3]; s_lap[3] = now; } };   // (no register to spare)
 
         // parities in one word (registers are short): bit 0 of the step, bit 1 of the updates so far, bit 2: there was one
         for (uint32_t st = 0u;; st ^= 1u) {
@@ -282,21 +504,70 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
 #pragma unroll
                 for (int k = 0; k < 4; ++k) add_r[k] = tok >= 0 ? g0r[(uint32_t)tok * (uint32_t)(4 * p.P) + (uint32_t)(k * p.P)] : 0.f;
             }
-            // ---- gates: recurrent term + gate table, cell update ----
+            // ---- gates: recurrent term + gate table, cell update; the second layer: its product with the first one's new state,
+            // recurrent term, biases ----
+            bool leave = false;
+#pragma unroll 1
+            for (int l = 0; l < NL; ++l) {
             if (live != 0u) {
-            if (ok && warp == 0 && lane == 0) mbar_expect_tx(&bar_pred, (uint32_t)(__popc(live) * p.H) * 2u);
-            if (st & 4u) {
-                if (ok) ok = cl_wait(&bar_acc_g, (~st >> 1) & 1u);
-                if (has_rem && ok) ok = cl_wait(&bar_acc_r, (~st >> 1) & 1u);
+            __nv_bfloat16* hst = reinterpret_cast<__nv_bfloat16*>(smem + L.hst) + l * CL_SLOTS * U;
+            float* c_mem = reinterpret_cast<float*>(smem + L.cell) + l * 3 * 128 + e;
+            if (l == 0) {
+                if (ok && warp == 0 && lane == 0) {
+                    mbar_expect_tx(&bar_pred, (uint32_t)(__popc(live) * p.H) * 2u);
+                    if constexpr (NL == 2) mbar_expect_tx(&bar_h0, (uint32_t)(__popc(live) * p.P) * 2u);
+                }
+                if (st & 4u) {
+                    if constexpr (NL == 1) {
+                        if (ok) ok = cl_wait(&bar_acc_g, (~st >> 1) & 1u);
+                        if (has_rem && ok) ok = cl_wait(&bar_acc_r, (~st >> 1) & 1u);
+                    }
+                }
             }
-            st = (st ^ 2u) | 4u;
+            float rec[NS], rec_r[4] = {0.f, 0.f, 0.f, 0.f};              // two layers: the recurrent term
+            if constexpr (NL == 2) {
+#pragma unroll
+                for (int s = 0; s < NS; ++s) rec[s] = 0.f;
+                // (of slots that start afresh too, for which it does not count: the next request has to follow the answer to the last)
+                const bool want_r = rem_on && ((live >> (e >> 3)) & 1u);
+                if (l == 0) {
+                    const float* mine = reinterpret_cast<const float*>(smem + L.rec);
+                    if (st & 4u) {
+                        if (ok) ok = cl_wait(&bar_rec, (~st >> 1) & 1u);
+#pragma unroll
+                        for (int s = 0; s < NS; ++s)
+                            if (u < U && s < NU) rec[s] = mine[s * 4 * U + e];
+                        if (want_r) {
+                            const float4 v = *reinterpret_cast<const float4*>(mine + (e >> 3) * 4 * U + 128 + 4 * (e & 7));
+                            rec_r[0] = v.x; rec_r[1] = v.y; rec_r[2] = v.z; rec_r[3] = v.w;
+                        }
+                    }
+                } else if ((st & 4u) && ok) {
+                    const unsigned long long* mine = rec_at(1);
+                    ok = cl_read_stamped<NS>(mine + e, (uint32_t)(4 * U), u < U ? live : 0u, updates, rec, &p.ctrl->abort,
+                                             mine + (e >> 3) * 4 * U + 128 + 4 * (e & 7), want_r, rec_r);
+                }
+            }
+            if (l == 1) {
+                if (ok) ok = cl_wait(&bar_acc_g, (st >> 1) & 1u);
+                if (has_rem && ok) ok = cl_wait(&bar_acc_r, (st >> 1) & 1u);
+            }
             tc_fence_after();
             {
                 float x[8];
-                tmem_ld8(tm_g + lane_off, x);
+                if (NL == 1 || l == 1) tmem_ld8(tm_g + lane_off, x);
+                if (NL == 2) {
+                    const float bias = l == 1 && u < U ? reinterpret_cast<const float*>(smem + L.b_gate)[e] : 0.f;
+#pragma unroll
+                    for (int s = 0; s < NS; ++s) {
+                        const float rs = (fresh >> s) & 1u ? 0.f : rec[s];
+                        if (l == 0) x[s] = rs;
+                        else add[s] = rs + bias;
+                    }
+                }
 #pragma unroll
                 for (int s = 0; s < 8; ++s) {
-                    if (s < NS) x[s] = fmaf(tanh_fast((((fresh >> s) & 1u ? 0.f : x[s]) + add[s]) * sc), sc, of);
+                    if (s < NS) x[s] = fmaf(tanh_fast(((NL == 1 && ((fresh >> s) & 1u) ? 0.f : x[s]) + add[s]) * sc), sc, of);
                     else x[s] = 0.f;
                 }
                 // lane 4 u + g holds gate g of all slots; it is to hold the four gates of slots 2 g and 2 g + 1
@@ -317,46 +588,75 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                     if (up2) { float t = own; own = g2; g2 = t; t = g1; g1 = g3; g3 = t; }
                     const float gi = own, gf = g1, gg = g2, go = g3;
                     const int s = 2 * g + k;
-                    if (u < U && s < NU) {
-                        if ((live >> s) & 1u) {
-                            const float cold = (fresh >> s) & 1u ? 0.f : c_st[k];
-                            const float cc = cell_update(gf, cold, gi, gg);
-                            c_st[k] = cc;
-                            h_st[k] = __float2bfloat16_rn(go * tanh_fast(cc));
-                        }
-                        hst[s * U + u] = h_st[k];
+                    if (u < U && s < NU && ((live >> s) & 1u)) {
+                        if constexpr (NL == 2) c_st[k] = c_mem[k * 128];
+                        const float cold = (fresh >> s) & 1u ? 0.f : c_st[k];
+                        const float cc = cell_update(gf, cold, gi, gg);
+                        c_st[k] = cc;
+                        if constexpr (NL == 2) c_mem[k * 128] = cc;
+                        hst[s * U + u] = __float2bfloat16_rn(go * tanh_fast(cc));
                     }
                 }
             }
             if (rem_on) {
                 const int s = e >> 3;
                 if ((live >> s) & 1u) {
-                    float4 x = *reinterpret_cast<const float4*>(gr + s * CL_GR_PITCH + 4 * (e & 7));
-                    if ((fresh >> s) & 1u) x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
+                    if (NL == 1 || l == 1) x = *reinterpret_cast<const float4*>(gr + s * CL_GR_PITCH + 4 * (e & 7));
+                    if (NL == 2) {
+                        if ((fresh >> s) & 1u) rec_r[0] = rec_r[1] = rec_r[2] = rec_r[3] = 0.f;
+                        if (l == 0) x = make_float4(rec_r[0], rec_r[1], rec_r[2], rec_r[3]);
+                        else {
+                            const float4 bias = *reinterpret_cast<const float4*>(smem + L.b_gate + 512 + 16 * (e & 7));
+                            add_r[0] = rec_r[0] + bias.x; add_r[1] = rec_r[1] + bias.y; add_r[2] = rec_r[2] + bias.z; add_r[3] = rec_r[3] + bias.w;
+                        }
+                    } else if ((fresh >> s) & 1u) x = make_float4(0.f, 0.f, 0.f, 0.f);
                     const float gi = fmaf(tanh_fast((x.x + add_r[0]) * 0.5f), 0.5f, 0.5f);
                     const float gf = fmaf(tanh_fast((x.y + add_r[1]) * 0.5f), 0.5f, 0.5f);
                     const float gg = fmaf(tanh_fast((x.z + add_r[2]) * 1.f), 1.f, 0.f);
                     const float go = fmaf(tanh_fast((x.w + add_r[3]) * 0.5f), 0.5f, 0.5f);
+                    if constexpr (NL == 2) c_rem = c_mem[2 * 128];
                     const float cold = (fresh >> s) & 1u ? 0.f : c_rem;
                     const float cc = cell_update(gf, cold, gi, gg);
                     c_rem = cc;
-                    h_rem = __float2bfloat16_rn(go * tanh_fast(cc));
+                    if constexpr (NL == 2) c_mem[2 * 128] = cc;
+                    hst[s * U + 32 + (e & 7)] = __float2bfloat16_rn(go * tanh_fast(cc));
                 }
-                hst[s * U + 32 + (e & 7)] = h_rem;
             }
             tc_fence_before();
             }
-            if (group_barrier_or<128>(1, !ok || idle)) break;
+            if (group_barrier_or<128>(1, !ok || idle)) { leave = true; break; }
             // h to all CTAs
+            const uint32_t h_from = NL == 2 ? (uint32_t)(l * CL_SLOTS * U) * 2u : 0u, h_to = NL == 2 && l == 0 ? L.h0 - L.h : 0u;
+            const uint32_t h_bar = NL == 2 && l == 0 ? smem_u32(&bar_h0) : smem_u32(&bar_h);
 #pragma unroll
             for (int k = 0; k < 2; ++k)
                 if (h_first + 32 * k < h_pieces && ((live >> (h_src[k] >> 24)) & 1u)) {
-                    const uint4 piece = *reinterpret_cast<const uint4*>(smem + (h_src[k] & 0xFFFFFFu));
+                    const uint4 piece = *reinterpret_cast<const uint4*>(smem + (h_src[k] & 0xFFFFFFu) + h_from);
                     for (int d0 = warp * (32 >> lpd_shift) + (lane >> lpd_shift); d0 < CL_SIZE; d0 += 128 >> lpd_shift) {
                         const uint32_t d = (uint32_t)(d0 + r) & (CL_SIZE - 1);
-                        st_async_16(cl_map(sbase, d) + h_dst[k], piece, cl_map(smem_u32(&bar_h), d));
+                        st_async_16(cl_map(sbase, d) + h_dst[k] + h_to, piece, cl_map(h_bar, d));
                     }
                 }
+            if constexpr (NL == 2) {
+                if (live == 0u) break;
+                // and, for the next step's recurrent term, to the cluster that has the layer's W_hh
+                if (warp == 3) {
+#pragma unroll
+                    for (int k = 0; k < 2; ++k)
+                        if (lane == h_first && h_first + 32 * k < h_pieces) {
+                            const uint32_t off = h_src[k] & 0xFFFFFFu, s = h_src[k] >> 24;
+                            const uint32_t row = (uint32_t)((cluster * 2 + l) * 2 + (int)((st >> 1) & 1u)) * 8u + s;
+                            *reinterpret_cast<uint4*>(p.hx + (size_t)row * p.P + r * U + ((off - L.hst) / 2u - s * (uint32_t)U)) = *reinterpret_cast<const uint4*>(smem + off + h_from);
+                        }
+                    fence_proxy_async_all();
+                    __syncwarp();
+                    if (lane == 0) red_release_add(p.req + l * CL_DECODERS + cluster, 1u);
+                }
+            }
+            }
+            if (leave) break;
+            if (live != 0u) { st = (st ^ 2u) | 4u; ++updates; }
             lap(1);
             // ---- the joint's operand z = act(enc_proj + pred_proj), in place ----
             if (ok) ok = cl_wait(&bar_enc, par);
@@ -370,7 +670,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         if (timed) {
             p.ctrl->active = 0;
             p.ctrl->loop_kernel = WIND_LOOP_CLUSTERS;
-            for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = cyc[k];
+            for (int k = 0; k < 3; ++k) p.ctrl->phase_cycles[k] = s_lap[k];
             p.ctrl->loop_ns = (long long)(globaltimer_ns() - ns0);
         }
     } else if (warp < 10) {
@@ -418,7 +718,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (half) *part = make_float4(acc[0], acc[1], acc[2], acc[3]);
             }
             if (group_barrier_or<192>(2, !ok || idle)) break;
-            if (lane == 0 && live != 0u) mbar_arrive(&bar_sync_mma);
+            if (NL == 1 && lane == 0 && live != 0u) mbar_arrive(&bar_sync_mma);
             if (half == 0 && mine && live != 0u) {
                 // the two K halves are added as loop_kernel adds its accumulators
                 const float4 o = *part;
@@ -469,44 +769,71 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     } else if (warp < 14) {
         // =====================================================================================
         // remainder units 32..: W_hh rows of units 32 + 2 k, + 1 (4 gates each: row 4 (u - 32) + gate) in warp 10 + k, one chain
-        // over all of K (as the gates' accumulator in loop_kernel), [slot, row] = h W_hh^T
+        // over all of K (as the gates' accumulator in loop_kernel), [slot, row] = h W_hh^T.  Two layers: W_ih of the second one, and
+        // behind the joint's operand these warps fetch the first layer's recurrent term, which the update of the next step begins with
+        // (fetched there it cost 600 to 1000 cycles; the second layer's is fetched under the product with the first one's new state)
         // =====================================================================================
-        if (has_rem) {
+        if (rem_warps) {
+            uint32_t updates = 0u;
             const int row = 8 * (warp - 10) + (lane >> 2), u = 32 + (row >> 2), g = row & 3;
             uint32_t wf[40][2];
-            const uint32_t* src = reinterpret_cast<const uint32_t*>(p.w_hh + ((size_t)g * p.P + r * U + min(u, U - 1)) * p.P) + (lane & 3);
+            const uint32_t* src = reinterpret_cast<const uint32_t*>(p.w_gate + ((size_t)g * p.P + r * U + min(u, U - 1)) * p.P) + (lane & 3);
 #pragma unroll
             for (int s0 = 0; s0 < 40; s0 += 8)
                 if (s0 < p.P / 16)
 #pragma unroll
                     for (int s = s0; s < s0 + 8; ++s) { wf[s][0] = src[s * 8]; wf[s][1] = src[s * 8 + 4]; }
+            const uint32_t back = NL == 2 ? L.h - L.h0 : 0u;             // two layers: the first one's state
             for (uint32_t st = 0u;; st ^= 1u) {          // bit 0: parity of the step, bit 1: of the updates so far
                 const uint32_t par = st & 1u;
                 ok = cl_wait_warp(&bar_dec, par);
                 if (all_idle() || !ok) break;
-                if (live_slots() != 0u) {
-                st ^= 2u;
-                ok = cl_wait_warp(&bar_h, (~st >> 1) & 1u);
+                const bool update = live_slots() != 0u;
+                if (update) st ^= 2u;
+                if (update && has_rem) {
+                ok = cl_wait_warp(NL == 2 ? &bar_h0 : &bar_h, (~st >> 1) & 1u);
                 if (!ok) break;
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
                 uint32_t a[2][4];
-                ldmatrix_x4(a[0], h_at(0));
+                ldmatrix_x4(a[0], h_at(0) - back);
 #pragma unroll
                 for (int s0 = 0; s0 < 40; s0 += 8)
                     if (s0 < p.P / 16)
 #pragma unroll
                         for (int s = s0; s < s0 + 8; s += 2) {
-                            ldmatrix_x4(a[(s / 2 + 1) & 1], h_at(s / 2 + 1));
+                            ldmatrix_x4(a[(s / 2 + 1) & 1], h_at(s / 2 + 1) - back);
                             mma_16816(acc, a[(s / 2) & 1][0], 0u, a[(s / 2) & 1][1], 0u, wf[s][0], wf[s][1]);
                             mma_16816(acc, a[(s / 2) & 1][2], 0u, a[(s / 2) & 1][3], 0u, wf[s + 1][0], wf[s + 1][1]);
                         }
                 *reinterpret_cast<float2*>(gr + (lane >> 2) * CL_GR_PITCH + (warp - 10) * 8 + (lane & 3) * 2) = make_float2(acc[0], acc[1]);
                 __syncwarp();
-                if (lane == 0) { mbar_arrive(&bar_acc_r); mbar_arrive(&bar_sync_mma); }
+                if (lane == 0) {
+                    mbar_arrive(&bar_acc_r);
+                    if constexpr (NL == 1) mbar_arrive(&bar_sync_mma);
+                }
                 }
                 ok = cl_wait_warp(&bar_enc, par) && cl_wait_warp(&bar_pred, (~st >> 1) & 1u);
                 if (!ok) break;
                 build_z(std::integral_constant<int, 1>{});
+                if constexpr (NL == 2) {
+                    if (update) {
+                        constexpr int AT_ONCE = NS <= 2 ? 3 : 5;
+                        const unsigned long long* src = rec_at(0);
+                        float* dst = reinterpret_cast<float*>(smem + L.rec);
+                        ++updates;
+                        for (int i = (int)threadIdx.x - 320; ok && i - lane < NU * 4 * U; i += 128 * AT_ONCE) {
+                            const int n_at = (NU * 4 * U - i + 127) >> 7;             // values of this thread's from i on (may be below 1)
+                            float v[AT_ONCE];
+                            ok = cl_read_stamped<AT_ONCE>(src + i, 128u, n_at >= AT_ONCE ? (1u << AT_ONCE) - 1u : (1u << max(n_at, 0)) - 1u, updates, v, &p.ctrl->abort);
+#pragma unroll
+                            for (int k = 0; k < AT_ONCE; ++k)
+                                if (k < n_at) dst[i + 128 * k] = v[k];
+                        }
+                        __syncwarp();
+                        if (!ok) break;
+                        if (lane == 0) mbar_arrive(&bar_rec);
+                    }
+                }
             }
         }
     } else if (warp == 14) {
@@ -535,12 +862,16 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (update) {
                     // mma.sync and tcgen05.mma exclude each other on the tensor cores: the short chains go first (when they are
                     // done, all of h is there as well)
-                    if (!(ok = cl_wait(&bar_sync_mma, n_g & 1u))) break;
+                    if constexpr (NL == 1) {
+                        if (!(ok = cl_wait(&bar_sync_mma, n_g & 1u))) break;
+                    } else if (!(ok = cl_wait(&bar_h0, n_g & 1u))) {
+                        break;
+                    }
                     fence_proxy_async_all();             // h came in through remote generic stores
                     tc_fence_after();
-                    uint64_t hd = smem_desc_sw128(sbase + L.h);
+                    uint64_t hd = smem_desc_sw128(sbase + (NL == 2 ? L.h0 : L.h));
 #pragma unroll 1
-                    for (int kb = 0; kb < kb_p; ++kb, hd += 2048 >> 4)
+                    for (int kb = 0; kb < kb_p; ++kb, hd += H_BLOCK >> 4)
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             tc_mma_bf16_ts(tm_g, tmem + (uint32_t)(kb * 32 + k * 8), hd + (uint64_t)(k * 2), id_g, (kb | k) != 0);
@@ -650,6 +981,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             announce(done ? p.blank : (emit ? lab : -1), done, par ^ 1u);          // what the step decided is recorded behind the answer
             const uint32_t bad = __ballot_sync(0xffffffffu, lane < n && lane <= first && broken);   // rows after the first non-blank one do not count
             n_rows += (unsigned)n; n_tok += emit; n_forced += forced;
+            if (NL == 2 && r == 0 && (step & 1023u) == 1023u && lane == 0) st_relaxed_u32(p.beat + cluster, step);
             if (lane == 0 && utt >= 0) {
                 s_hist[first] += 1;
                 if (emit) {
@@ -677,7 +1009,14 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
         tc_fence_after();
         tmem_dealloc(tmem, LOOP_TMEM_COLS);
     }
-    if (threadIdx.x == 0 && s_abort) { note_timeout(p.ctrl, 49 + s_abort, blockIdx.x); set_status(p.ctrl, WIND_ERR_TIMEOUT); }
+    if (threadIdx.x == 0) {
+        if (s_abort) {
+            note_timeout(p.ctrl, 49 + s_abort, blockIdx.x);
+            set_status(p.ctrl, WIND_ERR_TIMEOUT);
+            if constexpr (NL == 2) atomicExch(&p.ctrl->abort, 1);
+        }
+        if constexpr (NL == 2) red_release_add(p.done + cluster, 1u);
+    }
     __syncwarp();
     cl_barrier();                                        // no CTA leaves while another may still write into its shared memory
 }
@@ -764,17 +1103,27 @@ __global__ void __launch_bounds__(256) cl_choose_kernel(Ctrl* ctrl, const int32_
 static std::mutex g_cl_mutex;
 static int g_cl_clusters[64];          // per device: 0 not asked yet, -1 none, else clusters of 16 that are resident at a time
 
-template <int ACT>
+template <int ACT, int NL>
 static const void* cl_fn_act(int ns) {
     switch (ns) {
-        case 1: return (const void*)cl_kernel<1, ACT>;
-        case 2: return (const void*)cl_kernel<2, ACT>;
-        case 4: return (const void*)cl_kernel<4, ACT>;
-        default: return (const void*)cl_kernel<8, ACT>;
+        case 1: return (const void*)cl_kernel<1, ACT, NL>;
+        case 2: return (const void*)cl_kernel<2, ACT, NL>;
+        case 4: return (const void*)cl_kernel<4, ACT, NL>;
+        default: return (const void*)cl_kernel<8, ACT, NL>;
     }
 }
-static const void* cl_fn(int ns, int act) { return act == WIND_ACT_RELU ? cl_fn_act<WIND_ACT_RELU>(ns) : cl_fn_act<WIND_ACT_TANH>(ns); }
-static uint32_t cl_smem_bytes(int P, int H, int NV, int slots, int wp) { return cl_smem_layout(P, H, NV, slots, wp).total + 1024u; }
+static const void* cl_fn(int ns, int act, int layers) {
+    if (layers == 2) return act == WIND_ACT_RELU ? cl_fn_act<WIND_ACT_RELU, 2>(ns) : cl_fn_act<WIND_ACT_TANH, 2>(ns);
+    return act == WIND_ACT_RELU ? cl_fn_act<WIND_ACT_RELU, 1>(ns) : cl_fn_act<WIND_ACT_TANH, 1>(ns);
+}
+static uint32_t cl_smem_bytes(int P, int H, int NV, int slots, int wp, int layers) {
+    uint32_t bytes = cl_smem_layout(P, H, NV, slots, wp, layers).total;
+    if (layers == 2) {                                   // the CTAs of cl_recurrent: what its MMAs and its last ldmatrix may read
+        const uint32_t states = (uint32_t)((CL_DECODERS + 1) & ~1) * (uint32_t)P * 16u + 1024u;
+        if (bytes < states) bytes = states;
+    }
+    return bytes + 1024u;
+}
 
 // clusters of 16 CTAs the current device holds at a time (one CTA per SM); 0: none
 static int cl_clusters() {
@@ -785,14 +1134,16 @@ static int cl_clusters() {
         g_cl_clusters[dev] = -1;
         int optin = 0;
         if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-        const int want = (int)cl_smem_bytes(CL_MAX_DIM, CL_MAX_DIM, 16 * CL_MAX_LABELS, 2, 32);
+        const int want = (int)cl_smem_bytes(CL_MAX_DIM, CL_MAX_DIM, 16 * CL_MAX_LABELS, 8, 8, 2);
         if (want > optin - 1024) return 0;
-        for (int k = 0; k < 8; ++k)
-            if (cudaFuncSetAttribute(cl_fn(1 << (k & 3), k >> 2), cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
-                cudaFuncSetAttribute(cl_fn(1 << (k & 3), k >> 2), cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
+        for (int k = 0; k < 16; ++k) {
+            const void* fn = cl_fn(1 << (k & 3), k >> 2 & 1, 1 + (k >> 3));
+            if (cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
+                cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, want) != cudaSuccess) {
                 cudaGetLastError();
                 return 0;
             }
+        }
         cudaLaunchConfig_t cfg{};
         cfg.gridDim = dim3(CL_SIZE);
         cfg.blockDim = dim3(CL_THREADS);
@@ -803,7 +1154,7 @@ static int cl_clusters() {
         cfg.attrs = at;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, cl_fn(8, WIND_ACT_RELU), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
+        if (cudaOccupancyMaxActiveClusters(&n, cl_fn(8, WIND_ACT_RELU, 2), &cfg) != cudaSuccess) { cudaGetLastError(); n = 0; }
         if (n > 0) g_cl_clusters[dev] = n;
     }
     return g_cl_clusters[dev] > 0 ? g_cl_clusters[dev] : 0;
@@ -814,14 +1165,17 @@ static int cl_clusters() {
 // 3, 8 and 8 % rms.  Chosen by these, a decode takes 0.7 % longer than by the better kernel of each pair on the average; with a
 // constant ratio, 2.1 and 3.2 for windows of 8 and 16 rows, and clusters alone beyond that or for up to 64 utterances, it took 11 %
 // (64 utterances of 120 frames at W = 32: 1.53 ms against 1.32; 128: 2.84 against 1.79; 64 at W = 24, P = H = 384: 1.31 against 0.89).
+// Two layers: 112 pairs (P and H 256 and 640, W = 1 to 32, up to 128 utterances), 8 and 6 % rms in clusters, 8 % for grid barriers.
 static float cl_step_us(const wind_model_t& m, int W, int wp) {
     const float P = (float)m.P, H = (float)m.H, z = m.act == WIND_ACT_RELU ? 0.f : 0.0018f * H;
+    if (m.L == 2) return z + (wp == 8 ? 5.6f + 0.0085f * P + (0.0044f * (float)W / 8.f - 0.004f) * H : 5.2f + 0.0073f * P + 0.0015f * H);
     return z + (wp == 8 ? 4.3f + 0.0013f * P + (0.0009f + 0.0026f * (float)W / 8.f) * H : 4.25f + 0.0009f * P + 0.0028f * H);
 }
 static float other_step_us(const wind_model_t& m, const LoopPlan& pl, int B, int W) {
     const float P = (float)m.P, H = (float)m.H, rows = (float)B * (float)W;
     if (!pl.resident) return -2.5f + 3.8f * (float)pl.mt_count + 0.0053f * rows + 0.0177f * P + 0.0145f * H;
     const int waves = (pl.rg_count + pl.rg_stride - 1) / pl.rg_stride;
+    if (m.L == 2) return 12.3f + 0.0009f * H + 0.0043f * P + 0.0045f * rows + 0.018f * (float)B;
     return 10.1f + 0.005f * H + 0.002f * rows + (pl.dataflow ? 6.5f : 3.f) * (float)(waves - 1);
 }
 
@@ -831,12 +1185,23 @@ static float other_step_us(const wind_model_t& m, const LoopPlan& pl, int B, int
 static bool cl_supported(const Call& c) {
     const wind_model_t& m = c.m;
     const int nv = m.V + 1;
-    if (m.L != 1 || m.P % 128 || m.H % 128 || m.P > CL_MAX_DIM || m.H > CL_MAX_DIM || c.W > 32) return false;
+    if (m.L > 2 || m.P % 128 || m.H % 128 || m.P > CL_MAX_DIM || m.H > CL_MAX_DIM || c.W > 32) return false;
     if (cl_label_base(nv) + (cl_label_extra(nv) > 0 ? 8 : 0) > CL_MAX_LABELS) return false;
     if (c.mode != WIND_MODE_FIRST_NONBLANK || c.joint_iters > 0) return false;
     const LoopOptions o = loop_get_options();
     if (!o.resident || o.dataflow >= 0 || o.joint_placement >= 0) return false;
     return cl_clusters() > 0;
+}
+
+// Two layers: what the clusters hand one another lies in the workspace from the plain-ALU path's state (behind the utterances' order)
+// to the gate table: regions of other kernels, and where they are too small (few batch rows, H far below P) the other kernel decodes.
+struct ClExchange { size_t hx, rx, end; };
+static ClExchange cl_exchange(const Call& c, int n, int clusters, int slots) {
+    ClExchange x{};
+    x.hx = c.lay.h + align_up(sizeof(int32_t) * (size_t)n);
+    x.rx = align_up(x.hx + sizeof(__nv_bfloat16) * (size_t)clusters * 4 * 8 * c.m.P);
+    x.end = x.rx + sizeof(unsigned long long) * (size_t)clusters * 2 * slots * 4 * c.m.P;
+    return x;
 }
 
 // How a decode runs in clusters; false: it does not.  `other` is the plan by which another kernel could take it.
@@ -846,7 +1211,8 @@ static bool cl_supported(const Call& c) {
 // alone decide, for lengths whose mean is 0.6 of the longest, or rows that are refilled throughout.
 bool cl_plan(const Call& c, const LoopPlan& other, ClPlan* out) {
     if (!cl_supported(c)) return false;
-    const int n = c.N > 0 ? c.N : c.B, avail = cl_clusters();
+    const int n = c.N > 0 ? c.N : c.B, avail = c.m.L == 2 ? (cl_clusters() - 2 < CL_DECODERS ? cl_clusters() - 2 : CL_DECODERS) : cl_clusters();
+    if (avail < 1) return false;
     ClPlan q{};
     q.wp = c.W <= 8 ? 8 : (c.W <= 16 ? 16 : 32);
     // one slot per cluster as long as there are clusters, then more slots (a lock step of eight slots costs less than two of one)
@@ -854,6 +1220,10 @@ bool cl_plan(const Call& c, const LoopPlan& other, ClPlan* out) {
     q.clusters = n < avail ? n : avail;
     q.slots = (n + q.clusters - 1) / q.clusters < most ? (n + q.clusters - 1) / q.clusters : most;
     const int slots = q.slots * q.clusters;
+    // two layers: only where the other kernel has its weights on the chip (the same roundings); the clusters exchange states and
+    // recurrent terms in the regions of the other kernels' states
+    if (c.m.L == 2 && !other.resident) return false;
+    if (c.m.L == 2 && cl_exchange(c, n, q.clusters, q.slots).end > c.lay.g0) return false;
     q.rows = c.B < n ? c.B : n;
     q.cl_us = cl_step_us(c.m, c.W, q.wp);
     q.other_us = other_step_us(c.m, other, c.B, c.W);
@@ -877,6 +1247,7 @@ cudaError_t cl_loop(const Call& c, const ClPlan& q) {
     p.wp = q.wp;
     p.slots = q.slots;
     p.choose = q.choose;
+    p.smem = cl_smem_layout(m.P, m.H, p.NV, p.slots, p.wp, m.L);
     const int ns = p.slots <= 1 ? 1 : (p.slots <= 2 ? 2 : (p.slots <= 4 ? 4 : 8));
     p.queue_base = n < c.B ? n : c.B;
     long long cap = (long long)c.T * (c.S + 1) + 2;
@@ -885,7 +1256,7 @@ cudaError_t cl_loop(const Call& c, const ClPlan& q) {
     p.extra_arrivals = loop_extra_arrivals();
     p.enc_len = c.enc_len;
     p.g0 = c.g0();
-    p.w_hh = (const __nv_bfloat16*)c.w_hh[0]; p.w_pred = (const __nv_bfloat16*)m.w_pred; p.w_out = (const __nv_bfloat16*)m.w_out;
+    p.w_gate = (const __nv_bfloat16*)(m.L == 2 ? c.w_ih[1] : c.w_hh[0]); p.w_pred = (const __nv_bfloat16*)m.w_pred; p.w_out = (const __nv_bfloat16*)m.w_out;
     p.b_pred = m.b_pred; p.b_out = m.b_out;
     p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
     if (q.order) {
@@ -900,21 +1271,33 @@ cudaError_t cl_loop(const Call& c, const ClPlan& q) {
         cudaError_t e = cudaGetLastError();
         if (e != cudaSuccess) return e;
     }
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)(q.clusters * CL_SIZE));
-    cfg.blockDim = dim3(CL_THREADS);
-    cfg.dynamicSmemBytes = cl_smem_bytes(m.P, m.H, p.NV, p.slots, p.wp);
-    cfg.stream = c.stream;
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeClusterDimension;
-    at[0].val.clusterDim.x = CL_SIZE; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    CUtensorMap enc_map;
+    CUtensorMap enc_map, hx_map;
     cudaError_t e = loop_map3(&enc_map, c.enc_proj(), (uint64_t)n * c.T, m.H, 8);
     if (e != cudaSuccess) return e;
-    void* args[2] = {(void*)&enc_map, (void*)&p};
-    return cudaLaunchKernelExC(&cfg, cl_fn(ns, m.act), args);
+    hx_map = enc_map;
+    if (m.L == 2) {
+        const ClExchange x = cl_exchange(c, n, q.clusters, q.slots);
+        for (int l = 0; l < 2; ++l) p.w_rec[l] = (const __nv_bfloat16*)c.w_hh[l];
+        p.b_gate[0] = c.b_ih[1]; p.b_gate[1] = c.b_hh[1];
+        p.req = c.flags(); p.done = p.req + 2 * CL_DECODERS; p.beat = p.done + CL_DECODERS;   // (23 counters at the least)
+        p.hx = reinterpret_cast<__nv_bfloat16*>(c.ws + x.hx);
+        p.rx = reinterpret_cast<unsigned long long*>(c.ws + x.rx);
+        if ((e = loop_map3(&hx_map, p.hx, (uint64_t)q.clusters * 32, m.P, 8)) != cudaSuccess) return e;
+    }
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)((q.clusters + (m.L == 2 ? 2 : 0)) * CL_SIZE));
+    cfg.blockDim = dim3(CL_THREADS);
+    cfg.dynamicSmemBytes = cl_smem_bytes(m.P, m.H, p.NV, p.slots, p.wp, m.L);
+    cfg.stream = c.stream;
+    cudaLaunchAttribute at[2];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = CL_SIZE; at[0].val.clusterDim.y = 1; at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeCooperative;           // two layers: clusters wait for one another, so all have to be resident
+    at[1].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = m.L == 2 ? 2 : 1;
+    void* args[3] = {(void*)&enc_map, (void*)&hx_map, (void*)&p};
+    return cudaLaunchKernelExC(&cfg, cl_fn(ns, m.act, m.L), args);
 }
 
 }  // namespace wind

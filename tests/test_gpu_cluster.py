@@ -50,3 +50,52 @@ def test_remainder_units_round_like_the_others(pkg, seed, N, T, H, V, W, S):  # 
     want = pkg.decode(model, enc, lens, W, S)
     for a, b in zip(got[:3], want[:3]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("N,T,P,H,V,act,W,S", [
+    (1, 40, 128, 128, 127, 0, 1, 3),       # smallest dimensions, one decoding cluster
+    (6, 60, 640, 640, 1024, 0, 4, 10),     # remainder units; two slots in some clusters, one in others
+    (13, 30, 512, 640, 1151, 1, 8, 2),     # no remainder units; 72 labels in every CTA; three slots
+    (33, 20, 640, 128, 130, 0, 1, 3),      # states that need more shared memory than the decoding CTAs (P far above H)
+    (9, 30, 640, 128, 300, 0, 16, 2),      # padded window of 16
+    (40, 24, 640, 640, 1024, 0, 8, 3),     # all forty slots
+    (64, 30, 640, 640, 1024, 0, 8, 10),    # more utterances than slots: the queue, or the other kernel, as the lengths have it
+    (60, 16, 256, 384, 1000, 1, 5, 3),
+    (25, 20, 384, 256, 200, 0, 32, 3),     # widest window: ten slots, refilled
+    (50, 1, 640, 640, 200, 0, 2, 1),       # utterances of one frame: every update starts afresh
+])
+def test_two_layer_cluster_edges(pkg, N, T, P, H, V, act, W, S):  # noqa: F811
+    w, enc, lens = ragged_case(1300 + N + W, B=N, T=T, D=64, E=64, P=P, L=2, H=H, V=V, act=act,
+                               blank_id=0 if N % 2 else None, bias=1.5, dtype="bf16")
+    rep, out = check_against_oracle(pkg, w, enc, lens, W, S, kernels=2)
+    set_loop_mode(pkg, "barriers")
+    tok, frm, olen, stats, st = pkg.decode(pkg.WindModel(w), enc, lens, W, S)
+    assert st == 0 and stats["tokens"] == rep["stats"]["tokens"] and stats["jump_hist"] == rep["stats"]["jump_hist"]
+    for a, b in zip((tok, frm, olen), out):
+        assert np.array_equal(a, b)
+
+
+def test_two_layer_rows_refilled_in_clusters(pkg):  # noqa: F811
+    N, T, B, W, S = 150, 14, 32, 4, 3
+    w, enc, lens = ragged_case(1400, B=N, T=T, D=64, E=64, P=256, L=2, H=384, V=300, act=0, bias=2.0, dtype="bf16")
+    enc = np.nan_to_num(enc)
+    model = pkg.WindModel(w)
+    got = pkg.decode_refill(model, enc, lens, B, W, S)
+    set_loop_mode(pkg, "barriers")
+    want = pkg.decode_refill(model, enc, lens, B, W, S)
+    for a, b in zip(got[:3], want[:3]):
+        assert np.array_equal(a, b)
+
+
+def test_two_layer_decode_repeated(pkg):  # noqa: F811
+    # Small dimensions make short steps and few updates: the recurrent terms' answers come several steps late, over and over.
+    w, enc, lens = ragged_case(2402, B=6, T=30, D=64, E=64, P=128, L=2, H=128, V=200, bias=3.0, dtype="bf16")
+    enc = np.nan_to_num(enc)
+    model = pkg.WindModel(w)
+    set_loop_mode(pkg, "barriers")
+    want = pkg.decode(model, enc, lens, 8, 3)
+    pkg.wind_set_loop_options()
+    for _ in range(60):
+        got = pkg.decode(model, enc, lens, 8, 3)
+        for a, b in zip(got[:3], want[:3]):
+            assert np.array_equal(a, b)

@@ -15,6 +15,7 @@ pytestmark = pytest.mark.gpu
     ("CLUSTERS", "bf16", 3, 30, 64, 128, 1, 128, 200, 8, range(50, 66)),      # one slot per cluster
     ("CLUSTERS", "bf16", 60, 30, 64, 640, 1, 640, 200, 8, range(50, 66)),     # eight slots, remainder units, queue
     ("CLUSTERS", "bf16", 128, 40, 64, 256, 1, 256, 200, 32, range(50, 66)),   # the other kernel launched behind them
+    ("CLUSTERS", "bf16", 9, 30, 64, 640, 2, 256, 200, 8, range(50, 72)),      # two layers: the recurrent terms' clusters leave too
     ("WIDE", "bf16", 5, 30, 64, 192, 1, 1024, 600, 8, (3, 4)),
     ("GRID", "f32", 4, 24, 160, 320, 1, 300, 500, 8, (5,)),
 ])
