@@ -371,41 +371,37 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
     auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * H_BLOCK + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
 
-    // The joint's operand z = act(enc_proj + pred_proj), in place, by every warp that computes (0..13; it is bound by the shared
-    // memory's bandwidth: 30 KB per group of eight rows, 2110 cycles for eight groups).  Of a group the rows that count: three
-    // eighths of them to the four workers, the others to the W_pred and remainder warps, which have registers for one 16-byte piece
-    // at a time.  (Half to the workers, half to four W_pred warps: these took 4250 cycles for eight groups.)  Threads per row: a
-    // multiple of eight, one per 16-byte piece of a K block.
-    const int z_rows = p.wp == 8 ? p.W : 8, z_mine = warp < 4 ? (3 * z_rows + 4) / 8 : z_rows - (3 * z_rows + 4) / 8;
-    const int z_threads = warp < 4 ? 128 : (rem_warps ? 320 : 192), z_tid = warp < 4 ? (int)threadIdx.x : (int)threadIdx.x - 128;
-    const int z_tpr = (z_threads / max(z_mine, 1)) & ~7, z_at = z_tid / z_tpr;
-    const bool z_on = z_at < z_mine;
-    const int z_r = (warp < 4 ? 0 : z_rows - z_mine) + z_at, z_k0 = (z_tid % z_tpr) >> 3, z_kstep = z_tpr >> 3;
+    // The joint's operand z = act(enc_proj + pred_proj), in place, by every warp that computes (0..13).  It is bound by the shared
+    // memory's bandwidth, so a 16-byte piece of pred_proj is loaded once for several window rows: a unit of work is eight threads, a
+    // piece each of a K block, and p.z_rows of the rows of a group that count; units are dealt out evenly to all groups of eight threads.
+    // (Eight slots, W = 8: 22 KB per group of eight rows; with pred_proj loaded for every row and rows dealt out by role it was 30 KB:
+    // 128 utterances 9.04 -> 7.82 ms, 32 at W = 1 6.10 -> 5.54; one slot the same.)
+    const int z_rows = p.wp == 8 ? p.W : 8;
+    const int z_first = (int)(threadIdx.x >> 3) / kb_h << 8 | (int)(threadIdx.x >> 3) % kb_h;    // (group, part) << 8 | K block
     auto build_z = [&](auto which) {
-        constexpr int AT_ONCE = decltype(which)::value;               // pieces in flight per thread (the W_pred warps have registers for one)
-        if (z_on) {
-            uint8_t* zp = smem + L.z + (uint32_t)(z_r * 128 + (((lane & 7) ^ (z_r & 7)) << 4) + z_k0 * 1024);
-            const uint8_t* pp = smem + L.pred + (uint32_t)(z_k0 * 128 + (lane & 7) * 16);
+        constexpr int AT_ONCE = decltype(which)::value;               // rows in flight per thread (the W_pred warps have registers for one)
+        const uint32_t c = (uint32_t)(lane & 7);
 #pragma unroll 1
-            for (int gi = 0; gi < n_groups; ++gi, zp += p.H * 16) {
-                const uint8_t* py = pp + (uint32_t)(((gi << 3) >> wp_shift) * p.H * 2);
+        for (int at = z_first >> 8, kb = z_first & 255; at < n_groups << p.z_parts;) {
+            const int gi = at >> p.z_parts, r0 = (at & ((1 << p.z_parts) - 1)) * p.z_rows, r1 = min(r0 + p.z_rows, z_rows);
+            uint8_t* zp = smem + L.z + (uint32_t)(gi * p.H * 16 + kb * 1024);
+            const uint4 y = *reinterpret_cast<const uint4*>(smem + L.pred + (uint32_t)(((gi << 3) >> wp_shift) * p.H * 2 + kb * 128) + c * 16u);
 #pragma unroll 1
-                for (int j0 = 0; z_k0 + j0 * z_kstep < kb_h; j0 += AT_ONCE) {
-                    uint4 x[AT_ONCE], y[AT_ONCE];
+            for (int r = r0; r < r1; r += AT_ONCE) {
+                uint4 x[AT_ONCE];
 #pragma unroll
-                    for (int j = 0; j < AT_ONCE; ++j)
-                        if (z_k0 + (j0 + j) * z_kstep < kb_h) {
-                            x[j] = *reinterpret_cast<const uint4*>(zp + (j0 + j) * z_kstep * 1024);
-                            y[j] = *reinterpret_cast<const uint4*>(py + (j0 + j) * z_kstep * 128);
-                        }
+                for (int j = 0; j < AT_ONCE; ++j)
+                    if (j == 0 || r + j < r1) x[j] = *reinterpret_cast<const uint4*>(zp + (uint32_t)((r + j) * 128) + ((c ^ (uint32_t)(r + j)) << 4));
 #pragma unroll
-                    for (int j = 0; j < AT_ONCE; ++j)
-                        if (z_k0 + (j0 + j) * z_kstep < kb_h)
-                            *reinterpret_cast<uint4*>(zp + (j0 + j) * z_kstep * 1024) =
-                                make_uint4(act_add_bf16x2(x[j].x, y[j].x, ACT), act_add_bf16x2(x[j].y, y[j].y, ACT),
-                                           act_add_bf16x2(x[j].z, y[j].z, ACT), act_add_bf16x2(x[j].w, y[j].w, ACT));
-                }
+                for (int j = 0; j < AT_ONCE; ++j)
+                    if (j == 0 || r + j < r1)
+                        *reinterpret_cast<uint4*>(zp + (uint32_t)((r + j) * 128) + ((c ^ (uint32_t)(r + j)) << 4)) =
+                            make_uint4(act_add_bf16x2(x[j].x, y.x, ACT), act_add_bf16x2(x[j].y, y.y, ACT), act_add_bf16x2(x[j].z, y.z, ACT),
+                                       act_add_bf16x2(x[j].w, y.w, ACT));
             }
+            at += p.z_step >> 8;
+            kb += p.z_step & 255;
+            if (kb >= kb_h) { kb -= kb_h; ++at; }
         }
         fence_proxy_async();
         __syncwarp();
@@ -662,7 +658,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             if (ok) ok = cl_wait(&bar_enc, par);
             if (ok) ok = cl_wait(&bar_pred, (~st >> 1) & 1u);        // of the last update: this step's, or long there
             lap(2);
-            build_z(std::integral_constant<int, 2>{});
+            build_z(std::integral_constant<int, 4>{});
             if (ok) ok = cl_wait(&bar_acc_j, par);
             tc_fence_after();
             joint_argmax(std::integral_constant<int, 0>{});
@@ -1247,6 +1243,14 @@ cudaError_t cl_loop(const Call& c, const ClPlan& q) {
     p.wp = q.wp;
     p.slots = q.slots;
     p.choose = q.choose;
+    {
+        // units of the joint's operand: 448 threads (320 without warps 10-13) in eights; the fewer groups of rows, the fewer rows a unit
+        const int kb_h = m.H / 64, units = m.L == 2 || m.P / CL_SIZE > 32 ? 56 : 40, groups = p.slots * p.wp / 8, rows = p.wp == 8 ? p.W : 8;
+        p.z_parts = groups > 4 ? 1 : 2;
+        while ((1 << p.z_parts) > rows) --p.z_parts;
+        p.z_rows = (rows + (1 << p.z_parts) - 1) >> p.z_parts;
+        p.z_step = units / kb_h << 8 | units % kb_h;
+    }
     p.smem = cl_smem_layout(m.P, m.H, p.NV, p.slots, p.wp, m.L);
     const int ns = p.slots <= 1 ? 1 : (p.slots <= 2 ? 2 : (p.slots <= 4 ? 4 : 8));
     p.queue_base = n < c.B ? n : c.B;

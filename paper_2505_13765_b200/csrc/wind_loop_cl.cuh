@@ -35,6 +35,7 @@ struct ClParams {
     int queue_base;                    // value of ctrl->next_utt before the first utterance is taken from the queue
     int step_cap, extra_arrivals, choose;
     ClSmem smem;
+    int z_parts, z_rows, z_step;       // the joint's operand: log2 of the parts of a group of eight rows, rows of a part, (group, part) << 8 | K block from unit to unit
     const int32_t* order;              // [n_utt] order in which utterances are taken; null: 0, 1, ...
     const int32_t* enc_len;
     const float* g0;                   // [NV][4P]
