@@ -409,39 +409,46 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     };
 
     // Argmax of every window row over a share of this CTA's labels (HF), sent to the slots' owners.  With M = 64 accumulator row m
-    // lives in lane m % 16 of quadrant m / 16.
+    // lives in lane m % 16 of quadrant m / 16.  Read as 16 lanes x 256 bits, a thread holds a quarter of the columns of rows lane / 4 and
+    // lane / 4 + 8, so that all 32 threads have something to compare (a row a thread: 16 threads, four times the chain; 1008 -> 865
+    // cycles with eight slots, 995 -> 826 with one, of which a step keeps 195 and 33: the keys of the W_pred warps come last).
     auto joint_argmax = [&](auto which) {
         constexpr int HF = decltype(which)::value;
-        if (16 * q >= NU << wp_shift) return;                         // this warp's quadrant holds no window row
-        // CH columns at a time: their maximum, then the lowest label that has it (equal logits: the lower label)
-        constexpr int CH = HF ? 8 : 16;                                 // (the W_pred warps have registers for eight)
+        const int rows_here = (NU << wp_shift) - 16 * q;              // window rows of this warp's quadrant
+        if (rows_here <= 0) return;
+        constexpr int CH = HF ? 8 : 16;                                 // columns at a time (the W_pred warps have registers for eight)
         const int nh = (lab_n / 3) & ~7;                                // they take [0, nh), the workers [nh, lab_n)
-        float best = -INFINITY;
-        int lab = 0;
+        float best[2] = {-INFINITY, -INFINITY};
+        int lab[2] = {0, 0};
 #pragma unroll 1
         for (int c = HF ? 0 : nh; c < (HF ? nh : lab_n); c += CH) {
-            float v[CH];
-            if constexpr (CH == 16) tmem_ld16_sum(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
-            else tmem_ld8_sum(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
+            float v[CH / 2];                                            // of eight columns each: row lane / 4 twice, row lane / 4 + 8 twice
+            tmem_ld_quarter<CH / 8>(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
 #pragma unroll
-            for (int j = 0; j < CH; j += 4) {
-                const float4 b4 = *reinterpret_cast<const float4*>(s_bout + c + j);  // -inf behind the last label
-                v[j] += b4.x; v[j + 1] += b4.y; v[j + 2] += b4.z; v[j + 3] += b4.w;
+            for (int j = 0; j < CH / 8; ++j) {
+                const int at = c + 8 * j + 2 * (lane & 3);
+                const float2 b2 = *reinterpret_cast<const float2*>(s_bout + at);     // -inf behind the last label
+#pragma unroll
+                for (int k = 0; k < 2; ++k) {                           // equal logits: the lower label stays
+                    const float v0 = v[4 * j + 2 * k] + b2.x, v1 = v[4 * j + 2 * k + 1] + b2.y;
+                    if (v0 > best[k]) { best[k] = v0; lab[k] = at; }
+                    if (v1 > best[k]) { best[k] = v1; lab[k] = at + 1; }
+                }
             }
-            float m = v[0];
-#pragma unroll
-            for (int j = 1; j < CH; ++j) m = fmaxf(m, v[j]);
-            int at = CH;
-#pragma unroll
-            for (int j = CH - 1; j >= 0; --j) at = v[j] == m ? j : at;
-            if (m > best) { best = m; lab = c + at; }
         }
-        const int row = 16 * q + (lane & 15);
+        unsigned long long key[2];
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            key[k] = best[k] > -INFINITY ? pack_key(best[k], (uint32_t)(lab0 + lab[k])) : 0ull;
+            if (k == 0 || rows_here > 8) {
+                key[k] = max(key[k], __shfl_xor_sync(0xffffffffu, key[k], 1));
+                key[k] = max(key[k], __shfl_xor_sync(0xffffffffu, key[k], 2));
+            }
+        }
+        const int row = 16 * q + (lane >> 2) + 8 * (lane & 1);          // lanes 4 i: row i, 4 i + 1: row i + 8
         const int s = row >> wp_shift, w = row & (p.wp - 1);
-        if (lane < 16 && s < NU && w < p.W) {
-            const unsigned long long key = best > -INFINITY ? pack_key(best, (uint32_t)(lab0 + lab)) : 0ull;
-            st_async_8(cl_map(sbase + L.kbuf + (uint32_t)(w * CL_KEY_PITCH + 2 * r + HF) * 8u, s), key, cl_map(smem_u32(&bar_keys), s));
-        }
+        if ((lane & 2) == 0 && s < NU && w < p.W)
+            st_async_8(cl_map(sbase + L.kbuf + (uint32_t)(w * CL_KEY_PITCH + 2 * r + HF) * 8u, s), lane & 1 ? key[1] : key[0], cl_map(smem_u32(&bar_keys), s));
     };
 
     if (warp < 4) {

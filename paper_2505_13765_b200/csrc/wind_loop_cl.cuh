@@ -206,6 +206,32 @@ __device__ __forceinline__ bool cl_read_stamped(const unsigned long long* src, u
 // the same for a whole warp, with one answer for all its lanes
 __device__ __forceinline__ bool cl_wait_warp(uint64_t* bar, uint32_t parity) { return __all_sync(0xffffffffu, cl_wait(bar, parity)); }
 
+// Two accumulators of 16 rows (lanes) added, X times eight columns, rows spread over the warp as mma.sync spreads them: of columns
+// 8 x ..  v[4 x], v[4 x + 1]: row lane / 4, columns 2 (lane % 4), + 1;  v[4 x + 2], v[4 x + 3]: row lane / 4 + 8.
+template <int X>
+__device__ __forceinline__ void tmem_ld_quarter(uint32_t ta, uint32_t tb, float* v) {
+    uint32_t a[4 * X], b[4 * X];
+    if constexpr (X == 1) {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x1.b32 {%0,%1,%2,%3}, [%8];\n\t"
+            "tcgen05.ld.sync.aligned.16x256b.x1.b32 {%4,%5,%6,%7}, [%9];\n\t"
+            "tcgen05.wait::ld.sync.aligned;"
+            : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(b[0]), "=r"(b[1]), "=r"(b[2]), "=r"(b[3])
+            : "r"(ta), "r"(tb)
+            : "memory");
+    } else {
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%16];\n\t"
+            "tcgen05.ld.sync.aligned.16x256b.x2.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%17];\n\t"
+            "tcgen05.wait::ld.sync.aligned;"
+            : "=r"(a[0]), "=r"(a[1]), "=r"(a[2]), "=r"(a[3]), "=r"(a[4]), "=r"(a[5]), "=r"(a[6]), "=r"(a[7]), "=r"(b[0]), "=r"(b[1]),
+              "=r"(b[2]), "=r"(b[3]), "=r"(b[4]), "=r"(b[5]), "=r"(b[6]), "=r"(b[7])
+            : "r"(ta), "r"(tb)
+            : "memory");
+    }
+#pragma unroll
+    for (int i = 0; i < 4 * X; ++i) v[i] = __uint_as_float(a[i]) + __uint_as_float(b[i]);
+}
 __device__ __forceinline__ void ldmatrix_x4(uint32_t* r, uint32_t addr) {
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
