@@ -872,11 +872,277 @@ __global__ void __launch_bounds__(SL_THREADS, 1) simt_local_kernel(const SimtLoo
 }
 
 // ---------------------------------------------------------------------------
+// One-layer models of up to 64 units, joint units and labels: the same, with the weights in registers.
+//
+// A step of simt_local_kernel on the 64-unit model took 5300 cycles: 128 KB of gate weights through shared memory, seven block
+// barriers, and every phase's addresses worked out anew.  Here a thread keeps a gate row of W_hh (64 values), a quarter of a row of
+// W_pred and of W_out for the whole decode, W_ih and the embedding have become a table of all tokens' input terms in shared memory,
+// the four gates of a unit meet by shuffles, and every warp takes the decisions itself: three block barriers in a step that feeds a
+// token, two in one that does not.  What is left is issue slots, so few warps are better: with 16 a step takes 3650 cycles (and the
+// utterance of 44 steps 132 us in all).
+// ---------------------------------------------------------------------------
+constexpr int ST_MAX = 64;             // units, embedding, joint units, labels
+constexpr int ST_ROWS = 32;            // window rows
+constexpr int ST_THREADS = 4 * ST_MAX; // four threads a unit (its gates), a joint unit, a label (quarters of a row)
+constexpr int ST_WARPS = ST_THREADS / 32;
+
+// (ACT in the template: with both activations in the code, unrolled, its instructions do not fit the cache)
+template <typename TW, int ACT>
+__global__ void __launch_bounds__(ST_THREADS, 1) simt_tiny_kernel(const SimtLoopParams p) {
+    extern __shared__ __align__(16) float s_table[];               // [NV][4 unit + gate] W_ih emb + b_ih + b_hh
+    __shared__ __align__(16) float s_enc[2 * ST_ROWS * ST_MAX];    // enc_proj rows, a ring of 64: this window and the frames the next one may
+                                                                   // reach; before that the embedding
+    __shared__ __align__(16) float s_z[ACT == WIND_ACT_RELU ? 4 : ST_ROWS * ST_MAX];      // the joint's operand (ReLU: formed in registers)
+    __shared__ __align__(16) float s_h[2][ST_MAX];                 // [parity of the updates]
+    __shared__ __align__(16) float s_pred[ST_MAX];
+    __shared__ unsigned long long s_key[ST_WARPS][ST_ROWS];        // best key of a warp's eight labels per window row
+    __shared__ int s_hist[65];
+    if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int E = p.E, P = p.P, H = p.H, NV = p.NV;
+    const int item = tid >> 2, part = tid & 3;                     // unit and gate; joint unit or label, and quarter of its row
+    // n values of a row, 16 bytes at a time where rows allow it (element by element a matrix took 9 us); `in`: there is such a row
+    auto load_row = [](float* w, const void* m, size_t row, int n, bool in) {
+        constexpr int PIECE = 16 / (int)sizeof(TW);
+        const TW* src = static_cast<const TW*>(m) + row * n;
+        if (n % PIECE == 0 && reinterpret_cast<uintptr_t>(m) % 16 == 0) {
+#pragma unroll
+            for (int j = 0; j < ST_MAX; j += PIECE) {
+                const uint4 v = in && j < n ? __ldg(reinterpret_cast<const uint4*>(src + j)) : make_uint4(0, 0, 0, 0);
+                const uint32_t u[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int k = 0; k < 4; ++k)
+                    if constexpr (sizeof(TW) == 4) {
+                        w[j + k] = __uint_as_float(u[k]);
+                    } else {
+                        w[j + 2 * k] = __uint_as_float(u[k] << 16);
+                        w[j + 2 * k + 1] = __uint_as_float(u[k] & 0xffff0000u);
+                    }
+            }
+        } else {
+#pragma unroll
+            for (int j = 0; j < ST_MAX; ++j) w[j] = in && j < n ? (float)__ldg(src + j) : 0.f;
+        }
+    };
+    auto dot = [](const float* w, const float* x) {                // x in shared memory, the same for all threads
+        float a[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+        for (int j = 0; j < ST_MAX; j += 4) {
+            const float4 v = *reinterpret_cast<const float4*>(x + j);
+            a[0] = fmaf(w[j], v.x, a[0]); a[1] = fmaf(w[j + 1], v.y, a[1]); a[2] = fmaf(w[j + 2], v.z, a[2]); a[3] = fmaf(w[j + 3], v.w, a[3]);
+        }
+        return (a[0] + a[1]) + (a[2] + a[3]);
+    };
+
+    // ---- weights; table of the input terms ----
+    const size_t g_row = (size_t)part * P + min(item, P - 1);
+    float w[ST_MAX];
+    {
+        float e[ST_MAX * ST_MAX / ST_THREADS];                      // the embedding of all tokens
+#pragma unroll
+        for (int i = 0; i < ST_MAX * ST_MAX / ST_THREADS; ++i) {
+            const int v = (tid >> 6) + ST_THREADS / 64 * i, k = tid & 63;
+            e[i] = v < NV && k < E ? (float)__ldg(static_cast<const TW*>(p.emb) + (size_t)v * E + k) : 0.f;
+        }
+        load_row(w, p.w_ih[0], g_row, E, item < P);
+        const float bias = item < P ? p.b_ih[0][g_row] + p.b_hh[0][g_row] : 0.f;
+#pragma unroll
+        for (int i = 0; i < ST_MAX * ST_MAX / ST_THREADS; ++i) s_enc[tid + ST_THREADS * i] = e[i];
+        __syncthreads();
+#pragma unroll 2
+        for (int v = 0; v < NV; ++v) s_table[v * (4 * ST_MAX) + tid] = dot(w, s_enc + v * ST_MAX) + bias;
+    }
+    load_row(w, p.w_hh[0], g_row, P, item < P);
+    // a quarter of a row: four pieces of four values, 16 apart, so that the quarters' pieces lie side by side
+    float wp[16], wo[16];
+#pragma unroll
+    for (int j = 0; j < 16; ++j) {
+        const int k = (j >> 2) * 16 + part * 4 + (j & 3);
+        wp[j] = item < H && k < P ? (float)__ldg(static_cast<const TW*>(p.w_pred) + (size_t)item * P + k) : 0.f;
+        wo[j] = item < NV && k < H ? (float)__ldg(static_cast<const TW*>(p.w_out) + (size_t)item * H + k) : 0.f;
+    }
+    const float b_pred = item < H ? p.b_pred[item] : 0.f, b_out = item < NV ? p.b_out[item] : 0.f;
+#pragma unroll 1
+    for (int i = tid; i < 65; i += ST_THREADS) s_hist[i] = 0;
+
+    const int warps = (NV + 7) / 8;                                 // that have labels
+    s_key[warp][lane] = 0ull;
+    long long n_rows = 0, n_tok = 0, n_forced = 0;
+    int most_steps = 0;
+#pragma unroll 1
+    for (int utt = blockIdx.x; utt < p.B; utt += gridDim.x) {
+        const int len = min(max(p.enc_len[utt], 0), p.T);
+        // the utterance's state, the same in every thread
+        int t = 0, tok = p.blank, cnt = 0, pos = 0, steps = 0;
+        uint32_t par = 0u;
+        float c = 0.f;                                              // of unit `item`
+        // what the last step decided: recorded by the last warp when the others are at the joint
+        int r_first = -1, r_label = 0, r_t = 0, r_pos = 0;
+        bool r_emit = false, r_overflow = false, r_bad = false;
+        auto record = [&]() {
+            if (lane == 0 && r_first >= 0) {
+                s_hist[r_first] += 1;
+                if (r_emit) {
+                    p.out_tokens[(size_t)utt * p.max_out + r_pos] = r_label;
+                    p.out_frames[(size_t)utt * p.max_out + r_pos] = r_t;
+                }
+                if (r_overflow) set_status(p.ctrl, WIND_ERR_OUTPUT_OVERFLOW);
+                if (r_bad) set_status(p.ctrl, WIND_ERR_INTERNAL);
+            }
+        };
+        const TW* enc = static_cast<const TW*>(p.enc_proj) + (size_t)utt * p.T * H;
+        const int k_enc = tid & 63;
+        auto frame = [&](int f) { return k_enc < H ? (float)__ldg(enc + (size_t)f * H + k_enc) : 0.f; };
+        int have = min(len, 2 * p.W);                               // frames that are in the ring or on their way
+        __syncthreads();
+        if (tid < ST_MAX) s_h[0][tid] = 0.f;
+#pragma unroll 4
+        for (int f = tid >> 6; f < have; f += ST_THREADS / 64) s_enc[f * ST_MAX + k_enc] = frame(f);
+        __syncthreads();
+#pragma unroll 1
+        while (t < len) {
+            const int n = min(p.W, len - t);
+            // up to eight more frames, for the next step (a frame comes from L2: 900 cycles)
+            constexpr int AT_ONCE = 8 * 64 / ST_THREADS;
+            const int f0 = have + (tid >> 6);
+            have = min(len, t + 2 * p.W);
+            float e[AT_ONCE];
+#pragma unroll
+            for (int i = 0; i < AT_ONCE; ++i) e[i] = f0 + ST_THREADS / 64 * i < have ? frame(f0 + ST_THREADS / 64 * i) : 0.f;
+            if (tok >= 0) {
+                // ---- gates and cell: lanes 4 u + g hold gate g of a unit ----
+                float s = dot(w, s_h[par]) + s_table[tok * (4 * ST_MAX) + tid];
+                s = part == 2 ? tanhf(s) : 1.f / (1.f + expf(-s));
+                const int base = lane & 28;
+                const float gi = __shfl_sync(0xffffffffu, s, base), gf = __shfl_sync(0xffffffffu, s, base + 1), gg = __shfl_sync(0xffffffffu, s, base + 2),
+                            go = __shfl_sync(0xffffffffu, s, base + 3);
+                c = cell_update_fc(gf, c, gi, gg);
+                const float h = sl_round<TW>(go * tanhf(c));
+                par ^= 1u;
+                if (part == 0) s_h[par][item] = h;                  // (units past P: zero weights, and W_pred has none there)
+            }
+            auto quarter = [&](const float* x, float* v) {
+#pragma unroll
+                for (int j = 0; j < 4; ++j) *reinterpret_cast<float4*>(v + 4 * j) = *reinterpret_cast<const float4*>(x + 16 * j + part * 4);
+            };
+            if (tok >= 0) {
+                __syncthreads();
+                // ---- pred_proj ----
+                float x[16], a[4] = {0.f, 0.f, 0.f, 0.f};
+                quarter(s_h[par], x);
+#pragma unroll
+                for (int j = 0; j < 16; ++j) a[j & 3] = fmaf(wp[j], x[j], a[j & 3]);
+                float s = (a[0] + a[1]) + (a[2] + a[3]);
+                s += __shfl_xor_sync(0xffffffffu, s, 1);
+                s += __shfl_xor_sync(0xffffffffu, s, 2);
+                if (part == 0) s_pred[item] = s + b_pred;
+            }
+            __syncthreads();
+            // ---- joint ----
+            if constexpr (ACT != WIND_ACT_RELU) {                   // the operand in a loop of its own: one tanh in the code
+#pragma unroll 1
+                for (int i = tid; i < n * ST_MAX; i += ST_THREADS) s_z[i] = sl_round<TW>(tanhf(s_enc[((t + (i >> 6)) & 63) * ST_MAX + (i & 63)] + s_pred[i & 63]));
+                __syncthreads();
+            }
+            if (warp == ST_WARPS - 1) record();
+            if (warp < warps) {
+                float g[16];
+                quarter(s_pred, g);
+#pragma unroll 1
+                for (int r0 = 0; r0 < n; r0 += 4) {                 // four window rows at a time (behind the last: nobody looks)
+                    float a[4];
+#pragma unroll
+                    for (int r = 0; r < 4; ++r) {
+                        float x[16], b[4] = {0.f, 0.f, 0.f, 0.f};
+                        quarter(ACT == WIND_ACT_RELU ? s_enc + ((t + r0 + r) & 63) * ST_MAX : s_z + (r0 + r) * ST_MAX, x);
+#pragma unroll
+                        for (int j = 0; j < 16; ++j) b[j & 3] = fmaf(wo[j], ACT == WIND_ACT_RELU ? sl_round<TW>(fmaxf(x[j] + g[j], 0.f)) : x[j], b[j & 3]);
+                        a[r] = (b[0] + b[1]) + (b[2] + b[3]);
+                    }
+                    // lane 4 v + r: label v's logit of row r
+#pragma unroll
+                    for (int o = 2; o >= 1; o >>= 1) {
+                        const bool up = (part & o) != 0;
+#pragma unroll
+                        for (int r = 0; r < o; ++r) {
+                            const float send = up ? a[r] : a[r + o], keep = up ? a[r + o] : a[r];
+                            a[r] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+                        }
+                    }
+                    // the best of the warp's eight labels, the lowest of equals
+                    const float v = item < NV ? a[0] + b_out : -INFINITY;
+                    float m = v;
+#pragma unroll
+                    for (int o = 4; o < 32; o <<= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+                    const uint32_t equal = __ballot_sync(0xffffffffu, v == m) & (0x11111111u << part);
+                    if (lane < 4) s_key[warp][r0 + part] = m > -INFINITY ? pack_key(m, (uint32_t)(8 * warp + ((__ffs((int)equal) - 1) >> 2))) : 0ull;
+                }
+            }
+            // the frames requested above, behind those that this step looks at (the rest of them, with wide windows: now)
+#pragma unroll
+            for (int i = 0; i < AT_ONCE; ++i)
+                if (f0 + ST_THREADS / 64 * i < have) s_enc[((f0 + ST_THREADS / 64 * i) & 63) * ST_MAX + k_enc] = e[i];
+#pragma unroll 1
+            for (int f = f0 + 8; f < have; f += ST_THREADS / 64) s_enc[(f & 63) * ST_MAX + k_enc] = frame(f);
+            __syncthreads();
+            // ---- control (Algorithm 2's branch), by every warp ----
+            unsigned long long key = 0ull;                          // lane = window row; warps without labels have left 0
+#pragma unroll
+            for (int i = 0; i < ST_WARPS; ++i) key = max(key, s_key[i][lane]);
+            uint32_t label = key_label(key);
+            const bool broken = lane < n && (key == 0ull || label >= (uint32_t)NV);
+            if (broken || lane >= n) label = (uint32_t)p.blank;
+            const uint32_t hit = __ballot_sync(0xffffffffu, (int)label != p.blank);
+            const int first = hit ? __ffs((int)hit) - 1 : n, best = (int)__shfl_sync(0xffffffffu, label, first & 31);
+            const bool emit = hit && pos < p.max_out;
+            if (first > 0) cnt = 0;
+            t += first;
+            const int t_emit = t, at = pos;
+            bool forced = false;
+            if (emit) {
+                ++pos;
+                if (++cnt == p.S) { ++t; cnt = 0; forced = true; }
+            } else if (hit) {
+                t = len;                                            // no room for the token: this utterance stops here
+            }
+            tok = emit ? best : -1;
+            ++steps;
+            const bool stuck = steps >= p.step_cap && t < len;
+            if (stuck) t = len;
+            n_rows += n; n_tok += emit; n_forced += forced;
+            r_bad = __any_sync(0xffffffffu, broken && lane <= first) || stuck;
+            r_first = first; r_label = best; r_t = t_emit; r_pos = at; r_emit = emit; r_overflow = hit && !emit;
+        }
+        if (warp == ST_WARPS - 1) {
+            record();
+            if (lane == 0 && len > 0) p.out_len[utt] = pos;
+        }
+        most_steps = max(most_steps, steps);
+    }
+    __syncthreads();
+    if (tid == 0) {
+        atomicMax(&p.ctrl->step, most_steps);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->joint_rows), (unsigned long long)n_rows);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->tokens), (unsigned long long)n_tok);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->forced), (unsigned long long)n_forced);
+        if (blockIdx.x == 0) { p.ctrl->active = 0; p.ctrl->loop_kernel = WIND_LOOP_ONE_SM; }
+    }
+#pragma unroll 1
+    for (int k = tid; k < 65; k += ST_THREADS)
+        if (s_hist[k]) atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctrl->jump_hist[k]), (unsigned long long)s_hist[k]);
+}
+
+// ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
 template <typename TW>
 static const void* sl_fn(bool resident) {
     return resident ? (const void*)simt_grid_kernel<TW, true> : (const void*)simt_grid_kernel<TW, false>;
+}
+
+template <typename TW>
+static const void* st_fn(int act) {
+    return act == WIND_ACT_RELU ? (const void*)simt_tiny_kernel<TW, WIND_ACT_RELU> : (const void*)simt_tiny_kernel<TW, WIND_ACT_TANH>;
 }
 
 static std::mutex g_sl_mutex;
@@ -896,6 +1162,9 @@ static cudaError_t sl_device(int* optin) {
         for (const void* fn : {sl_fn<float>(false), sl_fn<float>(true), sl_fn<__nv_bfloat16>(false), sl_fn<__nv_bfloat16>(true),
                                (const void*)simt_local_kernel<float>, (const void*)simt_local_kernel<__nv_bfloat16>})
             if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn)) != cudaSuccess) return e;
+        // (its static shared memory: 13 KB)
+        for (const void* fn : {st_fn<float>(WIND_ACT_RELU), st_fn<float>(WIND_ACT_TANH), st_fn<__nv_bfloat16>(WIND_ACT_RELU), st_fn<__nv_bfloat16>(WIND_ACT_TANH)})
+            if ((e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, 16 * ST_MAX * ST_MAX)) != cudaSuccess) return e;
         g_sl_optin[dev] = n;
     }
     *optin = g_sl_optin[dev];
@@ -959,6 +1228,11 @@ cudaError_t simt_loop(const Call& c) {
     p.enc_proj = c.enc_proj(); p.enc_len = c.enc_len;
     p.h = c.h(0); p.c = c.c(); p.pred = c.pred_proj(); p.keys = c.keys();
     p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
+    if (local && m.L == 1 && m.E <= ST_MAX && m.P <= ST_MAX && m.H <= ST_MAX && p.NV <= ST_MAX && c.W <= ST_ROWS) {
+        void* args[1] = {(void*)&p};
+        return cudaLaunchKernel(m.dtype == WIND_DT_BF16 ? st_fn<__nv_bfloat16>(m.act) : st_fn<float>(m.act),
+                                dim3((unsigned)grid), dim3(ST_THREADS), args, (size_t)p.NV * 4 * ST_MAX * sizeof(float), c.stream);
+    }
     if (local) {
         int emb_here = emb;
         void* args[2] = {(void*)&p, (void*)&emb_here};

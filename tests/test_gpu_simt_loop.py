@@ -15,6 +15,10 @@ pytestmark = pytest.mark.gpu
     ("f32", 5, 30, 17, 19, 21, 1, 33, 29, 0, 9, 3),        # one SM, rows padded to four, window of more than eight rows
     ("f32", 3, 20, 20, 64, 32, 1, 16, 900, 0, 4, 3),       # one SM, embedding table in L2, more labels than threads
     ("f32", 2, 90, 16, 16, 16, 1, 16, 20, 0, 40, 3),       # one SM, window of more than 32 rows
+    ("f32", 160, 40, 30, 64, 64, 1, 64, 63, 1, 32, 2),     # weights in registers: all of them in use, widest window, more utterances than SMs
+    ("f32", 4, 30, 9, 1, 33, 1, 64, 1, 0, 17, 3),          # the same, barely: one more unit than half a row, one label, odd window
+    ("f32", 4, 30, 9, 65, 64, 1, 64, 63, 0, 8, 3),         # one embedding element too many
+    ("bf16", 5, 30, 24, 33, 61, 1, 35, 50, 1, 8, 3),
     ("f32", 9, 24, 32, 160, 320, 1, 300, 500, 0, 8, 4),    # grid: units in some CTAs only, three passes of utterances
     ("f32", 3, 24, 32, 130, 333, 2, 301, 449, 1, 5, 2),    # grid, rows padded to 32, two layers, tanh
     ("f32", 2, 10, 32, 640, 1024, 3, 1024, 4000, 0, 8, 2), # grid, weights too large for the chip
