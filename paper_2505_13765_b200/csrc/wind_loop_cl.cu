@@ -48,15 +48,21 @@ __device__ __forceinline__ void cl_gate_rows_to_tmem(const __nv_bfloat16* w, int
     const int q = warp & 3, U = P / CL_SIZE, u = 8 * q + (lane >> 2), g = lane & 3;
     const bool in = u < U;
     const uint4* src = reinterpret_cast<const uint4*>(w + ((size_t)g * P + r * U + (in ? u : 0)) * P);
+    // (five pieces under way: one at a time the ten of them took ten round trips)
+    constexpr int AT_ONCE = 5;
 #pragma unroll 1
-    for (int c0 = 16 * (warp >> 2); c0 < P / 2; c0 += 32) {
-        uint32_t v[16];
+    for (int c0 = 16 * (warp >> 2); c0 < P / 2; c0 += 32 * AT_ONCE) {
+        uint32_t v[AT_ONCE][16];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint4 x = in ? src[c0 / 4 + j] : make_uint4(0, 0, 0, 0);
-            v[4 * j] = x.x; v[4 * j + 1] = x.y; v[4 * j + 2] = x.z; v[4 * j + 3] = x.w;
-        }
-        tmem_st16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)c0, v);
+        for (int k = 0; k < AT_ONCE; ++k)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const uint4 x = in && c0 + 32 * k < P / 2 ? src[(c0 + 32 * k) / 4 + j] : make_uint4(0, 0, 0, 0);
+                v[k][4 * j] = x.x; v[k][4 * j + 1] = x.y; v[k][4 * j + 2] = x.z; v[k][4 * j + 3] = x.w;
+            }
+#pragma unroll
+        for (int k = 0; k < AT_ONCE; ++k)
+            if (c0 + 32 * k < P / 2) tmem_st16(tmem + ((uint32_t)(q * 32) << 16) + (uint32_t)(c0 + 32 * k), v[k]);
     }
     tmem_st_wait();
 }
@@ -331,9 +337,10 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     // ---- resident weights ----
 #pragma unroll 1
     for (int row = warp; row < lab_rows; row += CL_THREADS / 32)                  // W_out: K blocks of lab_rows x 128 bytes, 128-byte swizzle
-        for (int c = lane; c < p.H / 8; c += 32) {
-            const uint4 v = row < labs ? *reinterpret_cast<const uint4*>(p.w_out + (size_t)(lab0 + row) * p.H + c * 8) : make_uint4(0, 0, 0, 0);
-            *reinterpret_cast<uint4*>(smem + L.w_out + (c >> 3) * (lab_rows * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4)) = v;
+        for (int c = lane; c < p.H / 8; c += 32) {                                // (asynchronously: a row's copies were three round trips)
+            uint8_t* dst = smem + L.w_out + (c >> 3) * (lab_rows * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4);
+            if (row < labs) asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(dst)), "l"(p.w_out + (size_t)(lab0 + row) * p.H + c * 8) : "memory");
+            else *reinterpret_cast<uint4*>(dst) = make_uint4(0, 0, 0, 0);
         }
     for (uint32_t i = threadIdx.x; i < (L.pred - L.h0) / 16u; i += CL_THREADS)    // h of slots nobody uses must be numbers
         *reinterpret_cast<uint4*>(smem + L.h0 + i * 16) = make_uint4(0, 0, 0, 0);
@@ -347,7 +354,6 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     auto rec_at = [&](int l) { return p.rx + ((size_t)(cluster * 2 + l) * CL_SIZE + r) * (size_t)(NU * 4 * U); };
     if constexpr (NL == 2)
         for (int i = threadIdx.x; i < NU * 4 * U; i += CL_THREADS) rec_at(0)[i] = rec_at(1)[i] = 0ull;   // no update has number 0
-    fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -356,6 +362,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     const int q = warp & 3;                                                       // lane quadrant
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
     if (warp < 8) cl_gate_rows_to_tmem(p.w_gate, p.P, r, warp, lane, tmem);
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    fence_proxy_async();
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
