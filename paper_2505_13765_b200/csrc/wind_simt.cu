@@ -3,6 +3,7 @@
 // rounds them (enc_proj, the joint's activation output and the LSTM's h input go through
 // bf16), so both kernel sets compute the same quantities.
 #include "wind_internal.cuh"
+#include "wind_ptx.cuh"
 
 namespace wind {
 
@@ -70,6 +71,7 @@ __global__ void __launch_bounds__(256) enc_proj_simt_kernel(const TW* __restrict
                                                             TW* __restrict__ enc_proj, int B, int T, int D, int H) {
     __shared__ __align__(16) float As[2][16][68];
     __shared__ __align__(16) float Bs[2][16][68];
+    let_next_start();
     const long long rows = (long long)B * T;
     const long long r0 = (long long)blockIdx.x * 64;
     const int h0 = blockIdx.y * 64;

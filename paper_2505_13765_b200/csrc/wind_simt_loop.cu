@@ -897,7 +897,6 @@ __global__ void __launch_bounds__(ST_THREADS, 1) simt_tiny_kernel(const SimtLoop
     __shared__ __align__(16) float s_pred[ST_MAX];
     __shared__ unsigned long long s_key[ST_WARPS][ST_ROWS];        // best key of a warp's eight labels per window row
     __shared__ int s_hist[65];
-    if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int E = p.E, P = p.P, H = p.H, NV = p.NV;
     const int item = tid >> 2, part = tid & 3;                     // unit and gate; joint unit or label, and quarter of its row
@@ -965,6 +964,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) simt_tiny_kernel(const SimtLoop
 #pragma unroll 1
     for (int i = tid; i < 65; i += ST_THREADS) s_hist[i] = 0;
 
+    // (up to here, 11 us, under the encoder projection: the weights are the caller's)
+    wait_for_previous();
+    if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
     const int warps = (NV + 7) / 8;                                 // that have labels
     s_key[warp][lane] = 0ull;
     long long n_rows = 0, n_tok = 0, n_forced = 0;
@@ -1230,8 +1232,8 @@ cudaError_t simt_loop(const Call& c) {
     p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
     if (local && m.L == 1 && m.E <= ST_MAX && m.P <= ST_MAX && m.H <= ST_MAX && p.NV <= ST_MAX && c.W <= ST_ROWS) {
         void* args[1] = {(void*)&p};
-        return cudaLaunchKernel(m.dtype == WIND_DT_BF16 ? st_fn<__nv_bfloat16>(m.act) : st_fn<float>(m.act),
-                                dim3((unsigned)grid), dim3(ST_THREADS), args, (size_t)p.NV * 4 * ST_MAX * sizeof(float), c.stream);
+        return launch_overlapped(m.dtype == WIND_DT_BF16 ? st_fn<__nv_bfloat16>(m.act) : st_fn<float>(m.act),
+                                 dim3((unsigned)grid), dim3(ST_THREADS), args, (size_t)p.NV * 4 * ST_MAX * sizeof(float), c.stream);
     }
     if (local) {
         int emb_here = emb;

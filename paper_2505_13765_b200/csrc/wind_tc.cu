@@ -252,6 +252,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant__ C
         tmem_dealloc(tmem_base, GEMM_BN);
     }
     if (threadIdx.x == 0 && abort_flag) set_status(p.ctrl, WIND_ERR_TIMEOUT);
+    if (MODE == MODE_GATE_TABLE && blockIdx.x == 0 && threadIdx.x == 0) wait_for_previous();   // (whoever waits for this kernel waits for that one too)
 }
 
 // ---------------------------------------------------------------------------
@@ -300,6 +301,7 @@ enc_proj_kernel(const __grid_constant__ CUtensorMap map_a, const __grid_constant
     const int warp = uniform_warp_index(), lane = threadIdx.x & 31;
     const uint32_t el = lane == 0;   // the lane that executes the CTA-level instructions of an issuing warp
     uint8_t* smem = align_smem_1024(smem_raw);
+    let_next_start();
     if (p.ctrl->bad_input) return;   // a length outside [0, T]: nothing is read through it
 
     if (threadIdx.x == 0) {
@@ -504,8 +506,9 @@ cudaError_t tc_gate_table(const Call& c) {
     p.out_f32 = c.g0(); p.bias0 = c.b_ih[0]; p.bias1 = c.b_hh[0];
     constexpr int BN = GemmShape<MODE_GATE_TABLE>::BN;
     dim3 grid((unsigned)(((p.N + BN - 1) / BN) * ((p.rows + BM - 1) / BM)));
-    gemm_kernel<MODE_GATE_TABLE><<<grid, GEMM_THREADS, gemm_smem_bytes<MODE_GATE_TABLE>(), c.stream>>>(M.emb, M.w_ih0, p);
-    return cudaGetLastError();
+    // (beside the encoder projection, of which it needs nothing)
+    void* args[3] = {(void*)&M.emb, (void*)&M.w_ih0, (void*)&p};
+    return launch_overlapped((const void*)gemm_kernel<MODE_GATE_TABLE>, grid, dim3(GEMM_THREADS), args, gemm_smem_bytes<MODE_GATE_TABLE>(), c.stream);
 }
 
 int tc_setup_launches(const Call& c, int trace_step) { return 3 + loop_launches(c, trace_step); }  // init, projection, gate table; the loop's
