@@ -376,6 +376,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     auto live_slots = [&]() { return __ballot_sync(0xffffffffu, lane < NU && dec[min(lane, NU - 1)].tok >= 0); };
     // ldmatrix address of the state: two K steps of 16 at a time, matrix = 8 slots x 8 columns, lane = (column piece, slot)
     constexpr uint32_t H_BLOCK = NL == 2 ? 1024u : 2048u;
+    // With up to 32 window rows the gates' product with the state (960 cycles, for the next step) comes behind the joint's, which it would
+    // hold up by 350 of 8500.  Another CTA may be an update ahead by then, so there are two copies of the state, by parity of the updates
+    // (one more update needs this CTA's h, and that this product).  With more rows the joint's operand takes longer than the product, and
+    // there is no room.  One utterance of 100 s 2.20 -> 2.11 ms, seven short ones 0.683 -> 0.648.
+    const bool late = NL == 1 && NS <= 4 && cl_gates_late(NU, p.wp, NL);
+    const uint32_t h_copy = late ? (uint32_t)kb_p * H_BLOCK : 0u;
     const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
     auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * H_BLOCK + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };
 
@@ -638,7 +644,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             }
             if (group_barrier_or<128>(1, !ok || idle)) { leave = true; break; }
             // h to all CTAs
-            const uint32_t h_from = NL == 2 ? (uint32_t)(l * CL_SLOTS * U) * 2u : 0u, h_to = NL == 2 && l == 0 ? L.h0 - L.h : 0u;
+            const uint32_t h_from = NL == 2 ? (uint32_t)(l * CL_SLOTS * U) * 2u : 0u, h_to = NL == 2 && l == 0 ? L.h0 - L.h : ((st >> 1) & 1u) * h_copy;
             const uint32_t h_bar = NL == 2 && l == 0 ? smem_u32(&bar_h0) : smem_u32(&bar_h);
 #pragma unroll
             for (int k = 0; k < 2; ++k)
@@ -715,14 +721,15 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
             float acc[4] = {0.f, 0.f, 0.f, 0.f};
             if (mine && live != 0u) {
                 uint32_t b[2][4];
-                ldmatrix_x4(b[0], h_at(half * (k16s / 2)));
+                const uint32_t copy = ((~st >> 1) & 1u) * h_copy;
+                ldmatrix_x4(b[0], h_at(half * (k16s / 2)) + copy);
                 // (the state rows of the next two steps are requested a turn early; at the end they are rows nobody uses)
 #pragma unroll
                 for (int s0 = 0; s0 < 20; s0 += 4)
                     if (s0 < k16s)
 #pragma unroll
                         for (int s = s0; s < s0 + 4; s += 2) {
-                            ldmatrix_x4(b[(s / 2 + 1) & 1], h_at(half * (k16s / 2) + s / 2 + 1));
+                            ldmatrix_x4(b[(s / 2 + 1) & 1], h_at(half * (k16s / 2) + s / 2 + 1) + copy);
                             mma_16816(acc, wf[s][0], wf[s][1], wf[s][2], wf[s][3], b[(s / 2) & 1][0], b[(s / 2) & 1][1]);
                             mma_16816(acc, wf[s + 1][0], wf[s + 1][1], wf[s + 1][2], wf[s + 1][3], b[(s / 2) & 1][2], b[(s / 2) & 1][3]);
                         }
@@ -794,7 +801,6 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (s0 < p.P / 16)
 #pragma unroll
                     for (int s = s0; s < s0 + 8; ++s) { wf[s][0] = src[s * 8]; wf[s][1] = src[s * 8 + 4]; }
-            const uint32_t back = NL == 2 ? L.h - L.h0 : 0u;             // two layers: the first one's state
             for (uint32_t st = 0u;; st ^= 1u) {          // bit 0: parity of the step, bit 1: of the updates so far
                 const uint32_t par = st & 1u;
                 ok = cl_wait_warp(&bar_dec, par);
@@ -806,13 +812,14 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                 if (!ok) break;
                 float acc[4] = {0.f, 0.f, 0.f, 0.f};
                 uint32_t a[2][4];
-                ldmatrix_x4(a[0], h_at(0) - back);
+                const uint32_t copy = NL == 2 ? L.h0 - L.h : ((~st >> 1) & 1u) * h_copy;     // two layers: the first one's state
+                ldmatrix_x4(a[0], h_at(0) + copy);
 #pragma unroll
                 for (int s0 = 0; s0 < 40; s0 += 8)
                     if (s0 < p.P / 16)
 #pragma unroll
                         for (int s = s0; s < s0 + 8; s += 2) {
-                            ldmatrix_x4(a[(s / 2 + 1) & 1], h_at(s / 2 + 1) - back);
+                            ldmatrix_x4(a[(s / 2 + 1) & 1], h_at(s / 2 + 1) + copy);
                             mma_16816(acc, a[(s / 2) & 1][0], 0u, a[(s / 2) & 1][1], 0u, wf[s][0], wf[s][1]);
                             mma_16816(acc, a[(s / 2) & 1][2], 0u, a[(s / 2) & 1][3], 0u, wf[s + 1][0], wf[s + 1][1]);
                         }
@@ -870,17 +877,13 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                     const int s = (gi << 3) >> wp_shift;
                     tma_load_3d(smem + L.z + (uint32_t)(gi * p.H * 16), &enc_map, 0, (int)dec[s].row + ((gi << 3) & (p.wp - 1)), 0, &bar_enc);
                 }
-                if (update) {
+                auto gates = [&]() {
                     // mma.sync and tcgen05.mma exclude each other on the tensor cores: the short chains go first (when they are
                     // done, all of h is there as well)
-                    if constexpr (NL == 1) {
-                        if (!(ok = cl_wait(&bar_sync_mma, n_g & 1u))) break;
-                    } else if (!(ok = cl_wait(&bar_h0, n_g & 1u))) {
-                        break;
-                    }
+                    if (!(ok = cl_wait(NL == 1 ? &bar_sync_mma : &bar_h0, n_g & 1u))) return;
                     fence_proxy_async_all();             // h came in through remote generic stores
                     tc_fence_after();
-                    uint64_t hd = smem_desc_sw128(sbase + (NL == 2 ? L.h0 : L.h));
+                    uint64_t hd = smem_desc_sw128(sbase + (NL == 2 ? L.h0 : L.h + (n_g & 1u) * h_copy));
 #pragma unroll 1
                     for (int kb = 0; kb < kb_p; ++kb, hd += H_BLOCK >> 4)
 #pragma unroll
@@ -888,7 +891,8 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                             tc_mma_bf16_ts(tm_g, tmem + (uint32_t)(kb * 32 + k * 8), hd + (uint64_t)(k * 2), id_g, (kb | k) != 0);
                     tc_commit(&bar_acc_g);
                     ++n_g;
-                }
+                };
+                if (!late && update) { gates(); if (!ok) break; }
                 if (!(ok = cl_wait(&bar_z, par))) break;
                 tc_fence_after();
                 uint64_t bd = smem_desc_sw128(sbase + L.w_out), ad = ad0;
@@ -901,6 +905,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
                     for (int k = 1; k < 4; ++k) tc_mma_bf16(d, ad + (uint64_t)(k * 2), bd + (uint64_t)(k * 2), id_j, 1u);
                 }
                 tc_commit(&bar_acc_j);
+                if (late && update) { gates(); if (!ok) break; }
             }
             // copies and MMAs in flight must have completed before the memory they use goes back
             if (n_g > 0u) cl_wait(&bar_acc_g, (n_g - 1u) & 1u);
