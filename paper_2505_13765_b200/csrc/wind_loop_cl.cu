@@ -376,11 +376,12 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     auto live_slots = [&]() { return __ballot_sync(0xffffffffu, lane < NU && dec[min(lane, NU - 1)].tok >= 0); };
     // ldmatrix address of the state: two K steps of 16 at a time, matrix = 8 slots x 8 columns, lane = (column piece, slot)
     constexpr uint32_t H_BLOCK = NL == 2 ? 1024u : 2048u;
-    // With up to 32 window rows the gates' product with the state (960 cycles, for the next step) comes behind the joint's, which it would
-    // hold up by 350 of 8500.  Another CTA may be an update ahead by then, so there are two copies of the state, by parity of the updates
-    // (one more update needs this CTA's h, and that this product).  With more rows the joint's operand takes longer than the product, and
-    // there is no room.  One utterance of 100 s 2.20 -> 2.11 ms, seven short ones 0.683 -> 0.648.
-    const bool late = NL == 1 && NS <= 4 && cl_gates_late(NU, p.wp, NL);
+    // With one slot the gates' product with the state (960 cycles, for the next step) comes behind the joint's, which it would hold up by
+    // 350 of 8500.  Another CTA may be an update ahead by then, so there are two copies of the state, by parity of the updates (one more
+    // update needs this CTA's h, and that this product).  With more slots a copy would lack the state of slots that sat an update out,
+    // and from four on the joint's operand takes longer than the product.
+    // One utterance of 100 s 2.20 -> 2.11 ms, seven short ones 0.683 -> 0.648.
+    const bool late = NS == 1 && cl_gates_late(NU, NL);
     const uint32_t h_copy = late ? (uint32_t)kb_p * H_BLOCK : 0u;
     const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
     auto h_at = [&](int k32) { return h_row + (uint32_t)(k32 >> 1) * H_BLOCK + (uint32_t)((((k32 & 1) * 4 + (lane >> 3)) ^ (lane & 7)) << 4); };

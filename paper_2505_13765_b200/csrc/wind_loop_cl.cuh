@@ -68,7 +68,7 @@ __host__ __device__ inline int cl_label_extra(int NV) { return (NV - 16 * cl_lab
 __host__ __device__ inline uint32_t cl_h_block(int layers) { return layers == 2 ? 1024u : 2048u; }
 
 // whether the gates' product with the state follows the joint's, for which there are two copies of the state
-__host__ __device__ inline bool cl_gates_late(int slots, int wp, int layers) { return layers == 1 && slots * wp <= 32; }
+__host__ __device__ inline bool cl_gates_late(int slots, int layers) { return layers == 1 && slots == 1; }
 
 __host__ __device__ inline ClSmem cl_smem_layout(int P, int H, int NV, int slots, int wp, int layers) {
     ClSmem s{};
@@ -82,7 +82,7 @@ __host__ __device__ inline ClSmem cl_smem_layout(int P, int H, int NV, int slots
     if (off < reach) off = reach;
     const uint32_t state = (uint32_t)(P / 64) * cl_h_block(layers) + (layers == 2 ? 1024u : 0u);
     s.h0 = take(layers == 2 ? state : 0u, 1024);
-    s.h = take(cl_gates_late(slots, wp, layers) ? 2u * state : state, 1024);
+    s.h = take(cl_gates_late(slots, layers) ? 2u * state : state, 1024);
     s.pred = take(CL_SLOTS * (uint32_t)H * 2u, 1024);
     s.kbuf = take(CL_KEY_PITCH * (uint32_t)wp * 8u, 16);
     s.dec = take(CL_SLOTS * 16u, 16);

@@ -20,6 +20,8 @@ pytestmark = pytest.mark.gpu
     (13, 30, 512, 640, 1151, 1, 8, 2),     # no remainder units; 72 labels in every CTA; two slots
     (9, 30, 640, 128, 300, 0, 16, 2),      # padded window of 16
     (25, 24, 256, 384, 1000, 1, 5, 3),     # four slots, six K blocks, odd window
+    (28, 42, 512, 640, 552, 1, 1, 3),      # four slots, of which some sit most updates out
+    (18, 45, 128, 512, 353, 0, 2, 2),      # three
     (50, 24, 640, 512, 1030, 0, 4, 2),     # eight slots
     (109, 20, 640, 640, 140, 0, 8, 3),     # sixteen slots; some CTAs without a label
     (200, 16, 128, 640, 513, 1, 2, 2),     # more utterances than slots: the queue, longest first
