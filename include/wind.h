@@ -331,8 +331,8 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
  * The map, recombination and pruning run on the host; the model arithmetic (encoder projection, decoder updates of
  * surviving hypotheses, windowed joint, Eq. (1) and its K best entries) runs in kernels on `stream`.  For most shapes (E, P, H
  * multiples of 8, weights 16-byte aligned, one window's logits in shared memory) that is one kernel which stays for many
- * iterations: it takes each from page-locked host memory and leaves the K x K (label, offset, log-probability) triples there,
- * and the calling thread spins on them.  It has a block of 512 threads on every SM while it stays, so kernels of other
+ * iterations: it takes what to evaluate from page-locked host memory and leaves K (label, offset, log-probability) triples per
+ * hypothesis there, and the calling thread spins on them; what coming iterations will ask for is evaluated ahead.  It has a block of 512 threads on every SM while it stays, so kernels of other
  * streams that do not fit beside it (most that use shared memory or many registers) wait for it; it ends every 10 ms
  * (with prefix_search: after every iteration) and is launched again behind them.  Other shapes launch kernels per iteration
  * and synchronise `stream` to read the triples.  The call synchronises `stream` before it returns.
@@ -342,7 +342,8 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
  *   out_*      HOST: tokens/frames [max_hyps, max_out], lengths and scores [max_hyps], *n_hyps = hypotheses written
  *              (at most max_hyps, best first); a hypothesis longer than max_out is cut in the token arrays, its
  *              length is reported in full.  n_steps (may be null): iterations of the loop.
- *   workspace  DEVICE, at least wind_beam_workspace_bytes(m, T, W, K, max_symbols); 256-byte aligned.
+ *   workspace  DEVICE, wind_beam_workspace_bytes(m, T, W, K, max_symbols); 256-byte aligned.  (Without the part that
+ *              evaluating ahead takes the search runs too, more slowly.)
  * WIND_ERR_WORKSPACE also when the pool of decoder states (sized for K (W + 2) (min(max_symbols, 32) + 2) live
  * hypotheses) runs out.
  */

@@ -636,9 +636,9 @@ wind_status_t wind_beam_search(const wind_model_t* m, const void* enc, int32_t T
     Call cb;
     fill_call(cb, m, enc, nullptr, K, T, W, max_symbols, nullptr, nullptr, nullptr, 1, workspace, (cudaStream_t)stream);
     const BeamLayout bl = make_beam_layout(*m, T, W, K, max_symbols, cb.lay.total);
-    if (workspace_bytes < bl.total) return WIND_ERR_WORKSPACE;
+    if (workspace_bytes < bl.need) return WIND_ERR_WORKSPACE;
     cudaError_t ce = cudaSuccess;
-    s = beam_search_run(cb, bl, K, prefix_search != 0, max_hyps, max_out, out_tokens_host, out_frames_host, out_len_host, out_score_host,
+    s = beam_search_run(cb, bl, workspace_bytes >= bl.total, K, prefix_search != 0, max_hyps, max_out, out_tokens_host, out_frames_host, out_len_host, out_score_host,
                         n_hyps_host, n_steps_host, &ce);
     if (s == WIND_ERR_CUDA) return cuda_fail(ce, "beam search");
     return s;

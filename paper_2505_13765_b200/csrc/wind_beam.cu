@@ -11,6 +11,12 @@
 // carries (parent slot, label) until it survives the pruning of its frame, so at most K decoder updates are made per
 // iteration although K x K hypotheses are created.  Slots are reference-counted (a hypothesis created by the blank
 // entry shares its parent's slot).
+//
+// An iteration waits for the one before it, but what it evaluates (a token history at a frame) rarely depends on that one: most
+// hypotheses of the next frames' lists are there long before their turn.  So a command of the resident kernel is filled up with the
+// histories that the following iterations will most likely ask for (struct Ahead), and an iteration whose hypotheses have all been
+// evaluated needs no command.  What is evaluated is the same, in the same precision and summation order; only the guess when is not,
+// and a wrong one costs a row.  Beam 4, W = 8: 1.02 evaluations per one needed, 0.4 commands per iteration.
 #if defined(__x86_64__)
 #include <immintrin.h>
 #endif
@@ -114,6 +120,7 @@ inline void cpu_relax() {
 constexpr std::chrono::milliseconds kTurn(10);
 struct BeamDevice {
     const Call& c;
+    BeamShape shape;
     float *h_pool, *c_pool, *g_pool, *logits;
     unsigned long long* relay;
     bool single;                 // other kernels run on the stream between the iterations: one launch per command
@@ -137,12 +144,13 @@ struct BeamDevice {
         std::memset(mail, 0, sizeof(BeamMail));
         return cudaMemsetAsync(relay, 0, sizeof(unsigned long long) * kBeamWords, c.stream);
     }
-    void post(const int32_t* words, bool last) {        // 4 + 4 K values
+    int words() const { return 4 + 5 * shape.rows; }
+    void post(const int32_t* words_, bool last) {
         ++seq;
         volatile unsigned long long* out = mail->cmd;
-        for (int i = 0; i < 4 + 4 * c.B; ++i) {
+        for (int i = 0; i < words(); ++i) {
             const uint32_t flag = last && i == 1 ? kBeamLast : 0u;
-            out[i] = (unsigned long long)seq << 32 | ((uint32_t)words[i] | flag);
+            out[i] = (unsigned long long)seq << 32 | ((uint32_t)words_[i] | flag);
         }
     }
     // one command, until its result (nh * K entries) is there
@@ -154,7 +162,7 @@ struct BeamDevice {
             if (!running) {
                 // (a kernel that ends for want of commands took every CTA with it, between two commands)
                 if (++launches > 8) return WIND_ERR_TIMEOUT;
-                if ((*err = beam_step(c, mail, relay, seq, bar_base, h_pool, c_pool, g_pool, logits)) != cudaSuccess) return WIND_ERR_CUDA;
+                if ((*err = beam_step(c, shape, mail, relay, seq, bar_base, h_pool, c_pool, g_pool, logits)) != cudaSuccess) return WIND_ERR_CUDA;
                 running = true;
                 on_chip = false;
             }
@@ -188,13 +196,40 @@ struct BeamDevice {
     // Neither the mailbox nor the caller's workspace is given back before the kernel's end.
     ~BeamDevice() {
         if (!mail) return;
-        std::vector<int32_t> end(4 + 4 * (size_t)c.B, -1);
+        std::vector<int32_t> end((size_t)words(), -1);
         post(end.data(), false);
         cudaStreamSynchronize(c.stream);
         std::lock_guard<std::mutex> lock(g_mail_mutex);
         if (g_mail.size() < kMailKept) g_mail.push_back(mail);
         else cudaFreeHost(mail);
     }
+};
+
+// What is known and what will be asked for: per frame the evaluations made (a token history's K best entries), and a forecast of the
+// lists to come.  The list of a frame is worked off in rounds (a label without a jump leads to the next round of the same frame), so
+// a forecast is the K best hypotheses of each (frame, round) so far, from every evaluation made, wanted or not.
+// What followed from a hypothesis that fell out goes with it: commands filled up with such leftovers brought 2 rows per one needed.
+struct Eval {
+    int32_t node;           // the token history
+    int slot;               // its decoder state (one reference)
+    int32_t label[kMaxBeam], jump[kMaxBeam];
+    float logp[kMaxBeam];
+};
+struct Forecast {
+    uint64_t hash;
+    int32_t len, node;
+    int slot, parent;       // as in Hyp, one reference, none once `asked`
+    int count, from;        // from: frame of the hypothesis that most of its probability comes from, and that one's history
+    uint64_t from_hash;
+    bool asked;
+    double score, most;
+};
+struct Round { std::vector<Forecast> best; };
+struct Frame {
+    int rounds = 0, open = 0;                // rounds in use; forecasts not asked for yet
+    std::vector<Round> round;                // (kept from frame to frame)
+    std::vector<uint64_t> hash;              // of evals
+    std::vector<Eval> evals;
 };
 
 double log_add(double a, double b) {
@@ -211,36 +246,50 @@ BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, s
     size_t off = base;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
     const int s_eff = S < 32 ? S : 32;
-    L.slots = K * (W + 2) * (s_eff + 2) + 2 * K + 2;
-    L.h_pool = take(sizeof(float) * (size_t)L.slots * m.L * m.P);
-    L.c_pool = take(sizeof(float) * (size_t)L.slots * m.L * m.P);
-    L.g_pool = take(sizeof(float) * (size_t)L.slots * m.H);
+    L.own.slots = K * (W + 2) * (s_eff + 2) + 2 * K + 2;
+    L.own.h_pool = take(sizeof(float) * (size_t)L.own.slots * m.L * m.P);
+    L.own.c_pool = take(sizeof(float) * (size_t)L.own.slots * m.L * m.P);
+    L.own.g_pool = take(sizeof(float) * (size_t)L.own.slots * m.H);
     L.ints = take(sizeof(int32_t) * 8 * (size_t)K);
-    L.logits = take(sizeof(float) * (size_t)K * W * (m.V + 1));
+    L.own.logits = take(sizeof(float) * (size_t)K * W * (m.V + 1));
     L.top_label = take(sizeof(int32_t) * 3 * (size_t)K * K);   // labels, offsets, log-probabilities: one block, one copy
     L.top_jump = L.top_label + sizeof(int32_t) * (size_t)K * K;
     L.top_logp = L.top_jump + sizeof(int32_t) * (size_t)K * K;
     L.relay = take(sizeof(uint64_t) * kBeamWords);
-    L.total = off;
+    L.need = L.total = off;
+    // (a workspace of `need` bytes is enough: a command then has only the hypotheses of its iteration)
+    if (K > 1) {
+        const int rows = K > kBeamRows ? K : kBeamRows;
+        L.ahead.slots = L.own.slots + 32 * rows;
+        L.ahead.h_pool = take(sizeof(float) * (size_t)L.ahead.slots * m.L * m.P);
+        L.ahead.c_pool = take(sizeof(float) * (size_t)L.ahead.slots * m.L * m.P);
+        L.ahead.g_pool = take(sizeof(float) * (size_t)L.ahead.slots * m.H);
+        L.ahead.logits = take(sizeof(float) * (size_t)rows * W * (m.V + 1));
+        L.total = off;
+    }
     return L;
 }
 
 // cb: a call bundle with B = K rows (the beam), T, W, S of the utterance, enc = the utterance's frames [T, D];
 // its enc_len / out_len pointers are set here.  Outputs are HOST arrays.
-wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_search, int max_hyps, int max_out, int32_t* out_tokens,
+wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, bool ahead, int K, int prefix_search, int max_hyps, int max_out, int32_t* out_tokens,
                               int32_t* out_frames, int32_t* out_len, double* out_score, int32_t* n_hyps, int64_t* n_steps,
                               cudaError_t* cuda_err) {
     const wind_model_t& m = cb.m;
     const int T = cb.T, W = cb.W, S = cb.S, NV = m.V + 1, LP = m.L * m.P;
     cudaStream_t st = cb.stream;
     uint8_t* ws = cb.ws;
-    float* h_pool = reinterpret_cast<float*>(ws + bl.h_pool);
-    float* c_pool = reinterpret_cast<float*>(ws + bl.c_pool);
-    float* g_pool = reinterpret_cast<float*>(ws + bl.g_pool);
+    const bool resident = beam_step_supported(cb);
+    const BeamShape shape = resident ? beam_step_shape(cb, ahead && !prefix_search) : BeamShape{K, 0};
+    const int R = shape.rows;
+    const BeamPools& pools = shape.look > 0 ? bl.ahead : bl.own;
+    float* h_pool = reinterpret_cast<float*>(ws + pools.h_pool);
+    float* c_pool = reinterpret_cast<float*>(ws + pools.c_pool);
+    float* g_pool = reinterpret_cast<float*>(ws + pools.g_pool);
     int32_t* ints = reinterpret_cast<int32_t*>(ws + bl.ints);   // [0] src slots, [1] tokens, [2] dst slots, [3] expand slots, [4] lengths, [5] scratch, [6] frames
     int32_t *d_src = ints, *d_tok = ints + K, *d_dst = ints + 2 * K, *d_exp = ints + 3 * K, *d_len = ints + 4 * K,
             *d_scratch = ints + 5 * K, *d_t = ints + 6 * K;
-    float* logits = reinterpret_cast<float*>(ws + bl.logits);
+    float* logits = reinterpret_cast<float*>(ws + pools.logits);
     int32_t* d_top_label = reinterpret_cast<int32_t*>(ws + bl.top_label);
     int32_t* d_top_jump = reinterpret_cast<int32_t*>(ws + bl.top_jump);
     float* d_top_logp = reinterpret_cast<float*>(ws + bl.top_logp);
@@ -259,8 +308,8 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
     BEAM_CUDA(cudaMemsetAsync(h_pool, 0, sizeof(float) * LP, st));
     BEAM_CUDA(cudaMemsetAsync(c_pool, 0, sizeof(float) * LP, st));
 
-    std::vector<int> refs(bl.slots, 0), free_slots;
-    for (int s = bl.slots - 1; s >= 1; --s) free_slots.push_back(s);
+    std::vector<int> refs(pools.slots, 0), free_slots;
+    for (int s = pools.slots - 1; s >= 1; --s) free_slots.push_back(s);
     refs[0] = 1;   // the zero state stays
     auto release = [&](int s) { if (s > 0 && --refs[s] == 0) free_slots.push_back(s); };
 
@@ -271,10 +320,9 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
         refs[0]++;
         t2hyps[0].push_back(std::move(h0));
     }
-    BeamDevice dev{cb, h_pool, c_pool, g_pool, logits, reinterpret_cast<unsigned long long*>(ws + bl.relay), prefix_search != 0};
-    const bool resident = beam_step_supported(cb);
+    BeamDevice dev{cb, shape, h_pool, c_pool, g_pool, logits, reinterpret_cast<unsigned long long*>(ws + bl.relay), prefix_search != 0};
     if (resident) BEAM_CUDA(dev.open());
-    std::vector<int32_t> words(4 + 4 * (size_t)K);
+    std::vector<int32_t> words((size_t)dev.words());
     std::vector<int32_t> host_ints(4 * (size_t)K), top(3 * (size_t)K * K);
     const int32_t* top_label = top.data();
     const int32_t* top_jump = top.data() + (size_t)K * K;
@@ -437,8 +485,114 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
         }
     };
 
+    // ---- what is known of frames t .. t + look, and forecasts up to a window behind them ----
+    std::vector<Frame> frames((size_t)(shape.look + W + 2));
+    auto frame_at = [&](int t) -> Frame& { return frames[(size_t)t % frames.size()]; };
+    auto clear_frame = [&](Frame& f) {
+        for (const Eval& e : f.evals) release(e.slot);
+        f.evals.clear();
+        f.hash.clear();
+        for (int r = 0; r < f.rounds; ++r) {
+            for (const Forecast& c : f.round[(size_t)r].best)
+                if (!c.asked) release(c.slot >= 0 ? c.slot : c.parent);
+            f.round[(size_t)r].best.clear();
+        }
+        f.rounds = f.open = 0;
+    };
+    auto find_eval = [&](const Frame& f, int32_t node) {
+        const uint64_t h = node_hash(node);
+        for (size_t i = 0; i < f.hash.size(); ++i)
+            if (f.hash[i] == h && same_tokens(f.evals[i].node, node)) return (int)i;
+        return -1;
+    };
+    auto label_hash = [](uint64_t before, int label) { return (before ^ (uint64_t)(uint32_t)label) * 0x100000001B3ull + 0x9E3779B97F4A7C15ull; };
+    // (history, frame) fell out of a list
+    std::vector<std::pair<uint64_t, int>> fallen;
+    auto remove_fallen = [&] {
+        while (!fallen.empty()) {
+            const auto [hash, from] = fallen.back();
+            fallen.pop_back();
+            for (int t = from; t <= from + W + 1 && t < T; ++t) {
+                Frame& f = frame_at(t);
+                for (int r = 0; r < f.rounds; ++r) {
+                    std::vector<Forecast>& best = f.round[(size_t)r].best;
+                    for (size_t i = 0; i < best.size();) {
+                        if (best[i].from_hash != hash || best[i].from != from) { ++i; continue; }
+                        if (best[i].asked) {
+                            fallen.emplace_back(best[i].hash, t);
+                        } else {
+                            release(best[i].slot >= 0 ? best[i].slot : best[i].parent);
+                            --f.open;
+                        }
+                        best[i] = best.back();
+                        best.pop_back();
+                    }
+                }
+            }
+        }
+    };
+    // a hypothesis that will stand in round r of frame t: `label` (-1: none) behind the history `node`, whose state is in `slot`
+    auto forecast = [&](int t, int r, int from, int32_t node, int label, int slot, int count, double score) {
+        if (t >= T || r >= 64) return;
+        Frame& f = frame_at(t);
+        while (f.rounds <= r) {
+            if ((int)f.round.size() <= f.rounds) f.round.emplace_back();
+            ++f.rounds;
+        }
+        std::vector<Forecast>& best = f.round[(size_t)r].best;
+        const uint64_t h = label < 0 ? node_hash(node) : label_hash(node_hash(node), label);
+        const int len = node_len(node) + (label >= 0);
+        size_t worst = 0;
+        for (size_t i = 0; i < best.size(); ++i) {
+            if (best[i].hash == h && best[i].len == len) {                   // (a forecast: the hash is enough)
+                best[i].score = log_add(best[i].score, score);
+                if (score > best[i].most) { best[i].most = score; best[i].from = from; best[i].from_hash = node_hash(node); }
+                return;
+            }
+            if (best[i].score < best[worst].score) worst = i;
+        }
+        Forecast c{h, len, node, label < 0 ? slot : -1, label < 0 ? -1 : slot, count, from, node_hash(node), false, score, score};
+        if ((int)best.size() < K) {
+            best.emplace_back();
+            worst = best.size() - 1;
+        } else {
+            if (!(score > best[worst].score)) return;
+            if (best[worst].asked) {
+                fallen.emplace_back(best[worst].hash, t);
+            } else {
+                release(best[worst].slot >= 0 ? best[worst].slot : best[worst].parent);
+                --f.open;
+            }
+        }
+        if (label >= 0) {
+            nodes.push_back(Node{node, label, t, len, h});
+            c.node = (int32_t)nodes.size() - 1;
+        }
+        refs[(size_t)slot]++;
+        best[worst] = c;
+        ++f.open;
+    };
+    // what follows from an evaluation of frame t, for a hypothesis of its round r
+    auto forecast_children = [&](const Eval e, int t, int r, int count, double score) {
+        for (int k = 0; k < K; ++k) {
+            if (e.label[k] < 0 || !(e.logp[k] > -INFINITY)) continue;
+            const double s = score + (double)e.logp[k];
+            if (e.label[k] == m.blank_id) {
+                forecast(t + std::min(W, T - t), 0, t, e.node, -1, e.slot, 0, s);
+            } else {
+                const int now = e.jump[k] == 0 ? count + 1 : 1, to = t + e.jump[k] + (now == S);
+                forecast(to, to == t ? r + 1 : 0, t, e.node, e.label[k], e.slot, now == S ? 0 : now, s);
+            }
+        }
+    };
+    // the rows of a command: hypothesis, frame, round, score and count it counts with
+    struct Row { int eval, t, round, count; double score; };
+    std::vector<Row> rows;
+    std::vector<int> eval_of((size_t)K);
+    std::vector<int> parents;               // references to give back once the command is done
+
     for (int t = 0; t < T; ++t) {
-        while (!t2hyps[t].empty()) {
+        for (int round = 0; !t2hyps[t].empty(); ++round) {
             std::vector<Hyp> hyps;
             hyps.swap(t2hyps[t]);
             merge_duplicates(hyps);
@@ -450,37 +604,124 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
             const int nh = (int)hyps.size();
             const int n = W < T - t ? W : T - t;
             ++steps;
-            // ---- decoder update of the survivors that have no state yet ----
-            int nu = 0;
-            for (int b = 0; b < K; ++b) { host_ints[b] = -1; host_ints[K + b] = -1; host_ints[2 * K + b] = -1; host_ints[3 * K + b] = -1; }
-            for (int b = 0; b < nh; ++b) {
-                Hyp& h = hyps[b];
-                if (h.slot < 0) {
-                    if (free_slots.empty()) return WIND_ERR_WORKSPACE;
-                    const int s = free_slots.back();
-                    free_slots.pop_back();
-                    refs[s] = 1;
-                    host_ints[nu] = h.parent;
-                    host_ints[K + nu] = h.node < 0 ? m.blank_id : nodes[(size_t)h.node].tok;
-                    host_ints[2 * K + nu] = s;
-                    h.slot = s;
-                    ++nu;
-                }
-            }
-            for (int b = 0; b < nh; ++b) host_ints[3 * K + b] = hyps[b].slot;
             if (resident) {
-                words[0] = nu; words[1] = nh; words[2] = n; words[3] = t;
-                std::copy(host_ints.begin(), host_ints.end(), words.begin() + 4);
-                const wind_status_t rs = dev.run(words.data(), cuda_err);
-                if (rs != WIND_OK) return rs;
-                for (int u = 0; u < nu; ++u) release(host_ints[u]);
-                for (int i = 0; i < nh * K; ++i) {
-                    const uint32_t at = (uint32_t)dev.mail->top[2 * i], bits = (uint32_t)dev.mail->top[2 * i + 1];
-                    top[(size_t)i] = at == 0xffffffffu ? -1 : (int32_t)(at % (uint32_t)NV);
-                    top[(size_t)K * K + i] = at == 0xffffffffu ? -1 : (int32_t)(at / (uint32_t)NV);
-                    std::memcpy(&top[2 * (size_t)K * K + i], &bits, sizeof(float));
+                if ((int)free_slots.size() < K)                              // (evaluations and forecasts hold slots that the hypotheses need)
+                    for (Frame& f : frames) clear_frame(f);
+                std::fill(words.begin(), words.end(), -1);
+                rows.clear();
+                parents.clear();
+                int nu = 0, reach = t + n;
+                int32_t *c_src = words.data() + 4, *c_tok = c_src + R, *c_dst = c_tok + R, *c_slot = c_dst + R, *c_t = c_slot + R;
+                // one more hypothesis to evaluate; false: there is no slot for its state
+                auto add_row = [&](int32_t node, int slot, int parent, int at, int r, int count, double score) {
+                    if (slot < 0) {
+                        slot = take_slot();
+                        if (slot < 0) return false;
+                        c_src[nu] = parent;
+                        c_tok[nu] = node < 0 ? m.blank_id : nodes[(size_t)node].tok;
+                        c_dst[nu] = slot;
+                        ++nu;
+                    } else {
+                        refs[(size_t)slot]++;
+                    }
+                    const size_t i = rows.size();
+                    c_slot[i] = slot;
+                    c_t[i] = at;
+                    Frame& f = frame_at(at);
+                    rows.push_back(Row{(int)f.evals.size(), at, r, count, score});
+                    f.hash.push_back(node_hash(node));
+                    f.evals.emplace_back();
+                    f.evals.back().node = node;
+                    f.evals.back().slot = slot;
+                    std::fill(f.evals.back().label, f.evals.back().label + K, -1);       // (nothing follows from it yet)
+                    reach = std::max(reach, std::min(at + W, T));
+                    return true;
+                };
+                Frame& here = frame_at(t);
+                for (int b = 0; b < nh; ++b) {
+                    Hyp& h = hyps[b];
+                    int i = find_eval(here, h.node);
+                    if (i < 0) {
+                        i = (int)here.evals.size();
+                        if (!add_row(h.node, h.slot, h.parent, t, round, h.count, h.score)) return WIND_ERR_WORKSPACE;
+                    }
+                    eval_of[(size_t)b] = i;
+                    if (h.slot < 0) {
+                        h.slot = here.evals[(size_t)i].slot;
+                        refs[(size_t)h.slot]++;
+                        parents.push_back(h.parent);
+                    }
+                }
+                // what the forecast had in this list and the list has not
+                if (round < here.rounds)
+                    for (const Forecast& c : here.round[(size_t)round].best) {
+                        bool in = !c.asked;
+                        for (int b = 0; b < nh && !in; ++b) in = node_hash(hyps[(size_t)b].node) == c.hash;
+                        if (!in) fallen.emplace_back(c.hash, t);
+                    }
+                if (!rows.empty()) {
+                    remove_fallen();
+                    // the rest of the command: what comes next, frame by frame and round by round
+                    for (int at = t; shape.look > 0 && at <= t + shape.look && at < T && (int)rows.size() < R; ++at) {
+                        Frame& f = frame_at(at);
+                        for (int r = at == t ? round + 1 : 0; r < f.rounds && f.open > 0 && (int)rows.size() < R; ++r)
+                            for (size_t i = 0; i < f.round[(size_t)r].best.size(); ++i) {
+                                const Forecast c = f.round[(size_t)r].best[i];
+                                if (c.asked) continue;
+                                const int known = find_eval(f, c.node);
+                                if (known < 0) {
+                                    if ((int)rows.size() == R || (int)free_slots.size() <= K) break;
+                                    add_row(c.node, c.slot, c.parent, at, r, c.count, c.score);
+                                }
+                                f.round[(size_t)r].best[i].asked = true;
+                                --f.open;
+                                parents.push_back(c.slot >= 0 ? c.slot : c.parent);
+                                if (known >= 0) forecast_children(f.evals[(size_t)known], at, r, c.count, c.score);
+                            }
+                    }
+                    words[0] = nu; words[1] = (int32_t)rows.size(); words[2] = reach - t; words[3] = t;
+                    const wind_status_t rs = dev.run(words.data(), cuda_err);
+                    if (rs != WIND_OK) return rs;
+                    for (size_t i = 0; i < rows.size(); ++i) {
+                        const Row& row = rows[i];
+                        Eval& e = frame_at(row.t).evals[(size_t)row.eval];
+                        for (int k = 0; k < K; ++k) {
+                            const size_t o = 2 * (i * (size_t)K + (size_t)k);
+                            const uint32_t at = (uint32_t)dev.mail->top[o], bits = (uint32_t)dev.mail->top[o + 1];
+                            e.label[k] = at == 0xffffffffu ? -1 : (int32_t)(at % (uint32_t)NV);
+                            e.jump[k] = at == 0xffffffffu ? -1 : (int32_t)(at / (uint32_t)NV);
+                            std::memcpy(&e.logp[k], &bits, sizeof(float));
+                        }
+                    }
+                    if (shape.look > 0)
+                        for (const Row& row : rows) forecast_children(frame_at(row.t).evals[(size_t)row.eval], row.t, row.round, row.count, row.score);
+                }
+                for (int q : parents) release(q);
+                for (int b = 0; b < nh; ++b) {
+                    const Eval& e = here.evals[(size_t)eval_of[(size_t)b]];
+                    std::copy(e.label, e.label + K, top.begin() + (size_t)b * K);
+                    std::copy(e.jump, e.jump + K, top.begin() + (size_t)K * K + (size_t)b * K);
+                    std::memcpy(&top[2 * (size_t)K * K + (size_t)b * K], e.logp, sizeof(float) * (size_t)K);
                 }
             } else {
+                // ---- decoder update of the survivors that have no state yet ----
+                int nu = 0;
+                for (int b = 0; b < K; ++b) { host_ints[b] = -1; host_ints[K + b] = -1; host_ints[2 * K + b] = -1; host_ints[3 * K + b] = -1; }
+                for (int b = 0; b < nh; ++b) {
+                    Hyp& h = hyps[b];
+                    if (h.slot < 0) {
+                        if (free_slots.empty()) return WIND_ERR_WORKSPACE;
+                        const int s = free_slots.back();
+                        free_slots.pop_back();
+                        refs[s] = 1;
+                        host_ints[nu] = h.parent;
+                        host_ints[K + nu] = h.node < 0 ? m.blank_id : nodes[(size_t)h.node].tok;
+                        host_ints[2 * K + nu] = s;
+                        h.slot = s;
+                        ++nu;
+                    }
+                }
+                for (int b = 0; b < nh; ++b) host_ints[3 * K + b] = hyps[b].slot;
                 BEAM_CUDA(cudaMemcpyAsync(d_exp, host_ints.data() + 3 * K, sizeof(int32_t) * K, cudaMemcpyHostToDevice, st));
                 beam_gather_g_kernel<<<K, 128, 0, st>>>(g_pool, d_exp, cb.pred_proj(), d_t, t, T, m.H);   // sets the frames first
                 BEAM_CUDA(launch_set_t(cb, d_t));   // frames of the rows, and the control block's "active" word
@@ -507,7 +748,7 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
                         int tt = t + jump;
                         Node nd;
                         nd.parent = h.node; nd.tok = label; nd.frm = tt; nd.len = node_len(h.node) + 1;
-                        nd.hash = (node_hash(h.node) ^ (uint64_t)(uint32_t)label) * 0x100000001B3ull + 0x9E3779B97F4A7C15ull;
+                        nd.hash = label_hash(node_hash(h.node), label);
                         nodes.push_back(nd);
                         nhyp.node = (int32_t)nodes.size() - 1;
                         nhyp.count = jump == 0 ? h.count + 1 : 1;
@@ -525,7 +766,9 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_
                 }
             }
             for (int b = 0; b < nh; ++b) release(hyps[b].slot);
+            if (shape.look == 0) clear_frame(frame_at(t));
         }
+        clear_frame(frame_at(t));
     }
     std::vector<Hyp>& fin = t2hyps[T];
     merge_duplicates(fin);

@@ -31,7 +31,7 @@ namespace wind {
 
 constexpr int BS_THREADS = 512;
 constexpr int BS_WARPS = BS_THREADS / 32;
-constexpr int BS_UTTS = 4;            // updates of a pass
+constexpr int BS_UTTS = 4;            // updates of an item
 constexpr int BS_ROWS = 4;            // window rows of a joint item
 
 constexpr unsigned long long BS_IDLE_NS = 200000ull;
@@ -40,38 +40,52 @@ constexpr unsigned long long BS_IDLE_NS = 200000ull;
 struct BsPlan {
     int units, prows, labels;         // the most a CTA owns of each
     int k_l, k_p;                     // row lengths, rounded up to 32: of the gates (any layer), of W_pred
+    int rows, look;                   // as in BeamShape
     int zrows, k_z;                   // window rows of a joint pass; row length of the joint, rounded up to 32
     int resident;                     // the gates' weights of all layers stay; else a layer's are loaded in front of its use
     uint32_t layer, w_l, w_pred, w_out, bias, enc, x, z, total;   // layer: bytes of one layer's weights; z: later the window's logits
 };
-template <typename TW> static BsPlan bs_plan(int G, int W, int K, int E, int P, int L, int H, int NV, uint32_t budget) {
+template <typename TW> static BsPlan bs_plan_with(int G, int W, int rows, int look, int resident, int E, int P, int L, int H, int NV, uint32_t budget) {
     BsPlan s{};
     s.units = (P + G - 1) / G; s.prows = (H + G - 1) / G; s.labels = (NV + G - 1) / G;
     const int k0 = E + P, k1 = L > 1 ? 2 * P : 0, kmax = k0 > k1 ? k0 : k1;
     s.k_l = (kmax + 31) / 32 * 32; s.k_p = (P + 31) / 32 * 32;
     s.k_z = (H + 31) / 32 * 32;
-    const int all = (K * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
-    for (s.resident = 1; s.resident >= 0; --s.resident) {
-        unsigned long long off = 0;
-        auto take = [&](unsigned long long bytes) { const unsigned long long o = off; off += (bytes + 15) / 16 * 16; return (uint32_t)o; };
-        const unsigned long long layer = (unsigned long long)sizeof(TW) * s.units * 4 * s.k_l;
-        s.layer = (uint32_t)layer;
-        s.w_l = take(layer * (s.resident ? L : 1));
-        s.w_pred = take((unsigned long long)sizeof(TW) * ((s.prows + 3) / 4 * 4) * s.k_p);
-        s.w_out = take((unsigned long long)sizeof(TW) * ((s.labels + 3) / 4 * 4) * s.k_z);
-        s.bias = take(4ull * (4 * L * s.units + s.prows + s.labels));
-        s.enc = take((unsigned long long)sizeof(TW) * W * H);
-        const unsigned long long xa = 4ull * BS_UTTS * s.k_l, xb = 4ull * K * H;
-        s.x = take(xa > xb ? xa : xb);
-        s.z = (uint32_t)off;
-        const unsigned long long row = 4ull * s.k_z, window = 4ull * W * NV;
-        const unsigned long long fit = off < budget ? (budget - off) / row / BS_ROWS * BS_ROWS : 0;
-        s.zrows = fit < (unsigned long long)all ? (int)fit : all;
-        off += row * s.zrows > window ? row * s.zrows : window;
-        s.total = s.zrows == 0 || off > budget ? 0xffffffffu : (uint32_t)off;
-        if (s.total <= budget && s.zrows >= (s.resident && all > 16 ? 16 : BS_ROWS)) break;
+    s.rows = rows; s.look = look; s.resident = resident;
+    const int all = (rows * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
+    unsigned long long off = 0;
+    auto take = [&](unsigned long long bytes) { const unsigned long long o = off; off += (bytes + 15) / 16 * 16; return (uint32_t)o; };
+    const unsigned long long layer = (unsigned long long)sizeof(TW) * s.units * 4 * s.k_l;
+    s.layer = (uint32_t)layer;
+    s.w_l = take(layer * (resident ? L : 1));
+    s.w_pred = take((unsigned long long)sizeof(TW) * ((s.prows + 3) / 4 * 4) * s.k_p);
+    s.w_out = take((unsigned long long)sizeof(TW) * ((s.labels + 3) / 4 * 4) * s.k_z);
+    s.bias = take(4ull * (4 * L * s.units + s.prows + s.labels));
+    s.enc = take((unsigned long long)sizeof(TW) * (W + look) * H);
+    const unsigned long long xa = (unsigned long long)sizeof(TW) * BS_UTTS * ((rows + BS_UTTS - 1) / BS_UTTS) * s.k_l, xb = 4ull * rows * H;
+    s.x = take(xa > xb ? xa : xb);
+    s.z = (uint32_t)off;
+    const unsigned long long row = (unsigned long long)sizeof(TW) * s.k_z, window = 4ull * W * NV;
+    const unsigned long long fit = off < budget ? (budget - off) / row / BS_ROWS * BS_ROWS : 0;
+    s.zrows = fit < (unsigned long long)all ? (int)fit : all;
+    off += row * s.zrows > window ? row * s.zrows : window;
+    s.total = s.zrows == 0 || off > budget ? 0xffffffffu : (uint32_t)off;
+    return s;
+}
+// The weights stay if at least four row groups fit beside them; then as many rows and frames ahead as fit likewise.
+template <typename TW> static BsPlan bs_plan(int G, int W, int K, bool ahead, int E, int P, int L, int H, int NV, uint32_t budget) {
+    auto good = [&](const BsPlan& s) {
+        const int all = (s.rows * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
+        return s.total <= budget && s.zrows >= (s.resident && all > 16 ? 16 : BS_ROWS);
+    };
+    BsPlan s = bs_plan_with<TW>(G, W, K, 0, 1, E, P, L, H, NV, budget);
+    if (!good(s)) s = bs_plan_with<TW>(G, W, K, 0, 0, E, P, L, H, NV, budget);
+    if (!good(s) || !ahead || K < 2) return s;
+    const int rows = K > kBeamRows ? K : kBeamRows;
+    for (int look = kBeamLook; look > 0; look /= 2) {
+        const BsPlan a = bs_plan_with<TW>(G, W, rows, look, s.resident, E, P, L, H, NV, budget);
+        if (good(a)) return a;
     }
-    if (s.resident < 0) s.resident = 0;
     return s;
 }
 
@@ -84,7 +98,7 @@ struct BsParams {
     uint32_t extra_arrivals;
     BsPlan plan;
     int K;
-    int E, P, L, H, NV, blank, act, W;
+    int E, P, L, H, NV, blank, act, W, T;
     const void* emb;
     const void* w_ih[kMaxLayers];
     const void* w_hh[kMaxLayers];
@@ -98,9 +112,21 @@ struct BsParams {
     float *h_pool, *c_pool, *g_pool, *logits;
 };
 
-template <typename TW> __device__ __forceinline__ float bs_round(float x);
-template <> __device__ __forceinline__ float bs_round<float>(float x) { return x; }
-template <> __device__ __forceinline__ float bs_round<__nv_bfloat16>(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
+template <typename TW> __device__ __forceinline__ void bs_four(uint32_t at, float* v) {
+    if constexpr (sizeof(TW) == 2) {
+        uint32_t v0, v1;
+        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(at));
+        v[0] = __uint_as_float(v0 << 16); v[1] = __uint_as_float(v0 & 0xffff0000u);
+        v[2] = __uint_as_float(v1 << 16); v[3] = __uint_as_float(v1 & 0xffff0000u);
+    } else {
+        asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(at));
+    }
+}
+// four values (of type TW after rounding) to [k][4]
+template <typename TW> __device__ __forceinline__ void bs_put_four(TW* dst, float a, float b, float c, float d) {
+    if constexpr (sizeof(TW) == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(a, b), pack_bf16x2(c, d));
+    else *reinterpret_cast<float4*>(dst) = make_float4(a, b, c, d);
+}
 
 // Dot products of four rows of weights with four rows of x, both [k][4] in shared memory; the addresses are the lane's first
 // element (k = lane).  Afterwards lane l holds the one of weight row l >> 3 and x row (l >> 1) & 3.
@@ -114,15 +140,8 @@ __device__ __noinline__ float bs_dots(uint32_t w, uint32_t x, int steps) {
 #pragma unroll 4
     for (int i = 0; i < steps; ++i) {
         float wv[4], xv[4];
-        if constexpr (sizeof(TW) == 2) {
-            uint32_t v0, v1;
-            asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(w + 256u * i));
-            wv[0] = __uint_as_float(v0 << 16); wv[1] = __uint_as_float(v0 & 0xffff0000u);
-            wv[2] = __uint_as_float(v1 << 16); wv[3] = __uint_as_float(v1 & 0xffff0000u);
-        } else {
-            asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(wv[0]), "=f"(wv[1]), "=f"(wv[2]), "=f"(wv[3]) : "r"(w + 512u * i));
-        }
-        asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(xv[0]), "=f"(xv[1]), "=f"(xv[2]), "=f"(xv[3]) : "r"(x + 512u * i));
+        bs_four<TW>(w + 128u * (uint32_t)sizeof(TW) * i, wv);
+        bs_four<TW>(x + 128u * (uint32_t)sizeof(TW) * i, xv);
 #pragma unroll
         for (int j = 0; j < 4; ++j)
 #pragma unroll
@@ -169,14 +188,17 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
     const int G = gridDim.x, cta = blockIdx.x;
     const int P = p.P, H = p.H, NV = p.NV, K = p.K, LP = p.L * P;
     const BsPlan& M = p.plan;
+    const int R = M.rows;
     const int units = (P - cta + G - 1) / G, prows = (H - cta + G - 1) / G, labels = (NV - cta + G - 1) / G;
     TW* w_pred = reinterpret_cast<TW*>(sm + M.w_pred);
     TW* w_out = reinterpret_cast<TW*>(sm + M.w_out);
     TW* encs = reinterpret_cast<TW*>(sm + M.enc);
     float* b_gate = reinterpret_cast<float*>(sm + M.bias);                     // [layer][own unit][gate]
     float *b_pred = b_gate + 4 * p.L * M.units, *b_out = b_pred + M.prows;
-    float* xs = reinterpret_cast<float*>(sm + M.x);
-    float* zs = reinterpret_cast<float*>(sm + M.z);
+    TW* xs = reinterpret_cast<TW*>(sm + M.x);                    // operand of the gates or of W_pred, by fours of updates
+    float* gs = reinterpret_cast<float*>(sm + M.x);              // later pred_proj of the hypotheses
+    TW* za = reinterpret_cast<TW*>(sm + M.z);                    // the joint's operand
+    float* zs = reinterpret_cast<float*>(sm + M.z);              // later the logits of a window
     if (tid == 0) s_stop = 0;
 
     // n elements (whole 16-byte pieces) by one warp, asynchronously
@@ -261,7 +283,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
     auto take_command = [&](uint32_t seq) {
         __syncthreads();
         if (warp == 0) {
-            const int words = 4 + 4 * K;
+            const int words = 4 + 5 * R;
             const volatile unsigned long long* from = cta == 0 ? p.mail->cmd : p.relay;
             const unsigned long long limit = cta == 0 ? BS_IDLE_NS : kWaitLimitNs;
             unsigned long long v[(kBeamWords + 31) / 32], t0 = 0;
@@ -300,31 +322,31 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
 
     for (uint32_t seq = p.first_seq;; ++seq) {
         take_command(seq);
-        const int nu = s_cmd[0], nh = s_cmd[1] & (int)(kBeamLast - 1u), n = s_cmd[2], t = s_cmd[3];
+        const int nu = s_cmd[0], nh = s_cmd[1] & (int)(kBeamLast - 1u), span = s_cmd[2], t0 = s_cmd[3];
         const bool last = (s_cmd[1] & (int)kBeamLast) != 0;
         if (nu < 0) return;                                  // the end of the search, or no command for too long
-        const int *c_src = s_cmd + 4, *c_tok = c_src + K, *c_dst = c_tok + K, *c_slot = c_dst + K;
+        const int *c_src = s_cmd + 4, *c_tok = c_src + R, *c_dst = c_tok + R, *c_slot = c_dst + R, *c_t = c_slot + R;
         if (nu > 0 && !M.resident) load_layer(0);
 #pragma unroll 1
-        for (int w = warp; w < n; w += BS_WARPS) copy_row(encs + w * H, static_cast<const TW*>(p.enc_proj) + (size_t)(t + w) * H, H);
+        for (int w = warp; w < span; w += BS_WARPS) copy_row(encs + w * H, static_cast<const TW*>(p.enc_proj) + (size_t)(t0 + w) * H, H);
 
         // ---- decoder update: per layer the gates of this CTA's hidden units, then h and c into the new hypotheses' slots ----
+        const int quads = (nu + BS_UTTS - 1) / BS_UTTS;
+        auto update = [&](int quad, int u) { return min(quad * BS_UTTS + u, nu - 1); };      // (those behind the last repeat it)
         if (nu > 0) {
 #pragma unroll 1
             for (int l = 0; l < p.L; ++l) {
                 const int nin = l == 0 ? p.E : P, K32 = (nin + P + 31) / 32 * 32;
+                // an item: one of this CTA's units for four updates
+                auto c_of = [&](int item) { return p.c_pool + (size_t)c_src[update(item / units, col)] * LP + l * P + (item % units) * G + cta; };
+                float c_in = warp < units * quads ? __ldcg(c_of(warp)) : 0.f;          // requested ahead of everything else
+                // x and the state before it
 #pragma unroll 1
-                for (int u0 = 0; u0 < nu; u0 += BS_UTTS) {
-                    const int n_here = min(BS_UTTS, nu - u0);
-                    if (u0 > 0) __syncthreads();
-                    // x and the state before it of four updates (those behind the last repeat it)
+                for (int quad = 0; quad < quads; ++quad) {
                     int src[BS_UTTS], dst[BS_UTTS], tok[BS_UTTS];
 #pragma unroll
-                    for (int u = 0; u < BS_UTTS; ++u) { const int uu = u0 + min(u, n_here - 1); src[u] = c_src[uu]; dst[u] = c_dst[uu]; tok[u] = c_tok[uu]; }
-                    const int me = u0 + min(col, n_here - 1);
-                    auto c_of = [&](int ui) { return p.c_pool + (size_t)c_src[me] * LP + l * P + ui * G + cta; };
-                    float c_in = warp < units ? __ldcg(c_of(warp)) : 0.f;          // requested ahead of everything else
-#pragma unroll 1
+                    for (int u = 0; u < BS_UTTS; ++u) { const int uu = update(quad, u); src[u] = c_src[uu]; dst[u] = c_dst[uu]; tok[u] = c_tok[uu]; }
+#pragma unroll 2
                     for (int k = tid; k < K32; k += BS_THREADS) {
                         float x[BS_UTTS] = {0.f, 0.f, 0.f, 0.f};
                         if (k < nin && l == 0) {
@@ -333,26 +355,27 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                         } else if (k < nin + P) {
                             const int at = k < nin ? (l - 1) * P + k : l * P + k - nin;
 #pragma unroll
-                            for (int u = 0; u < BS_UTTS; ++u) x[u] = bs_round<TW>(__ldcg(p.h_pool + (size_t)(k < nin ? dst[u] : src[u]) * LP + at));
+                            for (int u = 0; u < BS_UTTS; ++u) x[u] = __ldcg(p.h_pool + (size_t)(k < nin ? dst[u] : src[u]) * LP + at);
                         }
-                        *reinterpret_cast<float4*>(xs + 4 * k) = make_float4(x[0], x[1], x[2], x[3]);
+                        bs_put_four<TW>(xs + 4 * (quad * M.k_l + k), x[0], x[1], x[2], x[3]);
                     }
-                    asm volatile("cp.async.wait_all;" ::: "memory");
-                    __syncthreads();
+                }
+                asm volatile("cp.async.wait_all;" ::: "memory");
+                __syncthreads();
 #pragma unroll 1
-                    for (int ui = warp; ui < units; ui += BS_WARPS) {
-                        const int j = ui * G + cta;
-                        const float mine = bs_dots<TW>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * lane), K32 / 32) + b_gate[4 * (l * M.units + ui) + grp];
-                        const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
-                                    ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
-                        const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
-                        const float cc = cell_update_fc(gf, c_in, gi, gg);
-                        if ((lane & 25) == 0 && col < n_here) {
-                            p.c_pool[(size_t)c_dst[me] * LP + l * P + j] = cc;
-                            p.h_pool[(size_t)c_dst[me] * LP + l * P + j] = go * tanhf(cc);
-                        }
-                        if (ui + BS_WARPS < units) c_in = __ldcg(c_of(ui + BS_WARPS));
+                for (int item = warp; item < units * quads; item += BS_WARPS) {
+                    const int quad = item / units, ui = item - quad * units, j = ui * G + cta;
+                    const float mine = bs_dots<TW>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * (quad * M.k_l + lane)), K32 / 32) + b_gate[4 * (l * M.units + ui) + grp];
+                    const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
+                                ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
+                    const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
+                    const float cc = cell_update_fc(gf, c_in, gi, gg);
+                    if ((lane & 25) == 0 && quad * BS_UTTS + col < nu) {
+                        const size_t to = (size_t)c_dst[quad * BS_UTTS + col] * LP + l * P + j;
+                        p.c_pool[to] = cc;
+                        p.h_pool[to] = go * tanhf(cc);
                     }
+                    if (item + BS_WARPS < units * quads) c_in = __ldcg(c_of(item + BS_WARPS));
                 }
                 arrive();
                 if (!M.resident && l + 1 < p.L) load_layer(l + 1);
@@ -360,40 +383,40 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
             }
             // ---- pred_proj of this CTA's joint units ----
 #pragma unroll 1
-            for (int u0 = 0; u0 < nu; u0 += BS_UTTS) {
-                const int n_here = min(BS_UTTS, nu - u0);
-                if (u0 > 0) __syncthreads();
+            for (int quad = 0; quad < quads; ++quad) {
                 int dst[BS_UTTS];
 #pragma unroll
-                for (int u = 0; u < BS_UTTS; ++u) dst[u] = c_dst[u0 + min(u, n_here - 1)];
-#pragma unroll 1
+                for (int u = 0; u < BS_UTTS; ++u) dst[u] = c_dst[update(quad, u)];
+#pragma unroll 2
                 for (int k = tid; k < M.k_p; k += BS_THREADS) {
                     float x[BS_UTTS] = {0.f, 0.f, 0.f, 0.f};
                     if (k < P) {
 #pragma unroll
-                        for (int u = 0; u < BS_UTTS; ++u) x[u] = bs_round<TW>(__ldcg(p.h_pool + (size_t)dst[u] * LP + (p.L - 1) * P + k));
+                        for (int u = 0; u < BS_UTTS; ++u) x[u] = __ldcg(p.h_pool + (size_t)dst[u] * LP + (p.L - 1) * P + k);
                     }
-                    *reinterpret_cast<float4*>(xs + 4 * k) = make_float4(x[0], x[1], x[2], x[3]);
+                    bs_put_four<TW>(xs + 4 * (quad * M.k_p + k), x[0], x[1], x[2], x[3]);
                 }
-                __syncthreads();
+            }
+            __syncthreads();
+            const int pgs = (prows + 3) / 4;
 #pragma unroll 1
-                for (int pg = warp; pg * 4 < prows; pg += BS_WARPS) {
-                    const int pi = pg * 4 + grp, o = min(pi, prows - 1) * G + cta;
-                    const float mine = bs_dots<TW>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * lane), M.k_p / 32) + b_pred[min(pi, prows - 1)];
-                    if ((lane & 1) == 0 && pi < prows && col < n_here) p.g_pool[(size_t)c_dst[u0 + col] * H + o] = mine;
-                }
+            for (int item = warp; item < pgs * quads; item += BS_WARPS) {
+                const int quad = item / pgs, pg = item - quad * pgs, pi = pg * 4 + grp, o = min(pi, prows - 1) * G + cta;
+                const float mine = bs_dots<TW>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * (quad * M.k_p + lane)), M.k_p / 32) + b_pred[min(pi, prows - 1)];
+                if ((lane & 1) == 0 && pi < prows && quad * BS_UTTS + col < nu) p.g_pool[(size_t)c_dst[quad * BS_UTTS + col] * H + o] = mine;
             }
             arrive();
             if (!wait()) return;
         }
 
         // ---- logits of this CTA's labels for every row of the window under every hypothesis ----
-        const int rows = nh * n;
+        // (windows as long as the first one's; of one that the end of the utterance cuts shorter the rows behind it repeat its last frame)
+        const int n = min(p.W, p.T - t0), rows = nh * n;
 #pragma unroll 1
         for (int b = warp >> 2; b < nh; b += BS_WARPS / 4)
 #pragma unroll 2
             for (int k = (tid & 127) * 4; k < H; k += 512)
-                *reinterpret_cast<float4*>(xs + b * H + k) = __ldcg(reinterpret_cast<const float4*>(p.g_pool + (size_t)c_slot[b] * H + k));
+                *reinterpret_cast<float4*>(gs + b * H + k) = __ldcg(reinterpret_cast<const float4*>(p.g_pool + (size_t)c_slot[b] * H + k));
         asm volatile("cp.async.wait_all;" ::: "memory");
 #pragma unroll 1
         for (int r0 = 0; r0 < rows; r0 += M.zrows) {
@@ -409,8 +432,8 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
 #pragma unroll
                 for (int j = 0; j < 4; ++j) {
                     const int row = min(r0 + rg * BS_ROWS + j, rows - 1), b = row / n;
-                    e4[j] = encs + (row - b * n) * H;
-                    g4[j] = xs + b * H;
+                    e4[j] = encs + min(c_t[b] - t0 + row - b * n, span - 1) * H;
+                    g4[j] = gs + b * H;
                 }
 #pragma unroll 2
                 for (int k = lane + 32 * (item - rg * cut); k < M.k_z; k += 32 * cut) {
@@ -429,8 +452,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                             }
                         }
                     }
-                    *reinterpret_cast<float4*>(zs + 4 * (rg * M.k_z + k)) =
-                        make_float4(bs_round<TW>(z[0]), bs_round<TW>(z[1]), bs_round<TW>(z[2]), bs_round<TW>(z[3]));
+                    bs_put_four<TW>(za + 4 * (rg * M.k_z + k), z[0], z[1], z[2], z[3]);
                 }
             }
             __syncthreads();
@@ -438,7 +460,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
 #pragma unroll 1
             for (int item = warp; item < lgs * nr4; item += BS_WARPS) {
                 const int rg = item / lgs, lg = item - rg * lgs, li = lg * 4 + grp, v = min(li, labels - 1) * G + cta;
-                const float mine = bs_dots<TW>(smem_u32(w_out + 4 * (lg * M.k_z + lane)), smem_u32(zs + 4 * (rg * M.k_z + lane)), M.k_z / 32) + b_out[min(li, labels - 1)];
+                const float mine = bs_dots<TW>(smem_u32(w_out + 4 * (lg * M.k_z + lane)), smem_u32(za + 4 * (rg * M.k_z + lane)), M.k_z / 32) + b_out[min(li, labels - 1)];
                 const int row = r0 + rg * BS_ROWS + col, b = row / n;
                 if ((lane & 1) == 0 && rg * BS_ROWS + col < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = mine;
             }
@@ -448,7 +470,7 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
             if (!wait()) return;
             // ---- Eq. (1) for hypothesis `cta`, the window's logits in shared memory ----
             const float* src = p.logits + (size_t)cta * p.W * NV;
-            const int total = n * NV;
+            const int n = min(p.W, p.T - c_t[cta]), total = n * NV;
 #pragma unroll 16
             for (int i = tid; i < total; i += BS_THREADS) zs[i] = __ldcg(src + i);
             __syncthreads();
@@ -561,10 +583,10 @@ static cudaError_t bs_device(int* optin) {
     return cudaSuccess;
 }
 
-static BsPlan bs_plan_of(const Call& c, int sms, uint32_t budget) {
+static BsPlan bs_plan_of(const Call& c, bool ahead, int sms, uint32_t budget) {
     const wind_model_t& m = c.m;
-    return m.dtype == WIND_DT_BF16 ? bs_plan<__nv_bfloat16>(sms, c.W, c.B, m.E, m.P, m.L, m.H, m.V + 1, budget)
-                                   : bs_plan<float>(sms, c.W, c.B, m.E, m.P, m.L, m.H, m.V + 1, budget);
+    return m.dtype == WIND_DT_BF16 ? bs_plan<__nv_bfloat16>(sms, c.W, c.B, ahead, m.E, m.P, m.L, m.H, m.V + 1, budget)
+                                   : bs_plan<float>(sms, c.W, c.B, ahead, m.E, m.P, m.L, m.H, m.V + 1, budget);
 }
 
 // Rows in whole 16-byte pieces (8 bf16; fp32 models take the same rule), a CTA's weights and one window's logits in shared
@@ -578,10 +600,18 @@ bool beam_step_supported(const Call& c) {
         if (!aligned(c.w_ih[l]) || !aligned(c.w_hh[l])) return false;
     int optin = 0, sms = 0;
     if (bs_device(&optin) != cudaSuccess || loop_sm_count(&sms) != cudaSuccess) { cudaGetLastError(); return false; }
-    return c.B <= sms && bs_plan_of(c, sms, (uint32_t)optin - 4096u).total <= (uint32_t)optin - 4096u;
+    return c.B <= sms && bs_plan_of(c, false, sms, (uint32_t)optin - 4096u).total <= (uint32_t)optin - 4096u;
 }
 
-cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
+// (of a call that beam_step_supported takes)
+BeamShape beam_step_shape(const Call& c, bool ahead) {
+    int optin = 0, sms = 0;
+    if (bs_device(&optin) != cudaSuccess || loop_sm_count(&sms) != cudaSuccess) { cudaGetLastError(); return {c.B, 0}; }
+    const BsPlan s = bs_plan_of(c, ahead, sms, (uint32_t)optin - 4096u);
+    return {s.rows, s.look};
+}
+
+cudaError_t beam_step(const Call& c, const BeamShape& shape, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
                       float* h_pool, float* c_pool, float* g_pool, float* logits) {
     int optin = 0, sms = 0;
     cudaError_t e = bs_device(&optin);
@@ -592,8 +622,8 @@ cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, 
     p.ctrl = c.ctrl(); p.mail = mail; p.relay = relay;
     p.first_seq = first_seq; p.bar_base = bar_base; p.K = c.B;
     p.extra_arrivals = (uint32_t)loop_extra_arrivals();
-    p.plan = bs_plan_of(c, sms, (uint32_t)optin - 4096u);
-    p.E = m.E; p.P = m.P; p.L = m.L; p.H = m.H; p.NV = m.V + 1; p.blank = m.blank_id; p.act = m.act; p.W = c.W;
+    p.plan = bs_plan_of(c, shape.look > 0, sms, (uint32_t)optin - 4096u);
+    p.E = m.E; p.P = m.P; p.L = m.L; p.H = m.H; p.NV = m.V + 1; p.blank = m.blank_id; p.act = m.act; p.W = c.W; p.T = c.T;
     p.emb = m.emb; p.w_pred = m.w_pred; p.b_pred = m.b_pred; p.w_out = m.w_out; p.b_out = m.b_out;
     for (int l = 0; l < m.L; ++l) { p.w_ih[l] = c.w_ih[l]; p.w_hh[l] = c.w_hh[l]; p.b_ih[l] = c.b_ih[l]; p.b_hh[l] = c.b_hh[l]; }
     p.enc_proj = c.enc_proj();

@@ -231,33 +231,40 @@ cudaError_t launch_fill_z(const Call& c);   // measurement aid: fixed joint acti
 
 // first-output distribution of a window (Eq. 1), in place on the window's logits
 // beam search (Algorithm 3): workspace regions behind the call's own layout, and the host-driven search
-struct BeamLayout {
+struct BeamPools {
     size_t h_pool, c_pool, g_pool;   // fp32 [slots][L][P] x 2, [slots][H]: decoder states of live hypotheses and their pred_proj
+    size_t logits;                   // fp32 [hypotheses of a command][W][V+1]
+    int slots;
+};
+struct BeamLayout {
+    BeamPools own, ahead;            // ahead, behind everything else: for commands with hypotheses of later iterations
     size_t ints;                     // int32 [8][K] per-iteration index arrays
-    size_t logits;                   // fp32 [K][W][V+1]
     size_t top_label, top_jump, top_logp;   // [K][K]
     size_t relay;                    // uint64 [kBeamWords]
-    size_t total;
-    int slots;
+    size_t need, total;              // without and with `ahead`
 };
 // Iterations on the device (wind_beam_step.cu): a kernel that takes commands from page-locked host memory and leaves each
 // hypothesis's K best entries there.  A word is (number of the command) << 32 | value.
 constexpr int kMaxBeam = 16;
-constexpr int kBeamWords = 4 + 4 * kMaxBeam;
+constexpr int kBeamRows = 12;          // hypotheses of a command, if a beam has not more (at most kMaxBeam)
+constexpr int kBeamLook = 12;          // a command's hypotheses stand at most this many frames behind its first
+constexpr int kBeamWords = 4 + 5 * kMaxBeam;
 constexpr uint32_t kBeamLast = 0x10000u;
 struct BeamMail {
-    // n_update (-1: end), n_hyps (and kBeamLast: the kernel ends behind this command), n_rows (the window, cut short by the end of the utterance), t; then for K updates each the
-    // slot of the state before, the token, the slot of the state after; then the states of K hypotheses
+    // n_update (-1: end), n_hyps (and kBeamLast: the kernel ends behind this command), frames from t to the last row of any window, t (the first hypothesis's frame);
+    // then, each for as many hypotheses as BeamShape::rows: of the updates the slot of the state before, the token, the slot of the state after; states and frames of the hypotheses
     alignas(128) unsigned long long cmd[kBeamWords];
     alignas(128) unsigned long long top[2 * kMaxBeam * kMaxBeam];   // per entry: offset * (V + 1) + label (all ones: none), fp32 bits of log P'
     alignas(128) uint32_t failed;                                   // a wait inside the kernel ran out
 };
+struct BeamShape { int rows, look; };  // most hypotheses of a command, most frames between them (0: they all stand at one)
+BeamShape beam_step_shape(const Call& c, bool ahead);
 bool beam_step_supported(const Call& c);
-cudaError_t beam_step(const Call& c, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
+cudaError_t beam_step(const Call& c, const BeamShape& shape, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
                       float* h_pool, float* c_pool, float* g_pool, float* logits);
 uint32_t beam_step_arrivals(const Call& c, int n_update);
 BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, size_t base);
-wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, int K, int prefix_search, int max_hyps, int max_out, int32_t* out_tokens,
+wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, bool ahead, int K, int prefix_search, int max_hyps, int max_out, int32_t* out_tokens,
                               int32_t* out_frames, int32_t* out_len, double* out_score, int32_t* n_hyps, int64_t* n_steps,
                               cudaError_t* cuda_err);
 

@@ -1,5 +1,7 @@
 """The beam search's iteration as one kernel, at the sizes where its split can go wrong, against the oracle: rows that are no
 multiple of 32, more updates than a pass takes, joint rows in several passes, every length of a thread's list of best entries."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -39,6 +41,44 @@ def test_beam_iteration_kernel(pkg, E, P, L, H, V, act, W, K, S):  # noqa: F811
         assert all(abs(a[k][2] - b[k][2]) < 1e-4 and list(a[k][1]) == list(b[k][1]) for k in a)
     print(f"[beam iteration] K={K} W={W}: {decided}/6 cases decidable and equal to the oracle")
     assert decided >= (1 if K < 8 else 0)
+
+
+def search(pkg, model, enc, W, K, S, short):
+    """wind_beam_search with a workspace that is `short` bytes smaller: (tokens, frames, lengths, scores, iterations)."""
+    L = pkg.load_library()
+    T = enc.shape[0]
+    dev = pkg.to_device_enc(model, enc[None])[0].contiguous()
+    n = ctypes.c_size_t(0)
+    assert L.wind_beam_workspace_bytes(model.ref, T, W, K, S, ctypes.byref(n)) == 0
+    ws = torch.empty(n.value + 256, dtype=torch.uint8, device="cuda")
+    tok, frm = np.full((64, T * S), -1, np.int32), np.full((64, T * S), -1, np.int32)
+    ln, sc, nh, steps = np.zeros(64, np.int32), np.zeros(64), ctypes.c_int32(0), ctypes.c_int64(0)
+    st = L.wind_beam_search(model.ref, dev.data_ptr(), T, W, K, S, 0, 64, T * S, tok.ctypes.data, frm.ctypes.data, ln.ctypes.data,
+                            sc.ctypes.data, ctypes.byref(nh), ctypes.byref(steps), ws.data_ptr() + -ws.data_ptr() % 256, n.value - short,
+                            torch.cuda.current_stream().cuda_stream)
+    assert st == 0
+    return tok, frm, ln, sc, nh.value, steps.value
+
+
+@pytest.mark.parametrize("dtype,T,E,P,L,H,V,act,W,K,S,bias", [
+    ("f32", 40, 24, 40, 1, 56, 35, 0, 1, 4, 3, 1.0),        # lists a frame apart
+    ("f32", 9, 16, 24, 2, 40, 60, 1, 8, 3, 2, 1.5),         # most windows cut short by the end of the utterance
+    ("f32", 200, 8, 8, 1, 8, 6, 0, 1, 2, 1, 0.0),           # smallest pool of states
+    ("bf16", 60, 40, 72, 1, 64, 300, 0, 5, 4, 10, 2.0),     # many rounds of a frame
+    ("bf16", 50, 32, 64, 2, 72, 150, 1, 16, 2, 3, 3.0),     # windows longer than the frames ahead
+    ("f32", 30, 32, 64, 1, 64, 200, 0, 64, 8, 3, 2.0),      # joint rows in several passes
+    ("bf16", 30, 32, 64, 1, 64, 100, 0, 4, 16, 2, 1.0),     # a command has no more rows than the beam
+    ("bf16", 60, 640, 640, 1, 640, 1024, 0, 8, 4, 10, 4.0),
+    ("f32", 40, 640, 640, 1, 640, 1024, 0, 8, 4, 10, 4.0),  # fewer frames ahead fit beside the weights
+])
+def test_evaluating_ahead_changes_nothing(pkg, dtype, T, E, P, L, H, V, act, W, K, S, bias):  # noqa: F811
+    r = np.random.default_rng(9700 + T + W)
+    w = random_weights(r, 16, E, P, L, H, V, act=act, blank_bias=bias, bias_scale=0.1)
+    w["dtype"] = dtype
+    model = pkg.WindModel(w)
+    enc = r.standard_normal((T, 16)).astype(np.float32)
+    for a, b in zip(search(pkg, model, enc, W, K, S, 0), search(pkg, model, enc, W, K, S, 256)):
+        assert np.array_equal(a, b)
 
 
 def test_other_streams_get_their_turn_during_a_search(pkg):  # noqa: F811
