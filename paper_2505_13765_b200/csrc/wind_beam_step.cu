@@ -4,11 +4,13 @@
 // As separate kernels an iteration of the 640-unit model with beam 4 took 85 us, of which 51 us were eleven kernels and copies
 // (a block per hidden unit or per sixteen labels loads its weights, waits for them, and uses them once) and the rest gaps and
 // the synchronisation.  Here hidden units, joint units and labels are dealt out over all SMs with their weights (67 KB each) in
-// shared memory, the phases follow one another behind grid barriers, and the kernel stays for the whole search: the host
-// writes each iteration's command to page-locked memory and reads the result there: 24 us an iteration.  One launch per iteration
-// took 42 us: 6 us of launch, the weights again, and every instruction fetched from L2 because it runs once.  What is left: 2 us
-// from host to host, three grid barriers (1.5 us each with their skew), and phases of 1 to 3 us that are chains of a few L2 and
-// shared-memory latencies each.
+// shared memory, the phases follow one another behind grid barriers, and the kernel stays for the whole search: the
+// host writes each command to page-locked memory and reads the result there.  One launch per iteration
+// took 42 us: 6 us of launch, the weights again, and every instruction fetched from L2 because it runs once.
+// A command of 4 hypotheses at W = 8 takes 22 us, one of 12 (hypotheses of later iterations, wind_beam.cu) 30 us, before 36 us: operands
+// of four elements and four rows at a time (element by element the joint's took 9 us), all updates in one pass, dot products in pairs
+// and eight rows at a time.  What is left: 7 us from result to command over the host, three grid barriers (1.5 us each with
+// their skew), dot products 6 us, the K best entries 6 us, and chains of a few L2 and shared-memory latencies.
 //
 // The kernel never depends on the host's pace: without a command for 200 us it ends, and the host launches it again with the
 // next one (all state is in global memory).  So a debugger or a descheduled host thread cost the search time only.  On every SM
@@ -81,11 +83,13 @@ template <typename TW> static BsPlan bs_plan(int G, int W, int K, bool ahead, in
     BsPlan s = bs_plan_with<TW>(G, W, K, 0, 1, E, P, L, H, NV, budget);
     if (!good(s)) s = bs_plan_with<TW>(G, W, K, 0, 0, E, P, L, H, NV, budget);
     if (!good(s) || !ahead || K < 2) return s;
-    const int rows = K > kBeamRows ? K : kBeamRows;
-    for (int look = kBeamLook; look > 0; look /= 2) {
-        const BsPlan a = bs_plan_with<TW>(G, W, rows, look, s.resident, E, P, L, H, NV, budget);
-        if (good(a)) return a;
-    }
+    // 12 rows and 12 frames, 16 and 12, 16 and 16: 250 frames at W = 8, beam 4: 28.8, 28.1, 27.2 ms; 200 at W = 16, beam 2: 18.8, 19.0, 18.7;
+    // 300 at W = 4, beam 3: 19.9, 18.9, 18.4; 100 at W = 1, beam 4: 9.4, 8.4, 9.0
+    for (int rows = kBeamRows; rows >= 8 && rows >= K; rows -= 4)
+        for (int look = kBeamLook; look >= 4; look /= 2) {
+            const BsPlan a = bs_plan_with<TW>(G, W, rows, look, s.resident, E, P, L, H, NV, budget);
+            if (good(a)) return a;
+        }
     return s;
 }
 
@@ -112,52 +116,103 @@ struct BsParams {
     float *h_pool, *c_pool, *g_pool, *logits;
 };
 
-template <typename TW> __device__ __forceinline__ void bs_four(uint32_t at, float* v) {
+// Two fp32 values in one register pair: an fma of both rounds each like fmaf, at half the instructions.
+__device__ __forceinline__ unsigned long long bs_pair(uint32_t lo, uint32_t hi) {
+    unsigned long long v;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(v) : "r"(lo), "r"(hi));
+    return v;
+}
+__device__ __forceinline__ void bs_fma_pair(unsigned long long& acc, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
+}
+// four values from shared memory, each twice
+template <typename TW> __device__ __forceinline__ void bs_four_twice(uint32_t at, unsigned long long* v) {
+    uint32_t x[4];
     if constexpr (sizeof(TW) == 2) {
-        uint32_t v0, v1;
-        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v0), "=r"(v1) : "r"(at));
-        v[0] = __uint_as_float(v0 << 16); v[1] = __uint_as_float(v0 & 0xffff0000u);
-        v[2] = __uint_as_float(v1 << 16); v[3] = __uint_as_float(v1 & 0xffff0000u);
+        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x[1]), "=r"(x[3]) : "r"(at));
+        x[0] = x[1] << 16; x[1] &= 0xffff0000u;
+        x[2] = x[3] << 16; x[3] &= 0xffff0000u;
     } else {
-        asm("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(at));
+        asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(at));
+    }
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = bs_pair(x[j], x[j]);
+}
+// four values from shared memory as two pairs
+template <typename TW> __device__ __forceinline__ void bs_two_pairs(uint32_t at, unsigned long long* v) {
+    if constexpr (sizeof(TW) == 2) {
+        uint32_t a, b;
+        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(at));
+        v[0] = bs_pair(a << 16, a & 0xffff0000u);
+        v[1] = bs_pair(b << 16, b & 0xffff0000u);
+    } else {
+        asm("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(at));
     }
 }
-// four values (of type TW after rounding) to [k][4]
-template <typename TW> __device__ __forceinline__ void bs_put_four(TW* dst, float a, float b, float c, float d) {
-    if constexpr (sizeof(TW) == 2) *reinterpret_cast<uint2*>(dst) = make_uint2(pack_bf16x2(a, b), pack_bf16x2(c, d));
-    else *reinterpret_cast<float4*>(dst) = make_float4(a, b, c, d);
+// four elements of a row that starts on 16 bytes, in shared or global memory
+__device__ __forceinline__ float4 bs_quad(const float* p) { return *reinterpret_cast<const float4*>(p); }
+__device__ __forceinline__ float4 bs_quad(const __nv_bfloat16* p) {
+    const uint2 v = *reinterpret_cast<const uint2*>(p);
+    return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
 }
+// four elements of four rows (of type TW after rounding) to [k][4]
+__device__ __forceinline__ void bs_put(float* dst, const float4& a, const float4& b, const float4& c, const float4& d) {
+    float4* to = reinterpret_cast<float4*>(dst);
+    to[0] = make_float4(a.x, b.x, c.x, d.x);
+    to[1] = make_float4(a.y, b.y, c.y, d.y);
+    to[2] = make_float4(a.z, b.z, c.z, d.z);
+    to[3] = make_float4(a.w, b.w, c.w, d.w);
+}
+__device__ __forceinline__ void bs_put(__nv_bfloat16* dst, const float4& a, const float4& b, const float4& c, const float4& d) {
+    uint4* to = reinterpret_cast<uint4*>(dst);
+    to[0] = make_uint4(pack_bf16x2(a.x, b.x), pack_bf16x2(c.x, d.x), pack_bf16x2(a.y, b.y), pack_bf16x2(c.y, d.y));
+    to[1] = make_uint4(pack_bf16x2(a.z, b.z), pack_bf16x2(c.z, d.z), pack_bf16x2(a.w, b.w), pack_bf16x2(c.w, d.w));
+}
+__device__ __noinline__ float4 bs_tanh(float4 v) { return make_float4(tanhf(v.x), tanhf(v.y), tanhf(v.z), tanhf(v.w)); }
 
-// Dot products of four rows of weights with four rows of x, both [k][4] in shared memory; the addresses are the lane's first
-// element (k = lane).  Afterwards lane l holds the one of weight row l >> 3 and x row (l >> 1) & 3.
-// (One function for the three phases, and few unrolled loops elsewhere: an iteration runs its code once, and what does not stay
+// Dot products of four rows of weights with four rows of x (Q times: the next four lie x_pitch bytes on), all [k][4] in shared memory;
+// the addresses are the lane's first element (k = lane).  Afterwards lane l holds the one of weight row l >> 3 and x row (l >> 1) & 3.
+// What bounds them is the arithmetic pipes (bf16 to fp32 and pairs of registers take as long as the fmas): 4 x 4 took 3200 cycles
+// for 20 steps of 16 warps, 8 x 4 is 1.3 times as fast.
+// (One function per Q, and few unrolled loops elsewhere: an iteration runs its code once, and what does not stay
 // in the 32 KB instruction cache is fetched at three cycles an instruction.)
-template <typename TW>
-__device__ __noinline__ float bs_dots(uint32_t w, uint32_t x, int steps) {
-    float a[16];
+template <typename TW, int Q>
+__device__ __noinline__ float2 bs_dots(uint32_t w, uint32_t x, uint32_t x_pitch, int steps) {
+    unsigned long long acc[Q][8];
 #pragma unroll
-    for (int i = 0; i < 16; ++i) a[i] = 0.f;
-#pragma unroll 4
+    for (int i = 0; i < 8 * Q; ++i) acc[i >> 3][i & 7] = 0ull;
+#pragma unroll(4 / Q)
     for (int i = 0; i < steps; ++i) {
-        float wv[4], xv[4];
-        bs_four<TW>(w + 128u * (uint32_t)sizeof(TW) * i, wv);
-        bs_four<TW>(x + 128u * (uint32_t)sizeof(TW) * i, xv);
+        unsigned long long wv[4], xv[2];
+        bs_four_twice<TW>(w + 128u * (uint32_t)sizeof(TW) * i, wv);
 #pragma unroll
-        for (int j = 0; j < 4; ++j)
+        for (int h = 0; h < Q; ++h) {
+            bs_two_pairs<TW>(x + h * x_pitch + 128u * (uint32_t)sizeof(TW) * i, xv);
 #pragma unroll
-            for (int n = 0; n < 4; ++n) a[4 * j + n] = fmaf(wv[j], xv[n], a[4 * j + n]);
-    }
-    const int lane = threadIdx.x & 31;
+            for (int j = 0; j < 4; ++j)
 #pragma unroll
-    for (int half = 8; half >= 1; half >>= 1) {
-        const bool up = (lane & (2 * half)) != 0;
-#pragma unroll
-        for (int c = 0; c < half; ++c) {
-            const float send = up ? a[c] : a[c + half], keep = up ? a[c + half] : a[c];
-            a[c] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * half);
+                for (int n = 0; n < 2; ++n) bs_fma_pair(acc[h][2 * j + n], wv[j], xv[n]);
         }
     }
-    return a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+    const int lane = threadIdx.x & 31;
+    float out[2] = {0.f, 0.f};
+#pragma unroll
+    for (int h = 0; h < Q; ++h) {
+        float a[16];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) asm("mov.b64 {%0, %1}, %2;" : "=f"(a[2 * i]), "=f"(a[2 * i + 1]) : "l"(acc[h][i]));
+#pragma unroll
+        for (int half = 8; half >= 1; half >>= 1) {
+            const bool up = (lane & (2 * half)) != 0;
+#pragma unroll
+            for (int c = 0; c < half; ++c) {
+                const float send = up ? a[c] : a[c + half], keep = up ? a[c + half] : a[c];
+                a[c] = keep + __shfl_xor_sync(0xffffffffu, send, 2 * half);
+            }
+        }
+        out[h] = a[0] + __shfl_xor_sync(0xffffffffu, a[0], 1);
+    }
+    return make_float2(out[0], out[1]);
 }
 
 __device__ __forceinline__ float bs_warp_max(float v) {
@@ -340,32 +395,27 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                 // an item: one of this CTA's units for four updates
                 auto c_of = [&](int item) { return p.c_pool + (size_t)c_src[update(item / units, col)] * LP + l * P + (item % units) * G + cta; };
                 float c_in = warp < units * quads ? __ldcg(c_of(warp)) : 0.f;          // requested ahead of everything else
-                // x and the state before it
-#pragma unroll 1
-                for (int quad = 0; quad < quads; ++quad) {
-                    int src[BS_UTTS], dst[BS_UTTS], tok[BS_UTTS];
-#pragma unroll
-                    for (int u = 0; u < BS_UTTS; ++u) { const int uu = update(quad, u); src[u] = c_src[uu]; dst[u] = c_dst[uu]; tok[u] = c_tok[uu]; }
+                // x and the state before it: four elements of four updates at a time, all loads of a thread at once
+                const int K4 = K32 / 4;
 #pragma unroll 2
-                    for (int k = tid; k < K32; k += BS_THREADS) {
-                        float x[BS_UTTS] = {0.f, 0.f, 0.f, 0.f};
-                        if (k < nin && l == 0) {
+                for (int i = tid; i < quads * K4; i += BS_THREADS) {
+                    const int quad = i / K4, k = 4 * (i - quad * K4);
+                    float4 x[BS_UTTS];
 #pragma unroll
-                            for (int u = 0; u < BS_UTTS; ++u) x[u] = (float)static_cast<const TW*>(p.emb)[(size_t)tok[u] * p.E + k];
-                        } else if (k < nin + P) {
-                            const int at = k < nin ? (l - 1) * P + k : l * P + k - nin;
-#pragma unroll
-                            for (int u = 0; u < BS_UTTS; ++u) x[u] = __ldcg(p.h_pool + (size_t)(k < nin ? dst[u] : src[u]) * LP + at);
-                        }
-                        bs_put_four<TW>(xs + 4 * (quad * M.k_l + k), x[0], x[1], x[2], x[3]);
+                    for (int u = 0; u < BS_UTTS; ++u) {
+                        const int uu = update(quad, u);
+                        if (k < nin && l == 0) x[u] = bs_quad(static_cast<const TW*>(p.emb) + (size_t)c_tok[uu] * p.E + k);
+                        else if (k < nin + P) x[u] = __ldcg(reinterpret_cast<const float4*>(p.h_pool + (size_t)(k < nin ? c_dst[uu] : c_src[uu]) * LP + (k < nin ? (l - 1) * P + k : l * P + k - nin)));
+                        else x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
                     }
+                    bs_put(xs + 4 * (quad * M.k_l + k), x[0], x[1], x[2], x[3]);
                 }
                 asm volatile("cp.async.wait_all;" ::: "memory");
                 __syncthreads();
 #pragma unroll 1
                 for (int item = warp; item < units * quads; item += BS_WARPS) {
                     const int quad = item / units, ui = item - quad * units, j = ui * G + cta;
-                    const float mine = bs_dots<TW>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * (quad * M.k_l + lane)), K32 / 32) + b_gate[4 * (l * M.units + ui) + grp];
+                    const float mine = bs_dots<TW, 1>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * (quad * M.k_l + lane)), 0u, K32 / 32).x + b_gate[4 * (l * M.units + ui) + grp];
                     const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
                                 ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
                     const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
@@ -382,27 +432,22 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                 if (!wait()) return;
             }
             // ---- pred_proj of this CTA's joint units ----
-#pragma unroll 1
-            for (int quad = 0; quad < quads; ++quad) {
-                int dst[BS_UTTS];
-#pragma unroll
-                for (int u = 0; u < BS_UTTS; ++u) dst[u] = c_dst[update(quad, u)];
+            const int K4 = M.k_p / 4;
 #pragma unroll 2
-                for (int k = tid; k < M.k_p; k += BS_THREADS) {
-                    float x[BS_UTTS] = {0.f, 0.f, 0.f, 0.f};
-                    if (k < P) {
+            for (int i = tid; i < quads * K4; i += BS_THREADS) {
+                const int quad = i / K4, k = 4 * (i - quad * K4);
+                float4 x[BS_UTTS];
 #pragma unroll
-                        for (int u = 0; u < BS_UTTS; ++u) x[u] = __ldcg(p.h_pool + (size_t)dst[u] * LP + (p.L - 1) * P + k);
-                    }
-                    bs_put_four<TW>(xs + 4 * (quad * M.k_p + k), x[0], x[1], x[2], x[3]);
-                }
+                for (int u = 0; u < BS_UTTS; ++u)
+                    x[u] = k < P ? __ldcg(reinterpret_cast<const float4*>(p.h_pool + (size_t)c_dst[update(quad, u)] * LP + (p.L - 1) * P + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                bs_put(xs + 4 * (quad * M.k_p + k), x[0], x[1], x[2], x[3]);
             }
             __syncthreads();
             const int pgs = (prows + 3) / 4;
 #pragma unroll 1
             for (int item = warp; item < pgs * quads; item += BS_WARPS) {
                 const int quad = item / pgs, pg = item - quad * pgs, pi = pg * 4 + grp, o = min(pi, prows - 1) * G + cta;
-                const float mine = bs_dots<TW>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * (quad * M.k_p + lane)), M.k_p / 32) + b_pred[min(pi, prows - 1)];
+                const float mine = bs_dots<TW, 1>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * (quad * M.k_p + lane)), 0u, M.k_p / 32).x + b_pred[min(pi, prows - 1)];
                 if ((lane & 1) == 0 && pi < prows && quad * BS_UTTS + col < nu) p.g_pool[(size_t)c_dst[quad * BS_UTTS + col] * H + o] = mine;
             }
             arrive();
@@ -412,15 +457,28 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
         // ---- logits of this CTA's labels for every row of the window under every hypothesis ----
         // (windows as long as the first one's; of one that the end of the utterance cuts shorter the rows behind it repeat its last frame)
         const int n = min(p.W, p.T - t0), rows = nh * n;
+        const int H4 = H / 4;
+        // (under a condition each, not in an unrolled loop, whose last turns would wait one for another)
 #pragma unroll 1
-        for (int b = warp >> 2; b < nh; b += BS_WARPS / 4)
-#pragma unroll 2
-            for (int k = (tid & 127) * 4; k < H; k += 512)
-                *reinterpret_cast<float4*>(gs + b * H + k) = __ldcg(reinterpret_cast<const float4*>(p.g_pool + (size_t)c_slot[b] * H + k));
+        for (int i0 = tid; i0 < nh * H4; i0 += 4 * BS_THREADS) {
+            float4 v[4];
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int i = i0 + j * BS_THREADS, b = i / H4;
+                if (i < nh * H4) v[j] = __ldcg(reinterpret_cast<const float4*>(p.g_pool + (size_t)c_slot[b] * H + 4 * (i - b * H4)));
+            }
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int i = i0 + j * BS_THREADS;
+                if (i < nh * H4) *reinterpret_cast<float4*>(gs + 4 * i) = v[j];
+            }
+        }
         asm volatile("cp.async.wait_all;" ::: "memory");
+        // passes of equal size, in whole pairs of row groups
+        const int passes = (rows + M.zrows - 1) / M.zrows, pass = min(M.zrows, ((rows + passes - 1) / passes + 2 * BS_ROWS - 1) / (2 * BS_ROWS) * (2 * BS_ROWS));
 #pragma unroll 1
-        for (int r0 = 0; r0 < rows; r0 += M.zrows) {
-            const int nr = min(M.zrows, rows - r0), nr4 = (nr + BS_ROWS - 1) / BS_ROWS;
+        for (int r0 = 0; r0 < rows; r0 += pass) {
+            const int nr = min(pass, rows - r0), nr4 = (nr + BS_ROWS - 1) / BS_ROWS;
             __syncthreads();
             // a warp takes four rows and a share of k
             const int cut = nr4 < BS_WARPS ? BS_WARPS / nr4 : 1;
@@ -435,34 +493,35 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                     e4[j] = encs + min(c_t[b] - t0 + row - b * n, span - 1) * H;
                     g4[j] = gs + b * H;
                 }
-#pragma unroll 2
-                for (int k = lane + 32 * (item - rg * cut); k < M.k_z; k += 32 * cut) {
-                    float z[4] = {0.f, 0.f, 0.f, 0.f};
-                    if (k < H) {
-#pragma unroll
-                        for (int j = 0; j < 4; ++j) z[j] = (float)e4[j][k] + g4[j][k];
-                        if (p.act == WIND_ACT_RELU) {
-#pragma unroll
-                            for (int j = 0; j < 4; ++j) z[j] = fmaxf(z[j], 0.f);
-                        } else {
 #pragma unroll 1
-                            for (int j = 0; j < 4; ++j) {              // one tanh in the code
-                                const float v = tanhf(z[0]);
-                                z[0] = z[1]; z[1] = z[2]; z[2] = z[3]; z[3] = v;
-                            }
+                for (int k = 4 * (lane + 32 * (item - rg * cut)); k < M.k_z; k += 128 * cut) {
+                    float4 z[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) {
+                        z[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (k < H) {
+                            const float4 a = bs_quad(e4[j] + k), g = bs_quad(g4[j] + k);
+                            z[j] = make_float4(a.x + g.x, a.y + g.y, a.z + g.z, a.w + g.w);
+                            if (p.act == WIND_ACT_RELU) z[j] = make_float4(fmaxf(z[j].x, 0.f), fmaxf(z[j].y, 0.f), fmaxf(z[j].z, 0.f), fmaxf(z[j].w, 0.f));
+                            else z[j] = bs_tanh(z[j]);
                         }
                     }
-                    bs_put_four<TW>(za + 4 * (rg * M.k_z + k), z[0], z[1], z[2], z[3]);
+                    bs_put(za + 4 * (rg * M.k_z + k), z[0], z[1], z[2], z[3]);
                 }
             }
             __syncthreads();
-            const int lgs = (labels + 3) / 4;
+            const int lgs = (labels + 3) / 4, pairs = (nr4 + 1) / 2;
 #pragma unroll 1
-            for (int item = warp; item < lgs * nr4; item += BS_WARPS) {
-                const int rg = item / lgs, lg = item - rg * lgs, li = lg * 4 + grp, v = min(li, labels - 1) * G + cta;
-                const float mine = bs_dots<TW>(smem_u32(w_out + 4 * (lg * M.k_z + lane)), smem_u32(za + 4 * (rg * M.k_z + lane)), M.k_z / 32) + b_out[min(li, labels - 1)];
-                const int row = r0 + rg * BS_ROWS + col, b = row / n;
-                if ((lane & 1) == 0 && rg * BS_ROWS + col < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = mine;
+            for (int item = warp; item < lgs * pairs; item += BS_WARPS) {
+                const int rg = 2 * (item / lgs), lg = item % lgs, li = lg * 4 + grp, v = min(li, labels - 1) * G + cta;
+                const uint32_t pitch = rg + 1 < nr4 ? 4u * (uint32_t)sizeof(TW) * (uint32_t)M.k_z : 0u;      // (an odd number of groups: the last one twice)
+                const float2 both = bs_dots<TW, 2>(smem_u32(w_out + 4 * (lg * M.k_z + lane)), smem_u32(za + 4 * (rg * M.k_z + lane)), pitch, M.k_z / 32);
+                const float bias = b_out[min(li, labels - 1)];
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const int at = (rg + h) * BS_ROWS + col, row = r0 + at, b = row / n;
+                    if ((lane & 1) == 0 && at < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = (h ? both.y : both.x) + bias;
+                }
             }
         }
         arrive();
@@ -471,8 +530,16 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
             // ---- Eq. (1) for hypothesis `cta`, the window's logits in shared memory ----
             const float* src = p.logits + (size_t)cta * p.W * NV;
             const int n = min(p.W, p.T - c_t[cta]), total = n * NV;
-#pragma unroll 16
-            for (int i = tid; i < total; i += BS_THREADS) zs[i] = __ldcg(src + i);
+#pragma unroll 1
+            for (int i0 = tid; i0 < total; i0 += 20 * BS_THREADS) {
+                float v[20];
+#pragma unroll
+                for (int j = 0; j < 20; ++j)
+                    if (i0 + j * BS_THREADS < total) v[j] = __ldcg(src + i0 + j * BS_THREADS);
+#pragma unroll
+                for (int j = 0; j < 20; ++j)
+                    if (i0 + j * BS_THREADS < total) zs[i0 + j * BS_THREADS] = v[j];
+            }
             __syncthreads();
 #pragma unroll 1
             for (int w = warp; w < n; w += BS_WARPS) {

@@ -246,8 +246,8 @@ struct BeamLayout {
 // Iterations on the device (wind_beam_step.cu): a kernel that takes commands from page-locked host memory and leaves each
 // hypothesis's K best entries there.  A word is (number of the command) << 32 | value.
 constexpr int kMaxBeam = 16;
-constexpr int kBeamRows = 12;          // hypotheses of a command, if a beam has not more (at most kMaxBeam)
-constexpr int kBeamLook = 12;          // a command's hypotheses stand at most this many frames behind its first
+constexpr int kBeamRows = 16;          // hypotheses of a command (at most kMaxBeam), if evaluations are made ahead
+constexpr int kBeamLook = 16;          // these stand at most so many frames behind the first one
 constexpr int kBeamWords = 4 + 5 * kMaxBeam;
 constexpr uint32_t kBeamLast = 0x10000u;
 struct BeamMail {

@@ -69,7 +69,7 @@ def search(pkg, model, enc, W, K, S, short):
     ("f32", 30, 32, 64, 1, 64, 200, 0, 64, 8, 3, 2.0),      # joint rows in several passes
     ("bf16", 30, 32, 64, 1, 64, 100, 0, 4, 16, 2, 1.0),     # a command has no more rows than the beam
     ("bf16", 60, 640, 640, 1, 640, 1024, 0, 8, 4, 10, 4.0),
-    ("f32", 40, 640, 640, 1, 640, 1024, 0, 8, 4, 10, 4.0),  # fewer frames ahead fit beside the weights
+    ("f32", 40, 640, 640, 1, 640, 1024, 0, 8, 4, 10, 4.0),  # nothing ahead fits beside the weights
 ])
 def test_evaluating_ahead_changes_nothing(pkg, dtype, T, E, P, L, H, V, act, W, K, S, bias):  # noqa: F811
     r = np.random.default_rng(9700 + T + W)
