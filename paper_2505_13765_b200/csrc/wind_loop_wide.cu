@@ -2,16 +2,17 @@
 // 1024 joint units: W_out has 65 tiles of 256 KB).
 //
 // loop_kernel streamed all of it every lock step: 768 KB of W_out and z through each SM for the joint and 384 KB for the decoder
-// (its 128-row state tile mostly padding), 34 us a step at 32 utterances x 16 window rows; here 17 to 19.  Here every weight stays on the chip,
+// (its 128-row state tile mostly padding), 34 us a step at 32 utterances x 16 window rows; here 16.  Here every weight stays on the chip,
 // because each CTA has one role only:
 //   L   a W_hh tile (4 gates x 16 units, shared memory); its GEMM for the next step runs behind the projection phase
-//   J   one vocabulary tile: the first 512 of K in tensor memory, the rest in shared memory; z comes through a ring
+//   J   one vocabulary tile: the first 768 of K in tensor memory, the rest in shared memory; z comes through a ring
 //   P   a W_pred tile (64 joint units, shared memory); builds z for all window rows
 //   C   one CTA records (tokens, frames, counters) and clears the keys
 // Every CTA takes the decisions of all utterances from the window's keys itself, so no decision travels; the cell state and the
 // hidden state stay in the registers of the thread that updates them.
 //
-// What bounds a step then is z: a J CTA reads every window row (54 KB/us through one SM: 4.7 us for 128 rows x 1024).  So a lock
+// What bounds a step then is z: a J CTA brings every window row into its shared memory and multiplies it from there (128 rows x 1024:
+// 4600 cycles of shared-memory bandwidth, 2048 each for the copy and for the MMAs, 512 for the part of W_out that lies there).  So a lock
 // step evaluates at most 128 rows: with more than 128 / W utterances alive a window is evaluated in parts, and one whose first
 // part holds a label needs no second.  Where labels are so rare that the second part would often follow, 256 rows (wide_rows).
 // Utterances sit in slots by length, so that the ones still decoding are a prefix and the window widens as they get fewer.
@@ -29,8 +30,13 @@ constexpr int WD_EPI = 256;
 constexpr int WD_NJ = 128;                 // window rows of a row group (an MMA of 64 rows takes as long as one of 128)
 constexpr int WD_ROWS = 256;               // most window rows of a step
 constexpr int WD_SLOTS = 64;               // most utterances
-constexpr int WD_MAX_STAGES = 16;
-constexpr int WD_TM_BLOCKS = 8;            // most K blocks of W_out in tensor memory (256 columns; two accumulators take the rest)
+constexpr int WD_MAX_STAGES = 8;
+// K blocks of a stage of z (two of them with more than 64 rows).  A stage costs its threads 300 to 450 cycles of waiting, issue and commit
+// whatever its size, so with one block each sixteen stages took 7700 cycles, and 7000 for 16 rows: now 6300 and 3700.
+constexpr int WD_UNIT = 4;
+// Most K blocks of W_out in tensor memory: 384 columns, an accumulator takes the rest (two of them up to 8 blocks).  What that leaves of
+// shared memory is the ring for z: nine blocks of 128 rows.
+constexpr int WD_TM_BLOCKS = 12;
 constexpr int WD_CHUNKS = 4;               // boxes of the state: several, so that the first MMAs start before the last rows are there
 constexpr uint32_t WD_Z_STAGE = WD_NJ * BK * 2;
 
@@ -58,7 +64,7 @@ struct WdMaps {
     CUtensorMap w_out;     // [V+1, H], box 128 rows x 1 block
     // z and the state lie in blocks of 64 columns, so that a box is one contiguous piece: with rows of H columns all CTAs read the
     // same few L2 slices at a time
-    CUtensorMap z[2];      // [H / 64][WD_ROWS][64], box 64 or 128 rows
+    CUtensorMap z[4];      // [H / 64][WD_ROWS][64], box 16, 32, 64 or 128 rows x 4, 4, 4 or 2 blocks
     CUtensorMap hb[2][2];  // [parity] [P / 64][nl][64], box blocks / chunks of 16 or of nl rows
 };
 
@@ -85,6 +91,43 @@ struct WdParams {
     const float* b_out;
     const __nv_bfloat16* w_out;
 };
+
+// 32 lanes x 32 columns of an accumulator, rows (lanes) spread over the warp as mma.sync spreads them: v[16 h + 4 x + 2 k + j] is lane
+// 16 h + 8 k + lane / 4, column 8 x + 2 (lane % 4) + j.
+__device__ __forceinline__ void wide_tmem_ld(uint32_t ta, float* v) {
+    uint32_t r[32];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+        asm volatile(
+            "tcgen05.ld.sync.aligned.16x256b.x4.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
+            : "=r"(r[16 * h]), "=r"(r[16 * h + 1]), "=r"(r[16 * h + 2]), "=r"(r[16 * h + 3]), "=r"(r[16 * h + 4]), "=r"(r[16 * h + 5]),
+              "=r"(r[16 * h + 6]), "=r"(r[16 * h + 7]), "=r"(r[16 * h + 8]), "=r"(r[16 * h + 9]), "=r"(r[16 * h + 10]), "=r"(r[16 * h + 11]),
+              "=r"(r[16 * h + 12]), "=r"(r[16 * h + 13]), "=r"(r[16 * h + 14]), "=r"(r[16 * h + 15])
+            : "r"(ta + ((uint32_t)(16 * h) << 16))
+            : "memory");
+    // (the registers pass through the wait, so that nothing reads them before it)
+    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+    for (int i = 0; i < 32; ++i) {
+        asm volatile("" : "+r"(r[i]));
+        v[i] = __uint_as_float(r[i]);
+    }
+}
+// Columns [0, 2 HALF) of a lane and of the lane WITH away become HALF of either, with the better (logit, label) of the two.
+template <int HALF, int WITH>
+__device__ __forceinline__ void wide_exchange(float* v, int* id, int lane) {
+    const bool up = (lane & WITH) != 0;
+#pragma unroll
+    for (int c = 0; c < HALF; ++c) {
+        const float sv = up ? v[c] : v[c + HALF], kv = up ? v[c + HALF] : v[c];
+        const int si = up ? id[c] : id[c + HALF], ki = up ? id[c + HALF] : id[c];
+        const float rv = __shfl_xor_sync(0xffffffffu, sv, WITH);
+        const int ri = __shfl_xor_sync(0xffffffffu, si, WITH);
+        const bool take = (rv > kv) || (rv == kv && ri < ki);   // lowest label on equal logits
+        v[c] = take ? rv : kv;
+        id[c] = take ? ri : ki;
+    }
+}
 
 __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_constant__ WdMaps M, const WdParams p) {
     extern __shared__ uint8_t smem_raw[];
@@ -136,8 +179,9 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_slot;
-    const uint32_t tm_acc = is_j ? tmem + (uint32_t)kb_t * (BK / 2) : tmem;      // J: behind W_out's blocks, two accumulators
+    const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
+    const uint32_t tm_acc = is_j ? tmem + (uint32_t)kb_t * (BK / 2) : tmem;      // J: behind W_out's blocks
+    const uint32_t two = (uint32_t)kb_t * (BK / 2) + 2 * WD_NJ <= LOOP_TMEM_COLS; // J: accumulators: row group n has number n & two
 
     // ---- weights ----
     const bool tile = !is_c && a_bytes > 0u;
@@ -218,10 +262,16 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
     uint4 ev[8];                                                   // P: enc_proj chunks of this thread's rows of the next window
     int kinds = 0, bw[8], bw_wi = -1;                              // 2 bits per row: 0 not written, 1 zeros, 2 a frame
     const float p_bias = is_p && e >= 0 ? p.b_pred[ht * 64 + 16 * q + (lane & 15)] : 0.f;
-    const float j_bias = is_j && e >= 0 && vt * 128 + q * 32 + lane < p.NV ? p.b_out[vt * 128 + q * 32 + lane] : 0.f;
+    float j_bias[4];                                               // J: of the thread's four vocabulary entries, lane / 4 + 8 k of its quadrant
+#pragma unroll
+    for (int k = 0; k < 4; ++k) {
+        const int v = vt * 128 + q * 32 + (lane >> 2) + 8 * k;
+        j_bias[k] = is_j && e >= 0 && v < p.NV ? p.b_out[v] : 0.f;
+    }
 
-    const int kb_first = is_j ? vt % p.kb_h : 0;     // the CTAs start at different K blocks: not all of them on the same lines of L2
-    uint32_t cur = 0, turn = 0;           // J: stage of the ring and how often it came round (TMA and MMA warps count alike)
+    // the CTAs start at different K blocks: not all of them on the same lines of L2
+    const int kb_first = is_j ? vt % ((p.kb_h + WD_UNIT - 1) / WD_UNIT) * WD_UNIT : 0;
+    uint32_t phases = warp == 0 ? 0xFFu : 0u;   // J, TMA and MMA warp: parity to wait for at each stage's barrier
     uint32_t gemm_n = 0;                  // L, P: GEMMs so far; J: row groups so far
     int wi = 0, live = 0;                 // window and slots of the joint phase just done, then of the next one
     float blanks = 0.f, labels = 0.f;     // of the last steps, fading (the same in every CTA)
@@ -408,8 +458,9 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
             }
         }
         if (!grid_sync(TR_L)) break;
-        live = max(s_live[0], s_live[1]);                          // (for the issuing warps; the same everywhere)
-        wi = s_window;
+        // (for the issuing warps; the same everywhere.  Out of a shuffle, so that the compiler knows that all lanes have the same)
+        live = __shfl_sync(0xffffffffu, max(s_live[0], s_live[1]), 0);
+        wi = __shfl_sync(0xffffffffu, s_window, 0);
         if (live == 0) break;
         if (step + 1 >= p.step_cap) { exit_status = WIND_ERR_INTERNAL; break; }
         // =====================================================================================
@@ -457,72 +508,93 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
         // J: logits of this CTA's vocabulary entries for every window row, best (logit, label) key of each row
         // =====================================================================================
         if (is_j) {
-            const int rows = live * wi, groups = (rows + WD_NJ - 1) / WD_NJ, box = rows > WD_NJ / 2;
-            const uint32_t z_bytes = (box ? WD_NJ : WD_NJ / 2) * BK * 2u;
+            const int rows = live * wi, groups = (rows + WD_NJ - 1) / WD_NJ, box = rows <= 16 ? 0 : (rows <= 32 ? 1 : (rows <= 64 ? 2 : 3));
+            // (few rows make short stages and more of them)
+            const int unit = box == 3 ? WD_UNIT / 2 : WD_UNIT, units = (p.kb_h + unit - 1) / unit;     // K blocks of a stage, stages of a row group
+            const uint32_t z_block = (16u << box) * BK * 2u, z_bytes = z_block * (uint32_t)unit, stages = min((uint32_t)WD_MAX_STAGES, (uint32_t)p.stages * WD_Z_STAGE / z_bytes);
+            const uint32_t loads = (uint32_t)(groups * units);
+            const uint32_t used = (loads / stages & 1u ? (1u << stages) - 1u : 0u) ^ ((1u << loads % stages) - 1u);   // stages used an odd number of times
+            uint32_t cur = 0, turn = 0;
             if (warp == 0) {
                 fence_proxy_async_all();
-                bool ok = true;
-                for (int rg = 0; rg < groups && ok; ++rg)
-                    for (int i = 0, kb = kb_first; i < p.kb_h; ++i, kb = kb + 1 == p.kb_h ? 0 : kb + 1) {
-                        if (!(ok = mbar_wait_warp(&empty_bar[cur], (turn & 1u) ^ 1u, &s_abort))) break;
-                        if (elect_one()) {
+                if (elect_one()) {
+                    bool ok = true;
+                    for (int rg = 0; rg < groups && ok; ++rg)
+                        for (int i = 0, kb = kb_first; i < units; ++i, kb = kb + unit >= p.kb_h ? 0 : kb + unit) {
+                            if (!(ok = mbar_wait(&empty_bar[cur], ((phases >> cur) ^ turn) & 1u, &s_abort))) break;
                             mbar_expect_tx(&full_bar[cur], z_bytes);
-                            tma_load_3d(ring + cur * WD_Z_STAGE, &M.z[box], 0, rg * WD_NJ, kb, &full_bar[cur]);
+                            tma_load_3d(ring + cur * z_bytes, &M.z[box], 0, rg * WD_NJ, kb, &full_bar[cur]);
+                            if (++cur == stages) { cur = 0; ++turn; }
                         }
-                        __syncwarp();
-                        if (++cur == (uint32_t)p.stages) { cur = 0; ++turn; }
-                    }
+                }
+                __syncwarp();
+                phases ^= used;
             } else if (warp == 1) {
+                // (the waits stand outside the elected thread's part: behind one in it the compiler no longer keeps the MMAs' operands in
+                // uniform registers, and an MMA took 50 cycles to issue)
                 tc_fence_after();
-                for (int rg = 0; rg < groups; ++rg, ++gemm_n) {
+                bool ok = true;
+                for (int rg = 0; rg < groups && ok; ++rg, ++gemm_n) {
                     const int cols = min(WD_NJ, (rows - rg * WD_NJ + 15) / 16 * 16);
-                    const uint32_t k_acc = gemm_n & 1u, idesc = idesc_bf16(128, cols), acc = tm_acc + k_acc * WD_NJ;
-                    bool ok = mbar_wait_warp(&acc_free[k_acc], ((gemm_n >> 1) & 1u) ^ 1u, &s_abort);
-                    if (!ok) break;
-                    tc_fence_after();
-                    for (int i = 0, kb = kb_first; i < p.kb_h; ++i, kb = kb + 1 == p.kb_h ? 0 : kb + 1) {
-                        if (!(ok = mbar_wait_warp(&full_bar[cur], turn & 1u, &s_abort))) break;
+                    const uint32_t k_acc = gemm_n & two, idesc = idesc_bf16(128, cols), acc = tm_acc + k_acc * WD_NJ;
+                    if (!(ok = mbar_wait_warp(&acc_free[k_acc], ((gemm_n >> two) & 1u) ^ 1u, &s_abort))) break;
+                    for (int i = 0, kb = kb_first; i < units; ++i, kb = kb + unit >= p.kb_h ? 0 : kb + unit) {
+                        if (!(ok = mbar_wait_warp(&full_bar[cur], ((phases >> cur) ^ turn) & 1u, &s_abort))) break;
                         tc_fence_after();
                         if (elect_one()) {
-                            const uint64_t bdesc = smem_desc_sw128(smem_u32(ring) + cur * WD_Z_STAGE);
-                            if (kb < kb_t) {
+                            uint64_t bdesc = smem_desc_sw128(smem_u32(ring) + cur * z_bytes);
+                            const int end = min(kb + unit, p.kb_h), end_t = min(end, kb_t);
+                            uint32_t more = i > 0;
+                            int b = kb;
+#pragma unroll 1
+                            for (; b < end_t; ++b, bdesc += z_block >> 4) {
 #pragma unroll
-                                for (int k = 0; k < BK / 16; ++k)
-                                    tc_mma_bf16_ts(acc, tmem + (uint32_t)(kb * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc, (i | k) != 0);
-                            } else {
-                                const uint64_t adesc = smem_desc_sw128(smem_u32(smem) + (uint32_t)(kb - kb_t) * 128u * BK * 2u);
+                                for (int k = 0; k < BK / 16; ++k, more = 1u) tc_mma_bf16_ts(acc, tmem + (uint32_t)(b * (BK / 2) + k * 8), bdesc + (uint64_t)(k * 2), idesc, more);
+                            }
+                            uint64_t adesc = smem_desc_sw128(smem_u32(smem) + (uint32_t)(b - kb_t) * 128u * BK * 2u);
+#pragma unroll 1
+                            for (; b < end; ++b, bdesc += z_block >> 4, adesc += (128u * BK * 2u) >> 4) {
 #pragma unroll
-                                for (int k = 0; k < BK / 16; ++k) tc_mma_bf16(acc, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (i | k) != 0);
+                                for (int k = 0; k < BK / 16; ++k, more = 1u) tc_mma_bf16(acc, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, more);
                             }
                             tc_commit(&empty_bar[cur]);
-                            if (i + 1 == p.kb_h) tc_commit(&acc_bar[k_acc]);
+                            if (i + 1 == units) tc_commit(&acc_bar[k_acc]);
                         }
                         __syncwarp();
-                        if (++cur == (uint32_t)p.stages) { cur = 0; ++turn; }
+                        if (++cur == stages) { cur = 0; ++turn; }
                     }
-                    if (!ok) break;
                 }
+                phases ^= used;
             } else {
                 unsigned long long* keys = p.keys + (size_t)((step + 1) & 1) * WD_ROWS;
-                const int v = vt * 128 + q * 32 + lane;
+                const int v0 = vt * 128 + q * 32 + (lane >> 2);
                 for (int rg = 0; rg < groups; ++rg, ++gemm_n) {
-                    const uint32_t k_acc = gemm_n & 1u;
-                    const bool ready = mbar_wait_warp(&acc_bar[k_acc], (gemm_n >> 1) & 1u, &s_abort);
+                    const uint32_t k_acc = gemm_n & two;
+                    const bool ready = mbar_wait_warp(&acc_bar[k_acc], (gemm_n >> two) & 1u, &s_abort);
                     tc_fence_after();
                     const int here = min(WD_NJ, rows - rg * WD_NJ);
+                    // A thread holds a quarter of the quadrant's entries of eight window rows: three comparisons each without an exchange,
+                    // then three exchanges  (A row of entries
+                    // per lane took five, with 31 instead of 7 pairs of shuffles: 3750 cycles for 128 rows against 1600.)
                     for (int c0 = 32 * sub; ready && c0 < here; c0 += 64) {
-                        float val[32];
-                        int id[32];
-                        tmem_ld16(tm_acc + lane_off + k_acc * WD_NJ + (uint32_t)c0, val);
-                        tmem_ld16(tm_acc + lane_off + k_acc * WD_NJ + (uint32_t)(c0 + 16), val + 16);
+                        float x[32], val[8];
+                        int id[8];
+                        wide_tmem_ld(tm_acc + lane_off + k_acc * WD_NJ + (uint32_t)c0, x);
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) { val[j] = v < p.NV ? val[j] + j_bias : -INFINITY; id[j] = v; }
-                        argmax_exchange<16>(val, id, lane);
-                        argmax_exchange<8>(val, id, lane);
-                        argmax_exchange<4>(val, id, lane);
-                        argmax_exchange<2>(val, id, lane);
-                        argmax_exchange<1>(val, id, lane);
-                        s_part[q * WD_NJ + c0 + lane] = val[0] > -INFINITY ? pack_key(val[0], (uint32_t)id[0]) : 0ull;
+                        for (int c = 0; c < 8; ++c) { val[c] = -INFINITY; id[c] = v0; }
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            if (v0 + 8 * k < p.NV)
+#pragma unroll
+                                for (int c = 0; c < 8; ++c) {
+                                    const float l = x[16 * (k >> 1) + 4 * (c >> 1) + 2 * (k & 1) + (c & 1)] + j_bias[k];
+                                    if (k == 0 || l > val[c]) { val[c] = l; id[c] = v0 + 8 * k; }
+                                }
+                        wide_exchange<4, 16>(val, id, lane);
+                        wide_exchange<2, 8>(val, id, lane);
+                        wide_exchange<1, 4>(val, id, lane);
+                        const int col = (lane & 16) + (lane & 8) + 2 * (lane & 3) + ((lane >> 2) & 1);
+                        s_part[q * WD_NJ + c0 + col] = val[0] > -INFINITY ? pack_key(val[0], (uint32_t)id[0]) : 0ull;
                     }
                     tc_fence_before();
                     __syncwarp();
@@ -611,7 +683,7 @@ static bool wd_plan(const Call& c, WdPlan* out) {
     const int l = tile + box + 4 * w.nl * 16 * 4, pp = tile + box + w.nl * 68 * 4;
     const int jw = (kb_h > WD_TM_BLOCKS ? kb_h - WD_TM_BLOCKS : 0) * 128 * BK * 2;
     w.stages = (budget - jw) / (int)WD_Z_STAGE;
-    if (w.stages > WD_MAX_STAGES) w.stages = WD_MAX_STAGES;
+    if (w.stages > 2 * WD_MAX_STAGES) w.stages = 2 * WD_MAX_STAGES;
     if (w.stages < 4) return false;
     int most = l > pp ? l : pp;
     if (most > budget) return false;
@@ -639,8 +711,9 @@ cudaError_t wide_loop(const Call& c) {
     if ((e = loop_map3(&M.w_hh, c.w_hh[0], 4ull * m.P, m.P, 16, 1)) != cudaSuccess) return e;
     if ((e = loop_map3(&M.w_pred, m.w_pred, m.H, m.P, 64, 1)) != cudaSuccess) return e;
     if ((e = loop_map3(&M.w_out, m.w_out, (uint64_t)m.V + 1, m.H, 128, 1)) != cudaSuccess) return e;
+    for (int k = 0; k < 4; ++k)
+        if ((e = loop_map_blocks(&M.z[k], c.z(), m.H / BK, WD_ROWS, 16 << k, k == 3 ? WD_UNIT / 2 : WD_UNIT)) != cudaSuccess) return e;
     for (int k = 0; k < 2; ++k) {
-        if ((e = loop_map_blocks(&M.z[k], c.z(), m.H / BK, WD_ROWS, k ? WD_NJ : WD_NJ / 2, 1)) != cudaSuccess) return e;
         for (int par = 0; par < 2; ++par)
             if ((e = loop_map_blocks(&M.hb[par][k], c.hb(par, 0), m.P / BK, w.nl, k ? w.nl : 16, m.P / BK / w.chunks)) != cudaSuccess) return e;
     }
