@@ -2,7 +2,7 @@
 // 1024 joint units: W_out has 65 tiles of 256 KB).
 //
 // loop_kernel streamed all of it every lock step: 768 KB of W_out and z through each SM for the joint and 384 KB for the decoder
-// (its 128-row state tile mostly padding), 34 us a step at 32 utterances x 16 window rows; here 16.  Here every weight stays on the chip,
+// (its 128-row state tile mostly padding), 34 us a step at 32 utterances x 16 window rows; here 15.  Here every weight stays on the chip,
 // because each CTA has one role only:
 //   L   a W_hh tile (4 gates x 16 units, shared memory); its GEMM for the next step runs behind the projection phase
 //   J   one vocabulary tile: the first 768 of K in tensor memory, the rest in shared memory; z comes through a ring
@@ -31,13 +31,13 @@ constexpr int WD_NJ = 128;                 // window rows of a row group (an MMA
 constexpr int WD_ROWS = 256;               // most window rows of a step
 constexpr int WD_SLOTS = 64;               // most utterances
 constexpr int WD_MAX_STAGES = 8;
-// K blocks of a stage of z (two of them with more than 64 rows).  A stage costs its threads 300 to 450 cycles of waiting, issue and commit
-// whatever its size, so with one block each sixteen stages took 7700 cycles, and 7000 for 16 rows: now 6300 and 3700.
-constexpr int WD_UNIT = 4;
+// K blocks of a stage of z (half of them with more than 64 rows, so that a stage is 64 KB at most).  A stage costs its threads 300 to
+// 450 cycles of waiting, issue and commit whatever its size: with one block each the joint of a step took 7.8 us at 32 utterances and
+// 6.2 with 16 rows; with 2 / 4 blocks 6.0 and 4.2, with 4 / 8 5.9 and 3.9.
+constexpr int WD_UNIT = 8;
 // Most K blocks of W_out in tensor memory: 384 columns, an accumulator takes the rest (two of them up to 8 blocks).  What that leaves of
 // shared memory is the ring for z: nine blocks of 128 rows.
 constexpr int WD_TM_BLOCKS = 12;
-constexpr int WD_CHUNKS = 4;               // boxes of the state: several, so that the first MMAs start before the last rows are there
 constexpr uint32_t WD_Z_STAGE = WD_NJ * BK * 2;
 
 // Window rows of a slot in the coming step.  `blanks` and `labels` are recent sums over all utterances: rows found blank, and
@@ -64,20 +64,20 @@ struct WdMaps {
     CUtensorMap w_out;     // [V+1, H], box 128 rows x 1 block
     // z and the state lie in blocks of 64 columns, so that a box is one contiguous piece: with rows of H columns all CTAs read the
     // same few L2 slices at a time
-    CUtensorMap z[4];      // [H / 64][WD_ROWS][64], box 16, 32, 64 or 128 rows x 4, 4, 4 or 2 blocks
-    CUtensorMap hb[2][2];  // [parity] [P / 64][nl][64], box blocks / chunks of 16 or of nl rows
+    CUtensorMap z[4];      // [H / 64][WD_ROWS][64], box 16, 32, 64 or 128 rows x 8, 8, 8 or 4 blocks
+    CUtensorMap hb[2][2];  // [parity] [P / 64][nl][64], box all blocks of 16 or of nl rows
 };
 
 struct WdPlan {
     int n_l, n_j, n_p, grid;              // CTAs of each role; recording CTA behind J
-    int nl, chunks, stages;
+    int nl, stages;
     uint32_t smem;
 };
 
 struct WdParams {
     Ctrl* ctrl;
     int B, T, W, S, max_out, H, P, NV, blank, act, step_cap, extra_arrivals;
-    int n_l, n_j, n_p, nl, chunks, stages, kb_h, kb_p;
+    int n_l, n_j, n_p, nl, stages, kb_h, kb_p;
     const int32_t* enc_len;
     unsigned long long* keys;             // [2][WD_ROWS]
     int32_t* out_tokens;
@@ -279,31 +279,29 @@ __global__ void __launch_bounds__(WD_THREADS, 1) wide_kernel(const __grid_consta
 
     // TMA and MMA of a 64-row weight tile with the state hb[par] (L and P)
     auto state_gemm = [&](int par) {
-        const int kc = p.kb_p / p.chunks, n_cols = live <= 16 ? 16 : p.nl;
+        const int n_cols = live <= 16 ? 16 : p.nl;
         const uint32_t block = (uint32_t)n_cols * BK * 2u;
+        // (one box and one wait: in four, so that the first MMAs start before the last rows are there, the phase took 4.7 us instead of 4.4)
         if (warp == 0) {
             fence_proxy_async_all();
             if (elect_one()) {
-                for (int c = 0; c < p.chunks; ++c) {
-                    mbar_expect_tx(&full_bar[c], (uint32_t)kc * block);
-                    tma_load_3d(ring + (uint32_t)(c * kc) * block, &M.hb[par][n_cols != 16], 0, 0, c * kc, &full_bar[c]);
-                }
+                mbar_expect_tx(&full_bar[0], (uint32_t)p.kb_p * block);
+                tma_load_3d(ring, &M.hb[par][n_cols != 16], 0, 0, 0, &full_bar[0]);
             }
             __syncwarp();
         } else if (warp == 1) {
             tc_fence_after();
             const uint32_t idesc = idesc_bf16(64, n_cols);
-            for (int c = 0; c < p.chunks; ++c) {
-                if (!mbar_wait_warp(&full_bar[c], gemm_n & 1u, &s_abort)) break;
+            if (mbar_wait_warp(&full_bar[0], gemm_n & 1u, &s_abort)) {
                 tc_fence_after();
                 if (elect_one()) {
-                    for (int kb = c * kc; kb < (c + 1) * kc; ++kb) {
+                    for (int kb = 0; kb < p.kb_p; ++kb) {
                         const uint64_t adesc = smem_desc_sw128(smem_u32(smem) + (uint32_t)kb * 64u * BK * 2u);
                         const uint64_t bdesc = smem_desc_sw128(smem_u32(ring) + (uint32_t)kb * block);
 #pragma unroll
                         for (int k = 0; k < BK / 16; ++k) tc_mma_bf16(tm_acc, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, (kb | k) != 0);
                     }
-                    if (c + 1 == p.chunks) tc_commit(&acc_bar[0]);
+                    tc_commit(&acc_bar[0]);
                 }
                 __syncwarp();
             }
@@ -678,7 +676,6 @@ static bool wd_plan(const Call& c, WdPlan* out) {
     w.grid = w.n_l + w.n_j + 1 + w.n_p;
     if (w.grid > sms) return false;
     w.nl = c.B <= 16 ? 16 : (c.B <= 32 ? 32 : 64);
-    w.chunks = kb_p % WD_CHUNKS == 0 ? WD_CHUNKS : 1;
     const int tile = kb_p * 64 * BK * 2, box = w.nl * m.P * 2;
     const int l = tile + box + 4 * w.nl * 16 * 4, pp = tile + box + w.nl * 68 * 4;
     const int jw = (kb_h > WD_TM_BLOCKS ? kb_h - WD_TM_BLOCKS : 0) * 128 * BK * 2;
@@ -715,7 +712,7 @@ cudaError_t wide_loop(const Call& c) {
         if ((e = loop_map_blocks(&M.z[k], c.z(), m.H / BK, WD_ROWS, 16 << k, k == 3 ? WD_UNIT / 2 : WD_UNIT)) != cudaSuccess) return e;
     for (int k = 0; k < 2; ++k) {
         for (int par = 0; par < 2; ++par)
-            if ((e = loop_map_blocks(&M.hb[par][k], c.hb(par, 0), m.P / BK, w.nl, k ? w.nl : 16, m.P / BK / w.chunks)) != cudaSuccess) return e;
+            if ((e = loop_map_blocks(&M.hb[par][k], c.hb(par, 0), m.P / BK, w.nl, k ? w.nl : 16, m.P / BK)) != cudaSuccess) return e;
     }
     WdParams p{};
     p.ctrl = c.ctrl();
@@ -723,7 +720,7 @@ cudaError_t wide_loop(const Call& c) {
     const long long cap = (long long)c.T * (c.S + 1) + 2;       // a part of a window moves by a frame or emits, like a whole one
     p.step_cap = cap > 0x7fffffff ? 0x7fffffff : (int)cap;
     p.extra_arrivals = loop_extra_arrivals();
-    p.n_l = w.n_l; p.n_j = w.n_j; p.n_p = w.n_p; p.nl = w.nl; p.chunks = w.chunks; p.stages = w.stages; p.kb_h = m.H / BK; p.kb_p = m.P / BK;
+    p.n_l = w.n_l; p.n_j = w.n_j; p.n_p = w.n_p; p.nl = w.nl; p.stages = w.stages; p.kb_h = m.H / BK; p.kb_p = m.P / BK;
     p.enc_len = c.enc_len;
     p.keys = c.keys();
     p.out_tokens = c.out_tokens; p.out_frames = c.out_frames; p.out_len = c.out_len;
