@@ -474,6 +474,13 @@ typedef struct {
 wind_status_t wind_debug_plan(const wind_model_t* m, int32_t B, int32_t W, int32_t sms, int32_t smem_optin, wind_plan_t* out);
 
 /*
+ * Dynamic shared memory of a CTA of the cluster kernel for a model, a window and a number of utterances per cluster (`slots`: 1 to 8
+ * for W <= 8, to 4 for W <= 16, to 2 for W <= 32), and what the kernel may ask for at most; host arithmetic only, for tests.
+ * WIND_ERR_UNSUPPORTED: the cluster kernel does not take the shapes.
+ */
+wind_status_t wind_debug_cluster_smem(const wind_model_t* m, int32_t W, int32_t slots, int32_t* bytes, int32_t* granted);
+
+/*
  * Which kernel ran the decoding loop of the last decode that used `workspace` (for tests and measurements; synchronises
  * `stream`).  Where two kernels are launched and the lengths decide between them on the device, it is the one that decoded.
  */

@@ -33,7 +33,7 @@ WIND_KERNELS_AUTO, WIND_KERNELS_SIMT, WIND_KERNELS_TENSOR = 0, 1, 2
 EXPORTS = [
     "wind_workspace_bytes", "wind_decode_greedy", "wind_decode_window_greedy", "wind_host_staging_bytes", "wind_decode_greedy_host",
     "wind_eval_joint_window", "wind_window_first_output", "wind_eval_joint_window_static", "wind_profile_decode", "wind_beam_workspace_bytes", "wind_beam_search", "wind_plan_batches", "wind_read_stats", "wind_set_trace", "wind_read_trace", "wind_debug_stall_barrier", "wind_set_kernels", "wind_status_string", "wind_last_cuda_error",
-    "wind_set_loop_options", "wind_debug_plan", "wind_bench_joint", "wind_refill_workspace_bytes", "wind_decode_greedy_refill", "wind_debug_loop_kernel",
+    "wind_set_loop_options", "wind_debug_plan", "wind_debug_cluster_smem", "wind_bench_joint", "wind_refill_workspace_bytes", "wind_decode_greedy_refill", "wind_debug_loop_kernel",
 ]
 
 _vp = C.c_void_p
@@ -153,6 +153,8 @@ def load_library():
     L.wind_set_loop_options.restype = None
     L.wind_debug_plan.argtypes = [mp, i32, i32, i32, i32, C.POINTER(wind_plan_t)]
     L.wind_debug_plan.restype = i32
+    L.wind_debug_cluster_smem.argtypes = [mp, i32, i32, C.POINTER(i32), C.POINTER(i32)]
+    L.wind_debug_cluster_smem.restype = i32
     L.wind_bench_joint.argtypes = [mp, i32, i32, i32, _vp, C.c_size_t, _vp, C.POINTER(wind_joint_bench_t)]
     L.wind_bench_joint.restype = i32
     L.wind_status_string.argtypes = [i32]
@@ -182,15 +184,28 @@ def wind_set_loop_options(resident: bool = True, joint_placement: int = -1, max_
     load_library().wind_set_loop_options(int(bool(resident)), int(joint_placement), int(max_joint_waves), int(dataflow))
 
 
-def wind_debug_plan(dims: Dict[str, int], B: int, W: int, sms: int = 148, smem_optin: int = 232448):
-    """The tile plan for bf16 model dimensions `dims` (D, E, P, L, H, V) on a device with the given SM count and
-    opt-in shared memory: host arithmetic only (no GPU needed).  Returns (status, dict of the plan's fields)."""
+def _model_of(dims: Dict[str, int], dtype: int = WIND_DT_BF16) -> wind_model_t:
+    """A model of dimensions `dims` (D, E, P, L, H, V) without weights, for the host-only entry points."""
     m = wind_model_t()
     for k in ("D", "E", "P", "L", "H", "V"):
         setattr(m, k, int(dims[k]))
     m.blank_id = int(dims.get("blank_id", dims["V"]))
     m.act = 0
-    m.dtype = WIND_DT_BF16
+    m.dtype = dtype
+    return m
+
+
+def wind_debug_cluster_smem(dims: Dict[str, int], W: int, slots: int):
+    """(status, bytes of shared memory a CTA of the cluster kernel asks for, bytes it may ask for): host arithmetic only."""
+    need, granted = C.c_int32(), C.c_int32()
+    st = load_library().wind_debug_cluster_smem(C.byref(_model_of(dims)), W, slots, C.byref(need), C.byref(granted))
+    return st, need.value, granted.value
+
+
+def wind_debug_plan(dims: Dict[str, int], B: int, W: int, sms: int = 148, smem_optin: int = 232448):
+    """The tile plan for bf16 model dimensions `dims` (D, E, P, L, H, V) on a device with the given SM count and
+    opt-in shared memory: host arithmetic only (no GPU needed).  Returns (status, dict of the plan's fields)."""
+    m = _model_of(dims)
     out = wind_plan_t()
     st = load_library().wind_debug_plan(C.byref(m), B, W, sms, smem_optin, C.byref(out))
     return st, out.as_dict()

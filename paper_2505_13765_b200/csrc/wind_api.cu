@@ -781,6 +781,17 @@ wind_status_t wind_debug_plan(const wind_model_t* m, int32_t B, int32_t W, int32
     return WIND_OK;
 }
 
+wind_status_t wind_debug_cluster_smem(const wind_model_t* m, int32_t W, int32_t slots, int32_t* bytes, int32_t* granted) {
+    wind_status_t s = check_model(m);
+    if (s != WIND_OK) return s;
+    if (!bytes || !granted || W < 1 || slots < 1) return WIND_ERR_INVALID_ARG;
+    if (m->dtype != WIND_DT_BF16 || !cl_fits(*m, W) || slots > (W <= 8 ? 8 : (W <= 16 ? 4 : 2))) return WIND_ERR_UNSUPPORTED;
+    uint32_t b = 0, g = 0;
+    cl_debug_smem(*m, W, slots, &b, &g);
+    *bytes = (int32_t)b; *granted = (int32_t)g;
+    return WIND_OK;
+}
+
 int32_t wind_set_trace(int32_t first_step) {
     int32_t prev = g_trace_step;
     g_trace_step = first_step < -1 ? -2 : first_step;

@@ -228,6 +228,9 @@ cudaError_t launch_set_t(const Call& c, const int32_t* t0);
 cudaError_t launch_gather_frames(const void* src, void* dst, const int32_t* enc_len, int B, int longest, size_t frame_bytes, size_t utt_bytes,
                                  cudaStream_t stream);   // src: device address of page-locked host memory
 cudaError_t launch_fill_z(const Call& c);   // measurement aid: fixed joint activations
+// cluster kernel (wind_loop_cl.cu): whether it takes a model and a window; its shared memory for a number of slots, and the most it is granted
+bool cl_fits(const wind_model_t& m, int W);
+void cl_debug_smem(const wind_model_t& m, int W, int slots, uint32_t* bytes, uint32_t* granted);
 
 // first-output distribution of a window (Eq. 1), in place on the window's logits
 // beam search (Algorithm 3): workspace regions behind the call's own layout, and the host-driven search

@@ -1141,6 +1141,23 @@ static uint32_t cl_smem_bytes(int P, int H, int NV, int slots, int wp, int layer
     }
     return bytes + 1024u;
 }
+// The most that a launch asks for: what every kernel is granted.  (The window's keys grow with its padding and the states with the
+// slots: with one layer one slot pair of 32 rows takes most, 219264 bytes against 212736 with eight slots of 8; with two 226944 against 224256.)
+static uint32_t cl_smem_most() {
+    uint32_t most = 0;
+    for (int layers = 1; layers <= 2; ++layers)
+        for (int wp = 8; wp <= 32; wp *= 2)
+            for (int slots = 1; slots <= 8 * CL_GROUPS / wp; ++slots) {
+                const uint32_t bytes = cl_smem_bytes(CL_MAX_DIM, CL_MAX_DIM, 16 * CL_MAX_LABELS, slots, wp, layers);
+                if (bytes > most) most = bytes;
+            }
+    return most;
+}
+static int cl_padded_window(int W) { return W <= 8 ? 8 : (W <= 16 ? 16 : 32); }
+void cl_debug_smem(const wind_model_t& m, int W, int slots, uint32_t* bytes, uint32_t* granted) {
+    *bytes = cl_smem_bytes(m.P, m.H, m.V + 1, slots, cl_padded_window(W), m.L);
+    *granted = cl_smem_most();
+}
 
 // clusters of 16 CTAs the current device holds at a time (one CTA per SM); 0: none
 static int cl_clusters() {
@@ -1151,7 +1168,7 @@ static int cl_clusters() {
         g_cl_clusters[dev] = -1;
         int optin = 0;
         if (cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) return 0;
-        const int want = (int)cl_smem_bytes(CL_MAX_DIM, CL_MAX_DIM, 16 * CL_MAX_LABELS, 8, 8, 2);
+        const int want = (int)cl_smem_most();
         if (want > optin - 1024) return 0;
         for (int k = 0; k < 16; ++k) {
             const void* fn = cl_fn(1 << (k & 3), k >> 2 & 1, 1 + (k >> 3));
@@ -1196,14 +1213,17 @@ static float other_step_us(const wind_model_t& m, const LoopPlan& pl, int B, int
     return 10.1f + 0.005f * H + 0.002f * rows + (pl.dataflow ? 6.5f : 3.f) * (float)(waves - 1);
 }
 
-// The shapes whose decoder fits one cluster: one LSTM layer, P and H multiples of 128 (a CTA's share is then whole 16-byte
-// pieces, and the K halves are equal) up to 640, at most 72 vocabulary entries per CTA, windows up to 32 rows.  Everything
-// else, and the FULL features (logits store, window-based decoding, timeline, forced loop modes), stays with loop_kernel.
-static bool cl_supported(const Call& c) {
-    const wind_model_t& m = c.m;
+// The shapes whose decoder fits one cluster (with two layers: one, and two clusters that all share): one or two LSTM layers, P and H
+// multiples of 128 (a CTA's share is then whole 16-byte pieces, and the K halves are equal) up to 640, at most 72 vocabulary entries per
+// CTA, windows up to 32 rows.  Everything else, and the FULL features (logits store, window-based decoding, timeline, forced loop
+// modes), stays with loop_kernel.
+bool cl_fits(const wind_model_t& m, int W) {
     const int nv = m.V + 1;
-    if (m.L > 2 || m.P % 128 || m.H % 128 || m.P > CL_MAX_DIM || m.H > CL_MAX_DIM || c.W > 32) return false;
-    if (cl_label_base(nv) + (cl_label_extra(nv) > 0 ? 8 : 0) > CL_MAX_LABELS) return false;
+    if (m.L > 2 || m.P % 128 || m.H % 128 || m.P > CL_MAX_DIM || m.H > CL_MAX_DIM || W > 32) return false;
+    return cl_label_base(nv) + (cl_label_extra(nv) > 0 ? 8 : 0) <= CL_MAX_LABELS;
+}
+static bool cl_supported(const Call& c) {
+    if (!cl_fits(c.m, c.W)) return false;
     if (c.mode != WIND_MODE_FIRST_NONBLANK || c.joint_iters > 0) return false;
     const LoopOptions o = loop_get_options();
     if (!o.resident || o.dataflow >= 0 || o.joint_placement >= 0) return false;
@@ -1231,7 +1251,7 @@ bool cl_plan(const Call& c, const LoopPlan& other, ClPlan* out) {
     const int n = c.N > 0 ? c.N : c.B, avail = c.m.L == 2 ? (cl_clusters() - 2 < CL_DECODERS ? cl_clusters() - 2 : CL_DECODERS) : cl_clusters();
     if (avail < 1) return false;
     ClPlan q{};
-    q.wp = c.W <= 8 ? 8 : (c.W <= 16 ? 16 : 32);
+    q.wp = cl_padded_window(c.W);
     // one slot per cluster as long as there are clusters, then more slots (a lock step of eight slots costs less than two of one)
     const int most = 8 * CL_GROUPS / q.wp;
     q.clusters = n < avail ? n : avail;

@@ -64,6 +64,8 @@ def test_remainder_units_round_like_the_others(pkg, seed, N, T, H, V, W, S):  # 
     (64, 30, 640, 640, 1024, 0, 8, 10),    # more utterances than slots: the queue, or the other kernel, as the lengths have it
     (60, 16, 256, 384, 1000, 1, 5, 3),
     (25, 20, 384, 256, 200, 0, 32, 3),     # widest window: ten slots, refilled
+    (6, 40, 640, 640, 1024, 0, 17, 3),     # padded window of 32 at the largest dimensions: the most shared memory, two slots in some clusters
+    (12, 40, 640, 640, 1024, 1, 32, 3),    # and more utterances than slots
     (50, 1, 640, 640, 200, 0, 2, 1),       # utterances of one frame: every update starts afresh
 ])
 def test_two_layer_cluster_edges(pkg, N, T, P, H, V, act, W, S):  # noqa: F811

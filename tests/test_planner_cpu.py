@@ -176,3 +176,21 @@ def test_no_utterance_group_spans_two_recording_ctas():
                     wide += pl["nl"] > 64 and B > 64
                     assert pl["nl"] <= 64 or pl["w_count"] <= 1, (P, L, B, pl)
     assert wide > 0
+
+
+def test_cluster_kernel_asks_for_no_more_shared_memory_than_it_is_granted():
+    seen = 0
+    for L in (1, 2):
+        for W, most in ((1, 8), (8, 8), (9, 4), (16, 4), (17, 2), (32, 2)):
+            for slots in range(1, most + 1):
+                for P in range(128, 641, 128):
+                    for H in range(128, 641, 128):
+                        for V in (127, 128, 300, 551, 552, 1015, 1024, 1030, 1151):
+                            st, need, granted = pkg.binding.wind_debug_cluster_smem(dict(D=64, E=64, P=P, L=L, H=H, V=V), W, slots)
+                            assert st == bd.WIND_OK and 0 < need <= granted, (L, W, slots, P, H, V, need, granted)
+                            assert granted <= 232448 - 1024          # beside the static part
+                            seen += need == granted
+    assert seen > 0                                                  # (and none too much)
+    large = dict(D=64, E=64, P=640, L=2, H=640, V=1024)
+    for dims, W, slots in ((large, 33, 1), (large, 8, 9), (large, 17, 3), (dict(large, L=3), 8, 1), (dict(large, P=192), 8, 1), (dict(large, V=1152), 8, 1)):
+        assert pkg.binding.wind_debug_cluster_smem(dims, W, slots)[0] == bd.WIND_ERR_UNSUPPORTED
