@@ -481,6 +481,19 @@ wind_status_t wind_debug_plan(const wind_model_t* m, int32_t B, int32_t W, int32
 wind_status_t wind_debug_cluster_smem(const wind_model_t* m, int32_t W, int32_t slots, int32_t* bytes, int32_t* granted);
 
 /*
+ * How the resident kernel of a beam search splits its work on a device with `sms` multiprocessors and `smem_optin` bytes of opt-in
+ * shared memory per block; host arithmetic only, for tests.  ahead: whether histories of coming iterations may fill up a command.
+ * WIND_ERR_UNSUPPORTED: the search runs as kernels per iteration.
+ */
+typedef struct {
+    int32_t rows, look;          /* most hypotheses of a command, most frames between them */
+    int32_t resident;            /* the gates' weights stay in shared memory */
+    int32_t updates, joint_rows; /* decoder updates and window rows of a pass */
+    int32_t smem_bytes;
+} wind_beam_plan_t;
+wind_status_t wind_debug_beam_plan(const wind_model_t* m, int32_t W, int32_t K, int32_t ahead, int32_t sms, int32_t smem_optin, wind_beam_plan_t* out);
+
+/*
  * Which kernel ran the decoding loop of the last decode that used `workspace` (for tests and measurements; synchronises
  * `stream`).  Where two kernels are launched and the lengths decide between them on the device, it is the one that decoded.
  */

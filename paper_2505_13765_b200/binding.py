@@ -33,7 +33,7 @@ WIND_KERNELS_AUTO, WIND_KERNELS_SIMT, WIND_KERNELS_TENSOR = 0, 1, 2
 EXPORTS = [
     "wind_workspace_bytes", "wind_decode_greedy", "wind_decode_window_greedy", "wind_host_staging_bytes", "wind_decode_greedy_host",
     "wind_eval_joint_window", "wind_window_first_output", "wind_eval_joint_window_static", "wind_profile_decode", "wind_beam_workspace_bytes", "wind_beam_search", "wind_plan_batches", "wind_read_stats", "wind_set_trace", "wind_read_trace", "wind_debug_stall_barrier", "wind_set_kernels", "wind_status_string", "wind_last_cuda_error",
-    "wind_set_loop_options", "wind_debug_plan", "wind_debug_cluster_smem", "wind_bench_joint", "wind_refill_workspace_bytes", "wind_decode_greedy_refill", "wind_debug_loop_kernel",
+    "wind_set_loop_options", "wind_debug_plan", "wind_debug_cluster_smem", "wind_debug_beam_plan", "wind_bench_joint", "wind_refill_workspace_bytes", "wind_decode_greedy_refill", "wind_debug_loop_kernel",
 ]
 
 _vp = C.c_void_p
@@ -90,6 +90,10 @@ class wind_joint_bench_t(C.Structure):
 
 class wind_trace_event_t(C.Structure):
     _fields_ = [("role", C.c_int32), ("phase", C.c_int32), ("event", C.c_int32), ("step", C.c_int32), ("clock", C.c_int64)]
+
+
+class wind_beam_plan_t(C.Structure):
+    _fields_ = [(n, C.c_int32) for n in ("rows", "look", "resident", "updates", "joint_rows", "smem_bytes")]
 
 
 _lib = None
@@ -155,6 +159,8 @@ def load_library():
     L.wind_debug_plan.restype = i32
     L.wind_debug_cluster_smem.argtypes = [mp, i32, i32, C.POINTER(i32), C.POINTER(i32)]
     L.wind_debug_cluster_smem.restype = i32
+    L.wind_debug_beam_plan.argtypes = [mp, i32, i32, i32, i32, i32, C.POINTER(wind_beam_plan_t)]
+    L.wind_debug_beam_plan.restype = i32
     L.wind_bench_joint.argtypes = [mp, i32, i32, i32, _vp, C.c_size_t, _vp, C.POINTER(wind_joint_bench_t)]
     L.wind_bench_joint.restype = i32
     L.wind_status_string.argtypes = [i32]
@@ -200,6 +206,13 @@ def wind_debug_cluster_smem(dims: Dict[str, int], W: int, slots: int):
     need, granted = C.c_int32(), C.c_int32()
     st = load_library().wind_debug_cluster_smem(C.byref(_model_of(dims)), W, slots, C.byref(need), C.byref(granted))
     return st, need.value, granted.value
+
+
+def wind_debug_beam_plan(dims: Dict[str, int], W: int, K: int, dtype: int, ahead: bool = False, sms: int = 148, smem_optin: int = 232448):
+    """(status, plan) of the beam search's resident kernel: host arithmetic only."""
+    out = wind_beam_plan_t()
+    st = load_library().wind_debug_beam_plan(C.byref(_model_of(dims, dtype)), W, K, int(ahead), sms, smem_optin, C.byref(out))
+    return st, {n: getattr(out, n) for n, _ in out._fields_}
 
 
 def wind_debug_plan(dims: Dict[str, int], B: int, W: int, sms: int = 148, smem_optin: int = 232448):

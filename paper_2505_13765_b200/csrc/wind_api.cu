@@ -792,6 +792,13 @@ wind_status_t wind_debug_cluster_smem(const wind_model_t* m, int32_t W, int32_t 
     return WIND_OK;
 }
 
+wind_status_t wind_debug_beam_plan(const wind_model_t* m, int32_t W, int32_t K, int32_t ahead, int32_t sms, int32_t smem_optin, wind_beam_plan_t* out) {
+    wind_status_t s = check_model(m);
+    if (s != WIND_OK) return s;
+    if (!out || W < 1 || W > kMaxWindow || K < 1 || K > kMaxBeam || sms < 1 || smem_optin < 4096) return WIND_ERR_INVALID_ARG;
+    return beam_step_debug_plan(*m, W, K, ahead != 0, sms, smem_optin, out) ? WIND_OK : WIND_ERR_UNSUPPORTED;
+}
+
 int32_t wind_set_trace(int32_t first_step) {
     int32_t prev = g_trace_step;
     g_trace_step = first_step < -1 ? -2 : first_step;

@@ -28,6 +28,7 @@
 #include "wind_ptx.cuh"
 
 #include <mutex>
+#include <type_traits>
 
 namespace wind {
 
@@ -43,17 +44,18 @@ struct BsPlan {
     int units, prows, labels;         // the most a CTA owns of each
     int k_l, k_p;                     // row lengths, rounded up to 32: of the gates (any layer), of W_pred
     int rows, look;                   // as in BeamShape
+    int quads;                        // fours of updates of a pass
     int zrows, k_z;                   // window rows of a joint pass; row length of the joint, rounded up to 32
     int resident;                     // the gates' weights of all layers stay; else a layer's are loaded in front of its use
     uint32_t layer, w_l, w_pred, w_out, bias, enc, x, z, total;   // layer: bytes of one layer's weights; z: later the window's logits
 };
-template <typename TW> static BsPlan bs_plan_with(int G, int W, int rows, int look, int resident, int E, int P, int L, int H, int NV, uint32_t budget) {
+template <typename TW> static BsPlan bs_plan_with(int G, int W, int rows, int look, int resident, int quads, int E, int P, int L, int H, int NV, uint32_t budget) {
     BsPlan s{};
     s.units = (P + G - 1) / G; s.prows = (H + G - 1) / G; s.labels = (NV + G - 1) / G;
     const int k0 = E + P, k1 = L > 1 ? 2 * P : 0, kmax = k0 > k1 ? k0 : k1;
     s.k_l = (kmax + 31) / 32 * 32; s.k_p = (P + 31) / 32 * 32;
     s.k_z = (H + 31) / 32 * 32;
-    s.rows = rows; s.look = look; s.resident = resident;
+    s.rows = rows; s.look = look; s.resident = resident; s.quads = quads;
     const int all = (rows * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
     unsigned long long off = 0;
     auto take = [&](unsigned long long bytes) { const unsigned long long o = off; off += (bytes + 15) / 16 * 16; return (uint32_t)o; };
@@ -64,7 +66,7 @@ template <typename TW> static BsPlan bs_plan_with(int G, int W, int rows, int lo
     s.w_out = take((unsigned long long)sizeof(TW) * ((s.labels + 3) / 4 * 4) * s.k_z);
     s.bias = take(4ull * (4 * L * s.units + s.prows + s.labels));
     s.enc = take((unsigned long long)sizeof(TW) * (W + look) * H);
-    const unsigned long long xa = (unsigned long long)sizeof(TW) * BS_UTTS * ((rows + BS_UTTS - 1) / BS_UTTS) * s.k_l, xb = 4ull * rows * H;
+    const unsigned long long xa = (unsigned long long)sizeof(TW) * BS_UTTS * quads * s.k_l, xb = 4ull * rows * H;
     s.x = take(xa > xb ? xa : xb);
     s.z = (uint32_t)off;
     const unsigned long long row = (unsigned long long)sizeof(TW) * s.k_z, window = 4ull * W * NV;
@@ -74,20 +76,32 @@ template <typename TW> static BsPlan bs_plan_with(int G, int W, int rows, int lo
     s.total = s.zrows == 0 || off > budget ? 0xffffffffu : (uint32_t)off;
     return s;
 }
-// The weights stay if at least four row groups fit beside them; then as many rows and frames ahead as fit likewise.
+// The weights stay if at least four row groups fit beside them, with all updates of a command in one pass or else in several; then as
+// many rows and frames ahead as fit likewise (those in one pass of updates).
 template <typename TW> static BsPlan bs_plan(int G, int W, int K, bool ahead, int E, int P, int L, int H, int NV, uint32_t budget) {
     auto good = [&](const BsPlan& s) {
         const int all = (s.rows * W + BS_ROWS - 1) / BS_ROWS * BS_ROWS;
         return s.total <= budget && s.zrows >= (s.resident && all > 16 ? 16 : BS_ROWS);
     };
-    BsPlan s = bs_plan_with<TW>(G, W, K, 0, 1, E, P, L, H, NV, budget);
-    if (!good(s)) s = bs_plan_with<TW>(G, W, K, 0, 0, E, P, L, H, NV, budget);
+    auto in_one = [](int rows) { return (rows + BS_UTTS - 1) / BS_UTTS; };
+    BsPlan s{};
+    s.total = 0xffffffffu;
+    for (int resident = 1; resident >= 0 && !good(s); --resident)
+        for (int quads = in_one(K); quads >= 1; --quads)
+            if (good(s = bs_plan_with<TW>(G, W, K, 0, resident, quads, E, P, L, H, NV, budget))) break;
     if (!good(s) || !ahead || K < 2) return s;
+    // Where weights stay only at the price of several passes, commands twice as long as the beam are worth more than that: two layers of
+    // 512 units in fp32, W = 8, K = 8: 46.2 us an iteration against 50.1 (K = 12, W = 4, where 16 rows are not twice the beam: 86 against 80).
+    if (s.resident && s.quads < in_one(K))
+        for (int look = kBeamLook; look >= 4 && kBeamRows >= 2 * K; look /= 2) {
+            const BsPlan a = bs_plan_with<TW>(G, W, kBeamRows, look, 0, in_one(kBeamRows), E, P, L, H, NV, budget);
+            if (good(a) && a.zrows >= 16) return a;
+        }
     // 12 rows and 12 frames, 16 and 12, 16 and 16: 250 frames at W = 8, beam 4: 28.8, 28.1, 27.2 ms; 200 at W = 16, beam 2: 18.8, 19.0, 18.7;
     // 300 at W = 4, beam 3: 19.9, 18.9, 18.4; 100 at W = 1, beam 4: 9.4, 8.4, 9.0
     for (int rows = kBeamRows; rows >= 8 && rows >= K; rows -= 4)
         for (int look = kBeamLook; look >= 4; look /= 2) {
-            const BsPlan a = bs_plan_with<TW>(G, W, rows, look, s.resident, E, P, L, H, NV, budget);
+            const BsPlan a = bs_plan_with<TW>(G, W, rows, look, s.resident, in_one(rows), E, P, L, H, NV, budget);
             if (good(a)) return a;
         }
     return s;
@@ -125,28 +139,15 @@ __device__ __forceinline__ unsigned long long bs_pair(uint32_t lo, uint32_t hi) 
 __device__ __forceinline__ void bs_fma_pair(unsigned long long& acc, unsigned long long a, unsigned long long b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
-// four values from shared memory, each twice
-template <typename TW> __device__ __forceinline__ void bs_four_twice(uint32_t at, unsigned long long* v) {
-    uint32_t x[4];
-    if constexpr (sizeof(TW) == 2) {
-        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(x[1]), "=r"(x[3]) : "r"(at));
-        x[0] = x[1] << 16; x[1] &= 0xffff0000u;
-        x[2] = x[3] << 16; x[3] &= 0xffff0000u;
-    } else {
-        asm("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(x[0]), "=r"(x[1]), "=r"(x[2]), "=r"(x[3]) : "r"(at));
-    }
-#pragma unroll
-    for (int j = 0; j < 4; ++j) v[j] = bs_pair(x[j], x[j]);
+// four values from shared memory: loaded, as fp32
+template <typename TW> __device__ __forceinline__ void bs_four(uint32_t at, uint32_t* v) {
+    if constexpr (sizeof(TW) == 2) asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v[1]), "=r"(v[3]) : "r"(at));
+    else asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
 }
-// four values from shared memory as two pairs
-template <typename TW> __device__ __forceinline__ void bs_two_pairs(uint32_t at, unsigned long long* v) {
+template <typename TW> __device__ __forceinline__ void bs_widen(uint32_t* v) {
     if constexpr (sizeof(TW) == 2) {
-        uint32_t a, b;
-        asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(a), "=r"(b) : "r"(at));
-        v[0] = bs_pair(a << 16, a & 0xffff0000u);
-        v[1] = bs_pair(b << 16, b & 0xffff0000u);
-    } else {
-        asm("ld.shared.v2.u64 {%0, %1}, [%2];" : "=l"(v[0]), "=l"(v[1]) : "r"(at));
+        v[0] = v[1] << 16; v[1] &= 0xffff0000u;
+        v[2] = v[3] << 16; v[3] &= 0xffff0000u;
     }
 }
 // four elements of a row that starts on 16 bytes, in shared or global memory
@@ -155,13 +156,16 @@ __device__ __forceinline__ float4 bs_quad(const __nv_bfloat16* p) {
     const uint2 v = *reinterpret_cast<const uint2*>(p);
     return make_float4(__uint_as_float(v.x << 16), __uint_as_float(v.x & 0xffff0000u), __uint_as_float(v.y << 16), __uint_as_float(v.y & 0xffff0000u));
 }
-// four elements of four rows (of type TW after rounding) to [k][4]
+// four elements of four rows (of type TW after rounding) to [k][4].  Neighbouring lanes' 64 bytes of fp32 lie behind one another: every
+// second lane begins a piece further on, so that eight lanes' stores meet all banks (in one order they took four times as long).
 __device__ __forceinline__ void bs_put(float* dst, const float4& a, const float4& b, const float4& c, const float4& d) {
-    float4* to = reinterpret_cast<float4*>(dst);
-    to[0] = make_float4(a.x, b.x, c.x, d.x);
-    to[1] = make_float4(a.y, b.y, c.y, d.y);
-    to[2] = make_float4(a.z, b.z, c.z, d.z);
-    to[3] = make_float4(a.w, b.w, c.w, d.w);
+    float4 t[4] = {make_float4(a.x, b.x, c.x, d.x), make_float4(a.y, b.y, c.y, d.y), make_float4(a.z, b.z, c.z, d.z), make_float4(a.w, b.w, c.w, d.w)};
+    const uint32_t first = (threadIdx.x >> 1) & 3u, at = smem_u32(dst);
+    if (first & 1u) { const float4 v = t[0]; t[0] = t[1]; t[1] = t[2]; t[2] = t[3]; t[3] = v; }
+    if (first & 2u) { float4 v = t[0]; t[0] = t[2]; t[2] = v; v = t[1]; t[1] = t[3]; t[3] = v; }
+#pragma unroll
+    for (uint32_t j = 0; j < 4; ++j)
+        asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(at + (((first + j) & 3u) << 4)), "f"(t[j].x), "f"(t[j].y), "f"(t[j].z), "f"(t[j].w) : "memory");
 }
 __device__ __forceinline__ void bs_put(__nv_bfloat16* dst, const float4& a, const float4& b, const float4& c, const float4& d) {
     uint4* to = reinterpret_cast<uint4*>(dst);
@@ -181,19 +185,43 @@ __device__ __noinline__ float2 bs_dots(uint32_t w, uint32_t x, uint32_t x_pitch,
     unsigned long long acc[Q][8];
 #pragma unroll
     for (int i = 0; i < 8 * Q; ++i) acc[i >> 3][i & 7] = 0ull;
-#pragma unroll(4 / Q)
-    for (int i = 0; i < steps; ++i) {
-        unsigned long long wv[4], xv[2];
-        bs_four_twice<TW>(w + 128u * (uint32_t)sizeof(TW) * i, wv);
+    // N steps' loads, then their arithmetic
+    auto some = [&](auto which, int i) {
+        constexpr int N = decltype(which)::value;
+        uint32_t wv[N][4], xv[N][Q][4];
 #pragma unroll
-        for (int h = 0; h < Q; ++h) {
-            bs_two_pairs<TW>(x + h * x_pitch + 128u * (uint32_t)sizeof(TW) * i, xv);
+        for (int n = 0; n < N; ++n) {
+            bs_four<TW>(w + 128u * (uint32_t)sizeof(TW) * (i + n), wv[n]);
 #pragma unroll
-            for (int j = 0; j < 4; ++j)
-#pragma unroll
-                for (int n = 0; n < 2; ++n) bs_fma_pair(acc[h][2 * j + n], wv[j], xv[n]);
+            for (int h = 0; h < Q; ++h) bs_four<TW>(x + h * x_pitch + 128u * (uint32_t)sizeof(TW) * (i + n), xv[n][h]);
         }
-    }
+#pragma unroll
+        for (int n = 0; n < N; ++n) {
+            unsigned long long ww[4];
+            bs_widen<TW>(wv[n]);
+#pragma unroll
+            for (int j = 0; j < 4; ++j) ww[j] = bs_pair(wv[n][j], wv[n][j]);
+#pragma unroll
+            for (int h = 0; h < Q; ++h) {
+                bs_widen<TW>(xv[n][h]);
+                const unsigned long long x0 = bs_pair(xv[n][h][0], xv[n][h][1]), x1 = bs_pair(xv[n][h][2], xv[n][h][3]);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    bs_fma_pair(acc[h][2 * j], ww[j], x0);
+                    bs_fma_pair(acc[h][2 * j + 1], ww[j], x1);
+                }
+            }
+        }
+    };
+    // (fp32 in steps of four written out: between phases that hold many registers the compiler otherwise let a step wait for its own
+    // loads, 40 steps 4600 cycles against 3600; bf16 was no faster by it)
+    constexpr int AT_ONCE = sizeof(TW) == 4 ? 4 / Q : 1;
+    int i = 0;
+    if constexpr (AT_ONCE > 1)
+#pragma unroll 1
+        for (; i + AT_ONCE <= steps; i += AT_ONCE) some(std::integral_constant<int, AT_ONCE>{}, i);
+#pragma unroll(4 / Q)
+    for (; i < steps; ++i) some(std::integral_constant<int, 1>{}, i);
     const int lane = threadIdx.x & 31;
     float out[2] = {0.f, 0.f};
 #pragma unroll
@@ -392,63 +420,72 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
 #pragma unroll 1
             for (int l = 0; l < p.L; ++l) {
                 const int nin = l == 0 ? p.E : P, K32 = (nin + P + 31) / 32 * 32;
-                // an item: one of this CTA's units for four updates
-                auto c_of = [&](int item) { return p.c_pool + (size_t)c_src[update(item / units, col)] * LP + l * P + (item % units) * G + cta; };
-                float c_in = warp < units * quads ? __ldcg(c_of(warp)) : 0.f;          // requested ahead of everything else
-                // x and the state before it: four elements of four updates at a time, all loads of a thread at once
                 const int K4 = K32 / 4;
-#pragma unroll 2
-                for (int i = tid; i < quads * K4; i += BS_THREADS) {
-                    const int quad = i / K4, k = 4 * (i - quad * K4);
-                    float4 x[BS_UTTS];
-#pragma unroll
-                    for (int u = 0; u < BS_UTTS; ++u) {
-                        const int uu = update(quad, u);
-                        if (k < nin && l == 0) x[u] = bs_quad(static_cast<const TW*>(p.emb) + (size_t)c_tok[uu] * p.E + k);
-                        else if (k < nin + P) x[u] = __ldcg(reinterpret_cast<const float4*>(p.h_pool + (size_t)(k < nin ? c_dst[uu] : c_src[uu]) * LP + (k < nin ? (l - 1) * P + k : l * P + k - nin)));
-                        else x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
-                    }
-                    bs_put(xs + 4 * (quad * M.k_l + k), x[0], x[1], x[2], x[3]);
-                }
-                asm volatile("cp.async.wait_all;" ::: "memory");
-                __syncthreads();
 #pragma unroll 1
-                for (int item = warp; item < units * quads; item += BS_WARPS) {
-                    const int quad = item / units, ui = item - quad * units, j = ui * G + cta;
-                    const float mine = bs_dots<TW, 1>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * (quad * M.k_l + lane)), 0u, K32 / 32).x + b_gate[4 * (l * M.units + ui) + grp];
-                    const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
-                                ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
-                    const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
-                    const float cc = cell_update_fc(gf, c_in, gi, gg);
-                    if ((lane & 25) == 0 && quad * BS_UTTS + col < nu) {
-                        const size_t to = (size_t)c_dst[quad * BS_UTTS + col] * LP + l * P + j;
-                        p.c_pool[to] = cc;
-                        p.h_pool[to] = go * tanhf(cc);
+                for (int q0 = 0; q0 < quads; q0 += M.quads) {
+                    const int here = min(M.quads, quads - q0);
+                    // an item: one of this CTA's units for four updates
+                    auto c_of = [&](int item) { return p.c_pool + (size_t)c_src[update(q0 + item / units, col)] * LP + l * P + (item % units) * G + cta; };
+                    float c_in = warp < units * here ? __ldcg(c_of(warp)) : 0.f;          // requested ahead of everything else
+                    if (q0 > 0) __syncthreads();
+                    // x and the state before it: four elements of four updates at a time, all loads of a thread at once
+#pragma unroll 2
+                    for (int i = tid; i < here * K4; i += BS_THREADS) {
+                        const int quad = i / K4, k = 4 * (i - quad * K4);
+                        float4 x[BS_UTTS];
+#pragma unroll
+                        for (int u = 0; u < BS_UTTS; ++u) {
+                            const int uu = update(q0 + quad, u);
+                            if (k < nin && l == 0) x[u] = bs_quad(static_cast<const TW*>(p.emb) + (size_t)c_tok[uu] * p.E + k);
+                            else if (k < nin + P) x[u] = __ldcg(reinterpret_cast<const float4*>(p.h_pool + (size_t)(k < nin ? c_dst[uu] : c_src[uu]) * LP + (k < nin ? (l - 1) * P + k : l * P + k - nin)));
+                            else x[u] = make_float4(0.f, 0.f, 0.f, 0.f);
+                        }
+                        bs_put(xs + 4 * (quad * M.k_l + k), x[0], x[1], x[2], x[3]);
                     }
-                    if (item + BS_WARPS < units * quads) c_in = __ldcg(c_of(item + BS_WARPS));
+                    asm volatile("cp.async.wait_all;" ::: "memory");
+                    __syncthreads();
+#pragma unroll 1
+                    for (int item = warp; item < units * here; item += BS_WARPS) {
+                        const int quad = item / units, ui = item - quad * units, j = ui * G + cta, at = (q0 + quad) * BS_UTTS + col;
+                        const float mine = bs_dots<TW, 1>(smem_u32(layer_at(l) + 4 * (ui * M.k_l + lane)), smem_u32(xs + 4 * (quad * M.k_l + lane)), 0u, K32 / 32).x + b_gate[4 * (l * M.units + ui) + grp];
+                        const float ai = __shfl_sync(0xffffffffu, mine, lane & 7), af = __shfl_sync(0xffffffffu, mine, 8 + (lane & 7)),
+                                    ag = __shfl_sync(0xffffffffu, mine, 16 + (lane & 7)), ao = __shfl_sync(0xffffffffu, mine, 24 + (lane & 7));
+                        const float gi = 1.f / (1.f + expf(-ai)), gf = 1.f / (1.f + expf(-af)), gg = tanhf(ag), go = 1.f / (1.f + expf(-ao));
+                        const float cc = cell_update_fc(gf, c_in, gi, gg);
+                        if ((lane & 25) == 0 && at < nu) {
+                            const size_t to = (size_t)c_dst[at] * LP + l * P + j;
+                            p.c_pool[to] = cc;
+                            p.h_pool[to] = go * tanhf(cc);
+                        }
+                        if (item + BS_WARPS < units * here) c_in = __ldcg(c_of(item + BS_WARPS));
+                    }
                 }
                 arrive();
                 if (!M.resident && l + 1 < p.L) load_layer(l + 1);
                 if (!wait()) return;
             }
             // ---- pred_proj of this CTA's joint units ----
-            const int K4 = M.k_p / 4;
-#pragma unroll 2
-            for (int i = tid; i < quads * K4; i += BS_THREADS) {
-                const int quad = i / K4, k = 4 * (i - quad * K4);
-                float4 x[BS_UTTS];
-#pragma unroll
-                for (int u = 0; u < BS_UTTS; ++u)
-                    x[u] = k < P ? __ldcg(reinterpret_cast<const float4*>(p.h_pool + (size_t)c_dst[update(quad, u)] * LP + (p.L - 1) * P + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
-                bs_put(xs + 4 * (quad * M.k_p + k), x[0], x[1], x[2], x[3]);
-            }
-            __syncthreads();
-            const int pgs = (prows + 3) / 4;
+            const int K4 = M.k_p / 4, pgs = (prows + 3) / 4;
 #pragma unroll 1
-            for (int item = warp; item < pgs * quads; item += BS_WARPS) {
-                const int quad = item / pgs, pg = item - quad * pgs, pi = pg * 4 + grp, o = min(pi, prows - 1) * G + cta;
-                const float mine = bs_dots<TW, 1>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * (quad * M.k_p + lane)), 0u, M.k_p / 32).x + b_pred[min(pi, prows - 1)];
-                if ((lane & 1) == 0 && pi < prows && quad * BS_UTTS + col < nu) p.g_pool[(size_t)c_dst[quad * BS_UTTS + col] * H + o] = mine;
+            for (int q0 = 0; q0 < quads; q0 += M.quads) {
+                const int here = min(M.quads, quads - q0);
+                if (q0 > 0) __syncthreads();
+#pragma unroll 2
+                for (int i = tid; i < here * K4; i += BS_THREADS) {
+                    const int quad = i / K4, k = 4 * (i - quad * K4);
+                    float4 x[BS_UTTS];
+#pragma unroll
+                    for (int u = 0; u < BS_UTTS; ++u)
+                        x[u] = k < P ? __ldcg(reinterpret_cast<const float4*>(p.h_pool + (size_t)c_dst[update(q0 + quad, u)] * LP + (p.L - 1) * P + k)) : make_float4(0.f, 0.f, 0.f, 0.f);
+                    bs_put(xs + 4 * (quad * M.k_p + k), x[0], x[1], x[2], x[3]);
+                }
+                __syncthreads();
+#pragma unroll 1
+                for (int item = warp; item < pgs * here; item += BS_WARPS) {
+                    const int quad = item / pgs, pg = item - quad * pgs, pi = pg * 4 + grp, o = min(pi, prows - 1) * G + cta, at = (q0 + quad) * BS_UTTS + col;
+                    const float mine = bs_dots<TW, 1>(smem_u32(w_pred + 4 * (pg * M.k_p + lane)), smem_u32(xs + 4 * (quad * M.k_p + lane)), 0u, M.k_p / 32).x + b_pred[min(pi, prows - 1)];
+                    if ((lane & 1) == 0 && pi < prows && at < nu) p.g_pool[(size_t)c_dst[at] * H + o] = mine;
+                }
             }
             arrive();
             if (!wait()) return;
@@ -493,34 +530,43 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
                     e4[j] = encs + min(c_t[b] - t0 + row - b * n, span - 1) * H;
                     g4[j] = gs + b * H;
                 }
+                auto act = [&](const float4& a, const float4& g) {
+                    const float4 v = make_float4(a.x + g.x, a.y + g.y, a.z + g.z, a.w + g.w);
+                    return p.act == WIND_ACT_RELU ? make_float4(fmaxf(v.x, 0.f), fmaxf(v.y, 0.f), fmaxf(v.z, 0.f), fmaxf(v.w, 0.f)) : bs_tanh(v);
+                };
+                if constexpr (sizeof(TW) == 4) {                // element by element: nothing to turn round, and even shares of k
+#pragma unroll 2
+                    for (int k = lane + 32 * (item - rg * cut); k < M.k_z; k += 32 * cut)
+                        *reinterpret_cast<float4*>(za + 4 * (rg * M.k_z + k)) =
+                            k < H ? act(make_float4(e4[0][k], e4[1][k], e4[2][k], e4[3][k]), make_float4(g4[0][k], g4[1][k], g4[2][k], g4[3][k])) : make_float4(0.f, 0.f, 0.f, 0.f);
+                } else {
 #pragma unroll 1
-                for (int k = 4 * (lane + 32 * (item - rg * cut)); k < M.k_z; k += 128 * cut) {
-                    float4 z[4];
+                    for (int k = 4 * (lane + 32 * (item - rg * cut)); k < M.k_z; k += 128 * cut) {
+                        float4 z[4];
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
-                        z[j] = make_float4(0.f, 0.f, 0.f, 0.f);
-                        if (k < H) {
-                            const float4 a = bs_quad(e4[j] + k), g = bs_quad(g4[j] + k);
-                            z[j] = make_float4(a.x + g.x, a.y + g.y, a.z + g.z, a.w + g.w);
-                            if (p.act == WIND_ACT_RELU) z[j] = make_float4(fmaxf(z[j].x, 0.f), fmaxf(z[j].y, 0.f), fmaxf(z[j].z, 0.f), fmaxf(z[j].w, 0.f));
-                            else z[j] = bs_tanh(z[j]);
+                        for (int j = 0; j < 4; ++j) {
+                            z[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+                            if (k < H) z[j] = act(bs_quad(e4[j] + k), bs_quad(g4[j] + k));
                         }
+                        bs_put(za + 4 * (rg * M.k_z + k), z[0], z[1], z[2], z[3]);
                     }
-                    bs_put(za + 4 * (rg * M.k_z + k), z[0], z[1], z[2], z[3]);
                 }
             }
             __syncthreads();
-            const int lgs = (labels + 3) / 4, pairs = (nr4 + 1) / 2;
+            // (fp32: one row group an item while that gives every warp one at most.  Large models have passes of four groups, and in pairs
+            // four of the sixteen warps had all the work)
+            const int lgs = (labels + 3) / 4, per = sizeof(TW) == 4 && lgs * nr4 <= BS_WARPS ? 1 : 2, items = lgs * ((nr4 + per - 1) / per);
 #pragma unroll 1
-            for (int item = warp; item < lgs * pairs; item += BS_WARPS) {
-                const int rg = 2 * (item / lgs), lg = item % lgs, li = lg * 4 + grp, v = min(li, labels - 1) * G + cta;
+            for (int item = warp; item < items; item += BS_WARPS) {
+                const int rg = per * (item / lgs), lg = item % lgs, li = lg * 4 + grp, v = min(li, labels - 1) * G + cta;
                 const uint32_t pitch = rg + 1 < nr4 ? 4u * (uint32_t)sizeof(TW) * (uint32_t)M.k_z : 0u;      // (an odd number of groups: the last one twice)
-                const float2 both = bs_dots<TW, 2>(smem_u32(w_out + 4 * (lg * M.k_z + lane)), smem_u32(za + 4 * (rg * M.k_z + lane)), pitch, M.k_z / 32);
+                const uint32_t wa = smem_u32(w_out + 4 * (lg * M.k_z + lane)), xa = smem_u32(za + 4 * (rg * M.k_z + lane));
+                const float2 both = per == 2 ? bs_dots<TW, 2>(wa, xa, pitch, M.k_z / 32) : bs_dots<TW, 1>(wa, xa, 0u, M.k_z / 32);
                 const float bias = b_out[min(li, labels - 1)];
 #pragma unroll
                 for (int h = 0; h < 2; ++h) {
                     const int at = (rg + h) * BS_ROWS + col, row = r0 + at, b = row / n;
-                    if ((lane & 1) == 0 && at < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = (h ? both.y : both.x) + bias;
+                    if (h < per && (lane & 1) == 0 && at < nr && li < labels) p.logits[((size_t)b * p.W + (row - b * n)) * NV + v] = (h ? both.y : both.x) + bias;
                 }
             }
         }
@@ -530,14 +576,15 @@ __global__ void __launch_bounds__(BS_THREADS, 1) beam_step_kernel(const BsParams
             // ---- Eq. (1) for hypothesis `cta`, the window's logits in shared memory ----
             const float* src = p.logits + (size_t)cta * p.W * NV;
             const int n = min(p.W, p.T - c_t[cta]), total = n * NV;
+            constexpr int AT_ONCE = sizeof(TW) == 4 ? 9 : 16;        // (with twenty the other phases were short of registers)
 #pragma unroll 1
-            for (int i0 = tid; i0 < total; i0 += 20 * BS_THREADS) {
-                float v[20];
+            for (int i0 = tid; i0 < total; i0 += AT_ONCE * BS_THREADS) {
+                float v[AT_ONCE];
 #pragma unroll
-                for (int j = 0; j < 20; ++j)
+                for (int j = 0; j < AT_ONCE; ++j)
                     if (i0 + j * BS_THREADS < total) v[j] = __ldcg(src + i0 + j * BS_THREADS);
 #pragma unroll
-                for (int j = 0; j < 20; ++j)
+                for (int j = 0; j < AT_ONCE; ++j)
                     if (i0 + j * BS_THREADS < total) zs[i0 + j * BS_THREADS] = v[j];
             }
             __syncthreads();
@@ -668,6 +715,16 @@ bool beam_step_supported(const Call& c) {
     int optin = 0, sms = 0;
     if (bs_device(&optin) != cudaSuccess || loop_sm_count(&sms) != cudaSuccess) { cudaGetLastError(); return false; }
     return c.B <= sms && bs_plan_of(c, false, sms, (uint32_t)optin - 4096u).total <= (uint32_t)optin - 4096u;
+}
+
+// the same on a device of `sms` SMs and `optin` bytes of shared memory a block, alignments aside
+bool beam_step_debug_plan(const wind_model_t& m, int W, int K, bool ahead, int sms, int optin, wind_beam_plan_t* out) {
+    const uint32_t budget = (uint32_t)optin - 4096u;
+    auto plan = [&](auto t) { return bs_plan<decltype(t)>(sms, W, K, ahead, m.E, m.P, m.L, m.H, m.V + 1, budget); };
+    const BsPlan s = m.dtype == WIND_DT_BF16 ? plan(__nv_bfloat16()) : plan(0.f);
+    if (m.E % 8 || m.P % 8 || m.H % 8 || K > sms || s.total > budget) return false;
+    *out = wind_beam_plan_t{s.rows, s.look, s.resident, 4 * s.quads, s.zrows, (int32_t)s.total};
+    return true;
 }
 
 // (of a call that beam_step_supported takes)

@@ -263,6 +263,7 @@ struct BeamMail {
 struct BeamShape { int rows, look; };  // most hypotheses of a command, most frames between them (0: they all stand at one)
 BeamShape beam_step_shape(const Call& c, bool ahead);
 bool beam_step_supported(const Call& c);
+bool beam_step_debug_plan(const wind_model_t& m, int W, int K, bool ahead, int sms, int optin, wind_beam_plan_t* out);
 cudaError_t beam_step(const Call& c, const BeamShape& shape, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,
                       float* h_pool, float* c_pool, float* g_pool, float* logits);
 uint32_t beam_step_arrivals(const Call& c, int n_update);

@@ -43,6 +43,26 @@ def test_beam_iteration_kernel(pkg, E, P, L, H, V, act, W, K, S):  # noqa: F811
     assert decided >= (1 if K < 8 else 0)
 
 
+@pytest.mark.parametrize("E,P,L,H,V,W,K,S,updates", [
+    (640, 640, 1, 96, 200, 32, 16, 2, 12),  # weights that stay beside twelve of the sixteen updates: two passes
+    (512, 512, 2, 512, 300, 8, 12, 2, 4),   # two layers beside four updates; joint items of one row group
+])
+def test_updates_in_passes_beside_resident_weights(pkg, E, P, L, H, V, W, K, S, updates):  # noqa: F811
+    plan = pkg.binding.wind_debug_beam_plan(dict(D=16, E=E, P=P, L=L, H=H, V=V), W, K, pkg.binding.WIND_DT_F32, True)[1]
+    assert plan["resident"] and plan["updates"] == updates < K
+    r = np.random.default_rng(9603 + K)
+    w = random_weights(r, 16, E, P, L, H, V, act=0, blank_bias=2.5, bias_scale=0.1)
+    w["dtype"] = "f32"
+    T = 3
+    enc = r.standard_normal((T, 16)).astype(np.float32)
+    want, gap, steps = oracle.beam_search(oracle.Model(w), enc, T, W, K, S, max_hyps=256)
+    got, gsteps, st = pkg.wind_beam_search(pkg.WindModel(w), enc, W, K, S, max_hyps=256)
+    assert st == 0 and gap > 2e-5            # (every pruning is decidable in fp32)
+    a, b = ({tuple(int(x) for x in h[0]): h for h in hyps} for hyps in (want, got))
+    assert gsteps == steps and set(a) == set(b)
+    assert all(abs(a[k][2] - b[k][2]) < 1e-4 and list(a[k][1]) == list(b[k][1]) for k in a)
+
+
 def search(pkg, model, enc, W, K, S, short):
     """wind_beam_search with a workspace that is `short` bytes smaller: (tokens, frames, lengths, scores, iterations)."""
     L = pkg.load_library()

@@ -194,3 +194,30 @@ def test_cluster_kernel_asks_for_no_more_shared_memory_than_it_is_granted():
     large = dict(D=64, E=64, P=640, L=2, H=640, V=1024)
     for dims, W, slots in ((large, 33, 1), (large, 8, 9), (large, 17, 3), (dict(large, L=3), 8, 1), (dict(large, P=192), 8, 1), (dict(large, V=1152), 8, 1)):
         assert pkg.binding.wind_debug_cluster_smem(dims, W, slots)[0] == bd.WIND_ERR_UNSUPPORTED
+
+
+# Beam search in one kernel: per (W, K) whether it takes the search, and with the gates' weights resident ("r") or loaded per command ("l").
+LARGE, XL = dict(D=512, E=640, P=640, L=1, H=640, V=1024), dict(D=1024, E=640, P=640, L=2, H=640, V=1024)
+U512, X512 = dict(D=512, E=512, P=512, L=1, H=512, V=4096), dict(D=512, E=512, P=512, L=2, H=512, V=1024)
+BEAMS = [(1, 4), (1, 16), (4, 4), (4, 8), (4, 12), (4, 16), (8, 4), (8, 8), (8, 12), (8, 16), (16, 4), (16, 16)]
+
+
+@pytest.mark.parametrize("dims,dtype,taken", [
+    (LARGE, bd.WIND_DT_F32, "r r r r r l r r l - - -"),
+    (XL, bd.WIND_DT_F32, "l l l l l l l l l - - -"),
+    (U512, bd.WIND_DT_F32, "r r r r - - - - - - - -"),
+    (X512, bd.WIND_DT_F32, "r r r r r l r r l l l l"),
+    (LARGE, bd.WIND_DT_BF16, "r r r r r r r r r r r r"),
+    (XL, bd.WIND_DT_BF16, "r r r r r r r r r r r l"),
+])
+def test_beam_searches_that_one_kernel_takes(dims, dtype, taken):
+    for (W, K), want in zip(BEAMS, taken.split()):
+        st, plan = pkg.binding.wind_debug_beam_plan(dims, W, K, dtype)
+        assert ("-" if st else "r" if plan["resident"] else "l") == want, (W, K, plan)
+        for ahead in (False, True):              # evaluating ahead neither refuses a search nor gives it less
+            s, p = pkg.binding.wind_debug_beam_plan(dims, W, K, dtype, ahead)
+            assert s == st
+            if st == bd.WIND_OK:
+                assert p["rows"] >= K and p["updates"] >= 1 and p["joint_rows"] >= 4 and p["smem_bytes"] <= 232448 - 4096
+                assert p["resident"] == plan["resident"] or p["rows"] >= 2 * K
+                assert (p["look"] > 0) or p["rows"] == K
