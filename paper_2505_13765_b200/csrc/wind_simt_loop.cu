@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(ST_THREADS, 1) simt_tiny_kernel(const SimtLoop
     for (int i = tid; i < 65; i += ST_THREADS) s_hist[i] = 0;
 
     // (up to here, 11 us, under the encoder projection: the weights are the caller's)
-    wait_for_previous();
+    wait_for_previous();                           // (what follows reads nothing by __ldg)
     if (p.ctrl->bad_input) return;                 // a length outside [0, T]: nothing is read through it
     const int warps = (NV + 7) / 8;                                 // that have labels
     s_key[warp][lane] = 0ull;
@@ -994,7 +994,9 @@ __global__ void __launch_bounds__(ST_THREADS, 1) simt_tiny_kernel(const SimtLoop
         };
         const TW* enc = static_cast<const TW*>(p.enc_proj) + (size_t)utt * p.T * H;
         const int k_enc = tid & 63;
-        auto frame = [&](int f) { return k_enc < H ? (float)__ldg(enc + (size_t)f * H + k_enc) : 0.f; };
+        // (an ordinary load: the kernel before this one may still have been writing enc_proj when this one began, and __ldg is only for
+        // what nobody writes in a kernel's lifetime)
+        auto frame = [&](int f) { return k_enc < H ? (float)enc[(size_t)f * H + k_enc] : 0.f; };
         int have = min(len, 2 * p.W);                               // frames that are in the ring or on their way
         __syncthreads();
         if (tid < ST_MAX) s_h[0][tid] = 0.f;

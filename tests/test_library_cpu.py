@@ -177,3 +177,17 @@ def test_product_path_does_not_touch_the_oracle():
             if f.endswith((".py", ".cu", ".cuh", ".h")):
                 src = open(os.path.join(dirpath, f)).read()
                 assert "oracle" not in src, f
+
+
+def test_overlapped_kernels_read_nothing_by_ldg_behind_their_wait():
+    # A kernel launched under the one before it shares that one's lifetime: what the other writes is not read-only for it.
+    csrc = os.path.join(ROOT, "paper_2505_13765_b200", "csrc")
+    kernels = 0
+    for name in sorted(os.listdir(csrc)):
+        text = open(os.path.join(csrc, name)).read()
+        for kernel in re.findall(r"^__global__ .*?^}", text, flags=re.S | re.M):
+            code = re.sub(r"//[^\n]*", "", kernel)
+            if "wait_for_previous();" in code:
+                kernels += 1
+                assert "__ldg" not in code.split("wait_for_previous();", 1)[1], name
+    assert kernels >= 2
