@@ -343,7 +343,7 @@ wind_status_t wind_profile_decode(const wind_model_t* m, const void* enc, const 
  *              (at most max_hyps, best first); a hypothesis longer than max_out is cut in the token arrays, its
  *              length is reported in full.  n_steps (may be null): iterations of the loop.
  *   workspace  DEVICE, wind_beam_workspace_bytes(m, T, W, K, max_symbols); 256-byte aligned.  (Without the part that
- *              evaluating ahead takes the search runs too, more slowly.)
+ *              evaluating ahead takes, 512 states and logits of up to 16 windows, the search runs too, more slowly.)
  * WIND_ERR_WORKSPACE also when the pool of decoder states (sized for K (W + 2) (min(max_symbols, 32) + 2) live
  * hypotheses) runs out.
  */

@@ -245,28 +245,28 @@ BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, s
     BeamLayout L{};
     size_t off = base;
     auto take = [&](size_t bytes) { size_t o = off; off = align_up(off + bytes); return o; };
-    const int s_eff = S < 32 ? S : 32;
-    L.own.slots = K * (W + 2) * (s_eff + 2) + 2 * K + 2;
-    L.own.h_pool = take(sizeof(float) * (size_t)L.own.slots * m.L * m.P);
-    L.own.c_pool = take(sizeof(float) * (size_t)L.own.slots * m.L * m.P);
-    L.own.g_pool = take(sizeof(float) * (size_t)L.own.slots * m.H);
     L.ints = take(sizeof(int32_t) * 8 * (size_t)K);
-    L.own.logits = take(sizeof(float) * (size_t)K * W * (m.V + 1));
     L.top_label = take(sizeof(int32_t) * 3 * (size_t)K * K);   // labels, offsets, log-probabilities: one block, one copy
     L.top_jump = L.top_label + sizeof(int32_t) * (size_t)K * K;
     L.top_logp = L.top_jump + sizeof(int32_t) * (size_t)K * K;
     L.relay = take(sizeof(uint64_t) * kBeamWords);
-    L.need = L.total = off;
+    // The pools come last: a search has them in one of two sizes, from the same place on.
+    const size_t pools = off;
+    auto pool = [&](BeamPools& p, int slots, int rows) {
+        off = pools;
+        p.slots = slots;
+        p.rows = rows;
+        p.h_pool = take(sizeof(float) * (size_t)slots * m.L * m.P);
+        p.c_pool = take(sizeof(float) * (size_t)slots * m.L * m.P);
+        p.g_pool = take(sizeof(float) * (size_t)slots * m.H);
+        p.logits = take(sizeof(float) * (size_t)rows * W * (m.V + 1));
+        return off;
+    };
+    const int s_eff = S < 32 ? S : 32;
+    L.need = L.total = pool(L.own, K * (W + 2) * (s_eff + 2) + 2 * K + 2, K);
     // (a workspace of `need` bytes is enough: a command then has only the hypotheses of its iteration)
-    if (K > 1) {
-        const int rows = K > kBeamRows ? K : kBeamRows;
-        L.ahead.slots = L.own.slots + 32 * rows;
-        L.ahead.h_pool = take(sizeof(float) * (size_t)L.ahead.slots * m.L * m.P);
-        L.ahead.c_pool = take(sizeof(float) * (size_t)L.ahead.slots * m.L * m.P);
-        L.ahead.g_pool = take(sizeof(float) * (size_t)L.ahead.slots * m.H);
-        L.ahead.logits = take(sizeof(float) * (size_t)rows * W * (m.V + 1));
-        L.total = off;
-    }
+    const BeamShape most = beam_step_most(m, W, K);
+    if (most.look > 0) L.total = pool(L.ahead, L.own.slots + 32 * most.rows, most.rows);
     return L;
 }
 
@@ -280,7 +280,8 @@ wind_status_t beam_search_run(Call& cb, const BeamLayout& bl, bool ahead, int K,
     cudaStream_t st = cb.stream;
     uint8_t* ws = cb.ws;
     const bool resident = beam_step_supported(cb);
-    const BeamShape shape = resident ? beam_step_shape(cb, ahead && !prefix_search) : BeamShape{K, 0};
+    BeamShape shape = resident ? beam_step_shape(cb, ahead && !prefix_search) : BeamShape{K, 0};
+    if (shape.look > 0 && shape.rows > bl.ahead.rows) shape = beam_step_shape(cb, false);
     const int R = shape.rows;
     const BeamPools& pools = shape.look > 0 ? bl.ahead : bl.own;
     float* h_pool = reinterpret_cast<float*>(ws + pools.h_pool);

@@ -727,6 +727,19 @@ bool beam_step_debug_plan(const wind_model_t& m, int W, int K, bool ahead, int s
     return true;
 }
 
+// (without a device: on a B200.  No context is made for this question.)
+BeamShape beam_step_most(const wind_model_t& m, int W, int K) {
+    int dev = 0, optin = 0, sms = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+        cudaGetLastError();
+        optin = 232448; sms = 148;
+    }
+    wind_beam_plan_t plan;
+    if (!beam_step_debug_plan(m, W, K, true, sms, optin, &plan)) return {K, 0};
+    return {plan.rows, plan.look};
+}
+
 // (of a call that beam_step_supported takes)
 BeamShape beam_step_shape(const Call& c, bool ahead) {
     int optin = 0, sms = 0;

@@ -237,10 +237,10 @@ void cl_debug_smem(const wind_model_t& m, int W, int slots, uint32_t* bytes, uin
 struct BeamPools {
     size_t h_pool, c_pool, g_pool;   // fp32 [slots][L][P] x 2, [slots][H]: decoder states of live hypotheses and their pred_proj
     size_t logits;                   // fp32 [hypotheses of a command][W][V+1]
-    int slots;
+    int slots, rows;                 // hypotheses of a command: rows
 };
 struct BeamLayout {
-    BeamPools own, ahead;            // ahead, behind everything else: for commands with hypotheses of later iterations
+    BeamPools own, ahead;            // one or the other; ahead: for commands with hypotheses of later iterations
     size_t ints;                     // int32 [8][K] per-iteration index arrays
     size_t top_label, top_jump, top_logp;   // [K][K]
     size_t relay;                    // uint64 [kBeamWords]
@@ -262,6 +262,7 @@ struct BeamMail {
 };
 struct BeamShape { int rows, look; };  // most hypotheses of a command, most frames between them (0: they all stand at one)
 BeamShape beam_step_shape(const Call& c, bool ahead);
+BeamShape beam_step_most(const wind_model_t& m, int W, int K);         // what a call with these shapes may come to on the current device
 bool beam_step_supported(const Call& c);
 bool beam_step_debug_plan(const wind_model_t& m, int W, int K, bool ahead, int sms, int optin, wind_beam_plan_t* out);
 cudaError_t beam_step(const Call& c, const BeamShape& shape, BeamMail* mail, unsigned long long* relay, uint32_t first_seq, uint32_t bar_base,

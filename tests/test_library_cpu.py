@@ -191,3 +191,22 @@ def test_overlapped_kernels_read_nothing_by_ldg_behind_their_wait():
                 kernels += 1
                 assert "__ldg" not in code.split("wait_for_previous();", 1)[1], name
     assert kernels >= 2
+
+
+@pytest.mark.parametrize("kw,W,K,S,rows", [
+    (dict(), 8, 4, 10, 16),                       # evaluates ahead: sixteen hypotheses a command
+    (dict(), 8, 1, 10, 0),                        # nothing to evaluate ahead
+    (dict(dtype=0), 8, 4, 10, 0),                 # no room for it beside fp32 weights
+    (dict(dtype=0), 1, 8, 10, 12),
+    (dict(L=2), 64, 16, 32, 0),                   # windows that only kernels per iteration take
+    (dict(P=644), 8, 4, 10, 0),                   # rows that are no multiple of eight: likewise
+])
+def test_beam_workspace_has_one_pool_of_states(lib, kw, W, K, S, rows):
+    m = large_model(**kw)
+    T = 300
+    n = C.c_size_t(0)
+    assert lib.wind_beam_workspace_bytes(C.byref(m), T, W, K, S, C.byref(n)) == bd.WIND_OK
+    slots = K * (W + 2) * (S + 2 if S < 32 else 34) + 2 * K + 2 + 32 * rows
+    floats = slots * (2 * m.L * m.P + m.H) + max(rows, K) * W * (m.V + 1)
+    rest = n.value - pkg.wind_workspace_bytes(m, K, T, W) - 4 * floats
+    assert 0 <= rest <= 12 * 256 + 32 * K + 12 * K * K + 8 * (4 + 5 * 16)     # index arrays, and each region up to the next 256 bytes
