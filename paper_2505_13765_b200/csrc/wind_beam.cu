@@ -263,8 +263,10 @@ BeamLayout make_beam_layout(const wind_model_t& m, int T, int W, int K, int S, s
         return off;
     };
     const int s_eff = S < 32 ? S : 32;
-    L.need = L.total = pool(L.own, K * (W + 2) * (s_eff + 2) + 2 * K + 2, K);
-    // (a workspace of `need` bytes is enough: a command then has only the hypotheses of its iteration)
+    L.need = pool(L.own, K * (W + 2) * (s_eff + 2) + 2 * K + 2, K);
+    // A workspace of `need` bytes is enough: a command then has only the hypotheses of its iteration.  (Asked for is a piece more at the
+    // least, so that what is left of an unaligned block behind its first aligned address is enough too.)
+    L.total = L.need + kAlign;
     const BeamShape most = beam_step_most(m, W, K);
     if (most.look > 0) L.total = pool(L.ahead, L.own.slots + 32 * most.rows, most.rows);
     return L;

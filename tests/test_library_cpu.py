@@ -209,4 +209,4 @@ def test_beam_workspace_has_one_pool_of_states(lib, kw, W, K, S, rows):
     slots = K * (W + 2) * (S + 2 if S < 32 else 34) + 2 * K + 2 + 32 * rows
     floats = slots * (2 * m.L * m.P + m.H) + max(rows, K) * W * (m.V + 1)
     rest = n.value - pkg.wind_workspace_bytes(m, K, T, W) - 4 * floats
-    assert 0 <= rest <= 12 * 256 + 32 * K + 12 * K * K + 8 * (4 + 5 * 16)     # index arrays, and each region up to the next 256 bytes
+    assert 0 <= rest <= 13 * 256 + 32 * K + 12 * K * K + 8 * (4 + 5 * 16)     # index arrays, and each region up to the next 256 bytes
