@@ -118,6 +118,7 @@ __device__ __noinline__ void cl_recurrent(const CUtensorMap& hx_map, const ClPar
             const uint32_t ready = __ballot_sync(0xffffffffu, on && n != total && mbar_test(&bar_full[c], n & 1u));
             if (__any_sync(0xffffffffu, s_abort) || __all_sync(0xffffffffu, !on || n == total)) break;
             if (ready) {
+                __syncwarp();                             // one lane has seen the barrier complete, all read what it stands for
                 work(ready);
                 n += (ready >> lane) & 1u;
             }
