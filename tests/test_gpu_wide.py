@@ -19,6 +19,8 @@ pytestmark = pytest.mark.gpu
     (33, 20, 64, 128, 320, 1024, 1000, 0, 1, 5),    # window of one frame, 64-row state box
     (9, 24, 64, 64, 1024, 640, 8000, 0, 16, 3),     # ten K blocks: the last stage of z is cut short, one accumulator
     (3, 24, 64, 64, 512, 896, 10000, 0, 10, 2),     # fourteen, two of them in shared memory; boxes of 32 and 16 rows
+    (33, 20, 64, 64, 512, 192, 10000, 0, 32, 3),    # three K blocks: boxes longer than the operand
+    (20, 20, 64, 64, 512, 1344, 3000, 1, 8, 3),     # twenty-one, nine of them in shared memory: one stage of 64 KB
 ])
 def test_large_vocabulary_kernel(pkg, B, T, D, E, P, H, V, act, W, S):  # noqa: F811
     w, enc, lens = ragged_case(1500 + B + P, B=B, T=T, D=D, E=E, P=P, L=1, H=H, V=V, act=act, blank_id=0 if B % 2 else None,
