@@ -1195,17 +1195,21 @@ static int cl_clusters() {
     return g_cl_clusters[dev] > 0 ? g_cl_clusters[dev] : 0;
 }
 
-// What a lock step costs, in us: of a cluster with all its slots, and of the other kernel with all its rows.  Fitted to 430 measured
-// pairs (P and H 128 to 640, 501 and 1025 labels, ReLU and tanh, W = 1 to 32, 29 to 600 utterances of equal and of ragged lengths):
-// 3, 8 and 8 % rms.  Chosen by these, a decode takes 0.7 % longer than by the better kernel of each pair on the average; with a
-// constant ratio, 2.1 and 3.2 for windows of 8 and 16 rows, and clusters alone beyond that or for up to 64 utterances, it took 11 %
-// (64 utterances of 120 frames at W = 32: 1.53 ms against 1.32; 128: 2.84 against 1.79; 64 at W = 24, P = H = 384: 1.31 against 0.89).
-// Two layers: 112 pairs (P and H 256 and 640, W = 1 to 32, up to 128 utterances), 8 and 6 % rms in clusters, 8 % for grid barriers.
+// What a lock step costs, in us: of a cluster with all its slots, and of the other kernel with all its rows.  Clusters: fitted to 104
+// steps of one layer (13 models: P and H 128 to 640, 500 and 1024 labels, ReLU and tanh; W = 1 to 32, every slot in use) and 68 of two
+// (9 models): 5.5 and 2.1 % rms for windows of up to 8 rows, 5.1 and 5.2 beyond, at most 19 off (tanh at W = 32 with few joint units).
+// Chosen by these, a decode takes 0.85 % longer than by the better kernel of each pair on the average where weights lie on the chip (961
+// pairs of one layer: 18 to 300 utterances of equal and of ragged lengths; 560 of two: 0.8 %), 1.7 % against streamed weights (235 pairs).
+// With the figures of earlier kernels, whose steps were 15 % longer, it took 1.7, 2.7 and 2.2 % longer (two layers, P = 640, H = 256, W = 1,
+// 41 utterances of 150 frames: 3.68 ms against 2.05).  What is lost most is a third: sizes where the joint of the other kernel fits well.
 static float cl_step_us(const wind_model_t& m, int W, int wp) {
-    const float P = (float)m.P, H = (float)m.H, z = m.act == WIND_ACT_RELU ? 0.f : 0.0018f * H;
-    if (m.L == 2) return z + (wp == 8 ? 5.6f + 0.0085f * P + (0.0044f * (float)W / 8.f - 0.004f) * H : 5.2f + 0.0073f * P + 0.0015f * H);
-    return z + (wp == 8 ? 4.3f + 0.0013f * P + (0.0009f + 0.0026f * (float)W / 8.f) * H : 4.25f + 0.0009f * P + 0.0028f * H);
+    const float P = (float)m.P, H = (float)m.H, NV = (float)(m.V + 1) / 1024.f, l = log2f((float)W), z = m.act == WIND_ACT_RELU ? 0.f : H;
+    if (m.L == 2) return wp == 8 ? 5.45f + 0.0023f * P + (0.0001f + 0.00124f * l + 0.00074f * NV) * H + 0.00013f * (float)W * z
+                                 : 5.65f + 0.0015f * P + (0.0028f + 0.0003f * NV) * H + 0.0014f * z;
+    return wp == 8 ? 3.3f + 0.0014f * P + (0.0017f + 0.00045f * l) * H + 0.23f * l + 0.00017f * (float)W * z
+                   : 3.77f + 0.0009f * P + 0.003f * H + 0.0015f * z;
 }
+// Other kernels: 430 pairs of one layer (8 % rms), 112 of two (8 %).
 static float other_step_us(const wind_model_t& m, const LoopPlan& pl, int B, int W) {
     const float P = (float)m.P, H = (float)m.H, rows = (float)B * (float)W;
     if (!pl.resident) return -2.5f + 3.8f * (float)pl.mt_count + 0.0053f * rows + 0.0177f * P + 0.0145f * H;

@@ -89,6 +89,28 @@ def test_which_kernel_decodes(pkg, B, W, T, lo, dim, want):  # noqa: F811
         assert np.array_equal(a, b)
 
 
+@pytest.mark.parametrize("L,B,W,T,lo,dim,want", [
+    (1, 36, 20, 150, 146, 384, "CLUSTERS"),     # three rounds of slots, and still ahead: 0.84 ms against 0.97
+    (1, 64, 12, 150, 146, 512, "CLUSTERS"),     # 0.82 against 0.97
+    (2, 41, 8, 150, 146, 640, "CLUSTERS"),      # one utterance more than slots: 0.94 against 1.28
+    (2, 128, 8, 60, 60, 512, "BARRIERS"),       # equal lengths: four rounds
+    (2, 128, 8, 60, 2, 512, "CLUSTERS"),        # ragged ones
+    (2, 64, 32, 60, 60, 128, "BARRIERS"),       # widest window: seven rounds
+])
+def test_which_kernel_decodes_near_the_line(pkg, L, B, W, T, lo, dim, want):  # noqa: F811
+    w, enc, _ = ragged_case(1970 + B + W + lo, B=B, T=T, D=64, E=64, P=dim, L=L, H=dim, V=200, bias=3.0, dtype="bf16")
+    lens = np.random.default_rng(B + lo).integers(lo, T + 1, size=B).astype(np.int32)
+    enc = np.nan_to_num(enc)
+    model = pkg.WindModel(w)
+    kernel, got = loop_kernel_of(pkg, model, enc, lens, W, 3)
+    assert kernel == getattr(pkg.binding, "WIND_LOOP_" + want)
+    set_loop_mode(pkg, "barriers")
+    kernel, ref = loop_kernel_of(pkg, model, enc, lens, W, 3)
+    assert kernel == pkg.binding.WIND_LOOP_BARRIERS
+    for a, b in zip(got, ref):
+        assert np.array_equal(a, b)
+
+
 @pytest.mark.parametrize("N,B,W,lo,want", [
     (384, 128, 16, 100, "BARRIERS"),        # rows refilled in the other kernel as well
     (300, 64, 8, 1, "CLUSTERS"),
