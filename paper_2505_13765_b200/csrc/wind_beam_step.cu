@@ -139,9 +139,9 @@ __device__ __forceinline__ unsigned long long bs_pair(uint32_t lo, uint32_t hi) 
 __device__ __forceinline__ void bs_fma_pair(unsigned long long& acc, unsigned long long a, unsigned long long b) {
     asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
-// four values from shared memory: loaded, as fp32
+// four values from shared memory: loaded, as fp32.  (volatile, or the compiler may take two loads for one, whatever barrier and stores lie between)
 template <typename TW> __device__ __forceinline__ void bs_four(uint32_t at, uint32_t* v) {
-    if constexpr (sizeof(TW) == 2) asm("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v[1]), "=r"(v[3]) : "r"(at));
+    if constexpr (sizeof(TW) == 2) asm volatile("ld.shared.v2.u32 {%0, %1}, [%2];" : "=r"(v[1]), "=r"(v[3]) : "r"(at));
     else asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];" : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3]) : "r"(at));
 }
 template <typename TW> __device__ __forceinline__ void bs_widen(uint32_t* v) {

@@ -193,6 +193,20 @@ def test_overlapped_kernels_read_nothing_by_ldg_behind_their_wait():
     assert kernels >= 2
 
 
+def test_loads_in_inline_assembly_are_volatile():
+    # Without that (and without a clobber) the compiler takes the statement for a function of its operands: a load may move over a barrier
+    # or be left out because the same address was loaded before.
+    csrc = os.path.join(ROOT, "paper_2505_13765_b200", "csrc")
+    loads = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for volatile, body in re.findall(r"\basm\s*(volatile)?\s*\((.*?)\);", text, flags=re.S):
+            if re.search(r'"[^"]*\b(ld|ldmatrix|atom|red|st)\.', body):
+                loads += 1
+                assert volatile, (name, body[:60])
+    assert loads > 25
+
+
 @pytest.mark.parametrize("kw,W,K,S,rows", [
     (dict(), 8, 4, 10, 16),                       # evaluates ahead: sixteen hypotheses a command
     (dict(), 8, 1, 10, 0),                        # nothing to evaluate ahead
