@@ -1,13 +1,14 @@
-// The decoding loop of the bf16 path for one-layer models whose decoder fits one thread-block cluster (sm_100a).
+// The decoding loop of the bf16 path for models of one or two layers whose decoder fits one thread-block cluster (sm_100a).
 //
 // A lock step is a chain of small dependent products, so what it costs is the latency of handing results from SM to SM.
 // Here every hand-over stays inside a cluster of 16 CTAs (st.async into distributed shared memory: about 0.25 us) instead of
 // going through L2 (a barrier over the chip alone is 1.3 us), and clusters share nothing but the queue of utterances.
 //
 // All weights of the loop stay on chip, cut over the 16 CTAs of a cluster (large model: 5.4 MB; a CTA holds 340 KB):
-//   tensor memory   W_hh rows of the CTA's first 32 hidden units (4 gates x 32 = the 128 lanes), operand A of the gates' MMA
+//   tensor memory   W_hh rows of the CTA's first 32 hidden units (4 gates x 32 = the 128 lanes), operand A of the gates' MMA; with two
+//                   layers the second one's W_ih (two more clusters hold W_hh, one a layer, for up to CL_DECODERS that decode: cl_recurrent)
 //   shared memory   W_out rows of its 1/16 of the vocabulary
-//   registers       W_pred rows of its 1/16 of the joint's hidden units and W_hh rows of its remaining hidden units, as
+//   registers       W_pred rows of its 1/16 of the joint's hidden units and W_hh (W_ih) rows of its remaining hidden units, as
 //                   mma.sync fragments (no register may be spilled: next to 220 KB of shared memory there is no first-
 //                   level cache left, and a spilled value comes from L2)
 // A cluster decodes up to 8 utterances ("slots") at a time; a lock step of a cluster is
@@ -16,7 +17,8 @@
 //           enc_proj rows start on their way (one TMA box per eight rows, in the layout of the joint's operand)
 //   (a step in which no slot feeds a token to its decoder goes from here to the joint, and only slots that do send anything in
 //   the next two phases: most steps of narrow windows emit nothing)
-//   gates   W_hh h was computed a step ahead; + the token's row of the gate table, cell update, new h to every CTA
+//   gates   W_hh h was computed a step ahead; + the token's row of the gate table, cell update, new h to every CTA (the second layer:
+//           W_ih times that, + its W_hh h, computed meanwhile in another cluster)
 //   pred    W_pred h, pred_proj to every CTA
 //   joint   z = act(enc_proj rows + pred_proj) in place, times the CTA's W_out rows on tcgen05 (window rows on the M axis, so
 //           that an accumulator lane is a window row and its argmax needs no exchange between lanes)
@@ -44,12 +46,13 @@ struct ClDec { int tok; uint32_t flags, row, unused; };   // what an owner sends
 constexpr uint32_t CL_FRESH = 1u, CL_IDLE = 2u, CL_ODD = 4u;   // CL_ODD: parity of the step it is for
 
 // W_hh (or the second layer's W_ih) rows of the CTA's hidden units 0..31 into tensor memory: lane 4 u + gate.  Warps 0-7.
+// AT_ONCE pieces are under way: five make short decodes of two layers 0.6 % faster; with one layer the registers they take lengthen every
+// step of several slots (128 utterances 8.61 -> 8.69 ms, 32 at W = 1 5.67 -> 5.71, one slot the same).
+template <int AT_ONCE>
 __device__ __forceinline__ void cl_gate_rows_to_tmem(const __nv_bfloat16* w, int P, int r, int warp, int lane, uint32_t tmem) {
     const int q = warp & 3, U = P / CL_SIZE, u = 8 * q + (lane >> 2), g = lane & 3;
     const bool in = u < U;
     const uint4* src = reinterpret_cast<const uint4*>(w + ((size_t)g * P + r * U + (in ? u : 0)) * P);
-    // (five pieces under way: one at a time the ten of them took ten round trips)
-    constexpr int AT_ONCE = 5;
 #pragma unroll 1
     for (int c0 = 16 * (warp >> 2); c0 < P / 2; c0 += 32 * AT_ONCE) {
         uint32_t v[AT_ONCE][16];
@@ -102,7 +105,7 @@ __device__ __noinline__ void cl_recurrent(const CUtensorMap& hx_map, const ClPar
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem = __shfl_sync(0xffffffffu, tmem_slot, 0);
-    if (warp < 8) cl_gate_rows_to_tmem(p.w_rec[layer], p.P, r, warp, lane, tmem);
+    if (warp < 8) cl_gate_rows_to_tmem<5>(p.w_rec[layer], p.P, r, warp, lane, tmem);
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
@@ -362,7 +365,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     const uint32_t tm_g = tmem + CL_MAX_DIM / 2, tm_j = tm_g + 32, tm_j2 = tm_j + 80;   // gates: 16 columns; joint: two copies of up to 72
     const int q = warp & 3;                                                       // lane quadrant
     const uint32_t lane_off = (uint32_t)(q * 32) << 16;
-    if (warp < 8) cl_gate_rows_to_tmem(p.w_gate, p.P, r, warp, lane, tmem);
+    if (warp < 8) cl_gate_rows_to_tmem<NL == 2 ? 5 : 1>(p.w_gate, p.P, r, warp, lane, tmem);
     asm volatile("cp.async.wait_all;" ::: "memory");
     fence_proxy_async();
     tc_fence_before();
@@ -381,7 +384,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     // 350 of 8500.  Another CTA may be an update ahead by then, so there are two copies of the state, by parity of the updates (one more
     // update needs this CTA's h, and that this product).  With more slots a copy would lack the state of slots that sat an update out,
     // and from four on the joint's operand takes longer than the product.
-    // One utterance of 100 s 2.20 -> 2.11 ms, seven short ones 0.683 -> 0.648.
+    // One utterance of 100 s 2.10 -> 2.00 ms, seven short ones 0.595 -> 0.567.
     const bool late = NS == 1 && cl_gates_late(NU, NL);
     const uint32_t h_copy = late ? (uint32_t)kb_p * H_BLOCK : 0u;
     const uint32_t h_row = sbase + L.h + (uint32_t)((lane & 7) * 128);
@@ -391,7 +394,7 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     // memory's bandwidth, so a 16-byte piece of pred_proj is loaded once for several window rows: a unit of work is eight threads, a
     // piece each of a K block, and p.z_rows of the rows of a group that count; units are dealt out evenly to all groups of eight threads.
     // (Eight slots, W = 8: 22 KB per group of eight rows; with pred_proj loaded for every row and rows dealt out by role it was 30 KB:
-    // 128 utterances 9.04 -> 7.82 ms, 32 at W = 1 6.10 -> 5.54; one slot the same.)
+    // 128 utterances 9.75 -> 8.63 ms, 32 at W = 1 6.07 -> 5.65; one slot the same.)
     const int z_rows = p.wp == 8 ? p.W : 8;
     const int z_first = (int)(threadIdx.x >> 3) / kb_h << 8 | (int)(threadIdx.x >> 3) % kb_h;    // (group, part) << 8 | K block
     auto build_z = [&](auto which) {
@@ -425,46 +428,80 @@ __global__ void __launch_bounds__(CL_THREADS, 1) cl_kernel(const __grid_constant
     };
 
     // Argmax of every window row over a share of this CTA's labels (HF), sent to the slots' owners.  With M = 64 accumulator row m
-    // lives in lane m % 16 of quadrant m / 16.  Read as 16 lanes x 256 bits, a thread holds a quarter of the columns of rows lane / 4 and
-    // lane / 4 + 8, so that all 32 threads have something to compare (a row a thread: 16 threads, four times the chain; 1008 -> 865
-    // cycles with eight slots, 995 -> 826 with one, of which a step keeps 195 and 33: the keys of the W_pred warps come last).
+    // lives in lane m % 16 of quadrant m / 16.
     auto joint_argmax = [&](auto which) {
         constexpr int HF = decltype(which)::value;
         const int rows_here = (NU << wp_shift) - 16 * q;              // window rows of this warp's quadrant
         if (rows_here <= 0) return;
         constexpr int CH = HF ? 8 : 16;                                 // columns at a time (the W_pred warps have registers for eight)
         const int nh = (lab_n / 3) & ~7;                                // they take [0, nh), the workers [nh, lab_n)
-        float best[2] = {-INFINITY, -INFINITY};
-        int lab[2] = {0, 0};
+        unsigned long long key;
+        int row;
+        bool mine;                                                      // this thread has the key of a row
+        if constexpr (NS <= NL) {
+            // Read as 16 lanes x 256 bits, a thread holds a quarter of the columns of rows lane / 4 and lane / 4 + 8, so that all 32 threads
+            // have something to compare, and the exchanges at the end are few.  One utterance of 100 s 2.05 -> 2.00 ms, seven short ones 0.585 -> 0.572,
+            // two layers with two slots 1.552 -> 1.540.
+            float best[2] = {-INFINITY, -INFINITY};
+            int lab[2] = {0, 0};
 #pragma unroll 1
-        for (int c = HF ? 0 : nh; c < (HF ? nh : lab_n); c += CH) {
-            float v[CH / 2];                                            // of eight columns each: row lane / 4 twice, row lane / 4 + 8 twice
-            tmem_ld_quarter<CH / 8>(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
+            for (int c = HF ? 0 : nh; c < (HF ? nh : lab_n); c += CH) {
+                float v[CH / 2];                                        // of eight columns each: row lane / 4 twice, row lane / 4 + 8 twice
+                tmem_ld_quarter<CH / 8>(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
 #pragma unroll
-            for (int j = 0; j < CH / 8; ++j) {
-                const int at = c + 8 * j + 2 * (lane & 3);
-                const float2 b2 = *reinterpret_cast<const float2*>(s_bout + at);     // -inf behind the last label
+                for (int j = 0; j < CH / 8; ++j) {
+                    const int at = c + 8 * j + 2 * (lane & 3);
+                    const float2 b2 = *reinterpret_cast<const float2*>(s_bout + at); // -inf behind the last label
 #pragma unroll
-                for (int k = 0; k < 2; ++k) {                           // equal logits: the lower label stays
-                    const float v0 = v[4 * j + 2 * k] + b2.x, v1 = v[4 * j + 2 * k + 1] + b2.y;
-                    if (v0 > best[k]) { best[k] = v0; lab[k] = at; }
-                    if (v1 > best[k]) { best[k] = v1; lab[k] = at + 1; }
+                    for (int k = 0; k < 2; ++k) {                       // equal logits: the lower label stays
+                        const float v0 = v[4 * j + 2 * k] + b2.x, v1 = v[4 * j + 2 * k + 1] + b2.y;
+                        if (v0 > best[k]) { best[k] = v0; lab[k] = at; }
+                        if (v1 > best[k]) { best[k] = v1; lab[k] = at + 1; }
+                    }
                 }
             }
-        }
-        unsigned long long key[2];
+            unsigned long long keys[2];
 #pragma unroll
-        for (int k = 0; k < 2; ++k) {
-            key[k] = best[k] > -INFINITY ? pack_key(best[k], (uint32_t)(lab0 + lab[k])) : 0ull;
-            if (k == 0 || rows_here > 8) {
-                key[k] = max(key[k], __shfl_xor_sync(0xffffffffu, key[k], 1));
-                key[k] = max(key[k], __shfl_xor_sync(0xffffffffu, key[k], 2));
+            for (int k = 0; k < 2; ++k) {
+                keys[k] = best[k] > -INFINITY ? pack_key(best[k], (uint32_t)(lab0 + lab[k])) : 0ull;
+                if (k == 0 || rows_here > 8) {
+                    keys[k] = max(keys[k], __shfl_xor_sync(0xffffffffu, keys[k], 1));
+                    keys[k] = max(keys[k], __shfl_xor_sync(0xffffffffu, keys[k], 2));
+                }
             }
+            key = lane & 1 ? keys[1] : keys[0];
+            row = 16 * q + (lane >> 2) + 8 * (lane & 1);                // lanes 4 i: row i, 4 i + 1: row i + 8
+            mine = (lane & 2) == 0;
+        } else {
+            // A row a thread.  (Spread over the warp as above, steps of several slots took 5 % longer: 128 utterances 8.60 -> 9.04 ms, 32 at W = 1
+            // 5.68 -> 5.94, two layers, 64 utterances, 12.77 -> 13.01.)  CH columns at a time: their maximum, then the lowest label that has it.
+            float best = -INFINITY;
+            int lab = 0;
+#pragma unroll 1
+            for (int c = HF ? 0 : nh; c < (HF ? nh : lab_n); c += CH) {
+                float v[CH];
+                if constexpr (CH == 16) tmem_ld16_sum(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
+                else tmem_ld8_sum(tm_j + lane_off + (uint32_t)c, tm_j2 + lane_off + (uint32_t)c, v);
+#pragma unroll
+                for (int j = 0; j < CH; j += 4) {
+                    const float4 b4 = *reinterpret_cast<const float4*>(s_bout + c + j);  // -inf behind the last label
+                    v[j] += b4.x; v[j + 1] += b4.y; v[j + 2] += b4.z; v[j + 3] += b4.w;
+                }
+                float m = v[0];
+#pragma unroll
+                for (int j = 1; j < CH; ++j) m = fmaxf(m, v[j]);
+                int at = CH;
+#pragma unroll
+                for (int j = CH - 1; j >= 0; --j) at = v[j] == m ? j : at;
+                if (m > best) { best = m; lab = c + at; }
+            }
+            key = best > -INFINITY ? pack_key(best, (uint32_t)(lab0 + lab)) : 0ull;
+            row = 16 * q + (lane & 15);
+            mine = lane < 16;
         }
-        const int row = 16 * q + (lane >> 2) + 8 * (lane & 1);          // lanes 4 i: row i, 4 i + 1: row i + 8
         const int s = row >> wp_shift, w = row & (p.wp - 1);
-        if ((lane & 2) == 0 && s < NU && w < p.W)
-            st_async_8(cl_map(sbase + L.kbuf + (uint32_t)(w * CL_KEY_PITCH + 2 * r + HF) * 8u, s), lane & 1 ? key[1] : key[0], cl_map(smem_u32(&bar_keys), s));
+        if (mine && s < NU && w < p.W)
+            st_async_8(cl_map(sbase + L.kbuf + (uint32_t)(w * CL_KEY_PITCH + 2 * r + HF) * 8u, s), key, cl_map(smem_u32(&bar_keys), s));
     };
 
     if (warp < 4) {
@@ -1198,10 +1235,11 @@ static int cl_clusters() {
 // What a lock step costs, in us: of a cluster with all its slots, and of the other kernel with all its rows.  Clusters: fitted to 104
 // steps of one layer (13 models: P and H 128 to 640, 500 and 1024 labels, ReLU and tanh; W = 1 to 32, every slot in use) and 68 of two
 // (9 models): 5.5 and 2.1 % rms for windows of up to 8 rows, 5.1 and 5.2 beyond, at most 19 off (tanh at W = 32 with few joint units).
-// Chosen by these, a decode takes 0.85 % longer than by the better kernel of each pair on the average where weights lie on the chip (961
-// pairs of one layer: 18 to 300 utterances of equal and of ragged lengths; 560 of two: 0.8 %), 1.7 % against streamed weights (235 pairs).
-// With the figures of earlier kernels, whose steps were 15 % longer, it took 1.7, 2.7 and 2.2 % longer (two layers, P = 640, H = 256, W = 1,
-// 41 utterances of 150 frames: 3.68 ms against 2.05).  What is lost most is a third: sizes where the joint of the other kernel fits well.
+// One layer's figures stand 2 to 7 % above its steps of today.  Chosen by these, a decode takes 1.1 % longer than by the better kernel of each
+// pair on the average where weights lie on the chip (961 pairs of one layer: 18 to 300 utterances of equal and of ragged lengths; 560 of
+// two: 0.8 %), 1.5 % against streamed weights (235 pairs); with 5 % less for one layer 0.6 and 1.7 %, but batches of the choice's tests
+// would change sides.  With the figures of earlier kernels, 15 to 20 % above, two layers took 2.7 % longer (P = 640, H = 256, W = 1, 41
+// utterances of 150 frames: 3.68 ms against 2.05).  What is lost most is 46 %: sizes where the joint of the other kernel fits well.
 static float cl_step_us(const wind_model_t& m, int W, int wp) {
     const float P = (float)m.P, H = (float)m.H, NV = (float)(m.V + 1) / 1024.f, l = log2f((float)W), z = m.act == WIND_ACT_RELU ? 0.f : H;
     if (m.L == 2) return wp == 8 ? 5.45f + 0.0023f * P + (0.0001f + 0.00124f * l + 0.00074f * NV) * H + 0.00013f * (float)W * z
