@@ -14,9 +14,9 @@
 //
 // An iteration waits for the one before it, but what it evaluates (a token history at a frame) rarely depends on that one: most
 // hypotheses of the next frames' lists are there long before their turn.  So a command of the resident kernel is filled up with the
-// histories that the following iterations will most likely ask for (struct Ahead), and an iteration whose hypotheses have all been
+// histories that the following iterations will most likely ask for (struct Forecast), and an iteration whose hypotheses have all been
 // evaluated needs no command.  What is evaluated is the same, in the same precision and summation order; only the guess when is not,
-// and a wrong one costs a row.  Beam 4, W = 8: 1.02 evaluations per one needed, 0.4 commands per iteration.
+// and a wrong one costs a row.  Beam 4, W = 8: 1.03 evaluations per one needed, 0.33 commands per iteration.
 #if defined(__x86_64__)
 #include <immintrin.h>
 #endif
